@@ -170,25 +170,32 @@ def phi_kernel_figure(kv, w, device, stream, sms, regimes=16, reps=2):
 
 def secondary_figures(kv, w, ctx, stream, sms, reps=2):
     """Beside the headline, outside its timed region, on the context that holds the workload's
-    samples: the native FP64 per-term kernel on the first regime (a full FP64 pass takes about
-    1000 s), and the two modes that are not per term -- the envelope sums and the exact dual over
+    samples: the native FP64 per-term kernel on the first regime (a full pass of it takes about
+    1000 s; the support is declared as 2^22 + 1, which is what routes FP64 requests to it), and the
+    two modes that are not per term -- the envelope sums and the exact dual over
     gamma >= 0 -- on the whole workload, in cells/s."""
     import torch
 
     M, E, K, R, NL = len(w.cp), len(w.eps), w.K, len(w.r), len(w.lam)
     dev = torch.device("cuda", torch.cuda.current_device())
 
-    def timed(fn):
+    def timed(fn, on=None):
         ms = []
         for i in range(reps + 1):
             fn()
             if i:
-                ms.append(kv.kvdro_last_grid_ms(ctx))
+                ms.append(kv.kvdro_last_grid_ms(on or ctx))
         return statistics.mean(ms)
 
     r1 = torch.empty((1, E, K), dtype=torch.int32, device=dev)
-    fp64_ms = timed(lambda: kv.kvdro_eval_grid(ctx, kv.KVDRO_FP64, R, w.r, NL, w.lam, E, w.eps, 1, w.cp[:1],
-                                               w.cw[:1], r_idx=r1, stream=stream))
+    big = kv.kvdro_create(dev.index)
+    try:
+        kv.kvdro_load_samples(big, K, w.offsets, torch.from_numpy(w.samples).to(dev), np.full(K, (1 << 22) + 1, np.int32),
+                              w.L_in, stream)
+        fp64_ms = timed(lambda: kv.kvdro_eval_grid(big, kv.KVDRO_FP64, R, w.r, NL, w.lam, E, w.eps, 1, w.cp[:1],
+                                                   w.cw[:1], r_idx=r1, stream=stream), big)
+    finally:
+        kv.kvdro_destroy(big)
     fp64_terms = R * NL * int(w.N.sum())
     fp64_rate = fp64_terms / (fp64_ms / 1e3)
     fp64_peak = sms * FP64_TERMS_PER_CLK_PER_SM * SM_MAX_MHZ_RECIPE * 1e6
@@ -197,7 +204,8 @@ def secondary_figures(kv, w, ctx, stream, sms, reps=2):
                                               r_idx=r_all, stream=stream))
     dual_ms = timed(lambda: kv.kvdro_eval_dual(ctx, R, w.r, E, w.eps, M, w.cp, w.cw, r_idx=r_all, stream=stream))
     return {"fp64_per_term": {"kernel": "k_grid<F64>: per term one DFMA, one max.f64, one DADD",
-                              "workload": f"{w.name}, first regime ({fp64_terms:.4g} terms)", "kernel_ms": fp64_ms,
+                              "workload": f"{w.name}, first regime ({fp64_terms:.4g} terms), support declared "
+                                          f"as 2^22 + 1", "kernel_ms": fp64_ms,
                               "achieved": fp64_rate, "unit": UNIT, "peak": fp64_peak, "frac": fp64_rate / fp64_peak,
                               "peak_basis": f"{sms} SMs x {FP64_TERMS_PER_CLK_PER_SM:.3f} terms/clk/SM (measured FP64 "
                                             f"pipe rates: 2.0 DFMA, 1.7 DADD / max.f64 per clk per SM) x "
@@ -528,7 +536,6 @@ def run_suite(args):
     dev = torch.device("cuda", 0)
     props = torch.cuda.get_device_properties(dev)
     peak32 = props.multi_processor_count * TERMS_PER_CLK_PER_SM * SM_MAX_MHZ_RECIPE * 1e6
-    peak64 = props.multi_processor_count * FP64_TERMS_PER_CLK_PER_SM * SM_MAX_MHZ_RECIPE * 1e6
     names = {kv.KVDRO_FP32: "fp32", kv.KVDRO_FP64: "fp64", kv.KVDRO_EXACT: "exact"}
     # bring the clocks up before the first measurement: a few seconds of the FP32 grid kernel
     warm = WORKLOADS["lognormal_k8_n1e5"]()
@@ -553,7 +560,7 @@ def run_suite(args):
         load_ms = (time.perf_counter() - t0) * 1e3
         for prec in precs:
             r_idx = torch.empty((M, E, K), dtype=torch.int32, device=dev)
-            reps = 1 if (prec == kv.KVDRO_FP64 or w.terms() > 1e13) else 3
+            reps = 1 if w.terms() > 1e13 else 3
             kv.kvdro_eval_grid(ctx, prec, R, w.r, NL, w.lam, E, w.eps, M, w.cp, w.cw, r_idx=r_idx)
             ms = []
             for _ in range(reps):
@@ -561,9 +568,8 @@ def run_suite(args):
                 ms.append(kv.kvdro_last_grid_ms(ctx))
             grid_ms = float(np.median(ms))
             rate = w.terms() / (grid_ms / 1e3)
-            peak = peak64 if prec == kv.KVDRO_FP64 else peak32
             print(json.dumps({"suite": True, "workload": w.name, "precision": names[prec], "terms": w.terms(),
-                              "grid_ms": grid_ms, "terms_per_s": rate, "peak": peak, "frac": rate / peak,
+                              "grid_ms": grid_ms, "terms_per_s": rate, "peak": peak32, "frac": rate / peak32,
                               "load_sort_ms_wall": load_ms}), flush=True)
         # not per term: the envelope mode (cells/s) and the exact dual over gamma ((m, e, k, r) cells/s)
         for mode, label in ((kv.KVDRO_ENVELOPE, "envelope"), ("dual", "dual")):

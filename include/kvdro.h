@@ -58,7 +58,9 @@ typedef enum {
     KVDRO_FP32 = 0,      /* FP32 outputs.  When every L_max <= 2^22 they are the KVDRO_EXACT
                             results rounded to FP32 (the exact kernel is also the fastest);
                             otherwise per-term arithmetic in FP32 with sums folded into FP64 */
-    KVDRO_FP64 = 1,      /* per-term arithmetic and sums in FP64 */
+    KVDRO_FP64 = 1,      /* FP64 outputs.  When every L_max <= 2^22 (and no cost times a class's
+                            L_max * N passes 1e300) they are the KVDRO_EXACT results, whose sums
+                            carry no rounding; otherwise per-term arithmetic and sums in FP64 */
     KVDRO_EXACT = 2,     /* per term, exact integer arithmetic on exact integer thresholds
                             (|x + 1 - t| summed exactly, half of the cells in packed FP32 adds,
                             half in integer absolute differences); exact integer counts and
@@ -112,7 +114,7 @@ int kvdro_quantiles(kvdro_ctx* ctx, int32_t F, const double* fractiles, int32_t*
  *   R, r       host int32[R], 1 <= R <= 2^20; every r must satisfy L_in_k <= r <= L_in_k + L_k for
  *              every class (the reservation domain of Sec. 2.2).
  *   NL, lam    host double[NL], finite, >= 0; 1 <= NL <= 256 (128 for KVDRO_FP64).  The exact
- *              kernel (KVDRO_EXACT, and KVDRO_FP32 when every L_max <= 2^22) takes 128 lam values
+ *              kernel (KVDRO_EXACT, and FP32 and FP64 as above) takes 128 lam values
  *              per launch; a larger grid runs as consecutive launches over blocks of 128 with the
  *              running minimum in context scratch (12 bytes per (regime, eps, class, r), at most
  *              256 MB at a time).

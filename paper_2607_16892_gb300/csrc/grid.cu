@@ -20,7 +20,7 @@
 //    multiply-add, one max and one add per sample and cell.  FP32: one saturating fused
 //    multiply-add on the excess scaled by a power of two (the clamp to [0, 1] is the max) and half
 //    a packed add per sample and cell.
-//  - EXACT (also FP32 requests whose supports are all <= 2^22): each cell's integer threshold t
+//  - EXACT (also FP32 and FP64 requests whose supports are all <= 2^22): each cell's integer threshold t
 //    (x >= t exactly when kappa x + d > 0), then per term the exact sum of |x + 1 - t|, half of a
 //    warp's cells on packed FP32 adds and half on integer absolute differences, so the FMA and ALU
 //    pipes work side by side; the epilogue puts every sample on its own branch (branch_sum).

@@ -105,7 +105,7 @@ def test_heavy_tail_k16_n1e6_exact_full_grid():
 
 
 def test_lognormal_k8_n1e5_fp64_full_grid():
-    """Native FP64 arithmetic per term on every cell of the 8-class grid (4096 r x 128 lam)."""
+    """FP64 requests on every cell of the 8-class grid (4096 r x 128 lam)."""
     w = lognormal_workload_k8_n1e5()
     gpu = run(w, kvdro.KVDRO_FP64)
     rep = compare_full(w, gpu, oracle_from_S(w, O.envelope_grid(w)), "fp64")
