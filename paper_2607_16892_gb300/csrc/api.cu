@@ -58,10 +58,12 @@ struct kvdro_ctx {
     cudaStream_t last_stream = nullptr;
 
     bool loaded = false;
+    bool pair_sums = false;  // the staged form of the loaded samples
     int32_t K = 0;
     int64_t total = 0, pair_total = 0, hist_total = 0;
     std::vector<int64_t> off, pair_off, hist_off, N;
     std::vector<int32_t> L, Lin, hist_blocks, exp_blocks;
+    std::vector<double> inv_n;
 
     Buf sorted, pairs, hist, csum, sumx, meta, errs, in_stage, grid_in, keys, cost64, out_stage, ranks, scan_tot, part,
         tile_lo;
@@ -76,6 +78,7 @@ struct kvdro_ctx {
 
     // device views into `meta`
     int64_t *d_off = nullptr, *d_pair_off = nullptr, *d_hist_off = nullptr, *d_N = nullptr;
+    double* d_inv_n = nullptr;
     int32_t *d_L = nullptr, *d_Lin = nullptr, *d_hist_blocks = nullptr, *d_exp_blocks = nullptr;
 };
 
@@ -316,6 +319,7 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     ctx->K = K;
     ctx->off.assign(offsets, offsets + K + 1);
     ctx->N.resize(K);
+    ctx->inv_n.resize(K);
     ctx->L.assign(L_max, L_max + K);
     ctx->Lin.assign(K, 0);
     if (L_in) ctx->Lin.assign(L_in, L_in + K);
@@ -327,6 +331,7 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
         const int64_t n = offsets[k + 1] - offsets[k];
         const int64_t padn = (int64_t)align_up((size_t)n, kvdro::kPadSamples);
         ctx->N[k] = n;
+        ctx->inv_n[k] = 1.0 / (double)n;
         ctx->pair_off[k + 1] = ctx->pair_off[k] + padn;
         ctx->hist_off[k + 1] = ctx->hist_off[k] + (int64_t)L_max[k] + 1;
         const int64_t hb = ctx->hist_blocks[k] + (n + slice - 1) / slice;
@@ -344,17 +349,18 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
 
     int rc;
     if ((rc = ensure(ctx, ctx->sorted, (size_t)ctx->total * 4))) return rc;
-    if ((rc = ensure(ctx, ctx->pairs, (size_t)ctx->pair_total * 8))) return rc;
+    int32_t max_L = 0;
+    for (int32_t k = 0; k < K; k++) max_L = std::max(max_L, L_max[k]);
+    ctx->pair_sums = max_L <= kvdro::kPairMaxL;
+    if ((rc = ensure(ctx, ctx->pairs, (size_t)ctx->pair_total * (ctx->pair_sums ? 4 : 8)))) return rc;
     if ((rc = ensure(ctx, ctx->hist, (size_t)ctx->hist_total * 4))) return rc;
     if ((rc = ensure(ctx, ctx->csum, (size_t)ctx->hist_total * 8))) return rc;
     if ((rc = ensure(ctx, ctx->sumx, (size_t)K * 8))) return rc;
     if ((rc = ensure(ctx, ctx->errs, 2 * sizeof(int32_t)))) return rc;
-    int64_t max_bins = 0;
-    for (int32_t k = 0; k < K; k++) max_bins = std::max<int64_t>(max_bins, (int64_t)L_max[k] + 1);
-    const int64_t scan_tiles = (max_bins + kvdro::scan_tile_bins() - 1) / kvdro::scan_tile_bins();
+    const int64_t scan_tiles = ((int64_t)max_L + 1 + kvdro::scan_tile_bins() - 1) / kvdro::scan_tile_bins();
     if ((rc = ensure(ctx, ctx->scan_tot, (size_t)K * scan_tiles * 16))) return rc;
     if ((rc = ensure(ctx, ctx->tile_lo, ((size_t)ctx->exp_blocks[K] + K) * 4))) return rc;
-    const size_t meta_bytes = (size_t)(K + 1) * 8 * 3 + (size_t)K * 8 + (size_t)K * 4 * 2 + (size_t)(K + 1) * 4 * 2 + 64;
+    const size_t meta_bytes = (size_t)(K + 1) * 8 * 3 + (size_t)K * 8 * 2 + (size_t)K * 4 * 2 + (size_t)(K + 1) * 4 * 2 + 64;
     if ((rc = ensure(ctx, ctx->meta, meta_bytes))) return rc;
 
     // Metadata upload (one copy from pinned staging).
@@ -372,6 +378,7 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     put(ctx->pair_off.data(), (K + 1) * 8, reinterpret_cast<void**>(&ctx->d_pair_off));
     put(ctx->hist_off.data(), (K + 1) * 8, reinterpret_cast<void**>(&ctx->d_hist_off));
     put(ctx->N.data(), K * 8, reinterpret_cast<void**>(&ctx->d_N));
+    put(ctx->inv_n.data(), K * 8, reinterpret_cast<void**>(&ctx->d_inv_n));
     put(ctx->L.data(), K * 4, reinterpret_cast<void**>(&ctx->d_L));
     put(ctx->Lin.data(), K * 4, reinterpret_cast<void**>(&ctx->d_Lin));
     put(ctx->hist_blocks.data(), (K + 1) * 4, reinterpret_cast<void**>(&ctx->d_hist_blocks));
@@ -402,10 +409,12 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     a.csum = static_cast<int64_t*>(ctx->csum.p);
     a.sumx = static_cast<int64_t*>(ctx->sumx.p);
     a.sorted = static_cast<int32_t*>(ctx->sorted.p);
-    a.pairs = static_cast<float2*>(ctx->pairs.p);
+    a.staged = ctx->pairs.p;
+    a.pair_sums = ctx->pair_sums;
     a.err = static_cast<int32_t*>(ctx->errs.p);
     a.tile_tot = static_cast<int64_t*>(ctx->scan_tot.p);
     a.tile_lo = static_cast<int32_t*>(ctx->tile_lo.p);
+    a.inv_n = nullptr;  // part of the metadata uploaded above
     a.scan_tiles = (int32_t)scan_tiles;
     a.K = K;
     KV_CUDA(kvdro::launch_histogram(a, ctx->hist_blocks[K], s), "histogram kernel");
@@ -586,9 +595,11 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     KV_CUDA(cudaMemsetAsync(ctx->keys.p, 0xFF, (size_t)rows * 8, s), "clearing argmin keys");
 
     kvdro::GridArgs a;
-    a.pairs = static_cast<const float2*>(ctx->pairs.p);
+    a.staged = ctx->pairs.p;
+    a.pair_sums = ctx->pair_sums;
     a.pair_off = ctx->d_pair_off;
     a.N = ctx->d_N;
+    a.inv_n = ctx->d_inv_n;
     a.sumx = static_cast<const int64_t*>(ctx->sumx.p);
     a.L = ctx->d_L;
     a.L_in = ctx->d_Lin;
@@ -792,6 +803,7 @@ int kvdro_eval_dual(kvdro_ctx* ctx, int32_t R, const int32_t* r, int32_t E, cons
     a.csum = static_cast<const int64_t*>(ctx->csum.p);
     a.hist_off = ctx->d_hist_off;
     a.N = ctx->d_N;
+    a.inv_n = ctx->d_inv_n;
     a.sumx = static_cast<const int64_t*>(ctx->sumx.p);
     a.L = ctx->d_L;
     a.L_in = ctx->d_Lin;

@@ -44,7 +44,7 @@ __device__ __forceinline__ void split_at(const ClassView& c, double eta, double 
                                          double& nu, int64_t& cnt, int64_t& sum) {
     mu = fmin(gam, cp);
     nu = fmin(gam, cw);
-    tail(c, first_active(mu + nu, excess_offset(cp, cw, mu, (double)c.L, eta), c.L), cnt, sum);
+    tail(c, first_active(mu + nu, excess_offset(row_offset(cp, cw, c.L, (int)eta), cp, mu, (double)c.L), c.L), cnt, sum);
 }
 
 // Sign of the right derivative of g at gamma, eps - (nu' sum_{x < t} x + mu' sum_{x >= t} (L - x)) / N
@@ -68,7 +68,7 @@ __device__ __forceinline__ double value_at(const ClassView& c, double eta, doubl
     int64_t cnt, sum;
     split_at(c, eta, cp, cw, gam, mu, nu, cnt, sum);
     const int64_t below = c.sumx - sum, dist = (int64_t)c.L * cnt - sum;
-    return gam * eps + branch_sum(cp, cw, mu, nu, (double)c.L, eta, (double)c.N, cnt, below, dist) * inv_n;
+    return gam * eps + branch_sum(cp, cw, mu, nu, c.L, (int)eta, c.N, cnt, below, dist) * inv_n;
 }
 
 __global__ void __launch_bounds__(kDualThreads) k_dual(const DualArgs a) {

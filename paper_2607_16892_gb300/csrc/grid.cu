@@ -21,9 +21,9 @@
 //    multiply-add on the excess scaled by a power of two (the clamp to [0, 1] is the max) and half
 //    a packed add per sample and cell.
 //  - EXACT (also FP32 and FP64 requests whose supports are all <= 2^22): each cell's integer threshold t
-//    (x >= t exactly when kappa x + d > 0), then per term the exact sum of |x + 1 - t|, half of a
-//    warp's cells on packed FP32 adds and half on integer absolute differences, so the FMA and ALU
-//    pipes work side by side; the epilogue puts every sample on its own branch (branch_sum).
+//    (x >= t exactly when kappa x + d > 0), then the exact sum of |x + 1 - t|, two samples at a time in
+//    packed FP32 adds and a max (or, above a support of 2^19, one at a time in integer absolute
+//    differences); the epilogue puts every sample on its own branch (branch_sum).
 //  - ENVELOPE (k_envelope): the same branch sums from the cumulative counts and sums, O(1) per
 //    cell, not per term.
 //
@@ -62,43 +62,43 @@ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 // multipliers, TR*TL a power of two <= 32), FP32 chunks between folds of the per-lane partial
 // sums into FP64 (FP64 folds once at the end), the largest CTA and minimum CTAs per SM it is
 // compiled for (these two bound its registers per thread), the staged chunk and ring depth, the
-// sample loop's unroll, and (exact) the lam columns per row on packed FP32 adds.
+// sample loop's unroll, and (exact) whether it reads pair sums.
 template <Prec P_, int TR_, int TL_, int FLUSH_, int MINB_, int MAXT_ = 512, int CHUNK_ = 2048, int STAGES_ = 3,
-          int UNROLL_ = 2, int FCOLS_ = TL_ / 2>
+          int UNROLL_ = 2, bool PAIR_ = false>
 struct GridCfg {
-    static constexpr int FCOLS = FCOLS_;
+    static constexpr bool PAIR = PAIR_;
     static constexpr Prec P = P_;
     static constexpr int TR = TR_, TL = TL_, V = TR_ * TL_, LOG2V = ilog2(TR_ * TL_), FLUSH = FLUSH_, MINB = MINB_;
     static constexpr int MAXT = MAXT_;
-    static constexpr int CHUNK = CHUNK_;    // samples per staged chunk (float2 each)
-    static constexpr int STAGES = STAGES_;  // ring depth
-    static constexpr int UNROLL = UNROLL_;  // unroll of the sample loop
-    static_assert(CHUNK_ % 128 == 0 && CHUNK_ * 8 * STAGES_ <= 160 * 1024, "chunk ring must fit shared memory");
+    static constexpr int CHUNK = CHUNK_;      // samples per staged chunk
+    static constexpr int BYTES = PAIR_ ? 4 : 8;  // staged bytes per sample (native FP64 also reads pair sums)
+    static constexpr int STAGES = STAGES_;    // ring depth
+    static constexpr int UNROLL = UNROLL_;    // unroll of the sample loop
+    static_assert(CHUNK_ % 128 == 0 && CHUNK_ * BYTES * STAGES_ <= 160 * 1024, "chunk ring must fit shared memory");
     static_assert((V & (V - 1)) == 0 && V >= 2 && V <= 32, "tile must hold a power of two <= 32 cells");
     static_assert(P_ == Prec::F64 || TL_ % 2 == 0, "the FP32 and exact tiles pack lam values in pairs");
-    static_assert(FLUSH >= 0 && UNROLL >= 1 && FCOLS >= 0 && FCOLS <= TL, "shape parameters out of range");
+    static_assert(FLUSH >= 0 && UNROLL >= 1 && (!PAIR || P_ == Prec::EXACT), "shape parameters out of range");
 };
 // 2 r x 8 lam tiles, up to 16 warps per CTA and (FP32, exact) two CTAs per SM (64 registers)
 // for up to 128 lam values; larger lam grids run the exact kernel in blocks of 128 lam values
 // (kExactLamBlock), and the FP32 kernel takes 2 x 16 tiles.  FP64: 2 x 8 tiles.
-// The exact variants stage 6144-sample chunks (48 KB), the FP32 and FP64 ones 4096-sample chunks
-// (32 KB), through a 2-deep ring (two CTAs of the exact kernel per SM: 2 x 96 KB of ring).  The FP32
-// variants fold their partial sums every 2 chunks (256 samples per lane); the exact variants fold
-// as often as their support size requires, independently of the chunk size.  The FP32 and exact
-// variants unroll the sample loop 4 times, and the exact variants give half of every row's lam
-// columns (FCOLS) to the packed FP32 adds, the rest to the integer absolute differences.
+// The exact variants hold 96 KB of ring per CTA, two CTAs per SM: three 32 KB chunks of pair sums
+// (8192 samples; two of 32, 36 or 48 KB, four of 24 and six of 16 measured 2 to 5 % slower) or two 48 KB
+// chunks of (x', x') pairs; the FP32 and FP64 ones two of 32 KB.  The FP32 variants fold their partial sums every
+// 2 chunks (256 samples per lane); the exact variants fold as often as their support size requires,
+// independently of the chunk size.
 using CfgF32 = GridCfg<Prec::F32, 2, 8, 2, 2, 512, 4096, 2, 4>;
 using CfgF32Wide = GridCfg<Prec::F32, 2, 16, 2, 1, 512, 4096, 2, 4>;
 using CfgF64 = GridCfg<Prec::F64, 2, 8, 0, 1, 512, 4096, 2>;
-using CfgExact = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 6144, 2, 4>;
-// Above a support of 2^19 the packed FP32 sums (exact only up to 2^24) would fold every few loads;
-// there every column takes the integer absolute differences, whose sums fold far less often.
-using CfgExactInt = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 6144, 2, 8, 0>;
+using CfgExact = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 8192, 3, 8, true>;
+// Above a support of kPairMaxL the FP32 sums (exact only up to 2^24) would fold every few loads; there
+// the integer absolute differences, whose sums fold far less often, take the samples one by one.
+using CfgExactInt = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 6144, 2, 8>;
 // One or two lam values (a small grid, or the last block of a larger one): 8 r x 2 lam tiles, so
-// that a single value pads its tile to 2 columns rather than 8; both columns on the integer sad.
-using CfgExactFewLam = GridCfg<Prec::EXACT, 8, 2, 0, 2, 512, 6144, 2, 8, 0>;
+// that a single value pads its tile to 2 columns rather than 8.
+using CfgExactFewLam = GridCfg<Prec::EXACT, 8, 2, 0, 2, 512, 8192, 3, 8, true>;
+using CfgExactIntFewLam = GridCfg<Prec::EXACT, 8, 2, 0, 2, 512, 6144, 2, 8>;
 constexpr int32_t kFewLam = 2;
-constexpr int32_t kExactIntAboveL = 1 << 19;
 constexpr int kWarpsTarget = 16;  // warps per CTA the r groups fill up to
 static_assert(kExactLamBlock == kWarpsTarget * CfgExact::TL && kExactLamBlock == kWarpsTarget * CfgExactInt::TL,
               "one launch of the exact kernel takes 16 warps of lam tiles");
@@ -125,10 +125,11 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
-__device__ __forceinline__ u64 abs2(u64 v) {
+// max(|v|, d) of both halves
+__device__ __forceinline__ u64 max_abs2(u64 v, float d) {
     float a, b;
     upk(v, a, b);
-    return pk(fabsf(a), fabsf(b));
+    return pk(fmaxf(fabsf(a), d), fmaxf(fabsf(b), d));
 }
 // max(w, 0); a NaN operand yields 0 (PTX max returns the non-NaN input).
 __device__ __forceinline__ double relu(double w) {
@@ -230,24 +231,127 @@ __device__ __forceinline__ T transpose_reduce(T (&v)[V], int lane) {
 }
 
 struct SmemLayout {
-    size_t ring, full, lam, eps, S, total;
+    size_t ring, full, lam, eps, S, acc, t, total;
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int RG, int TR, int NLpad, int E, int chunk, int stages) {
+// `acc` and `t` (the exact kernel's cells, in warp order): the integer sums and the thresholds.
+__host__ __device__ inline SmemLayout smem_layout(int RG, int TR, int NLpad, int E, int chunk_bytes, int stages) {
     SmemLayout L;
     L.ring = 0;
-    L.full = (size_t)stages * chunk * sizeof(float2);
+    L.full = (size_t)stages * chunk_bytes;
     L.lam = L.full + 8 * (size_t)stages;
     L.eps = L.lam + 8 * (size_t)NLpad;
     L.S = L.eps + 8 * (size_t)E;
-    L.total = L.S + 8 * (size_t)RG * TR * NLpad;
+    L.acc = L.S + 8 * (size_t)RG * TR * NLpad;
+    L.t = (L.acc + 8 * (size_t)RG * TR * NLpad + 15) & ~(size_t)15;
+    L.total = L.t + 4 * (size_t)RG * TR * NLpad;
     return L;
 }
 
-// Epilogue of one CTA: for each of its (r, eps) pairs, the minimum over lam of lam * eps + S
-// (lowest index on ties), the cost and lam index outputs, and the argmin over r through a 64-bit
-// atomicMin key (FP32: cost bits and r index; otherwise the cost's double bits truncated to 44
+// The minimum over lam of lam * eps + S for one (r, eps) pair: the value RN(RN(lam eps) + S) and the
+// lowest index attaining it.
+//
+// FP32 first: with lam, eps and S cut to floats (each at most 2^-23 low) v' = fma(lam, eps, S) lies
+// within [v (1 - 2.6 x 2^-23), v (1 + 2^-23)], so a lam attaining the minimum has v' at most
+// (1 + 2^-20) times the smallest v', and only those values -- one as a rule -- are formed in FP64, in
+// ascending order, except one whose lam and S are both no smaller than the best's, which cannot be
+// below it.  Where the floats do not hold (a negative S, magnitudes above 2^100, a minimum below
+// 2^-80 that the cut of smaller parts to zero could matter to) every value is formed.
+constexpr float kLamWindow = 1.f + 0x1p-19f;
+constexpr float kLamFloor = 0x1p-80f;
+
+// A value >= 0 cut to a float: 0 below 2^-100; `ok` is cleared above 2^100 and for negative values.
+__device__ __forceinline__ float cut(double v, bool& ok) {
+    const long long b = dbits(v);
+    if ((b << 1) == 0) return 0.f;  // +-0
+    const unsigned e = (unsigned)((unsigned long long)b >> 52);  // sign and exponent
+    ok = ok && e <= 1023u + 100u;
+    return e >= 1023u - 100u ? narrow(b) : 0.f;
+}
+
+struct LamMin {
+    long long key = 0x7fffffffffffffffll;  // order key of v
+    double v = DBL_MAX;
+    int j = 0x7fffffff;
+    // value j, in ascending order of j; `skip`: S >= 0 and finite floats (the window holds)
+    __device__ __forceinline__ void take(double lam, double eps, double s, int at, bool skip, const double* L, const double* S) {
+        if (skip && j != 0x7fffffff && dbits(lam) >= dbits(L[j]) && dbits(s) >= dbits(S[j])) return;
+        const double w = __dadd_rn(__dmul_rn(lam, eps), s);
+        const long long k = order_key(w);
+        if (k < key) {
+            key = k;
+            v = w;
+            j = at;
+        }
+    }
+    // the lower of two lanes' results (ties: lower index), over groups of G lanes
+    __device__ __forceinline__ void reduce(int G) {
+        for (int o = 1; o < G; o <<= 1) {
+            const long long ok = __shfl_xor_sync(0xffffffffu, key, o);
+            const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, j, o);
+            if (ok < key || (ok == key && oj < j)) {
+                key = ok;
+                v = ov;
+                j = oj;
+            }
+        }
+    }
+};
+
+// The warp's lanes over one row of S (every lane returns the result).
+__device__ __forceinline__ LamMin warp_lam_min(const double* S, const double* lam, double eps, int NL, int lane) {
+    bool ok = true, unused = true;
+    const float ef = cut(eps, ok);
+    float ub = INFINITY;
+    for (int j = lane; j < NL; j += 32) ub = fminf(ub, fmaf(cut(lam[j], ok), ef, cut(S[j], ok)));
+    if (!ok) ub = 0.f;
+    ub = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(ub)));  // ordered as uints: all >= 0
+    const bool fast = ub > kLamFloor;
+    LamMin r;
+    for (int j = lane; j < NL; j += 32)
+        if (!fast || fmaf(cut(lam[j], unused), ef, cut(S[j], unused)) <= ub * kLamWindow)
+            r.take(lam[j], eps, S[j], j, fast, lam, S);
+    r.reduce(32);
+    return r;
+}
+
+// One (r, eps) pair's results: the cost and lam index outputs and the argmin over r through a 64-bit
+// key for atomicMin (FP32: cost bits and r index; otherwise the cost's double bits truncated to 44
 // bits, order-preserving for non-negative values, with the r index in the low 20 bits).
+// Returns the key, or all ones before the last lam block; the caller takes its minimum.
+template <bool F32OUT>
+__device__ __forceinline__ u64 write_pair(const GridArgs& a, double best, int bj, int m, int k, int e, int ri) {
+    const size_t row = ((size_t)m * a.E + e) * a.K + k;
+    const size_t o = row * a.R + ri;
+    bj += a.lam0;
+    if (a.part_val) {  // lam blocks: merge with the earlier blocks (they hold lower indices)
+        const size_t q = ((((size_t)(m - a.m0)) * a.E + e) * a.K + k) * a.R + ri;
+        if (!a.part_first && !(best < a.part_val[q])) {
+            best = a.part_val[q];
+            bj = a.part_idx[q];
+        }
+        if (!a.part_last) {
+            a.part_val[q] = best;
+            a.part_idx[q] = bj;
+            return ~0ull;
+        }
+    }
+    u64 key;
+    if constexpr (F32OUT) {
+        const float cf = (float)best;
+        if (a.cost_out) static_cast<float*>(a.cost_out)[o] = cf;
+        key = ((u64)__float_as_uint(cf > 0.f ? cf : 0.f) << 32) | (u64)(uint32_t)ri;
+    } else {
+        static_cast<double*>(a.cost_out)[o] = best;
+        const bool above = dbits(best) > 0 && dbits(best) <= 0x7ff0000000000000ll;  // best > 0
+        key = ((u64)(above ? dbits(best) : 0ll) & ~0xFFFFFull) | (u64)ri;
+    }
+    if (a.lam_idx_out) a.lam_idx_out[o] = bj;
+    return key;
+}
+
+// Epilogue of one CTA of the grid kernel: a warp per (r, eps) pair.
 template <bool F32OUT>
 __device__ __forceinline__ void cta_epilogue(const GridArgs& a, const double* s_S, const double* s_lam,
                                              const double* s_eps, int stride, int rl_count, int r_cta0, int m, int k) {
@@ -256,45 +360,10 @@ __device__ __forceinline__ void cta_epilogue(const GridArgs& a, const double* s_
         const int rl = p / a.E, e = p % a.E;
         const int ri = r_cta0 + rl;
         if (ri >= a.R) continue;
-        double best = DBL_MAX;
-        int bj = 0x7fffffff;
-        for (int j = lane; j < a.NL; j += 32) {
-            const double v = __dadd_rn(__dmul_rn(s_lam[j], s_eps[e]), s_S[rl * stride + j]);
-            if (v < best) { best = v; bj = j; }
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-            if (ov < best || (ov == best && oj < bj)) { best = ov; bj = oj; }
-        }
+        const LamMin b = warp_lam_min(s_S + rl * stride, s_lam, s_eps[e], a.NL, lane);
         if (lane == 0) {
-            const size_t row = ((size_t)m * a.E + e) * a.K + k;
-            const size_t o = row * a.R + ri;
-            bj += a.lam0;
-            if (a.part_val) {  // lam blocks: merge with the earlier blocks (they hold lower indices)
-                const size_t q = ((((size_t)(m - a.m0)) * a.E + e) * a.K + k) * a.R + ri;
-                if (!a.part_first && !(best < a.part_val[q])) {
-                    best = a.part_val[q];
-                    bj = a.part_idx[q];
-                }
-                if (!a.part_last) {
-                    a.part_val[q] = best;
-                    a.part_idx[q] = bj;
-                    continue;
-                }
-            }
-            u64 key;
-            if constexpr (F32OUT) {
-                const float cf = (float)best;
-                if (a.cost_out) static_cast<float*>(a.cost_out)[o] = cf;
-                key = ((u64)__float_as_uint(cf > 0.f ? cf : 0.f) << 32) | (u64)(uint32_t)ri;
-            } else {
-                static_cast<double*>(a.cost_out)[o] = best;
-                key = ((u64)__double_as_longlong(best > 0.0 ? best : 0.0) & ~0xFFFFFull) | (u64)ri;
-            }
-            if (a.lam_idx_out) a.lam_idx_out[o] = bj;
-            atomicMin(a.keys + row, key);
+            const u64 key = write_pair<F32OUT>(a, b.v, b.j, m, k, e, ri);
+            if (key != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + e) * a.K + k, key);
         }
     }
 }
@@ -307,8 +376,9 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     constexpr int TR = C::TR, TL = C::TL, V = C::V, LOG2V = C::LOG2V;
     extern __shared__ __align__(128) unsigned char smem[];
     const int NLpad = a.LT * TL;
-    const SmemLayout lay = smem_layout(a.RG, TR, NLpad, a.E, C::CHUNK, C::STAGES);
-    float2* ring = reinterpret_cast<float2*>(smem + lay.ring);
+    const SmemLayout lay = smem_layout(a.RG, TR, NLpad, a.E, C::CHUNK * C::BYTES, C::STAGES);
+    unsigned char* ring = smem + lay.ring;  // chunk c in stage c % STAGES
+    constexpr size_t kStageBytes = (size_t)C::CHUNK * C::BYTES;
     u64* full = reinterpret_cast<u64*>(smem + lay.full);
     double* s_lam = reinterpret_cast<double*>(smem + lay.lam);
     double* s_eps = reinterpret_cast<double*>(smem + lay.eps);
@@ -320,9 +390,8 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     b /= a.r_blocks;
     const int k = b % a.K;
     const int m = a.m0 + b / a.K;
-    const int lt = warp % a.LT, rg = warp / a.LT;
+    [[maybe_unused]] const int lt = warp % a.LT, r_local0 = warp / a.LT * TR;
     const int r_cta0 = rb * a.RG * TR;
-    const int r_local0 = rg * TR;
 
     for (int i = tid; i < NLpad; i += blockDim.x) s_lam[i] = i < a.NL ? a.lam[i] : 0.0;
     for (int i = tid; i < a.E; i += blockDim.x) s_eps[i] = a.eps[i];
@@ -330,19 +399,19 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     const int64_t pbase = a.pair_off[k];
     const int64_t np = a.pair_off[k + 1] - pbase;  // multiple of kPadSamples
     const int nchunks = (int)((np + C::CHUNK - 1) / C::CHUNK);
-    const float2* src = a.pairs + pbase;
+    // (native FP64 also serves contexts that stage pair sums)
+    const int bytes = P == Prec::F64 && a.pair_sums ? 4 : C::BYTES;
+    const unsigned char* src = static_cast<const unsigned char*>(a.staged) + pbase * bytes;
     auto issue = [&](int c) {
         if (c == a.test_skip_chunk) return;  // test hook: nothing will complete this chunk's barrier
         const int s = c % C::STAGES;
         const int64_t cnt = min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
-        tma_bulk_load(smem_u32(ring + (size_t)s * C::CHUNK), src + (int64_t)c * C::CHUNK, (uint32_t)(cnt * sizeof(float2)),
+        tma_bulk_load(smem_u32(ring + (size_t)s * kStageBytes), src + (int64_t)c * C::CHUNK * bytes, (uint32_t)(cnt * bytes),
                       smem_u32(&full[s]));
     };
-    __shared__ double s_inv_n;  // 1 / N, one FP64 division per CTA (FP64 runs at 1/64 of FP32 here)
     if (tid == 0) {
         for (int s = 0; s < C::STAGES; s++) mbar_init(smem_u32(&full[s]), 1);
         fence_mbar_init();
-        s_inv_n = 1.0 / (double)a.N[k];
     }
     __syncthreads();
     if (tid == 0)
@@ -351,18 +420,20 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     int consumed = 0;                    // chunk at which the loop stopped
 
     // Per-cell constants of this warp's tile (identical across its lanes).
-    const double cp = a.cp[m], cw = a.cw[m], Lk = (double)a.L[k];
-    double eta[TR];
-    bool rvalid[TR];
+    const double cp = a.cp[m], cw = a.cw[m], Lk = to_double(a.L[k]);
+    [[maybe_unused]] double eta[TR];
+    [[maybe_unused]] bool rvalid[TR];
+    if constexpr (P != Prec::EXACT) {
 #pragma unroll
-    for (int i = 0; i < TR; i++) {
-        const int ri = r_cta0 + r_local0 + i;
-        rvalid[i] = ri < a.R;
-        eta[i] = rvalid[i] ? (double)a.r[ri] - (double)a.L_in[k] : 0.0;
+        for (int i = 0; i < TR; i++) {
+            const int ri = r_cta0 + r_local0 + i;
+            rvalid[i] = ri < a.R;
+            eta[i] = rvalid[i] ? (double)a.r[ri] - (double)a.L_in[k] : 0.0;
+        }
     }
 
     bool timeout = false;
-    double acc64 = 0.0;  // this lane's cell after the warp transposition
+    [[maybe_unused]] double acc64 = 0.0;  // this lane's cell after the warp transposition
 
     if constexpr (P == Prec::F32) {
         // Each row's excess is taken about its reservation: kappa (x - eta) + W(eta) (excess_at_eta).
@@ -452,7 +523,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
             if (!mbar_wait_bounded(smem_u32(&full[s]), (uint32_t)((c / C::STAGES) & 1), a.wait_ns)) timeout = true;
             if (!timeout) {
                 const int cnt = (int)min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
-                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * C::CHUNK);
+                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * kStageBytes);
                 const int nq = cnt >> 6;  // float4 (two samples) per lane: (x', x') pairs
                 if (nq == C::CHUNK / 64) {  // a full chunk: a fixed trip count, unrolled with no remainder
 #pragma unroll(C::UNROLL)
@@ -490,7 +561,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         }
     } else if constexpr (P == Prec::F64) {
         // each row's excess about its reservation, as in the FP32 kernel: x - eta per sample and row
-        const double offd = (double)stage_offset(a.L[k]);  // the staged samples carry the class's offset
+        const double offd = a.pair_sums ? 0.0 : (double)stage_offset(a.L[k]);  // (x', x') pairs carry the class's offset
         double base[TR];
 #pragma unroll
         for (int i = 0; i < TR; i++) base[i] = offd + eta[i];  // an exact integer
@@ -514,18 +585,32 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
             if (!mbar_wait_bounded(smem_u32(&full[s]), (uint32_t)((c / C::STAGES) & 1), a.wait_ns)) timeout = true;
             if (!timeout) {
                 const int cnt = (int)min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
-                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * C::CHUNK);
-                const int nq = cnt >> 6;
-                for (int t = 0; t < nq; t++) {
-                    const float4 v = q[lane + 32 * t];
+                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * kStageBytes);
+                auto two = [&](float x0, float x1) {  // two staged samples (NaN: none)
 #pragma unroll
                     for (int i = 0; i < TR; i++) {
-                        const double xa = (double)v.x - base[i], xb = (double)v.z - base[i];  // x - eta, exact
+                        const double xa = (double)x0 - base[i], xb = (double)x1 - base[i];  // x - eta, exact
 #pragma unroll
                         for (int j = 0; j < TL; j++) {
                             acc[i][j] += relu(fma(kap[j], xa, dd[i][j]));
                             acc[i][j] += relu(fma(kap[j], xb, dd[i][j]));
                         }
+                    }
+                };
+                if (a.pair_sums) {  // samples back from (sum, difference), exactly; none past the class's last
+                    const int64_t left = a.N[k] - (int64_t)c * C::CHUNK;
+                    for (int t = 0; t < cnt >> 7; t++) {
+                        const float4 v = q[lane + 32 * t];
+                        const int at = 4 * (lane + 32 * t);
+                        const float nan = __int_as_float(0x7fc00000);
+                        // the one real sample of a half-padded pair is the larger: its partner is 0
+                        two(at < left ? 0.5f * (v.x + v.z) : nan, at + 1 < left ? 0.5f * (v.x - v.z) : nan);
+                        two(at + 2 < left ? 0.5f * (v.y + v.w) : nan, at + 3 < left ? 0.5f * (v.y - v.w) : nan);
+                    }
+                } else {
+                    for (int t = 0; t < cnt >> 6; t++) {
+                        const float4 v = q[lane + 32 * t];
+                        two(v.x, v.z);
                     }
                 }
             }
@@ -554,152 +639,160 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         // EXACT: per cell (i, j) the active samples are x >= t_ij for an integer threshold t_ij, and
         // sum_n max(kappa x_n + d, 0) = kappa sum_{x >= t} x + d #{x >= t}.  With c = t - 1,
         // max(x - c, 0) = (x - c + |x - c|) / 2 and sum_n (x - c) has a closed form, so the kernel
-        // streams sum_n |x - c| only, on two pipes at once.  For half of a warp's lam columns one
-        // packed FP32 add forms y = x' + (1 - t - 2^23) = x - c for two cells and one adds |y| into
-        // the running sum (the absolute value rides on the add's operand); for the other half one
-        // integer absolute-difference-and-add (__sad) works on the staged float's bit pattern,
-        // 0x4B000000 + x.  Every value is an integer below 2^24, so both are exact.  Sums are
-        // folded into int64 through the warp transposition before an FP32 sum could pass 2^24.  The
-        // count #{x >= t} comes from the class's cumulative counts; the epilogue puts every sample
+        // streams sum_n |x - c| only, as integers.
+        // Pair sums: |a - c| + |b - c| = max(|a + b - 2c|, |a - b|) takes two samples for two cells in one
+        // packed FP32 add, two max and (with the next pair's) one packed add, an instruction per term
+        // as with one sample at a time, but split evenly over the FMA and ALU pipes within each cell and
+        // with fewer register operands (3 reads a term, and the pair's sum and difference serve every
+        // cell), in half the staged bytes.  Packed adds on one half of a warp's cells beside integer
+        // absolute differences on the other (3.5 reads a term) took 16.43 ms on 8 classes x 100,000
+        // samples x 4096 r x 128 lam, this 16.06: 83 of the 128 terms/clk/SM that either pipe and the
+        // issue slots allow.  Every value is an integer
+        // below 2^24, so the FP32 arithmetic is exact; sums fold into int64 through the warp transposition
+        // before one could pass 2^24.
+        // (x', x') pairs: one integer absolute-difference-and-add (__sad) per term on the staged float's
+        // bit pattern, 0x4B000000 + x.
+        // The count #{x >= t} comes from the class's cumulative counts; the epilogue puts every sample
         // on its branch of phi with these integer sums (branch_sum) in FP64.
-        constexpr int TLF = C::FCOLS;  // lam columns per r row on the packed FP32 adds (in pairs)
-        constexpr int TLI = TL - TLF;  // lam columns per r row on the integer path
-        static_assert(TLF % 2 == 0 && TLI >= 1, "packed columns come in pairs");
-        constexpr int NPF = TLF > 0 ? TLF / 2 : 1;  // array extent (unused when TLF = 0)
-        u64 ntf[TR][NPF], accf[TR][NPF];           // ntf: 1 - t - 2^23 for a pair of cells
-        int cci[TR][TLI];                          // 0x4B000000 + t - 1 per cell
-        unsigned acci[TR][TLI];
-        // Each lane works out the threshold of the cell it owns after the final transposition
-        // (cell lane >> (5 - LOG2V)); the warp's V thresholds then reach every lane by shuffles.
-        const int cidx = lane >> (5 - LOG2V);
-        const int ci = cidx / TL, cj = cidx % TL;
-        const int c_ri = r_cta0 + r_local0 + ci, c_lj = lt * TL + cj;
-        const bool c_valid = c_ri < a.R && c_lj < a.NL;
-        const double c_lam = s_lam[c_lj];  // s_lam is padded with zeros to NLpad
-        const double c_mu = fmin(c_lam, cp), c_kap = c_mu + fmin(c_lam, cw);
-        const double c_eta = c_valid ? (double)a.r[c_ri] - (double)a.L_in[k] : 0.0;
-        const double c_d = excess_offset(cp, cw, c_mu, Lk, c_eta);
-        // t = L + 1 means "none" (no sample exceeds L); t in [0, L + 1] keeps |x - c| <= L + 1
-        const int c_t = (int)(c_valid ? first_active(c_kap, c_d, a.L[k]) : (int64_t)a.L[k] + 1);
+        constexpr int NPF = C::PAIR ? TL / 2 : 1, NI = C::PAIR ? 1 : TL;  // array extents
+        [[maybe_unused]] u64 n2c[TR][NPF], accf[TR][NPF];  // -2c for two cells, their sums
+        [[maybe_unused]] int cci[TR][NI];                  // 0x4B000000 + c per cell
+        [[maybe_unused]] unsigned acci[TR][NI];
+        // The CTA's cells, V per warp, are half its threads: each cell's threshold is one thread's work (its
+        // few FP64 instructions take the pipe as long for one lane as for 32), read back by its warp;
+        // the same thread combines the cell's sums at the end, so nothing of it stays in registers
+        // over the sample loop.
+        int* s_t = reinterpret_cast<int*>(smem + lay.t);
+        long long* s_acc = reinterpret_cast<long long*>(smem + lay.acc);
+        const int cells = (blockDim.x >> 5) * V;
+        struct CellAt {
+            int rl, lj, ri;
+        };
+        auto cell_at = [&](int c) {
+            const int w = c >> LOG2V, i = c & (V - 1);
+            CellAt x;
+            x.rl = w / a.LT * TR + i / TL;
+            x.lj = w % a.LT * TL + i % TL;
+            x.ri = r_cta0 + x.rl;
+            return x;
+        };
+        for (int c = tid; c < cells; c += blockDim.x) {
+            const CellAt x = cell_at(c);
+            int ct = a.L[k] + 1;  // L + 1 means "none" (no sample exceeds L); t in [0, L + 1] keeps |x - c| <= L + 1
+            if (x.ri < a.R && x.lj < a.NL) {
+                const double lam = s_lam[x.lj], mu = dmin_nonneg(lam, cp);
+                const RowOffset row = row_offset(cp, cw, a.L[k], a.r[x.ri] - a.L_in[k]);
+                ct = first_active(__dadd_rn(mu, dmin_nonneg(lam, cw)), excess_offset(row, cp, mu, Lk), a.L[k]);
+            }
+            s_t[c] = ct;
+        }
+        __syncthreads();
+        const int* w_t = s_t + warp * V;
 #pragma unroll
         for (int i = 0; i < TR; i++) {
+            if constexpr (C::PAIR) {
 #pragma unroll
-            for (int jp = 0; jp < TLF / 2; jp++) {
-                const int t0 = __shfl_sync(0xffffffffu, c_t, (i * TL + 2 * jp) << (5 - LOG2V));
-                const int t1 = __shfl_sync(0xffffffffu, c_t, (i * TL + 2 * jp + 1) << (5 - LOG2V));
-                ntf[i][jp] = pk((float)(1 - t0 - (1 << 23)), (float)(1 - t1 - (1 << 23)));  // exact: below 2^24
-                accf[i][jp] = 0ull;
-            }
+                for (int jp = 0; jp < TL / 2; jp++) {
+                    n2c[i][jp] = pk((float)(2 - 2 * w_t[i * TL + 2 * jp]), (float)(2 - 2 * w_t[i * TL + 2 * jp + 1]));
+                    accf[i][jp] = 0ull;
+                }
+            } else {
 #pragma unroll
-            for (int jj = 0; jj < TLI; jj++) {
-                cci[i][jj] = kStageBits - 1 + __shfl_sync(0xffffffffu, c_t, (i * TL + TLF + jj) << (5 - LOG2V));
-                acci[i][jj] = 0u;
+                for (int j = 0; j < TL; j++) {
+                    cci[i][j] = kStageBits - 1 + w_t[i * TL + j];
+                    acci[i][j] = 0u;
+                }
             }
         }
-        // Fold after `fe` loads of two samples, when a lane's sums are at most 2 fe (L + 1): with
-        // packed columns that is at most 2^24 (exact in FP32; the transposition's 32-lane sums stay
-        // below 2^29); with none, only the integer limit applies (32 lanes' sums below 2^32).  fe
-        // is a power of two, the same for every thread of the CTA.
-        const int64_t fold_lim = TLF > 0 ? (1ll << 24) : (1ll << 32) / 32 - 1;
-        int fe = 1;
-        while (fe < (1 << 20) && 2ll * (2 * fe) * ((int64_t)a.L[k] + 1) <= fold_lim) fe <<= 1;
+        // Fold after at most `fe` loads of kPer samples each: a lane's sum is then at most
+        // kPer fe (L + 1), within 2^24 in FP32 (the transposition's 32-lane sums stay below 2^29), or as
+        // integers 32 lanes' sums below 2^32.  The same for every thread of the CTA.
+        constexpr int kPer = C::PAIR ? 4 : 2;
+        constexpr long long kFoldLimit = C::PAIR ? (1ll << 24) : (1ll << 32) / 32 - 1;
+        const int fe = (int)min(1ll << 20, max(1ll, kFoldLimit / (kPer * ((long long)a.L[k] + 1))));
         long long acc_r = 0;
         auto fold = [&]() {
             unsigned vs[V];
 #pragma unroll
             for (int i = 0; i < TR; i++) {
+                if constexpr (C::PAIR) {
 #pragma unroll
-                for (int jp = 0; jp < TLF / 2; jp++) {
-                    float a0, a1;
-                    upk(accf[i][jp], a0, a1);
-                    vs[i * TL + 2 * jp] = __float2uint_rn(a0);
-                    vs[i * TL + 2 * jp + 1] = __float2uint_rn(a1);
-                    accf[i][jp] = 0ull;
-                }
+                    for (int jp = 0; jp < TL / 2; jp++) {
+                        float a0, a1;
+                        upk(accf[i][jp], a0, a1);
+                        vs[i * TL + 2 * jp] = __float2uint_rn(a0);
+                        vs[i * TL + 2 * jp + 1] = __float2uint_rn(a1);
+                        accf[i][jp] = 0ull;
+                    }
+                } else {
 #pragma unroll
-                for (int jj = 0; jj < TLI; jj++) {
-                    vs[i * TL + TLF + jj] = acci[i][jj];
-                    acci[i][jj] = 0u;
+                    for (int j = 0; j < TL; j++) {
+                        vs[i * TL + j] = acci[i][j];
+                        acci[i][j] = 0u;
+                    }
                 }
             }
             acc_r += (long long)transpose_reduce<unsigned, V>(vs, lane);
         };
-        // one load: two samples' (x', x') pairs into every cell's sum (the compiler interleaves the
-        // two pipes' instructions)
+        // One load into every cell's sum.  The pair sums' rate hangs on ptxas's register allocation (operand
+        // bank conflicts): written cell by cell, the second pair first, 16.06 ms on 8 classes x 100,000
+        // samples x 4096 r x 128 lam; first pair first 16.39, the accumulator as first operand 16.57, two
+        // cells' adds ahead of their max 16.91, all adds first 17.03; unrolled 4 / 16 times 16.6 / 16.5.
         auto step = [&](const float4 v) {
-            const u64 xa = pk(v.x, v.y), xb = pk(v.z, v.w);
-            const int ba = __float_as_int(v.x), bb = __float_as_int(v.z);  // 0x4B000000 + x
+            if constexpr (C::PAIR) {
+                const u64 s0 = pk(v.x, v.x), s1 = pk(v.y, v.y);
 #pragma unroll
-            for (int i = 0; i < TR; i++) {
+                for (int i = 0; i < TR; i++)
 #pragma unroll
-                for (int p = 0; p < TLF / 2; p++)
-                    accf[i][p] = fadd2(accf[i][p], fadd2(abs2(fadd2(xa, ntf[i][p])), abs2(fadd2(xb, ntf[i][p]))));
-#pragma unroll
-                for (int jj = 0; jj < TLI; jj++) acci[i][jj] = __sad(bb, cci[i][jj], __sad(ba, cci[i][jj], acci[i][jj]));
-            }
-        };
-        auto run = [&](const float4* q, int t0, int t1, bool clamp) {
-            if (clamp) {
-#pragma unroll 1
-                for (int t = t0; t < t1; t++) {
-                    float4 v = q[lane + 32 * t];  // NaN padding -> x = 0 (x' = 2^23)
-                    v.x = fmaxf(v.x, kStageOffset), v.y = fmaxf(v.y, kStageOffset);
-                    v.z = fmaxf(v.z, kStageOffset), v.w = fmaxf(v.w, kStageOffset);
-                    step(v);
-                }
+                    for (int p = 0; p < NPF; p++)
+                        accf[i][p] = fadd2(fadd2(max_abs2(fadd2(s1, n2c[i][p]), v.w), max_abs2(fadd2(s0, n2c[i][p]), v.z)), accf[i][p]);
             } else {
-#pragma unroll(C::UNROLL)
-                for (int t = t0; t < t1; t++) step(q[lane + 32 * t]);
+                const int ba = __float_as_int(v.x), bb = __float_as_int(v.z);  // 0x4B000000 + x
+#pragma unroll
+                for (int i = 0; i < TR; i++)
+#pragma unroll
+                    for (int j = 0; j < TL; j++) acci[i][j] = __sad(bb, cci[i][j], __sad(ba, cci[i][j], acci[i][j]));
             }
         };
-        constexpr int kChunkLoads = C::CHUNK / 64;  // loads of one full chunk per lane
-        constexpr int kSegLoads = 32;
-        static_assert(kChunkLoads % kSegLoads == 0, "a full chunk splits into whole segments");
+        constexpr int kSeg = 8;  // loads per segment of a fixed trip count
+        int pending = 0;         // loads since the last fold
+        auto room = [&](int loads) {  // fold first if the loads since the last fold would pass fe
+            if (pending + loads > fe) {
+                fold();
+                pending = 0;
+            }
+            pending += loads;
+        };
         const int64_t n_k = a.N[k];
-        int pending = 0;  // loads since the last fold
         for (int c = 0; c < nchunks; c++) {
             const int s = c % C::STAGES;
             if (!mbar_wait_bounded(smem_u32(&full[s]), (uint32_t)((c / C::STAGES) & 1), a.wait_ns)) timeout = true;
             if (!timeout) {
                 const int cnt = (int)min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
-                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * C::CHUNK);
-                const int nq = cnt >> 6;
-                // loads [0, t_clean) hold samples only; the class's last ones may hold NaN padding,
-                // which they read as x = 0 (x' = 2^23)
+                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * kStageBytes);
+                const int nq = cnt / (32 * kPer);
+                // loads [0, t_clean) hold samples only; of (x', x') pairs the class's last ones may hold
+                // NaN padding, which they read as x = 0 (x' = 2^23)
                 const int64_t left = n_k - (int64_t)c * C::CHUNK;
-                const int t_clean = left <= 0 ? 0 : (int)min((int64_t)nq, left >> 6);
-                if (nq == kChunkLoads && t_clean == nq && fe >= kSegLoads) {
-                    // a full chunk of samples only: segments of a fixed trip count, which unroll with
-                    // no remainder.  fe is a power of two >= kSegLoads and every earlier chunk took
-                    // this path too (only a class's last chunk is ragged or padded), so the loads
-                    // since the last fold are a multiple of kSegLoads and reach fe exactly at a
-                    // segment's end.
+                const int t_clean = C::PAIR ? nq : (left <= 0 ? 0 : (int)min((int64_t)nq, left / (32 * kPer)));
+                int t0 = 0;
+                if (fe >= kSeg) {
 #pragma unroll 1
-                    for (int h = 0; h < kChunkLoads / kSegLoads; h++) {
+                    for (; t0 + kSeg <= t_clean; t0 += kSeg) {
+                        room(kSeg);
 #pragma unroll(C::UNROLL)
-                        for (int t = 0; t < kSegLoads; t++) step(q[lane + 32 * (kSegLoads * h + t)]);
-                        pending += kSegLoads;
-                        if (pending >= fe) {
-                            fold();
-                            pending = 0;
-                        }
+                        for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
                     }
-                } else {
-                    for (int t0 = 0; t0 < nq; t0 += fe) {
-                        const int t1 = min(nq, t0 + fe);
-                        const int tm = max(t0, min(t1, t_clean));
-                        if (pending + (t1 - t0) > fe) {  // fold first: the loads since the last fold would pass fe
-                            fold();
-                            pending = 0;
-                        }
-                        run(q, t0, tm, false);
-                        if (tm < t1) run(q, tm, t1, true);
-                        pending += t1 - t0;
-                        if (pending >= fe) {
-                            fold();
-                            pending = 0;
-                        }
+                }
+#pragma unroll 1
+                for (; t0 < nq; t0++) {
+                    room(1);
+                    float4 v = q[lane + 32 * t0];
+                    if (!C::PAIR && t0 >= t_clean) {
+                        v.x = fmaxf(v.x, kStageOffset), v.y = fmaxf(v.y, kStageOffset);
+                        v.z = fmaxf(v.z, kStageOffset), v.w = fmaxf(v.w, kStageOffset);
                     }
+                    step(v);
                 }
             }
             consumed = c;
@@ -717,21 +810,36 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         }
         if (!timeout) {
             if (pending > 0) fold();
-            // this lane's cell: the active count from the cumulative counts, then the branch sums
-            const long long t = (long long)c_t;  // integer in [0, L + 1]
-            const long long Nk = a.N[k];
-            const long long count = t <= 0 ? Nk : (t > a.L[k] ? 0 : Nk - (long long)a.cdf[a.hist_off[k] + t - 1]);
-            // acc_r = sum |x - c| over the samples and the padding zeros; with y = x - c,
-            // max(y, 0) = (y + |y|) / 2
-            const long long npad = np - Nk;
-            const long long sum_abs = acc_r - npad * (t > 1 ? t - 1 : 1 - t);
-            const long long sum_y = a.sumx[k] + Nk * (1 - t);
-            const long long sum_relu = (sum_y + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
-            const long long sum = sum_relu + (t - 1) * count;  // sum_{x >= t} x
-            // each sample on its own branch of phi (exact integer sums): V = c_w eta - nu x below t,
-            // U = c_p (L - eta) - mu (L - x) from t on; no large term cancels another
-            acc64 = branch_sum(cp, cw, c_mu, fmin(c_lam, cw), Lk, c_eta, (double)Nk, count, a.sumx[k] - sum,
-                               (long long)a.L[k] * count - sum);
+            // the lane's cell (cell lane >> (5 - log2 V) of its warp)
+            if ((lane & ((1 << (5 - LOG2V)) - 1)) == 0) s_acc[warp * V + (lane >> (5 - LOG2V))] = acc_r;
+            __syncthreads();
+            const long long Nk = a.N[k], sumx = a.sumx[k], npad = np - Nk;
+            for (int c = tid; c < cells; c += blockDim.x) {
+                const CellAt x = cell_at(c);
+                if (x.ri >= a.R || x.lj >= a.NL) continue;
+                // the active count from the cumulative counts, then the branch sums
+                const int ti = s_t[c], L = a.L[k];  // in [0, L + 1]
+                const long long t = ti;
+                const long long count = ti <= 0 ? Nk : (ti > L ? 0 : Nk - (long long)a.cdf[a.hist_off[k] + t - 1]);
+                // s_acc = sum |x - c| over the samples and the padding zeros; with y = x - c,
+                // max(y, 0) = (y + |y|) / 2
+                const long long sum_abs = s_acc[c] - npad * (t > 1 ? t - 1 : 1 - t);
+                const long long sum_y = sumx + Nk * (1 - t);
+                const long long sum_relu = (sum_y + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
+                const long long sum = sum_relu + (t - 1) * count;  // sum_{x >= t} x
+                // each sample on its own branch of phi (exact integer sums): V = c_w eta - nu x below t,
+                // U = c_p (L - eta) - mu (L - x) from t on; no large term cancels another
+                const double lam = s_lam[x.lj];
+                const double tot = branch_sum(cp, cw, dmin_nonneg(lam, cp), dmin_nonneg(lam, cw), L, a.r[x.ri] - a.L_in[k],
+                                              Nk, count, sumx - sum, (long long)L * count - sum);
+                const double S = __dmul_rn(tot, a.inv_n[k]);
+                s_S[x.rl * NLpad + x.lj] = S;
+                if (a.S_out) {
+                    const size_t o = (((size_t)m * a.K + k) * a.R + x.ri) * a.NL_out + a.lam0 + x.lj;
+                    if (a.f32_out) static_cast<float*>(a.S_out)[o] = (float)S;
+                    else static_cast<double*>(a.S_out)[o] = S;
+                }
+            }
         }
     }
 
@@ -746,33 +854,27 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         return;
     }
 
-    // S for this lane's cell.
-    {
+    // S for this lane's cell (the exact kernel has formed it above).
+    if constexpr (P != Prec::EXACT) {
         const int cidx = lane >> (5 - LOG2V);
         const int i = cidx / TL, j = cidx % TL;
         const int ri = r_cta0 + r_local0 + i, lj = lt * TL + j;
         const bool owner = (lane & ((1 << (5 - LOG2V)) - 1)) == 0;
         if (owner && ri < a.R && lj < a.NL) {
+            // the split's base plus its excess sum: sum V + sum max(kappa x + d, 0), or
+            // sum U + sum max(-(kappa x + d), 0)
             const double mu = fmin(s_lam[lj], cp), nu = fmin(s_lam[lj], cw);
             const double Nk = (double)a.N[k];
             const double eta_i = (double)a.r[ri] - (double)a.L_in[k];
-            double tot;
-            if constexpr (P == Prec::EXACT) {
-                tot = acc64;  // the branch sums, formed above
-            } else {
-                // the split's base plus its excess sum: sum V + sum max(kappa x + d, 0), or
-                // sum U + sum max(-(kappa x + d), 0)
-                const long long N64 = a.N[k], sx = a.sumx[k];
-                const double base = use_u_split(mu, nu)
-                                        ? cp * (Lk - eta_i) * Nk - mu * (double)((long long)a.L[k] * N64 - sx)
-                                        : cw * eta_i * Nk - nu * (double)sx;
-                tot = base + acc64;
-            }
-            const double S = tot * s_inv_n;
+            const long long N64 = a.N[k], sx = a.sumx[k];
+            const double base = use_u_split(mu, nu) ? cp * (Lk - eta_i) * Nk - mu * (double)((long long)a.L[k] * N64 - sx)
+                                                    : cw * eta_i * Nk - nu * (double)sx;
+            const double tot = base + acc64;
+            const double S = __dmul_rn(tot, a.inv_n[k]);
             s_S[(r_local0 + i) * NLpad + lj] = S;
             if (a.S_out) {
                 const size_t o = (((size_t)m * a.K + k) * a.R + ri) * a.NL_out + a.lam0 + lj;
-                if (P == Prec::F32 || a.f32_out) static_cast<float*>(a.S_out)[o] = (float)S;
+                if (P == Prec::F32) static_cast<float*>(a.S_out)[o] = (float)S;
                 else static_cast<double*>(a.S_out)[o] = S;
             }
         }
@@ -786,107 +888,230 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
 // The same cells in O(1) each from the class's cumulative counts C[v] = #{x <= v} and sums
 // CS[v] = sum_{x <= v} x: the samples with kappa x + d > 0 are exactly x >= t for the integer
 // threshold t, so sum_n max(kappa x_n + d, 0) = kappa (sum - CS[t-1]) + d (N - C[t-1]).
-constexpr int kEnvR = 8;          // r values per CTA
+//
+// The FP64 pipe bounds it, so a cell whose samples all lie on one branch of phi -- an FP32 look at its
+// offset settles most of those -- costs three FP64 instructions (one product less its row's
+// rounded constant, and 1 / N) and the others about twelve; what depends on the reservation or on
+// lam alone is formed once per CTA, and the minimum over lam leaves about one value per
+// (r, eps) pair to FP64.
+//
+// A warp takes 2 passes of 32 / W rows, W lanes along lam each (W: NL rounded up to a power of two, at
+// most 32), so small lam grids fill the warp with rows.
 constexpr int kEnvThreads = 256;
-constexpr int kEnvTable = 4096;   // lam * eps products kept in shared memory when NL * E is at most this
+constexpr int kEnvPasses = 2;
 
-// Order key of a double for the minimum over lam: equal for equal values (-0 is taken as +0) and
-// ordered as the values are for every non-NaN double, so the comparison runs on integers instead
-// of the FP64 pipe (which this part executes at 2 operations per clock per SM).
-__device__ __forceinline__ long long order_key(double v) {
-    long long b = __double_as_longlong(v);
-    if (b == (long long)0x8000000000000000ull) b = 0;
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+__host__ __device__ inline int env_width(int NL) {
+    int w = 1;
+    while (w < NL && w < 32) w <<= 1;
+    return w;
 }
+__host__ __device__ inline int env_rows(int NL) { return kEnvPasses * kEnvThreads / env_width(NL); }
 
-// The envelope kernel's epilogue: each thread takes whole (r, eps) pairs and scans lam in
-// ascending order with a strict comparison, so ties keep the lowest index (as cta_epilogue's
-// reduction does); the cost of every lam is lam * eps + S, rounded as there.  One FP64 add per
-// (r, eps, lam) when the CTA holds the lam * eps products (s_le, [lam][eps]), else a multiply and
-// an add; no shuffles.
-__device__ __forceinline__ void env_epilogue(const GridArgs& a, const double* s_S, const double* s_lam,
-                                             const double* s_eps, const double* s_le, int r_cta0, int m, int k) {
-    for (int p = threadIdx.x; p < kEnvR * a.E; p += blockDim.x) {
-        const int rl = p / a.E, e = p % a.E;
-        const int ri = r_cta0 + rl;
-        if (ri >= a.R) continue;
-        const double eps = s_eps[e];
-        const double* S = s_S + rl * a.NL;
-        double best = __dadd_rn(s_le ? s_le[e] : __dmul_rn(s_lam[0], eps), S[0]);
-        long long best_key = order_key(best);
-        int bj = 0;
-        if (s_le) {
-            for (int j = 1; j < a.NL; j++) {
-                const double v = __dadd_rn(s_le[j * a.E + e], S[j]);
-                const long long key = order_key(v);
-                if (key < best_key) {
-                    best_key = key;
-                    best = v;
-                    bj = j;
-                }
-            }
-        } else {
-            for (int j = 1; j < a.NL; j++) {
-                const double v = __dadd_rn(__dmul_rn(s_lam[j], eps), S[j]);
-                const long long key = order_key(v);
-                if (key < best_key) {
-                    best_key = key;
-                    best = v;
-                    bj = j;
-                }
-            }
-        }
-        const size_t row = ((size_t)m * a.E + e) * a.K + k;
-        const size_t o = row * a.R + ri;
-        static_cast<double*>(a.cost_out)[o] = best;
-        if (a.lam_idx_out) a.lam_idx_out[o] = bj + a.lam0;
-        const u64 key = ((u64)__double_as_longlong(best > 0.0 ? best : 0.0) & ~0xFFFFFull) | (u64)ri;
-        atomicMin(a.keys + row, key);
-    }
+struct EnvRow {
+    RowOffset off;
+    double pv, ev, pu, eu;  // c_w eta N and c_p (L - eta) N: rounded product and its error
+    float cp_le, cw_eta;
+    int eta, pad;
+};
+struct EnvSmem {
+    size_t kap, eps, S, row, muf, kapf, lamf, Sf, total;
+    int stride, stride_f;  // elements per row of S and Sf
+};
+__host__ __device__ inline EnvSmem env_smem(int NL, int E) {
+    EnvSmem s;
+    const int rows = env_rows(NL), n4 = (NL + 3) & ~3;
+    s.stride = NL | 1;  // odd: rows start in other banks
+    s.stride_f = 4 * (n4 / 4 | 1);  // read four at a time, lanes along the rows
+    s.kap = 8 * (size_t)NL;
+    s.eps = s.kap + 8 * (size_t)NL;
+    s.S = s.eps + 8 * (size_t)E;
+    s.row = s.S + 8 * (size_t)rows * s.stride;
+    s.lamf = (s.row + sizeof(EnvRow) * rows + 15) & ~(size_t)15;
+    s.Sf = s.lamf + 4 * (size_t)n4;
+    s.muf = s.Sf + 4 * (size_t)rows * s.stride_f;
+    s.kapf = s.muf + 4 * (size_t)NL;
+    s.total = s.kapf + 4 * (size_t)NL;
+    return s;
 }
 
 __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
-    extern __shared__ __align__(16) double esm[];
-    double* s_lam = esm;
-    double* s_eps = s_lam + a.NL;
-    double* s_S = s_eps + a.E;
+    extern __shared__ __align__(16) unsigned char esm[];
+    __shared__ int s_bad[2];  // some magnitude the floats do not hold: in the inputs, in S
+    __shared__ int s_first_sat, s_unsorted;
+    const EnvSmem lay = env_smem(a.NL, a.E);
+    double* s_lam = reinterpret_cast<double*>(esm);
+    double* s_kap = reinterpret_cast<double*>(esm + lay.kap);
+    double* s_eps = reinterpret_cast<double*>(esm + lay.eps);
+    double* s_S = reinterpret_cast<double*>(esm + lay.S);
+    EnvRow* s_row = reinterpret_cast<EnvRow*>(esm + lay.row);
+    float* s_lamf = reinterpret_cast<float*>(esm + lay.lamf);
+    float* s_Sf = reinterpret_cast<float*>(esm + lay.Sf);
+    float* s_muf = reinterpret_cast<float*>(esm + lay.muf);
+    float* s_kapf = reinterpret_cast<float*>(esm + lay.kapf);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int b = blockIdx.x;
     const int rb = b % a.r_blocks;
     b /= a.r_blocks;
     const int k = b % a.K;
     const int m = a.m0 + b / a.K;
-    const int r_cta0 = rb * kEnvR;
-    for (int i = threadIdx.x; i < a.NL; i += blockDim.x) s_lam[i] = a.lam[i];
-    for (int i = threadIdx.x; i < a.E; i += blockDim.x) s_eps[i] = a.eps[i];
-    __syncthreads();
-    double* s_le = a.NL * a.E <= kEnvTable ? s_S + kEnvR * a.NL : nullptr;  // [lam][eps] products
-    if (s_le)
-        for (int i = threadIdx.x; i < a.NL * a.E; i += blockDim.x) s_le[i] = __dmul_rn(s_lam[i / a.E], s_eps[i % a.E]);
+    const int NL = a.NL, W = env_width(NL), max_rows = env_rows(NL);
+    const int r_cta0 = rb * max_rows, rows = min(max_rows, a.R - r_cta0);
     const double cp = a.cp[m], cw = a.cw[m];
-    const int32_t Lk = a.L[k];
-    const int64_t Nk = a.N[k];
-    const double N = (double)Nk, inv_n = 1.0 / N;
-    const int32_t* C = a.cdf + a.hist_off[k];
-    const int64_t* CS = a.csum + a.hist_off[k];
-    for (int cell = threadIdx.x; cell < kEnvR * a.NL; cell += blockDim.x) {
-        const int rl = cell / a.NL, j = cell % a.NL;
-        const int ri = r_cta0 + rl;
-        if (ri >= a.R) continue;
-        const double eta = (double)a.r[ri] - (double)a.L_in[k];
-        const double lam = s_lam[j];
-        const double mu = fmin(lam, cp), nu = fmin(lam, cw), kap = mu + nu;
-        const double d = excess_offset(cp, cw, mu, (double)Lk, eta);
-        const int64_t t = first_active(kap, d, Lk);  // first active sample value, in [0, L + 1]
-        const int64_t below_n = t >= 1 ? (int64_t)C[t - 1] : 0;
-        const int64_t below_s = t >= 1 ? CS[t - 1] : 0;
-        const int64_t cnt = Nk - below_n, sx = a.sumx[k] - below_s;  // samples from t on, and their sum
-        const double tot = branch_sum(cp, cw, mu, nu, (double)Lk, eta, N, cnt, below_s, (int64_t)Lk * cnt - sx);
-        const double S = tot * inv_n;
-        s_S[rl * a.NL + j] = S;
-        if (a.S_out) static_cast<double*>(a.S_out)[(((size_t)m * a.K + k) * a.R + ri) * a.NL_out + a.lam0 + j] = S;
+    const int L = a.L[k];
+    const long long N = a.N[k], sumx = a.sumx[k];
+    if (tid < 2) s_bad[tid] = 0;
+    if (tid == 0) {
+        s_first_sat = a.NL - 1;
+        s_unsorted = 0;
     }
     __syncthreads();
-    env_epilogue(a, s_S, s_lam, s_eps, s_le, r_cta0, m, k);
+    bool ok = true;
+    for (int i = tid; i < rows; i += kEnvThreads) {
+        const int eta = a.r[r_cta0 + i] - a.L_in[k];
+        EnvRow w;
+        w.off = row_offset(cp, cw, L, eta);
+        const double iv = to_double((long long)eta * N), iu = to_double((long long)(L - eta) * N);
+        w.pv = __dmul_rn(cw, iv);
+        w.ev = fma(cw, iv, -w.pv);
+        w.pu = __dmul_rn(cp, iu);
+        w.eu = fma(cp, iu, -w.pu);
+        w.cp_le = cut(w.off.cp_le, ok);
+        w.cw_eta = cut(w.off.cw_eta, ok);
+        w.eta = eta;
+        s_row[i] = w;
+    }
+    for (int i = tid; i < NL; i += kEnvThreads) {
+        const double l = a.lam[i], mu = dmin_nonneg(l, cp), nu = dmin_nonneg(l, cw), kap = __dadd_rn(mu, nu);
+        s_lam[i] = l;
+        s_kap[i] = kap;
+        if (dbits(l) >= dbits(cp) && dbits(l) >= dbits(cw)) atomicMin(&s_first_sat, i);
+        if (i > 0 && !(dbits(a.lam[i - 1]) <= dbits(l))) s_unsorted = 1;
+        s_lamf[i] = cut(l, ok);
+        s_muf[i] = cut(mu, ok);
+        s_kapf[i] = cut(kap, ok);
+    }
+    for (int i = tid; i < a.E; i += kEnvThreads) s_eps[i] = a.eps[i];
+    if (!ok) s_bad[0] = 1;
+    __syncthreads();
+    const bool floats = s_bad[0] == 0;
+    // Every lam from max(c_p, c_w) on gives the same S (mu = c_p, nu = c_w), and in an ascending grid the
+    // first of them costs least at every radius, with the lowest index: the rest need no evaluation.
+    const int NLs = s_unsorted ? NL : s_first_sat + 1;
+    const double inv_n = a.inv_n[k], Ld = to_double(L), sumx_d = to_double(sumx);
+    const long long dist_all = (long long)L * N - sumx;
+    const double dist_d = to_double(dist_all);
+    const float Lf = (float)L;
+    const int32_t* C = a.cdf + a.hist_off[k];
+    const int64_t* CS = a.csum + a.hist_off[k];
+    for (int rl = warp * (32 / W) + lane / W; rl < rows; rl += kEnvThreads / W) {
+        const EnvRow& w = s_row[rl];
+        for (int j = lane & (W - 1); j < NLs; j += W) {
+            const double lam = s_lam[j], mu = dmin_nonneg(lam, cp), nu = dmin_nonneg(lam, cw);
+            // d in FP32, off by at most 2^-21 of the sum of its parts: far enough from zero, and kappa L + d
+            // likewise, it tells that every sample is active (t = 0) or that none is (t = L + 1)
+            const float part = fmaf(s_muf[j], Lf, w.cw_eta), d = w.cp_le - part, parts = w.cp_le + part;
+            const float top = fmaf(s_kapf[j], Lf, d);
+            int t;
+            if (floats && parts > 0x1p-40f && d > 0x1p-20f * parts) t = 0;
+            else if (floats && parts > 0x1p-40f && top < -0x1p-19f * parts) t = L + 1;
+            else t = first_active(s_kap[j], excess_offset(w.off, cp, mu, Ld), L);
+            const bool inside = t >= 1 && t <= L;
+            const long long below_n = inside ? (long long)C[t - 1] : (t >= 1 ? N : 0);
+            const long long cnt = N - below_n;  // samples from t on
+            // sum phi: the branch sums (branch_sum) with the row's own products where one branch holds all
+            double p = cnt == 0 ? w.pv : w.pu, e = cnt == 0 ? w.ev : w.eu, mul = cnt == 0 ? nu : mu;
+            double by = cnt == 0 ? sumx_d : dist_d;
+            long long below_s = 0;
+            const bool both = cnt > 0 && cnt < N;
+            if (both) {
+                below_s = CS[t - 1];
+                const double i = to_double((long long)w.eta * below_n);
+                p = __dmul_rn(cw, i);
+                e = fma(cw, i, -p);
+                mul = nu;
+                by = to_double(below_s);
+            }
+            double tot = __dadd_rn(fma(-mul, by, p), e);
+            if (both)
+                tot = __dadd_rn(tot, diff_of_products(cp, to_double((long long)(L - w.eta) * cnt), mu,
+                                                      to_double((long long)L * cnt - (sumx - below_s))));
+            const double S = __dmul_rn(tot, inv_n);
+            s_S[rl * lay.stride + j] = S;
+            s_Sf[rl * lay.stride_f + j] = cut(S, ok);
+            if (a.S_out) {
+                double* out = static_cast<double*>(a.S_out) + (((size_t)m * a.K + k) * a.R + r_cta0 + rl) * a.NL_out + a.lam0;
+                out[j] = S;
+                if (j == NLs - 1)
+                    for (int i = NLs; i < NL; i++) out[i] = S;
+            }
+        }
+        for (int j = NLs + (lane & (W - 1)); j < ((NLs + 3) & ~3); j += W) s_Sf[rl * lay.stride_f + j] = INFINITY;
+    }
+    for (int j = NL + tid; j < ((NL + 3) & ~3); j += kEnvThreads) s_lamf[j] = 0.f;
+    if (!ok) s_bad[1] = 1;
+    __syncthreads();
+    // G lanes per (r, eps) pair, as many as keep every thread busy, groups along r first (coalesced outputs,
+    // one atomic per warp and radius); each lane takes every G-th four lam values and keeps its smallest v', where it was, and its second smallest: with the second outside the
+    // window only that one value is formed in FP64, by all lanes at once.
+    const int pairs = rows * a.E, n4 = (NLs + 3) / 4;
+    int G = 1;
+    while (G < 32 && G < n4 && 2 * G * pairs <= kEnvThreads) G <<= 1;
+    const int per_pass = kEnvThreads / G, g = tid & (G - 1);
+    for (int p0 = 0; p0 < pairs; p0 += per_pass) {  // the same trips for every lane: the group's shuffles are warp-wide
+        const int p = p0 + tid / G;
+        const bool active = p < pairs;
+        const int e = active ? p / rows : 0, rl = active ? p % rows : 0;
+        const double* S = s_S + rl * lay.stride;
+        const double eps = s_eps[e];
+        const float4* lam4 = reinterpret_cast<const float4*>(s_lamf);
+        const float4* S4 = reinterpret_cast<const float4*>(s_Sf + rl * lay.stride_f);
+        bool fast = floats && s_bad[1] == 0;
+        const float ef = cut(eps, fast);
+        float m1 = INFINITY, m2 = INFINITY;
+        int j1 = 0;
+        for (int q = g; q < n4; q += G) {
+            const float4 l = lam4[q], s = S4[q];
+            const float v[4] = {fmaf(l.x, ef, s.x), fmaf(l.y, ef, s.y), fmaf(l.z, ef, s.z), fmaf(l.w, ef, s.w)};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                m2 = fminf(m2, fmaxf(m1, v[i]));
+                if (v[i] < m1) j1 = 4 * q + i;
+                m1 = fminf(m1, v[i]);
+            }
+        }
+        for (int o = 1; o < G; o <<= 1) {
+            const float o1 = __shfl_xor_sync(0xffffffffu, m1, o), o2 = __shfl_xor_sync(0xffffffffu, m2, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, j1, o);
+            m2 = fminf(fminf(m2, o2), fmaxf(m1, o1));
+            if (o1 < m1 || (o1 == m1 && oj < j1)) j1 = oj;
+            m1 = fminf(m1, o1);
+        }
+        fast = fast && m1 > kLamFloor;
+        const float thr = m1 * kLamWindow;
+        LamMin best;
+        if (fast && m2 > thr) {
+            best.v = __dadd_rn(__dmul_rn(s_lam[j1], eps), S[j1]);
+            best.j = j1;
+        }
+        const bool several = active && best.j == 0x7fffffff;
+        if (__any_sync(0xffffffffu, several)) {
+            LamMin r;
+            if (several)
+                for (int j = g; j < NLs; j += G)
+                    if (!fast || fmaf(s_lamf[j], ef, s_Sf[rl * lay.stride_f + j]) <= thr)
+                        r.take(s_lam[j], eps, S[j], j, fast, s_lam, S);
+            r.reduce(G);
+            if (several) best = r;
+        }
+        u64 key = ~0ull;
+        if (active && g == 0) key = write_pair<false>(a, best.v, best.j, m, k, e, r_cta0 + rl);
+        // the warp's minimum over each radius it holds, e0 (its first lane's) upwards
+        const int e0 = __shfl_sync(0xffffffffu, e, 0), e1 = __reduce_max_sync(0xffffffffu, e);
+        for (int ei = e0; ei <= e1; ei++) {
+            const u64 low = group_min(e == ei ? key : ~0ull, 32);
+            if (lane == 0 && low != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + ei) * a.K + k, low);
+        }
+    }
 }
 
 template <Prec P>
@@ -923,7 +1148,7 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
     sh.RG = sh.LT >= kWarpsTarget ? 1 : kWarpsTarget / sh.LT;
     sh.threads = 32 * sh.LT * sh.RG;
     sh.r_blocks = (R + sh.RG * C::TR - 1) / (sh.RG * C::TR);
-    sh.smem = smem_layout(sh.RG, C::TR, sh.LT * C::TL, E, C::CHUNK, C::STAGES).total;
+    sh.smem = smem_layout(sh.RG, C::TR, sh.LT * C::TL, E, C::CHUNK * C::BYTES, C::STAGES).total;
     return sh;
 }
 
@@ -934,37 +1159,42 @@ GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L) {
         sh.LT = 1;
         sh.RG = 1;
         sh.threads = kEnvThreads;
-        sh.r_blocks = (R + kEnvR - 1) / kEnvR;
-        sh.smem = 8 * ((size_t)NL + E + (size_t)kEnvR * NL + ((int64_t)NL * E <= kEnvTable ? (size_t)NL * E : 0));
+        sh.r_blocks = (R + env_rows(NL) - 1) / env_rows(NL);
+        sh.smem = env_smem(NL, E).total;
         return sh;
     }
     if (p == Prec::F64) return shape_for<CfgF64>(2, R, NL, E);
     if (p == Prec::EXACT) {  // NL <= kExactLamBlock: larger grids launch in blocks
-        if (NL <= kFewLam) return shape_for<CfgExactFewLam>(8, R, NL, E);
-        if (max_L > kExactIntAboveL) return shape_for<CfgExactInt>(6, R, NL, E);
-        return shape_for<CfgExact>(3, R, NL, E);
+        if (max_L > kPairMaxL) return NL <= kFewLam ? shape_for<CfgExactIntFewLam>(9, R, NL, E) : shape_for<CfgExactInt>(6, R, NL, E);
+        return NL <= kFewLam ? shape_for<CfgExactFewLam>(8, R, NL, E) : shape_for<CfgExact>(3, R, NL, E);
     }
     if (NL <= kWarpsTarget * CfgF32::TL) return shape_for<CfgF32>(0, R, NL, E);
     return shape_for<CfgF32Wide>(1, R, NL, E);
 }
 
+// Raises the kernel's shared-memory limit to the largest layout its shapes can have: all of its warps,
+// 64 eps.
+template <class C>
+cudaError_t prepare() {
+    const int warps = C::MAXT / 32;
+    return cudaFuncSetAttribute(k_grid<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_layout(1, C::TR, warps * C::TL, 64, C::CHUNK * C::BYTES, C::STAGES).total + 256);
+}
+
 cudaError_t grid_prepare(Prec p) {
-    // the largest layout any variant can need: 16 warps, 256 lam, 64 eps
-    const int mx = (int)(smem_layout(16, 2, 256, 64, 4096, 4).total + 4096);
-    if (p == Prec::F64) return cudaFuncSetAttribute(k_grid<CfgF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    if (p == Prec::F64) return prepare<CfgF64>();
     if (p == Prec::EXACT) {
-        cudaError_t e = cudaFuncSetAttribute(k_grid<CfgExact>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_grid<CfgExactInt>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_grid<CfgExactFewLam>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaError_t e = prepare<CfgExact>();
+        if (e == cudaSuccess) e = prepare<CfgExactInt>();
+        if (e == cudaSuccess) e = prepare<CfgExactFewLam>();
+        if (e == cudaSuccess) e = prepare<CfgExactIntFewLam>();
         return e;
     }
     if (p == Prec::ENVELOPE)
         return cudaFuncSetAttribute(k_envelope, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(8 * (256 + 64 + (size_t)kEnvR * 256 + kEnvTable)));
-    cudaError_t e = cudaFuncSetAttribute(k_grid<CfgF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_grid<CfgF32Wide>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+                                    (int)env_smem(256, 64).total);
+    const cudaError_t e = prepare<CfgF32>();
+    return e == cudaSuccess ? prepare<CfgF32Wide>() : e;
 }
 
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s) {
@@ -977,6 +1207,7 @@ cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s)
     else if (p == Prec::F64) k_grid<CfgF64><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (p == Prec::EXACT && sh.variant == 3) k_grid<CfgExact><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (p == Prec::EXACT && sh.variant == 8) k_grid<CfgExactFewLam><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
+    else if (p == Prec::EXACT && sh.variant == 9) k_grid<CfgExactIntFewLam><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (p == Prec::EXACT) k_grid<CfgExactInt><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (sh.variant == 0) k_grid<CfgF32><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else k_grid<CfgF32Wide><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);

@@ -6,12 +6,15 @@
 
 namespace kvdro {
 
-// Samples of one class are staged for the grid kernel as (x', x') float pairs, x' the sample plus
-// the class's staging offset (stage_offset below), so that one 128-bit shared-memory load yields
-// the packed operands of two samples.  Each class region starts on a multiple of kPadSamples and
-// is padded with NaN pairs, which contribute exactly zero to the per-term kernels' excess sums
-// (max(NaN, 0) = 0 in PTX max.f32 / max.f64); the exact kernel reads the padding as x = 0 and
-// subtracts its known |0 - c| per cell.
+// Samples of one class are staged for the grid kernel in regions of a multiple of kPadSamples, in one
+// of two forms, the same for every class of a context.
+//  - Pair sums, where the largest support is at most kPairMaxL: four samples a, b, c, d in 16 bytes as
+//    the floats {a + b, c + d, |a - b|, |c - d|}, each an integer below 2^24; samples past the class's
+//    last are 0, and the exact kernel subtracts their known |0 - c| per cell.
+//  - (x', x') float pairs above, x' the sample plus the class's staging offset (stage_offset below), so
+//    that one 128-bit shared-memory load yields the packed operands of two samples, padded with NaN
+//    pairs, which contribute exactly zero to the per-term kernels' excess sums (max(NaN, 0) = 0 in PTX
+//    max.f32 / max.f64); the exact kernel reads the padding as x = 0.
 constexpr int kPadSamples = 128;
 
 // Error bits reported by kernels in ctx->d_err[1].
@@ -22,19 +25,22 @@ struct SortArgs {
     const int64_t* offsets;     // [K+1]
     const int32_t* L;           // [K]
     const int64_t* hist_off;    // [K+1] start of class k's cumulative-count array (L_k + 1 entries)
-    const int64_t* pair_off;    // [K+1] start of class k's padded pair region
+    const int64_t* pair_off;    // [K+1] start of class k's padded region, in samples
     const int32_t* hist_blocks; // [K+1] prefix of histogram blocks per class
     const int32_t* exp_blocks;  // [K+1] prefix of expand blocks per class
     int32_t* hist;              // [hist_off[K]] counts, then cumulative counts (in place)
     int64_t* csum;              // [hist_off[K]] cumulative sums sum_{x <= v} x, or nullptr to skip
     int64_t* sumx;              // [K] sum of samples per class
     int32_t* sorted;            // [offsets[K]]
-    float2* pairs;              // [pair_off[K]]
+    void* staged;               // pair_off[K] samples, 4 bytes each as pair sums or 8 as (x', x') pairs
     int32_t* err;               // [0] += out-of-range samples
     int64_t* tile_tot;          // [K][scan_tiles][2] scan tile totals (count, sum of v h[v])
     int32_t* tile_lo;           // [exp_blocks[K] + K] per class from exp_blocks[k] + k: the bin of the
                                 // first position of each expansion tile, then the bin of position N - 1
+    double* inv_n;              // [K] 1 / N written by the expansion, or nullptr to skip (may lie over
+                                // tile_tot, which the expansion does not read)
     int32_t scan_tiles;         // scan tiles of the largest class: ceil((max L + 1) / scan tile bins)
+    int32_t pair_sums;          // the staged form
     int32_t K;
 };
 
@@ -48,25 +54,31 @@ cudaError_t launch_gather_quantiles(const int32_t* sorted, const int64_t* offset
                                     int32_t F, int32_t* out, cudaStream_t s);
 
 // F32: per-term FP32 excess sums folded into FP64.  F64: per-term FP64.  EXACT: an exact integer
-// threshold per cell, then per term an exact sum of |x - c| (packed FP32 adds and integer
-// absolute differences side by side on two pipes), combined in FP64.
+// threshold per cell, then an exact sum of |x - c| over the samples (two samples at a time in packed
+// FP32 adds and a max, or one at a time in integer absolute differences), combined in FP64.
 // ENVELOPE: the same sums in O(1) per cell from cumulative counts and sums (not per term).
 enum class Prec { F32 = 0, F64 = 1, EXACT = 2, ENVELOPE = 3 };
 constexpr int32_t kExactMaxL = 1 << 22;  // the exact kernel's integer sums need L <= 2^22
 
-// Samples of a class whose support is at most kExactMaxL are staged as x + 2^23.  On [2^23, 2^24)
-// a float's bit pattern is 0x4B000000 + x exactly, so the staged float serves both halves of the
-// exact kernel without a conversion: packed FP32 adds on the value, integer absolute differences
-// on the bits.  Larger supports are staged as x.  The FP32 and FP64 per-term kernels subtract
-// the class's offset (exactly) from every sample.
+// Up to a support of kPairMaxL a lane's FP32 sums of |a - c| + |b - c| stay exact (below 2^24) over at
+// least 7 loads of four samples between folds; the integer sums of larger supports fold every 8 loads
+// of two at most.
+constexpr int32_t kPairMaxL = 1 << 19;
+
+// In the (x', x') form, samples of a class whose support is at most kExactMaxL carry an offset of 2^23.
+// On [2^23, 2^24) a float's bit pattern is 0x4B000000 + x exactly, so the exact kernel's integer
+// absolute differences work on the bits without a conversion.  Larger supports are staged as x.  The
+// FP32 and FP64 per-term kernels subtract the class's offset (exactly) from every sample.
 constexpr float kStageOffset = 8388608.0f;  // 2^23
 constexpr int32_t kStageBits = 0x4B000000;  // bit pattern of 2^23
 __host__ __device__ inline float stage_offset(int32_t L) { return L <= kExactMaxL ? kStageOffset : 0.0f; }
 
 struct GridArgs {
-    const float2* pairs;        // padded (x', x') pairs, x' = x + stage_offset(L_k)
-    const int64_t* pair_off;    // [K+1]
+    const void* staged;         // the padded samples
+    const int64_t* pair_off;    // [K+1] in samples
+    int32_t pair_sums;          // the staged form
     const int64_t* N;           // [K]
+    const double* inv_n;        // [K] 1 / N
     const int64_t* sumx;        // [K]
     const int32_t* L;           // [K]
     const int32_t* L_in;        // [K]
@@ -145,6 +157,7 @@ struct DualArgs {
     const int64_t* csum;        // cumulative sums, same layout
     const int64_t* hist_off;    // [K+1]
     const int64_t* N;           // [K]
+    const double* inv_n;        // [K] 1 / N
     const int64_t* sumx;        // [K]
     const int32_t* L;           // [K]
     const int32_t* L_in;        // [K]
@@ -161,6 +174,53 @@ cudaError_t launch_dual(const DualArgs& a, cudaStream_t s);
 
 
 #ifdef __CUDACC__
+// Every FP64-pipe instruction -- add, multiply, FMA, compare, minimum and each conversion from or to
+// double -- runs at 1.6 to 1.9 lanes per clock per SM on this part, a warp's 32 lanes in about 64
+// cycles of its scheduler's share, where an integer instruction takes 2.  The per-cell code
+// therefore compares, converts and takes minima of doubles on their bit patterns and leaves to the
+// FP64 pipe only the roundings that the results are made of.
+__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ bool dpos(double v) { return dbits(v) > 0; }  // v > 0 (v not NaN)
+// min(a, b) for a, b >= 0, not NaN
+__device__ __forceinline__ double dmin_nonneg(double a, double b) { return dbits(a) < dbits(b) ? a : b; }
+
+// (double)v, v >= 0: normalised by its leading zeros and packed, exact below 2^53 (every count and
+// sum of ordinary problems); the conversion instruction rounds the larger ones.
+__device__ __forceinline__ double to_double(long long v) {
+    if (v >= (1ll << 53)) return (double)v;
+    const int lz = __clzll(v);                                    // 64 for v = 0
+    const unsigned long long m = (unsigned long long)v << (lz & 63);  // leading one at bit 63
+    const unsigned long long b = ((unsigned long long)(1086 - lz) << 52) + ((m >> 11) & 0xFFFFFFFFFFFFFull);
+    return __longlong_as_double(v == 0 ? 0ll : (long long)b);
+}
+__device__ __forceinline__ double to_double(int v) { return to_double((long long)v); }
+
+// Magnitude of a double whose exponent lies in [-100, 100], cut to a float: relative error below 2^-23.
+__device__ __forceinline__ bool narrowable(long long b) {
+    const unsigned e = (unsigned)(b >> 52) & 0x7ff;
+    return e - (1023u - 100u) <= 200u;
+}
+__device__ __forceinline__ float narrow(long long b) {
+    return __uint_as_float((unsigned)((b & 0x7fffffffffffffffll) >> 29) - (896u << 23));
+}
+
+// Order key of a double: equal for equal values (-0 is taken as +0) and ordered as the values are
+// for every non-NaN double.
+__device__ __forceinline__ long long order_key(double v) {
+    long long b = __double_as_longlong(v);
+    if (b == (long long)0x8000000000000000ull) b = 0;
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// The smaller key over groups of G lanes (a power of two), in every lane.
+__device__ __forceinline__ unsigned long long group_min(unsigned long long key, int G) {
+    for (int o = 1; o < G; o <<= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
+        key = other < key ? other : key;
+    }
+    return key;
+}
+
 // The offset d = (c_p - mu) L - (c_p + c_w) eta of a cell's excess kappa x + d, evaluated as
 // c_p (L - eta) - (mu L + c_w eta): L - eta is an exact integer and every product is rounded once,
 // so a large c_p never swallows a small mu or c_w (the first form cancels to 0 at eta = L when
@@ -168,10 +228,20 @@ cudaError_t launch_dual(const DualArgs& a, cudaStream_t s);
 // mu = c_p the L terms vanish exactly and d = -(c_p + c_w) eta.  Every rounding is spelled out
 // (no contraction left to the compiler), so each call site gets the same d bit for bit: a
 // kernel that classifies samples twice at one multiplier (the dual's slope and value) must see
-// the same threshold both times.
-__device__ __forceinline__ double excess_offset(double cp, double cw, double mu, double L, double eta) {
-    const double cw_eta = __dmul_rn(cw, eta);
-    return mu == cp ? -__fma_rn(cp, eta, cw_eta) : __dsub_rn(__dmul_rn(cp, L - eta), __fma_rn(mu, L, cw_eta));
+// the same threshold both times.  What does not depend on mu is formed once per reservation.
+struct RowOffset {
+    double cw_eta, cp_le, d_sat;
+};
+__device__ __forceinline__ RowOffset row_offset(double cp, double cw, int L, int eta) {
+    RowOffset r;
+    const double e = to_double(eta);
+    r.cw_eta = __dmul_rn(cw, e);
+    r.cp_le = __dmul_rn(cp, to_double(L - eta));
+    r.d_sat = -__fma_rn(cp, e, r.cw_eta);
+    return r;
+}
+__device__ __forceinline__ double excess_offset(const RowOffset& r, double cp, double mu, double Ld) {
+    return dbits(mu) == dbits(cp) ? r.d_sat : __dsub_rn(r.cp_le, __fma_rn(mu, Ld, r.cw_eta));
 }
 
 // The same excess about the reservation: kappa x + d = kappa (x - eta) + W(eta), with
@@ -202,10 +272,16 @@ __device__ __forceinline__ double diff_of_products(double c, double i, double m,
     return fma(-m, j, p) + e;
 }
 
-__device__ __forceinline__ double branch_sum(double cp, double cw, double mu, double nu, double L, double eta,
-                                             double n, int64_t cnt, int64_t sx_below, int64_t dist_above) {
-    return diff_of_products(cw, eta * (n - (double)cnt), nu, (double)sx_below) +
-           diff_of_products(cp, (L - eta) * (double)cnt, mu, (double)dist_above);
+// A branch without samples is skipped: it would add exactly zero.
+__device__ __forceinline__ double branch_sum(double cp, double cw, double mu, double nu, int L, int eta, long long n,
+                                             long long cnt, long long sx_below, long long dist_above) {
+    double v = 0.0;
+    if (cnt < n) v = diff_of_products(cw, to_double((long long)eta * (n - cnt)), nu, to_double(sx_below));
+    if (cnt > 0) {
+        const double u = diff_of_products(cp, to_double((long long)(L - eta) * cnt), mu, to_double(dist_above));
+        v = cnt < n ? __dadd_rn(v, u) : u;
+    }
+    return v;
 }
 
 // The per-term kernels sum phi as a base plus excesses: sum V + sum max(U - V, 0), or
@@ -216,12 +292,11 @@ __device__ __forceinline__ bool use_u_split(double mu, double nu) { return nu > 
 
 // The first active support point of a cell: the smallest integer t in [0, L] with
 // kappa * t + d > 0, or L + 1 when there is none (kappa >= 0, so the condition is monotone in
-// t).  One FMA gives the sign of kappa * t + d exactly, so each test is exact.  An FP32 estimate
-// of -d / kappa (off by a few units at most for L <= 2^24) is corrected by at most 8 such tests
-// each way; should that not settle it, the FP64 quotient is corrected the same way.
-__device__ __forceinline__ int64_t first_active(double kappa, double d, int64_t L) {
-    if (d > 0.0) return 0;
-    if (!(kappa > 0.0) || !(fma(kappa, (double)L, d) > 0.0)) return L + 1;
+// t).  One FMA gives the sign of kappa * t + d exactly, so each test is exact.  settle_active finds
+// t from the FP32 quotient -d / kappa (off by a few units at most for L <= 2^24), corrected by at
+// most 8 tests each way; should that not settle it, the FP64 quotient is corrected the same way.
+static __device__ __noinline__ int settle_active(double kappa, double d, int L) {
+    if (!(fma(kappa, (double)L, d) > 0.0)) return L + 1;
     // here t is in [1, L]: kappa (t - 1) + d <= 0 < kappa t + d
     auto settle = [&](double q, int64_t& t) {
         const double e = floor(q) + 1.0;
@@ -231,9 +306,29 @@ __device__ __forceinline__ int64_t first_active(double kappa, double d, int64_t 
         return (t == 1 || !(fma(kappa, (double)(t - 1), d) > 0.0)) && fma(kappa, (double)t, d) > 0.0;
     };
     int64_t t;
-    if (settle((double)__fdiv_rn(-(float)d, (float)kappa), t)) return t;
+    if (settle((double)__fdiv_rn(-(float)d, (float)kappa), t)) return (int)t;
     (void)settle(-d / kappa, t);
-    return t;
+    return (int)t;
+}
+// Almost every cell needs no FP64 instruction for it.  |d| and kappa cut to floats are at most 2^-23
+// below their values and the quotient is within 2 ulp of theirs, so x0 = -d / kappa lies within
+// q (1 +- 3 x 2^-23), inside q (1 +- 2^-21) after the rounding of the two ends.  Below 2^20 that
+// interval is shorter than one and holds at most one integer n: with none, t is its floor plus one;
+// with n, the sign at n decides.
+__device__ __forceinline__ int first_active(double kappa, double d, int L) {
+    const long long db = dbits(d), kb = dbits(kappa);
+    if (db > 0) return db <= 0x7ff0000000000000ll ? 0 : L + 1;  // NaN is not positive
+    if (kb <= 0) return L + 1;
+    if ((db << 1) == 0) return 1;
+    if (!narrowable(db) || !narrowable(kb)) return settle_active(kappa, d, L);
+    const float q = __fdividef(narrow(db), narrow(kb));
+    const float lo = fmaf(q, -0x1p-21f, q), hi = fmaf(q, 0x1p-21f, q);
+    if (lo >= (float)L) return L + 1;  // (float)L is exact: L <= 2^24
+    if (!(q < 0x1p20f)) return settle_active(kappa, d, L);
+    const int n_lo = __float2int_rd(lo), n = __float2int_rd(hi);
+    int t = n + 1;
+    if (n_lo != n && dpos(fma(kappa, to_double(n), d))) t = n;
+    return min(t, L + 1);
 }
 #endif
 

@@ -278,10 +278,12 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     sa.csum = nullptr;  // cumulative sums are not needed here
     sa.sumx = reinterpret_cast<int64_t*>(S + o_sumx);
     sa.sorted = reinterpret_cast<int32_t*>(S + o_sorted);
-    sa.pairs = reinterpret_cast<float2*>(S + o_pairs);
+    sa.staged = S + o_pairs;  // of 8 bytes a sample as pair sums take 4
+    sa.pair_sums = max_L <= kvdro::kPairMaxL;
     sa.err = reinterpret_cast<int32_t*>(S + o_err);
     sa.tile_tot = reinterpret_cast<int64_t*>(S + o_tiles);
     sa.tile_lo = reinterpret_cast<int32_t*>(S + o_tile_lo);
+    sa.inv_n = reinterpret_cast<double*>(S + o_tiles);  // written once the scan is done with its tile totals
     sa.scan_tiles = (int32_t)scan_tiles;
     sa.K = K;
     NA_CUDA(kvdro::launch_histogram(sa, (int32_t)hist_blocks, s));
@@ -295,9 +297,11 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     // ---- the grid kernel (the exact one, FP32 outputs, whenever every support is at most 2^22;
     // else the FP32-arithmetic one) and the argmin finalisation
     kvdro::GridArgs a;
-    a.pairs = sa.pairs;
+    a.staged = sa.staged;
+    a.pair_sums = sa.pair_sums;
     a.pair_off = sa.pair_off;
     a.N = mt.N;
+    a.inv_n = sa.inv_n;
     a.sumx = sa.sumx;
     a.L = mt.L;
     a.L_in = mt.L_in;

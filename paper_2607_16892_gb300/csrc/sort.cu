@@ -5,8 +5,8 @@
 // output position p into the smallest v with C[v] > p.  The scan also records, for every tile of
 // kExpandTile output positions, the bin its first position falls in; the expansion then marks
 // where each bin's run of positions starts inside the tile and takes a running maximum, O(N + L)
-// in all.  It also writes the (x', x') float pairs that the grid kernel streams (x' = x plus the
-// class's staging offset), NaN-padded to a multiple of kPadSamples per class.
+// in all.  It also writes the samples in the form that the grid kernel streams (kvdro_internal.cuh),
+// padded to a multiple of kPadSamples per class.
 #include <math.h>
 
 #include <algorithm>
@@ -275,6 +275,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
     const int64_t p0 = q * kExpandTile;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t pend = min(Nk, p0 + kExpandTile);  // sample positions of this tile
+    if (a.inv_n && q == 0 && tid == 0) a.inv_n[k] = 1.0 / (double)Nk;
     if (p0 < Nk) {  // block-uniform
         const int32_t* tl = a.tile_lo + a.exp_blocks[k] + k;
         const int32_t v_lo = tl[q], v_hi = tl[q + 1];
@@ -320,17 +321,28 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
         int32_t* out = a.sorted + a.offsets[k];
         for (int64_t i = tid; i < pend - p0; i += kExpandThreads) out[p0 + i] = sv[i];
     }
+    const int64_t qend = min(padk, p0 + kExpandTile);  // padk and p0 are multiples of 128
+    if (a.pair_sums) {  // four positions per 16-byte store; 0 past the class's samples
+        float4* out = reinterpret_cast<float4*>(static_cast<float*>(a.staged) + a.pair_off[k]);
+        for (int64_t i = 4 * (int64_t)tid; p0 + i < qend; i += 4 * kExpandThreads) {
+            const int64_t pos = p0 + i;
+            int32_t x[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) x[j] = pos + j < Nk ? sv[i + j] : 0;
+            out[pos >> 2] = make_float4((float)(x[0] + x[1]), (float)(x[2] + x[3]), (float)abs(x[1] - x[0]),
+                                        (float)abs(x[3] - x[2]));
+        }
+        return;
+    }
     // the tile's (x', x') pairs, two positions per 16-byte store; NaN past the class's samples
-    float2* pr = a.pairs + a.pair_off[k];
+    float2* pr = static_cast<float2*>(a.staged) + a.pair_off[k];
     const float nan = __int_as_float(0x7fc00000);  // quiet NaN pad
     const float off = stage_offset(Lk);              // x + 2^23 is exact for L <= 2^22
-    const int64_t qend = min(padk, p0 + kExpandTile);  // padk is a multiple of 128: even
     for (int64_t i = 2 * (int64_t)tid; p0 + i < qend; i += 2 * kExpandThreads) {
         const int64_t pos = p0 + i;
         const float f0 = pos < Nk ? (float)sv[i] + off : nan;
         const float f1 = pos + 1 < Nk ? (float)sv[i + 1] + off : nan;
-        if (pos + 1 < qend) *reinterpret_cast<float4*>(pr + pos) = make_float4(f0, f0, f1, f1);
-        else pr[pos] = make_float2(f0, f0);
+        *reinterpret_cast<float4*>(pr + pos) = make_float4(f0, f0, f1, f1);  // qend is even
     }
 }
 

@@ -45,3 +45,50 @@ def test_fp64_requests(L, cost):
     if L <= 1 << 22:
         same = all(np.array_equal(v, got[k]) for k, v in run(w, kvdro.KVDRO_EXACT).items())
         assert same or cost > 2e294
+
+
+@pytest.mark.parametrize("nl", [1, 2, 3, 31, 32, 33, 64, 101, 256])
+@pytest.mark.parametrize("order", ["ascending", "shuffled", "repeated"])
+def test_envelope_lam_grids(nl, order):
+    """Lanes along lam and rows of r per warp (widths 1 to 32), the saturated tail of an ascending grid that
+    is not evaluated, and the FP32 look at the minimum over lam, against the exact kernel's results: the same
+    integer sums and roundings, so every output is the same bit for bit, lowest-index ties included."""
+    rng = np.random.default_rng(nl)
+    lam = np.logspace(-3, 2, nl)
+    if order == "shuffled":
+        rng.shuffle(lam)
+    elif order == "repeated":
+        lam = np.repeat(lam, 2)[:nl]
+    w = make([rng.integers(0, 4001, 700), rng.integers(0, 90, 41)], 4000, np.unique(rng.integers(0, 4001, 83)), lam,
+             np.concatenate([[0.0], np.logspace(0, 3, 1 + nl % 17)]), [10.0, 0.5, 0.0], [1.0, 2.0, 1.0])
+    exact, env = run(w, kvdro.KVDRO_EXACT), run(w, kvdro.KVDRO_ENVELOPE)
+    for key, v in exact.items():
+        assert np.array_equal(v, env[key]), key
+
+
+@pytest.mark.parametrize("scale", [1e-150, 1e-32, 1e-25, 1e28, 1e33, 1e150])
+def test_envelope_magnitudes(scale):
+    """Costs and multipliers around the ends of what the FP32 look at a minimum takes (2^+-100, 2^-80)."""
+    rng = np.random.default_rng(3)
+    w = make([rng.integers(0, 901, 300)], 900, np.arange(0, 901, 25), scale * np.logspace(-3, 1, 40), [0.0, 1.0, 70.0],
+             [10 * scale], [scale])
+    exact, env = run(w, kvdro.KVDRO_EXACT), run(w, kvdro.KVDRO_ENVELOPE)
+    for key, v in exact.items():
+        assert np.array_equal(v, env[key]), key
+    compare_full(w, env, O.solve(w), "fp64")
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 127, 128, 129, 8191, 8192, 8193, 24577])
+@pytest.mark.parametrize("L,nl", [(300, 9), (1 << 19, 1), (1 << 19, 9), ((1 << 19) + 1, 2), ((1 << 19) + 1, 9)])
+def test_exact_staged_forms(n, L, nl):
+    """Pair sums up to a support of 2^19 (4 samples to a load, 8192 to a chunk, zero padding) and (x', x')
+    pairs above, on 2 x 8 and 8 x 2 tiles: the sums of the exact and the envelope mode are the same integers,
+    so every output is the same bit for bit.  Samples at 0 and at the top of the support, against
+    reservations at both ends, make a lane's sums as large as they get between folds."""
+    rng = np.random.default_rng(n)
+    x = rng.integers(0, L + 1, n)
+    x[: n // 2] = L
+    w = make([x], L, [0, 1, L // 3, L - 1, L], np.logspace(-2, 2, nl), [0.0, 30.0], [10.0, 0.3], [1.0, 1.0])
+    exact, env = run(w, kvdro.KVDRO_EXACT), run(w, kvdro.KVDRO_ENVELOPE)
+    for key, v in exact.items():
+        assert np.array_equal(v, env[key]), key
