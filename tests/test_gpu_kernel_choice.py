@@ -92,3 +92,26 @@ def test_exact_staged_forms(n, L, nl):
     exact, env = run(w, kvdro.KVDRO_EXACT), run(w, kvdro.KVDRO_ENVELOPE)
     for key, v in exact.items():
         assert np.array_equal(v, env[key]), key
+
+
+@pytest.mark.parametrize("L", [1, 2, 7, 400])
+@pytest.mark.parametrize("cp,cw", [(10.0, 1.0), (1.0, 10.0), (3.0, 3.0), (5.0, 0.0), (0.0, 5.0), (0.0, 0.0), (1e6, 1.0),
+                                   (1.0, 1e6)])
+def test_dual_on_each_side_of_the_smaller_cost(L, cp, cw):
+    """The search runs below min(c_p, c_w) or between the costs, over thresholds that rise or fall with gamma,
+    with minima at 0, at the smaller cost, at the larger and between; every integer r, radii from 0 past L."""
+    rng = np.random.default_rng(L)
+    w = make([rng.integers(0, L + 1, 60), np.full(5, L), np.zeros(4)], L, np.arange(L + 1), [1.0],
+             np.concatenate([[0.0], np.logspace(-3, np.log10(2.0 * L + 1.0), 37)]), cp, cw)
+    ctx = kvdro.kvdro_create(0)
+    try:
+        kvdro.kvdro_load_samples(ctx, w.K, w.offsets, torch.from_numpy(w.samples).cuda(), w.L, w.L_in)
+        shape = (1, len(w.eps), w.K, len(w.r))
+        cost, gamma = np.empty(shape), np.empty(shape)
+        kvdro.kvdro_eval_dual(ctx, len(w.r), w.r, len(w.eps), w.eps, 1, w.cp, w.cw, cost=cost, gamma=gamma)
+    finally:
+        kvdro.kvdro_destroy(ctx)
+    ref = O.solve_dual(w)["cost"]
+    size = cw * L + cp * L + max(cp, cw) * L  # the lines that cross at a minimiser are no larger
+    assert np.all(np.abs(cost - ref) <= 1e-12 * np.abs(ref) + 16 * np.finfo(float).eps * size)
+    assert np.all((gamma >= 0) & (gamma <= max(cp, cw)))
