@@ -36,7 +36,6 @@ constexpr int32_t kMaxF = 65536;
 constexpr int64_t kMaxKF = 1 << 22;
 constexpr long long kTestWaitNs = 1000000;  // the wait test's bound: 1 ms
 constexpr int32_t kMaxNLf32 = 256;
-constexpr int64_t kPartBytes = 256LL << 20;  // cap of the running-minimum buffer of lam blocks
 constexpr int32_t kMaxNLf64 = 128;
 // Host outputs of a grid over several regimes return in up to this many regime blocks, each
 // copied while the next evaluates.
@@ -51,6 +50,7 @@ struct Buf {
 
 struct kvdro_ctx {
     int device = 0;
+    int sms = 0;  // of the device
     std::string err;
     int fail_after = -1;  // test hook: the fail_after-th allocation of this context fails
     int skip_chunk = -1;  // test hook: grid kernels never copy this chunk, so their waits run out
@@ -65,7 +65,7 @@ struct kvdro_ctx {
     std::vector<int32_t> L, Lin, hist_blocks, exp_blocks;
     std::vector<double> inv_n;
 
-    Buf sorted, pairs, hist, csum, sumx, meta, errs, in_stage, grid_in, keys, cost64, out_stage, ranks, scan_tot, part,
+    Buf sorted, pairs, hist, csum, sumx, meta, errs, in_stage, grid_in, keys, cost64, out_stage, ranks, scan_tot,
         tile_lo;
     void* pin = nullptr;  // pinned host staging
     size_t pin_bytes = 0;
@@ -254,7 +254,7 @@ int kvdro_create(kvdro_ctx** out, int device_ordinal) {
     if (const char* f = std::getenv("KVDRO_TEST_FAIL_ALLOC")) ctx->fail_after = std::atoi(f);
     if (const char* f = std::getenv("KVDRO_TEST_SKIP_CHUNK")) ctx->skip_chunk = std::atoi(f);
     DeviceGuard g(device_ordinal);
-    if (!g.ok || kvdro::grid_prepare(Prec::F32) != cudaSuccess || kvdro::grid_prepare(Prec::F64) != cudaSuccess ||
+    if (!g.ok || kvdro::sm_count(&ctx->sms) != cudaSuccess || kvdro::grid_prepare(Prec::F32) != cudaSuccess || kvdro::grid_prepare(Prec::F64) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->pin_free, cudaEventDisableTiming) != cudaSuccess ||
         kvdro::grid_prepare(Prec::EXACT) != cudaSuccess || kvdro::grid_prepare(Prec::ENVELOPE) != cudaSuccess ||
         cudaEventCreate(&ctx->grid_t0) != cudaSuccess ||
@@ -276,7 +276,7 @@ int kvdro_destroy(kvdro_ctx* ctx) {
     if (ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
     cudaDeviceSynchronize();
     for (Buf* b : {&ctx->sorted, &ctx->scan_tot, &ctx->pairs, &ctx->hist, &ctx->csum, &ctx->sumx, &ctx->meta, &ctx->errs, &ctx->in_stage,
-                   &ctx->grid_in, &ctx->keys, &ctx->cost64, &ctx->out_stage, &ctx->ranks, &ctx->part, &ctx->tile_lo})
+                   &ctx->grid_in, &ctx->keys, &ctx->cost64, &ctx->out_stage, &ctx->ranks, &ctx->tile_lo})
         release(*b);
     if (ctx->pin) cudaFreeHost(ctx->pin);
     if (ctx->pin_free) cudaEventDestroy(ctx->pin_free);
@@ -524,14 +524,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     if (!g.ok) return fail(ctx, KVDRO_ECUDA, "cannot select device %d", ctx->device);
     ctx->last_stream = s;
 
-    // Launch shape: lam tiles x r groups of warps per CTA.  The exact kernel takes at most
-    // kExactLamBlock lam values per launch; a larger grid runs as consecutive launches over blocks
-    // of it (the last block may be smaller and take its own shape).
-    const int32_t lam_blk = KP == Prec::EXACT ? kvdro::kExactLamBlock : NL;
-    const int32_t nblk = (NL + lam_blk - 1) / lam_blk;
-    const int32_t NL_last = NL - (nblk - 1) * lam_blk;
-    const kvdro::GridShape shape = kvdro::grid_shape(KP, R, std::min(NL, lam_blk), E, max_L);
-    const kvdro::GridShape shape_last = kvdro::grid_shape(KP, R, NL_last, E, max_L);
+    const kvdro::GridShape shape = kvdro::grid_shape(KP, R, NL, E, max_L, (int64_t)M * ctx->K, ctx->sms);
 
     // Grid parameters in one upload.
     const size_t gbytes = align_up((size_t)R * 4, 8) + 8 * ((size_t)NL + E + 2 * (size_t)M);
@@ -626,23 +619,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     // chunk.  It travels with this context's launches only.
     a.test_skip_chunk = ctx->skip_chunk;
     a.wait_ns = ctx->skip_chunk >= 0 ? kTestWaitNs : 0;
-    a.lam0 = 0;
-    a.NL_out = NL;
-    a.part_val = nullptr;
-    a.part_idx = nullptr;
-    a.part_first = a.part_last = 1;
-    const int64_t per_m = (int64_t)ctx->K * std::max(shape.r_blocks, shape_last.r_blocks);
-    int64_t m_step = std::max<int64_t>(1, 0x7fffffffLL / per_m);
-    if (nblk > 1) {
-        // the running minimum over lam blocks, 12 bytes per (regime, eps, class, r), for at most
-        // kPartBytes worth of regimes at a time
-        const int64_t per_regime = (int64_t)E * ctx->K * R * 12;
-        m_step = std::max<int64_t>(1, std::min<int64_t>(m_step, kPartBytes / per_regime));
-        const int64_t cells = std::min<int64_t>(m_step, M) * (per_regime / 12);
-        if ((rc = ensure(ctx, ctx->part, (size_t)cells * 12))) return rc;
-        a.part_val = static_cast<double*>(ctx->part.p);
-        a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(ctx->part.p) + (size_t)cells * 8);
-    }
+    int64_t m_step = std::max<int64_t>(1, 0x7fffffffLL / ((int64_t)ctx->K * shape.r_blocks));
     // Host outputs laid out regime-major (S, cost, lam index) go back in blocks of regimes on the
     // context's copy stream, each block as soon as its launches are done, so the copies overlap the
     // evaluation of later regimes instead of following the whole grid.
@@ -662,14 +639,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     for (int64_t m0 = 0; m0 < M; m0 += m_step) {
         a.m0 = (int32_t)m0;
         a.m_count = (int32_t)std::min<int64_t>(m_step, M - m0);
-        for (int32_t b = 0; b < nblk; b++) {
-            a.lam = d_lam + (size_t)b * lam_blk;
-            a.NL = b + 1 < nblk ? lam_blk : NL_last;
-            a.lam0 = b * lam_blk;
-            a.part_first = b == 0;
-            a.part_last = b + 1 == nblk;
-            KV_CUDA(kvdro::launch_grid(KP, b + 1 < nblk ? shape : shape_last, a, s), "grid kernel");
-        }
+        KV_CUDA(kvdro::launch_grid(KP, shape, a, s), "grid kernel");
         if (pipe) {
             KV_CUDA(cudaEventRecord(ctx->copy_ready, s), "recording a regime block");
             KV_CUDA(cudaStreamWaitEvent(ctx->copy_stream, ctx->copy_ready, 0), "ordering a copy");

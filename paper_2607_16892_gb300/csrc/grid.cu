@@ -38,6 +38,9 @@
 #include <float.h>
 #include <math.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "kvdro_internal.cuh"
 
 namespace kvdro {
@@ -58,50 +61,47 @@ constexpr unsigned kWaitPollCap = 1u << 28;
 
 constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 
-// Shape of one instantiation of the grid kernel: precision, warp tile (TR reservations x TL
-// multipliers, TR*TL a power of two <= 32), FP32 chunks between folds of the per-lane partial
-// sums into FP64 (FP64 folds once at the end), the largest CTA and minimum CTAs per SM it is
-// compiled for (these two bound its registers per thread), the staged chunk and ring depth, the
-// sample loop's unroll, and (exact) whether it reads pair sums.
+// Shape of one instantiation of the FP32- or FP64-arithmetic kernel: precision, warp tile (TR
+// reservations x TL multipliers, TR*TL a power of two <= 32), FP32 chunks between folds of the per-lane
+// partial sums into FP64 (FP64 folds once at the end), the largest CTA and minimum CTAs per SM it is
+// compiled for (these two bound its registers per thread), the staged chunk and ring depth, and the
+// sample loop's unroll.
 template <Prec P_, int TR_, int TL_, int FLUSH_, int MINB_, int MAXT_ = 512, int CHUNK_ = 2048, int STAGES_ = 3,
-          int UNROLL_ = 2, bool PAIR_ = false>
+          int UNROLL_ = 2>
 struct GridCfg {
-    static constexpr bool PAIR = PAIR_;
     static constexpr Prec P = P_;
     static constexpr int TR = TR_, TL = TL_, V = TR_ * TL_, LOG2V = ilog2(TR_ * TL_), FLUSH = FLUSH_, MINB = MINB_;
     static constexpr int MAXT = MAXT_;
-    static constexpr int CHUNK = CHUNK_;      // samples per staged chunk
-    static constexpr int BYTES = PAIR_ ? 4 : 8;  // staged bytes per sample (native FP64 also reads pair sums)
-    static constexpr int STAGES = STAGES_;    // ring depth
-    static constexpr int UNROLL = UNROLL_;    // unroll of the sample loop
-    static_assert(CHUNK_ % 128 == 0 && CHUNK_ * BYTES * STAGES_ <= 160 * 1024, "chunk ring must fit shared memory");
+    static constexpr int CHUNK = CHUNK_;    // samples per staged chunk
+    static constexpr int BYTES = 8;         // staged bytes per sample (native FP64 also reads pair sums, 4)
+    static constexpr int STAGES = STAGES_;  // ring depth
+    static constexpr int UNROLL = UNROLL_;  // unroll of the sample loop
+    static_assert(P_ != Prec::EXACT && CHUNK_ % 128 == 0 && CHUNK_ * BYTES * STAGES_ <= 160 * 1024, "chunk ring must fit");
     static_assert((V & (V - 1)) == 0 && V >= 2 && V <= 32, "tile must hold a power of two <= 32 cells");
-    static_assert(P_ == Prec::F64 || TL_ % 2 == 0, "the FP32 and exact tiles pack lam values in pairs");
-    static_assert(FLUSH >= 0 && UNROLL >= 1 && (!PAIR || P_ == Prec::EXACT), "shape parameters out of range");
+    static_assert(P_ == Prec::F64 || TL_ % 2 == 0, "the FP32 tiles pack lam values in pairs");
+    static_assert(FLUSH >= 0 && UNROLL >= 1, "shape parameters out of range");
 };
-// 2 r x 8 lam tiles, up to 16 warps per CTA and (FP32, exact) two CTAs per SM (64 registers)
-// for up to 128 lam values; larger lam grids run the exact kernel in blocks of 128 lam values
-// (kExactLamBlock), and the FP32 kernel takes 2 x 16 tiles.  FP64: 2 x 8 tiles.
-// The exact variants hold 96 KB of ring per CTA, two CTAs per SM: three 32 KB chunks of pair sums
-// (8192 samples; two of 32, 36 or 48 KB, four of 24 and six of 16 measured 2 to 5 % slower) or two 48 KB
-// chunks of (x', x') pairs; the FP32 and FP64 ones two of 32 KB.  The FP32 variants fold their partial sums every
-// 2 chunks (256 samples per lane); the exact variants fold as often as their support size requires,
-// independently of the chunk size.
+// FP32: 2 r x 8 lam tiles, up to 16 warps per CTA and two CTAs per SM (64 registers) for up to 128 lam
+// values, 2 x 16 tiles above.  FP64: 2 x 8 tiles.  Both stage 32 KB chunks through a 2-deep ring; the FP32
+// variants fold their partial sums every 2 chunks (256 samples per lane) and unroll the sample loop 4 times.
 using CfgF32 = GridCfg<Prec::F32, 2, 8, 2, 2, 512, 4096, 2, 4>;
 using CfgF32Wide = GridCfg<Prec::F32, 2, 16, 2, 1, 512, 4096, 2, 4>;
 using CfgF64 = GridCfg<Prec::F64, 2, 8, 0, 1, 512, 4096, 2>;
-using CfgExact = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 8192, 3, 8, true>;
-// Above a support of kPairMaxL the FP32 sums (exact only up to 2^24) would fold every few loads; there
-// the integer absolute differences, whose sums fold far less often, take the samples one by one.
-using CfgExactInt = GridCfg<Prec::EXACT, 2, 8, 0, 2, 512, 6144, 2, 8>;
-// One or two lam values (a small grid, or the last block of a larger one): 8 r x 2 lam tiles, so
-// that a single value pads its tile to 2 columns rather than 8.
-using CfgExactFewLam = GridCfg<Prec::EXACT, 8, 2, 0, 2, 512, 8192, 3, 8, true>;
-using CfgExactIntFewLam = GridCfg<Prec::EXACT, 8, 2, 0, 2, 512, 6144, 2, 8>;
-constexpr int32_t kFewLam = 2;
 constexpr int kWarpsTarget = 16;  // warps per CTA the r groups fill up to
-static_assert(kExactLamBlock == kWarpsTarget * CfgExact::TL && kExactLamBlock == kWarpsTarget * CfgExactInt::TL,
-              "one launch of the exact kernel takes 16 warps of lam tiles");
+
+// The exact kernel: 16 cells per warp, up to 16 warps per CTA and two CTAs per SM (64 registers).  A CTA
+// takes whole rows of lam values, laid over its warps without regard to rows (a warp needs 16 thresholds,
+// whatever cells they are), in one pass over the class's samples or several (exact_shape).
+constexpr int kExactV = 16;
+constexpr int kExactLog2V = 4;
+constexpr int kExactWarps = 16;
+constexpr int kExactMaxPasses = 4;
+constexpr size_t kExactSmem = (228 * 1024 - 2 * 1024) / 2 - 256;  // two CTAs in an SM's 228 KB, 1 KB reserved for each
+template <bool PAIR>
+struct ExactCfg {
+    static constexpr int kBytes = PAIR ? 4 : 8, kPer = PAIR ? 4 : 2;  // staged bytes per sample, samples per load
+    static constexpr int kChunk = PAIR ? 8192 : 6144;                 // samples per staged chunk at most
+};
 
 // ---------------------------------------------------------------- PTX helpers
 
@@ -231,21 +231,45 @@ __device__ __forceinline__ T transpose_reduce(T (&v)[V], int lane) {
 }
 
 struct SmemLayout {
-    size_t ring, full, lam, eps, S, acc, t, total;
+    size_t ring, full, lam, eps, S, lamf, Sf, total;
+    int stride_f;
 };
 
-// `acc` and `t` (the exact kernel's cells, in warp order): the integer sums and the thresholds.
+__host__ __device__ inline int four(int n) { return (n + 3) & ~3; }
+// Floats per row of S cut to floats: read four at a time with lanes along the rows, so an odd number of fours.
+__host__ __device__ inline int float_stride(int NL) { return 4 * ((NL + 3) / 4 | 1); }
+
 __host__ __device__ inline SmemLayout smem_layout(int RG, int TR, int NLpad, int E, int chunk_bytes, int stages) {
     SmemLayout L;
+    L.stride_f = float_stride(NLpad);
     L.ring = 0;
     L.full = (size_t)stages * chunk_bytes;
     L.lam = L.full + 8 * (size_t)stages;
     L.eps = L.lam + 8 * (size_t)NLpad;
     L.S = L.eps + 8 * (size_t)E;
-    L.acc = L.S + 8 * (size_t)RG * TR * NLpad;
-    L.t = (L.acc + 8 * (size_t)RG * TR * NLpad + 15) & ~(size_t)15;
-    L.total = L.t + 4 * (size_t)RG * TR * NLpad;
+    L.lamf = (L.S + 8 * (size_t)RG * TR * NLpad + 15) & ~(size_t)15;
+    L.Sf = L.lamf + 4 * (size_t)four(NLpad);
+    L.total = L.Sf + 4 * (size_t)RG * TR * L.stride_f;
     return L;
+}
+
+// The exact kernel's: `S` holds the cells' integer sums first, then their S, `t` their thresholds.
+struct ExactSmem {
+    size_t full, lam, eps, S, t, lamf, Sf, total;
+    int stride_f;
+};
+__host__ __device__ inline ExactSmem exact_smem(int rows, int NL, int E, int tiles, int ring_bytes) {
+    ExactSmem s;
+    s.stride_f = float_stride(NL);
+    s.full = ring_bytes;
+    s.lam = s.full + 32;
+    s.eps = s.lam + 8 * (size_t)NL;
+    s.S = s.eps + 8 * (size_t)E;
+    s.t = (s.S + 8 * (size_t)tiles * kExactV + 15) & ~(size_t)15;
+    s.lamf = s.t + 4 * (size_t)tiles * kExactV;
+    s.Sf = s.lamf + 4 * (size_t)four(NL);
+    s.total = s.Sf + 4 * (size_t)rows * s.stride_f;
+    return s;
 }
 
 // The minimum over lam of lam * eps + S for one (r, eps) pair: the value RN(RN(lam eps) + S) and the
@@ -299,76 +323,104 @@ struct LamMin {
     }
 };
 
-// The warp's lanes over one row of S (every lane returns the result).
-__device__ __forceinline__ LamMin warp_lam_min(const double* S, const double* lam, double eps, int NL, int lane) {
-    bool ok = true, unused = true;
-    const float ef = cut(eps, ok);
-    float ub = INFINITY;
-    for (int j = lane; j < NL; j += 32) ub = fminf(ub, fmaf(cut(lam[j], ok), ef, cut(S[j], ok)));
-    if (!ok) ub = 0.f;
-    ub = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(ub)));  // ordered as uints: all >= 0
-    const bool fast = ub > kLamFloor;
-    LamMin r;
-    for (int j = lane; j < NL; j += 32)
-        if (!fast || fmaf(cut(lam[j], unused), ef, cut(S[j], unused)) <= ub * kLamWindow)
-            r.take(lam[j], eps, S[j], j, fast, lam, S);
-    r.reduce(32);
-    return r;
-}
-
 // One (r, eps) pair's results: the cost and lam index outputs and the argmin over r through a 64-bit
 // key for atomicMin (FP32: cost bits and r index; otherwise the cost's double bits truncated to 44
 // bits, order-preserving for non-negative values, with the r index in the low 20 bits).
-// Returns the key, or all ones before the last lam block; the caller takes its minimum.
 template <bool F32OUT>
 __device__ __forceinline__ u64 write_pair(const GridArgs& a, double best, int bj, int m, int k, int e, int ri) {
-    const size_t row = ((size_t)m * a.E + e) * a.K + k;
-    const size_t o = row * a.R + ri;
-    bj += a.lam0;
-    if (a.part_val) {  // lam blocks: merge with the earlier blocks (they hold lower indices)
-        const size_t q = ((((size_t)(m - a.m0)) * a.E + e) * a.K + k) * a.R + ri;
-        if (!a.part_first && !(best < a.part_val[q])) {
-            best = a.part_val[q];
-            bj = a.part_idx[q];
-        }
-        if (!a.part_last) {
-            a.part_val[q] = best;
-            a.part_idx[q] = bj;
-            return ~0ull;
-        }
-    }
-    u64 key;
+    const size_t o = (((size_t)m * a.E + e) * a.K + k) * a.R + ri;
+    if (a.lam_idx_out) a.lam_idx_out[o] = bj;
     if constexpr (F32OUT) {
         const float cf = (float)best;
         if (a.cost_out) static_cast<float*>(a.cost_out)[o] = cf;
-        key = ((u64)__float_as_uint(cf > 0.f ? cf : 0.f) << 32) | (u64)(uint32_t)ri;
+        return ((u64)__float_as_uint(cf > 0.f ? cf : 0.f) << 32) | (u64)(uint32_t)ri;
     } else {
         static_cast<double*>(a.cost_out)[o] = best;
         const bool above = dbits(best) > 0 && dbits(best) <= 0x7ff0000000000000ll;  // best > 0
-        key = ((u64)(above ? dbits(best) : 0ll) & ~0xFFFFFull) | (u64)ri;
+        return ((u64)(above ? dbits(best) : 0ll) & ~0xFFFFFull) | (u64)ri;
     }
-    if (a.lam_idx_out) a.lam_idx_out[o] = bj;
-    return key;
 }
 
-// Epilogue of one CTA of the grid kernel: a warp per (r, eps) pair.
+// The CTA's rows of S in shared memory, as doubles and cut to floats (INFINITY past NL up to a multiple of
+// four), with the lam values likewise (0 past NL).
+struct LamRows {
+    const double *S, *lam, *eps;
+    const float *Sf, *lamf;
+    int stride, stride_f;
+    int rows, NL;
+    bool floats;  // every lam and S is >= 0 and small enough for its float
+};
+
+// The end of every grid kernel, by all threads of the CTA (whole warps): for each (r, eps) pair the minimum
+// over lam, its outputs and the argmin over r.
+//
+// G lanes per pair, as many as keep every thread busy, groups along r first (outputs side by side, one
+// atomic per warp and radius: one per pair held the envelope at 7.8 ms where it now takes 3.7); each lane
+// takes every G-th four lam values and keeps its smallest v', where it was, and its second smallest: with
+// the second outside the window only that one value is formed in FP64, by all lanes at once.
 template <bool F32OUT>
-__device__ __forceinline__ void cta_epilogue(const GridArgs& a, const double* s_S, const double* s_lam,
-                                             const double* s_eps, int stride, int rl_count, int r_cta0, int m, int k) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int p = warp; p < rl_count * a.E; p += nwarps) {
-        const int rl = p / a.E, e = p % a.E;
-        const int ri = r_cta0 + rl;
-        if (ri >= a.R) continue;
-        const LamMin b = warp_lam_min(s_S + rl * stride, s_lam, s_eps[e], a.NL, lane);
-        if (lane == 0) {
-            const u64 key = write_pair<F32OUT>(a, b.v, b.j, m, k, e, ri);
-            if (key != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + e) * a.K + k, key);
+__device__ __forceinline__ void lam_min_epilogue(const GridArgs& a, const LamRows& x, int r_cta0, int m, int k) {
+    const int tid = threadIdx.x, lane = tid & 31, threads = blockDim.x;
+    const int pairs = x.rows * a.E, n4 = (x.NL + 3) / 4;
+    int G = 1;
+    while (G < 32 && G < n4 && 2 * G * pairs <= threads) G <<= 1;
+    const int per_pass = threads / G, g = tid & (G - 1);
+    for (int p0 = 0; p0 < pairs; p0 += per_pass) {  // the same trips for every lane: the group's shuffles are warp-wide
+        const int p = p0 + tid / G;
+        const bool active = p < pairs;
+        const int e = active ? p / x.rows : 0, rl = active ? p % x.rows : 0;
+        const double* S = x.S + rl * x.stride;
+        const float* Sf = x.Sf + rl * x.stride_f;
+        const double eps = x.eps[e];
+        bool fast = x.floats;
+        const float ef = cut(eps, fast);
+        float m1 = INFINITY, m2 = INFINITY;
+        int j1 = 0;
+        for (int q = g; q < n4; q += G) {
+            const float4 l = reinterpret_cast<const float4*>(x.lamf)[q], s = reinterpret_cast<const float4*>(Sf)[q];
+            const float v[4] = {fmaf(l.x, ef, s.x), fmaf(l.y, ef, s.y), fmaf(l.z, ef, s.z), fmaf(l.w, ef, s.w)};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                m2 = fminf(m2, fmaxf(m1, v[i]));
+                if (v[i] < m1) j1 = 4 * q + i;
+                m1 = fminf(m1, v[i]);
+            }
+        }
+        for (int o = 1; o < G; o <<= 1) {
+            const float o1 = __shfl_xor_sync(0xffffffffu, m1, o), o2 = __shfl_xor_sync(0xffffffffu, m2, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, j1, o);
+            m2 = fminf(fminf(m2, o2), fmaxf(m1, o1));
+            if (o1 < m1 || (o1 == m1 && oj < j1)) j1 = oj;
+            m1 = fminf(m1, o1);
+        }
+        fast = fast && m1 > kLamFloor;
+        const float thr = m1 * kLamWindow;
+        LamMin best;
+        if (fast && m2 > thr) {
+            best.v = __dadd_rn(__dmul_rn(x.lam[j1], eps), S[j1]);
+            best.j = j1;
+        }
+        const bool several = active && best.j == 0x7fffffff;
+        if (__any_sync(0xffffffffu, several)) {
+            LamMin r;
+            if (several)
+                for (int j = g; j < x.NL; j += G)
+                    if (!fast || fmaf(x.lamf[j], ef, Sf[j]) <= thr) r.take(x.lam[j], eps, S[j], j, fast, x.lam, S);
+            r.reduce(G);
+            if (several) best = r;
+        }
+        u64 key = ~0ull;
+        if (active && g == 0) key = write_pair<F32OUT>(a, best.v, best.j, m, k, e, r_cta0 + rl);
+        // the warp's minimum over each radius it holds, e0 (its first lane's) upwards
+        const int e0 = __shfl_sync(0xffffffffu, e, 0), e1 = __reduce_max_sync(0xffffffffu, e);
+        for (int ei = e0; ei <= e1; ei++) {
+            const u64 low = group_min(e == ei ? key : ~0ull, 32);
+            if (lane == 0 && low != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + ei) * a.K + k, low);
         }
     }
 }
 
-// ---------------------------------------------------------------- the grid kernel
+// ---------------------------------------------------------------- the FP32- and FP64-arithmetic kernels
 
 template <class C>
 __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
@@ -383,6 +435,8 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     double* s_lam = reinterpret_cast<double*>(smem + lay.lam);
     double* s_eps = reinterpret_cast<double*>(smem + lay.eps);
     double* s_S = reinterpret_cast<double*>(smem + lay.S);
+    float* s_lamf = reinterpret_cast<float*>(smem + lay.lamf);
+    float* s_Sf = reinterpret_cast<float*>(smem + lay.Sf);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int b = blockIdx.x;
@@ -390,7 +444,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     b /= a.r_blocks;
     const int k = b % a.K;
     const int m = a.m0 + b / a.K;
-    [[maybe_unused]] const int lt = warp % a.LT, r_local0 = warp / a.LT * TR;
+    const int lt = warp % a.LT, r_local0 = warp / a.LT * TR;
     const int r_cta0 = rb * a.RG * TR;
 
     for (int i = tid; i < NLpad; i += blockDim.x) s_lam[i] = i < a.NL ? a.lam[i] : 0.0;
@@ -420,20 +474,18 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     int consumed = 0;                    // chunk at which the loop stopped
 
     // Per-cell constants of this warp's tile (identical across its lanes).
-    const double cp = a.cp[m], cw = a.cw[m], Lk = to_double(a.L[k]);
-    [[maybe_unused]] double eta[TR];
-    [[maybe_unused]] bool rvalid[TR];
-    if constexpr (P != Prec::EXACT) {
+    const double cp = a.cp[m], cw = a.cw[m], Lk = (double)a.L[k];
+    double eta[TR];
+    bool rvalid[TR];
 #pragma unroll
-        for (int i = 0; i < TR; i++) {
-            const int ri = r_cta0 + r_local0 + i;
-            rvalid[i] = ri < a.R;
-            eta[i] = rvalid[i] ? (double)a.r[ri] - (double)a.L_in[k] : 0.0;
-        }
+    for (int i = 0; i < TR; i++) {
+        const int ri = r_cta0 + r_local0 + i;
+        rvalid[i] = ri < a.R;
+        eta[i] = rvalid[i] ? (double)a.r[ri] - (double)a.L_in[k] : 0.0;
     }
 
     bool timeout = false;
-    [[maybe_unused]] double acc64 = 0.0;  // this lane's cell after the warp transposition
+    double acc64 = 0.0;  // this lane's cell after the warp transposition
 
     if constexpr (P == Prec::F32) {
         // Each row's excess is taken about its reservation: kappa (x - eta) + W(eta) (excess_at_eta).
@@ -635,212 +687,6 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
                 for (int j = 0; j < TL; j++) vals[i * TL + j] = acc[i][j];
             acc64 = transpose_reduce<double, V>(vals, lane);
         }
-    } else {
-        // EXACT: per cell (i, j) the active samples are x >= t_ij for an integer threshold t_ij, and
-        // sum_n max(kappa x_n + d, 0) = kappa sum_{x >= t} x + d #{x >= t}.  With c = t - 1,
-        // max(x - c, 0) = (x - c + |x - c|) / 2 and sum_n (x - c) has a closed form, so the kernel
-        // streams sum_n |x - c| only, as integers.
-        // Pair sums: |a - c| + |b - c| = max(|a + b - 2c|, |a - b|) takes two samples for two cells in one
-        // packed FP32 add, two max and (with the next pair's) one packed add, an instruction per term
-        // as with one sample at a time, but split evenly over the FMA and ALU pipes within each cell and
-        // with fewer register operands (3 reads a term, and the pair's sum and difference serve every
-        // cell), in half the staged bytes.  Packed adds on one half of a warp's cells beside integer
-        // absolute differences on the other (3.5 reads a term) took 16.43 ms on 8 classes x 100,000
-        // samples x 4096 r x 128 lam, this 16.06: 83 of the 128 terms/clk/SM that either pipe and the
-        // issue slots allow.  Every value is an integer
-        // below 2^24, so the FP32 arithmetic is exact; sums fold into int64 through the warp transposition
-        // before one could pass 2^24.
-        // (x', x') pairs: one integer absolute-difference-and-add (__sad) per term on the staged float's
-        // bit pattern, 0x4B000000 + x.
-        // The count #{x >= t} comes from the class's cumulative counts; the epilogue puts every sample
-        // on its branch of phi with these integer sums (branch_sum) in FP64.
-        constexpr int NPF = C::PAIR ? TL / 2 : 1, NI = C::PAIR ? 1 : TL;  // array extents
-        [[maybe_unused]] u64 n2c[TR][NPF], accf[TR][NPF];  // -2c for two cells, their sums
-        [[maybe_unused]] int cci[TR][NI];                  // 0x4B000000 + c per cell
-        [[maybe_unused]] unsigned acci[TR][NI];
-        // The CTA's cells, V per warp, are half its threads: each cell's threshold is one thread's work (its
-        // few FP64 instructions take the pipe as long for one lane as for 32), read back by its warp;
-        // the same thread combines the cell's sums at the end, so nothing of it stays in registers
-        // over the sample loop.
-        int* s_t = reinterpret_cast<int*>(smem + lay.t);
-        long long* s_acc = reinterpret_cast<long long*>(smem + lay.acc);
-        const int cells = (blockDim.x >> 5) * V;
-        struct CellAt {
-            int rl, lj, ri;
-        };
-        auto cell_at = [&](int c) {
-            const int w = c >> LOG2V, i = c & (V - 1);
-            CellAt x;
-            x.rl = w / a.LT * TR + i / TL;
-            x.lj = w % a.LT * TL + i % TL;
-            x.ri = r_cta0 + x.rl;
-            return x;
-        };
-        for (int c = tid; c < cells; c += blockDim.x) {
-            const CellAt x = cell_at(c);
-            int ct = a.L[k] + 1;  // L + 1 means "none" (no sample exceeds L); t in [0, L + 1] keeps |x - c| <= L + 1
-            if (x.ri < a.R && x.lj < a.NL) {
-                const double lam = s_lam[x.lj], mu = dmin_nonneg(lam, cp);
-                const RowOffset row = row_offset(cp, cw, a.L[k], a.r[x.ri] - a.L_in[k]);
-                ct = first_active(__dadd_rn(mu, dmin_nonneg(lam, cw)), excess_offset(row, cp, mu, Lk), a.L[k]);
-            }
-            s_t[c] = ct;
-        }
-        __syncthreads();
-        const int* w_t = s_t + warp * V;
-#pragma unroll
-        for (int i = 0; i < TR; i++) {
-            if constexpr (C::PAIR) {
-#pragma unroll
-                for (int jp = 0; jp < TL / 2; jp++) {
-                    n2c[i][jp] = pk((float)(2 - 2 * w_t[i * TL + 2 * jp]), (float)(2 - 2 * w_t[i * TL + 2 * jp + 1]));
-                    accf[i][jp] = 0ull;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < TL; j++) {
-                    cci[i][j] = kStageBits - 1 + w_t[i * TL + j];
-                    acci[i][j] = 0u;
-                }
-            }
-        }
-        // Fold after at most `fe` loads of kPer samples each: a lane's sum is then at most
-        // kPer fe (L + 1), within 2^24 in FP32 (the transposition's 32-lane sums stay below 2^29), or as
-        // integers 32 lanes' sums below 2^32.  The same for every thread of the CTA.
-        constexpr int kPer = C::PAIR ? 4 : 2;
-        constexpr long long kFoldLimit = C::PAIR ? (1ll << 24) : (1ll << 32) / 32 - 1;
-        const int fe = (int)min(1ll << 20, max(1ll, kFoldLimit / (kPer * ((long long)a.L[k] + 1))));
-        long long acc_r = 0;
-        auto fold = [&]() {
-            unsigned vs[V];
-#pragma unroll
-            for (int i = 0; i < TR; i++) {
-                if constexpr (C::PAIR) {
-#pragma unroll
-                    for (int jp = 0; jp < TL / 2; jp++) {
-                        float a0, a1;
-                        upk(accf[i][jp], a0, a1);
-                        vs[i * TL + 2 * jp] = __float2uint_rn(a0);
-                        vs[i * TL + 2 * jp + 1] = __float2uint_rn(a1);
-                        accf[i][jp] = 0ull;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < TL; j++) {
-                        vs[i * TL + j] = acci[i][j];
-                        acci[i][j] = 0u;
-                    }
-                }
-            }
-            acc_r += (long long)transpose_reduce<unsigned, V>(vs, lane);
-        };
-        // One load into every cell's sum.  The pair sums' rate hangs on ptxas's register allocation (operand
-        // bank conflicts): written cell by cell, the second pair first, 16.06 ms on 8 classes x 100,000
-        // samples x 4096 r x 128 lam; first pair first 16.39, the accumulator as first operand 16.57, two
-        // cells' adds ahead of their max 16.91, all adds first 17.03; unrolled 4 / 16 times 16.6 / 16.5.
-        auto step = [&](const float4 v) {
-            if constexpr (C::PAIR) {
-                const u64 s0 = pk(v.x, v.x), s1 = pk(v.y, v.y);
-#pragma unroll
-                for (int i = 0; i < TR; i++)
-#pragma unroll
-                    for (int p = 0; p < NPF; p++)
-                        accf[i][p] = fadd2(fadd2(max_abs2(fadd2(s1, n2c[i][p]), v.w), max_abs2(fadd2(s0, n2c[i][p]), v.z)), accf[i][p]);
-            } else {
-                const int ba = __float_as_int(v.x), bb = __float_as_int(v.z);  // 0x4B000000 + x
-#pragma unroll
-                for (int i = 0; i < TR; i++)
-#pragma unroll
-                    for (int j = 0; j < TL; j++) acci[i][j] = __sad(bb, cci[i][j], __sad(ba, cci[i][j], acci[i][j]));
-            }
-        };
-        constexpr int kSeg = 8;  // loads per segment of a fixed trip count
-        int pending = 0;         // loads since the last fold
-        auto room = [&](int loads) {  // fold first if the loads since the last fold would pass fe
-            if (pending + loads > fe) {
-                fold();
-                pending = 0;
-            }
-            pending += loads;
-        };
-        const int64_t n_k = a.N[k];
-        for (int c = 0; c < nchunks; c++) {
-            const int s = c % C::STAGES;
-            if (!mbar_wait_bounded(smem_u32(&full[s]), (uint32_t)((c / C::STAGES) & 1), a.wait_ns)) timeout = true;
-            if (!timeout) {
-                const int cnt = (int)min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
-                const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * kStageBytes);
-                const int nq = cnt / (32 * kPer);
-                // loads [0, t_clean) hold samples only; of (x', x') pairs the class's last ones may hold
-                // NaN padding, which they read as x = 0 (x' = 2^23)
-                const int64_t left = n_k - (int64_t)c * C::CHUNK;
-                const int t_clean = C::PAIR ? nq : (left <= 0 ? 0 : (int)min((int64_t)nq, left / (32 * kPer)));
-                int t0 = 0;
-                if (fe >= kSeg) {
-#pragma unroll 1
-                    for (; t0 + kSeg <= t_clean; t0 += kSeg) {
-                        room(kSeg);
-#pragma unroll(C::UNROLL)
-                        for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
-                    }
-                }
-#pragma unroll 1
-                for (; t0 < nq; t0++) {
-                    room(1);
-                    float4 v = q[lane + 32 * t0];
-                    if (!C::PAIR && t0 >= t_clean) {
-                        v.x = fmaxf(v.x, kStageOffset), v.y = fmaxf(v.y, kStageOffset);
-                        v.z = fmaxf(v.z, kStageOffset), v.w = fmaxf(v.w, kStageOffset);
-                    }
-                    step(v);
-                }
-            }
-            consumed = c;
-            if (__syncthreads_or(timeout)) {
-                timeout = true;
-                break;
-            }
-            if (c + C::STAGES < nchunks) {
-                if (tid == 0) {
-                    fence_proxy_async();
-                    issue(c + C::STAGES);
-                }
-                issued = c + C::STAGES + 1;
-            }
-        }
-        if (!timeout) {
-            if (pending > 0) fold();
-            // the lane's cell (cell lane >> (5 - log2 V) of its warp)
-            if ((lane & ((1 << (5 - LOG2V)) - 1)) == 0) s_acc[warp * V + (lane >> (5 - LOG2V))] = acc_r;
-            __syncthreads();
-            const long long Nk = a.N[k], sumx = a.sumx[k], npad = np - Nk;
-            for (int c = tid; c < cells; c += blockDim.x) {
-                const CellAt x = cell_at(c);
-                if (x.ri >= a.R || x.lj >= a.NL) continue;
-                // the active count from the cumulative counts, then the branch sums
-                const int ti = s_t[c], L = a.L[k];  // in [0, L + 1]
-                const long long t = ti;
-                const long long count = ti <= 0 ? Nk : (ti > L ? 0 : Nk - (long long)a.cdf[a.hist_off[k] + t - 1]);
-                // s_acc = sum |x - c| over the samples and the padding zeros; with y = x - c,
-                // max(y, 0) = (y + |y|) / 2
-                const long long sum_abs = s_acc[c] - npad * (t > 1 ? t - 1 : 1 - t);
-                const long long sum_y = sumx + Nk * (1 - t);
-                const long long sum_relu = (sum_y + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
-                const long long sum = sum_relu + (t - 1) * count;  // sum_{x >= t} x
-                // each sample on its own branch of phi (exact integer sums): V = c_w eta - nu x below t,
-                // U = c_p (L - eta) - mu (L - x) from t on; no large term cancels another
-                const double lam = s_lam[x.lj];
-                const double tot = branch_sum(cp, cw, dmin_nonneg(lam, cp), dmin_nonneg(lam, cw), L, a.r[x.ri] - a.L_in[k],
-                                              Nk, count, sumx - sum, (long long)L * count - sum);
-                const double S = __dmul_rn(tot, a.inv_n[k]);
-                s_S[x.rl * NLpad + x.lj] = S;
-                if (a.S_out) {
-                    const size_t o = (((size_t)m * a.K + k) * a.R + x.ri) * a.NL_out + a.lam0 + x.lj;
-                    if (a.f32_out) static_cast<float*>(a.S_out)[o] = (float)S;
-                    else static_cast<double*>(a.S_out)[o] = S;
-                }
-            }
-        }
     }
 
     if (timeout) {
@@ -854,8 +700,9 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         return;
     }
 
-    // S for this lane's cell (the exact kernel has formed it above).
-    if constexpr (P != Prec::EXACT) {
+    // S for this lane's cell.
+    bool ok = true;
+    {
         const int cidx = lane >> (5 - LOG2V);
         const int i = cidx / TL, j = cidx % TL;
         const int ri = r_cta0 + r_local0 + i, lj = lt * TL + j;
@@ -872,17 +719,284 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
             const double tot = base + acc64;
             const double S = __dmul_rn(tot, a.inv_n[k]);
             s_S[(r_local0 + i) * NLpad + lj] = S;
+            s_Sf[(r_local0 + i) * lay.stride_f + lj] = cut(S, ok);
             if (a.S_out) {
-                const size_t o = (((size_t)m * a.K + k) * a.R + ri) * a.NL_out + a.lam0 + lj;
+                const size_t o = (((size_t)m * a.K + k) * a.R + ri) * a.NL + lj;
                 if (P == Prec::F32) static_cast<float*>(a.S_out)[o] = (float)S;
                 else static_cast<double*>(a.S_out)[o] = S;
             }
         }
     }
+    // the floats past the last lam value; `ok` over the CTA
+    for (int i = tid; i < a.RG * TR * 4; i += blockDim.x)
+        if (a.NL + (i & 3) < four(a.NL)) s_Sf[(i >> 2) * lay.stride_f + a.NL + (i & 3)] = INFINITY;
+    for (int j = tid; j < four(a.NL); j += blockDim.x) s_lamf[j] = j < a.NL ? cut(s_lam[j], ok) : 0.f;
+    const bool floats = __syncthreads_and(ok);
+    const LamRows rows = {s_S, s_lam, s_eps, s_Sf, s_lamf, NLpad, lay.stride_f, min(a.RG * TR, a.R - r_cta0), a.NL, floats};
+    lam_min_epilogue<P == Prec::F32>(a, rows, r_cta0, m, k);
+}
+
+// ---------------------------------------------------------------- the exact kernel
+//
+// Per cell the active samples are x >= t for an integer threshold t, and
+// sum_n max(kappa x_n + d, 0) = kappa sum_{x >= t} x + d #{x >= t}.  With c = t - 1,
+// max(x - c, 0) = (x - c + |x - c|) / 2 and sum_n (x - c) has a closed form, so the kernel streams
+// sum_n |x - c| only, as integers.
+//
+// Pair sums: |a - c| + |b - c| = max(|a + b - 2c|, |a - b|) takes two samples for two cells in one packed
+// FP32 add, two max and (with the next pair's) one packed add, an instruction per term as with one sample
+// at a time, but split evenly over the FMA and ALU pipes within each cell and with fewer register operands
+// (3 reads a term, and the pair's sum and difference serve every cell), in half the staged bytes.  Packed
+// adds on one half of a warp's cells beside integer absolute differences on the other (3.5 reads a term)
+// took 16.43 ms on 8 classes x 100,000 samples x 4096 r x 128 lam, this 16.06: 83 of the 128 terms/clk/SM
+// that either pipe and the issue slots allow.  Every value is an integer below 2^24, so the FP32
+// arithmetic is exact; sums fold into int64 through the warp transposition before one could pass 2^24.
+//
+// (x', x') pairs (supports above kPairMaxL): one integer absolute-difference-and-add (__sad) per term on
+// the staged float's bit pattern, 0x4B000000 + x; 23.1 ms there.
+//
+// The count #{x >= t} comes from the class's cumulative counts; every sample then goes on its branch of
+// phi with these integer sums (branch_sum) in FP64.
+template <bool PAIR>
+__global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a) {
+    using X = ExactCfg<PAIR>;
+    constexpr int V = kExactV, kOwn = 5 - kExactLog2V;  // lane l owns cell l >> kOwn after the transposition
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NL = a.NL;
+    int b = blockIdx.x;
+    const int r_cta0 = b % a.r_blocks * a.rows;
+    b /= a.r_blocks;
+    const int k = b % a.K;
+    const int m = a.m0 + b / a.K;
+    const int rows = min(a.rows, a.R - r_cta0), cells = rows * NL;
+    const int chunk = a.chunk, stage_bytes = chunk * X::kBytes, nwarps = blockDim.x >> 5;
+    const ExactSmem lay = exact_smem(a.rows, NL, a.E, nwarps * a.passes, a.stages * stage_bytes);
+    unsigned char* ring = smem;  // chunk c in stage c % stages
+    u64* full = reinterpret_cast<u64*>(smem + lay.full);
+    double* s_lam = reinterpret_cast<double*>(smem + lay.lam);
+    double* s_eps = reinterpret_cast<double*>(smem + lay.eps);
+    double* s_S = reinterpret_cast<double*>(smem + lay.S);
+    int* s_t = reinterpret_cast<int*>(smem + lay.t);
+    float* s_lamf = reinterpret_cast<float*>(smem + lay.lamf);
+    float* s_Sf = reinterpret_cast<float*>(smem + lay.Sf);
+
+    const int64_t pbase = a.pair_off[k];
+    const int64_t np = a.pair_off[k + 1] - pbase;  // multiple of kPadSamples
+    const int nchunks = (int)((np + chunk - 1) / chunk), total = nchunks * a.passes;  // over all passes
+    const unsigned char* src = static_cast<const unsigned char*>(a.staged) + pbase * X::kBytes;
+    auto issue = [&](int c, int s) {  // the class's chunk c into stage s
+        if (c == a.test_skip_chunk) return;  // test hook: nothing will complete this chunk's barrier
+        const int64_t cnt = min((int64_t)chunk, np - (int64_t)c * chunk);
+        tma_bulk_load(smem_u32(ring + (size_t)s * stage_bytes), src + (int64_t)c * stage_bytes, (uint32_t)(cnt * X::kBytes),
+                      smem_u32(&full[s]));
+    };
+    // the chunk `ahead` places after the class's chunk c, passes wrapping
+    auto chunk_after = [&](int c, int ahead) { return (c + ahead) % nchunks; };
+    if (tid == 0) {  // no other thread touches a barrier before the __syncthreads below
+        s_bad = 0;
+        for (int s = 0; s < a.stages; s++) mbar_init(smem_u32(&full[s]), 1);
+        fence_mbar_init();
+        for (int i = 0; i < a.stages && i < total; i++) issue(chunk_after(0, i), i);
+    }
+    for (int i = tid; i < NL; i += blockDim.x) s_lam[i] = a.lam[i];
+    for (int i = tid; i < a.E; i += blockDim.x) s_eps[i] = a.eps[i];
     __syncthreads();
 
-    if (P == Prec::F32 || a.f32_out) cta_epilogue<true>(a, s_S, s_lam, s_eps, NLpad, a.RG * TR, r_cta0, m, k);
-    else cta_epilogue<false>(a, s_S, s_lam, s_eps, NLpad, a.RG * TR, r_cta0, m, k);
+    // Each cell's threshold is one thread's work (its few FP64 instructions take the pipe as long for one
+    // lane as for 32) and read back by its warp; a thread combines the cell's sums at the end, so
+    // nothing of it stays in registers over the sample loop.
+    const double cp = a.cp[m], cw = a.cw[m];
+    for (int c = tid; c < nwarps * a.passes * V; c += blockDim.x) {
+        int t = a.L[k] + 1;  // "none" (no sample exceeds L); t in [0, L + 1] keeps |x - c| <= L + 1
+        if (c < cells) {
+            const double lam = s_lam[c % NL], mu = dmin_nonneg(lam, cp);
+            const RowOffset row = row_offset(cp, cw, a.L[k], a.r[r_cta0 + c / NL] - a.L_in[k]);
+            t = first_active(__dadd_rn(mu, dmin_nonneg(lam, cw)), excess_offset(row, cp, mu, to_double(a.L[k])), a.L[k]);
+        }
+        s_t[c] = t;
+    }
+    __syncthreads();
+    constexpr int NP = PAIR ? V / 2 : 1, NI = PAIR ? 1 : V;  // array extents
+    [[maybe_unused]] u64 n2c[NP], accf[NP];                  // -2c for two cells, their sums
+    [[maybe_unused]] int cci[NI];                            // 0x4B000000 + c per cell
+    [[maybe_unused]] unsigned acci[NI];
+    // Fold after at most `fe` loads of kPer samples each: a lane's sum is then at most kPer fe (L + 1),
+    // within 2^24 in FP32 (the transposition's 32-lane sums stay below 2^29), or as integers 32 lanes'
+    // sums below 2^32.  The same for every thread of the CTA.
+    constexpr long long kFoldLimit = PAIR ? (1ll << 24) : (1ll << 32) / 32 - 1;
+    const int fe = (int)min(1ll << 20, max(1ll, kFoldLimit / (X::kPer * ((long long)a.L[k] + 1))));
+    long long acc_r = 0;
+    auto fold = [&]() {
+        unsigned vs[V];
+        if constexpr (PAIR) {
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                float a0, a1;
+                upk(accf[p], a0, a1);
+                vs[2 * p] = __float2uint_rn(a0);
+                vs[2 * p + 1] = __float2uint_rn(a1);
+                accf[p] = 0ull;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; j++) {
+                vs[j] = acci[j];
+                acci[j] = 0u;
+            }
+        }
+        acc_r += (long long)transpose_reduce<unsigned, V>(vs, lane);
+    };
+    // One load into every cell's sum.  The pair sums' rate hangs on ptxas's register allocation (operand
+    // bank conflicts): written cell by cell, the second pair first, 16.06 ms on 8 classes x 100,000
+    // samples x 4096 r x 128 lam; first pair first 16.39, the accumulator as first operand 16.57, two
+    // cells' adds ahead of their max 16.91, all adds first 17.03; unrolled 4 / 16 times 16.6 / 16.5.
+    auto step = [&](const float4 v) {
+        if constexpr (PAIR) {
+            const u64 s0 = pk(v.x, v.x), s1 = pk(v.y, v.y);
+#pragma unroll
+            for (int p = 0; p < NP; p++)
+                accf[p] = fadd2(fadd2(max_abs2(fadd2(s1, n2c[p]), v.w), max_abs2(fadd2(s0, n2c[p]), v.z)), accf[p]);
+        } else {
+            const int ba = __float_as_int(v.x), bb = __float_as_int(v.z);  // 0x4B000000 + x
+#pragma unroll
+            for (int j = 0; j < V; j++) acci[j] = __sad(bb, cci[j], __sad(ba, cci[j], acci[j]));
+        }
+    };
+    constexpr int kSeg = 8;  // loads per segment of a fixed trip count
+    int pending = 0;         // loads since the last fold
+    auto room = [&](int loads) {  // fold first if the loads since the last fold would pass fe
+        if (pending + loads > fe) {
+            fold();
+            pending = 0;
+        }
+        pending += loads;
+    };
+    bool timeout = false;
+    int at = 0, c = 0, s = 0;  // chunk over all passes, of the class, its stage
+    uint32_t phase = 0;
+    const int* w_t = s_t + warp * V;  // the pass's thresholds
+    for (; at < total; at++) {
+        if (c == 0) {
+            if constexpr (PAIR) {
+#pragma unroll
+                for (int p = 0; p < NP; p++) {
+                    n2c[p] = pk((float)(2 - 2 * w_t[2 * p]), (float)(2 - 2 * w_t[2 * p + 1]));
+                    accf[p] = 0ull;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; j++) {
+                    cci[j] = kStageBits - 1 + w_t[j];
+                    acci[j] = 0u;
+                }
+            }
+        }
+        if (!mbar_wait_bounded(smem_u32(&full[s]), phase, a.wait_ns)) timeout = true;
+        if (!timeout) {
+            const int cnt = (int)min((int64_t)chunk, np - (int64_t)c * chunk);
+            const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * stage_bytes);
+            const int nq = cnt / (32 * X::kPer);
+            // loads [0, t_clean) hold samples only; of (x', x') pairs the class's last ones may hold NaN
+            // padding, which they read as x = 0 (x' = 2^23)
+            const int64_t left = a.N[k] - (int64_t)c * chunk;
+            const int t_clean = PAIR ? nq : (left <= 0 ? 0 : (int)min((int64_t)nq, left / (32 * X::kPer)));
+            int t0 = 0;
+            if (fe >= kSeg) {
+#pragma unroll 1
+                for (; t0 + kSeg <= t_clean; t0 += kSeg) {
+                    room(kSeg);
+#pragma unroll
+                    for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
+                }
+            }
+#pragma unroll 1
+            for (; t0 < nq; t0++) {
+                room(1);
+                float4 v = q[lane + 32 * t0];
+                if (!PAIR && t0 >= t_clean) {
+                    v.x = fmaxf(v.x, kStageOffset), v.y = fmaxf(v.y, kStageOffset);
+                    v.z = fmaxf(v.z, kStageOffset), v.w = fmaxf(v.w, kStageOffset);
+                }
+                step(v);
+            }
+        }
+        if (__syncthreads_or(timeout)) {
+            timeout = true;
+            break;
+        }
+        if (tid == 0 && at + a.stages < total) {
+            fence_proxy_async();
+            issue(chunk_after(c, a.stages), s);
+        }
+        if (++s == a.stages) {
+            s = 0;
+            phase ^= 1;
+        }
+        if (++c == nchunks) {  // the pass's sums
+            c = 0;
+            if (pending > 0) fold();
+            pending = 0;
+            if ((lane & ((1 << kOwn) - 1)) == 0)
+                reinterpret_cast<long long*>(s_S)[w_t - s_t + (lane >> kOwn)] = acc_r;
+            acc_r = 0;
+            w_t += nwarps * V;
+        }
+    }
+    if (timeout) {
+        // Report, then let every copy this CTA issued land before the CTA's shared memory is released:
+        // chunks up to `at` + stages - 1 were issued.
+        if (tid == 0) {
+            atomicOr(a.err + 1, kErrTimeout);
+            for (const int end = min(at + a.stages, total); at < end; at++) {
+                (void)mbar_wait_bounded(smem_u32(&full[s]), phase, a.wait_ns);
+                if (++s == a.stages) {
+                    s = 0;
+                    phase ^= 1;
+                }
+            }
+        }
+        __syncthreads();
+        return;
+    }
+    __syncthreads();
+    bool ok = true;
+    {
+        const long long N = a.N[k], sumx = a.sumx[k], npad = np - N;
+        const int L = a.L[k];
+        for (int i = tid; i < cells; i += blockDim.x) {
+            // the active count from the cumulative counts, then the branch sums
+            const int ti = s_t[i], rl = i / NL, lj = i % NL;  // ti in [0, L + 1]
+            const long long t = ti;
+            const long long count = ti <= 0 ? N : (ti > L ? 0 : N - (long long)a.cdf[a.hist_off[k] + t - 1]);
+            // sum |x - c| over the samples and the padding zeros; with y = x - c, max(y, 0) = (y + |y|) / 2
+            const long long sum_abs = dbits(s_S[i]) - npad * (t > 1 ? t - 1 : 1 - t);
+            const long long sum_y = sumx + N * (1 - t);
+            const long long sum_relu = (sum_y + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
+            const long long sum = sum_relu + (t - 1) * count;  // sum_{x >= t} x
+            // each sample on its own branch of phi (exact integer sums): V = c_w eta - nu x below t,
+            // U = c_p (L - eta) - mu (L - x) from t on; no large term cancels another
+            const double lam = s_lam[lj];
+            const double tot = branch_sum(cp, cw, dmin_nonneg(lam, cp), dmin_nonneg(lam, cw), L,
+                                          a.r[r_cta0 + rl] - a.L_in[k], N, count, sumx - sum, (long long)L * count - sum);
+            const double S = __dmul_rn(tot, a.inv_n[k]);
+            s_S[i] = S;  // in place of the sum, which only this thread reads
+            s_Sf[rl * lay.stride_f + lj] = cut(S, ok);
+            if (a.S_out) {
+                const size_t o = (((size_t)m * a.K + k) * a.R + r_cta0 + rl) * NL + lj;
+                if (a.f32_out) static_cast<float*>(a.S_out)[o] = (float)S;
+                else static_cast<double*>(a.S_out)[o] = S;
+            }
+        }
+        for (int i = tid; i < rows * 4; i += blockDim.x)
+            if (NL + (i & 3) < four(NL)) s_Sf[(i >> 2) * lay.stride_f + NL + (i & 3)] = INFINITY;
+        for (int j = tid; j < four(NL); j += blockDim.x) s_lamf[j] = j < NL ? cut(s_lam[j], ok) : 0.f;
+    }
+    if (!ok) s_bad = 1;
+    __syncthreads();
+    const LamRows x = {s_S, s_lam, s_eps, s_Sf, s_lamf, NL, lay.stride_f, rows, NL, s_bad == 0};
+    if (a.f32_out) lam_min_epilogue<true>(a, x, r_cta0, m, k);
+    else lam_min_epilogue<false>(a, x, r_cta0, m, k);
 }
 
 // The same cells in O(1) each from the class's cumulative counts C[v] = #{x <= v} and sums
@@ -919,9 +1033,9 @@ struct EnvSmem {
 };
 __host__ __device__ inline EnvSmem env_smem(int NL, int E) {
     EnvSmem s;
-    const int rows = env_rows(NL), n4 = (NL + 3) & ~3;
+    const int rows = env_rows(NL), n4 = four(NL);
     s.stride = NL | 1;  // odd: rows start in other banks
-    s.stride_f = 4 * (n4 / 4 | 1);  // read four at a time, lanes along the rows
+    s.stride_f = float_stride(NL);
     s.kap = 8 * (size_t)NL;
     s.eps = s.kap + 8 * (size_t)NL;
     s.S = s.eps + 8 * (size_t)E;
@@ -1039,79 +1153,19 @@ __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
             s_S[rl * lay.stride + j] = S;
             s_Sf[rl * lay.stride_f + j] = cut(S, ok);
             if (a.S_out) {
-                double* out = static_cast<double*>(a.S_out) + (((size_t)m * a.K + k) * a.R + r_cta0 + rl) * a.NL_out + a.lam0;
+                double* out = static_cast<double*>(a.S_out) + (((size_t)m * a.K + k) * a.R + r_cta0 + rl) * a.NL;
                 out[j] = S;
                 if (j == NLs - 1)
                     for (int i = NLs; i < NL; i++) out[i] = S;
             }
         }
-        for (int j = NLs + (lane & (W - 1)); j < ((NLs + 3) & ~3); j += W) s_Sf[rl * lay.stride_f + j] = INFINITY;
+        for (int j = NLs + (lane & (W - 1)); j < four(NLs); j += W) s_Sf[rl * lay.stride_f + j] = INFINITY;
     }
-    for (int j = NL + tid; j < ((NL + 3) & ~3); j += kEnvThreads) s_lamf[j] = 0.f;
+    for (int j = NL + tid; j < four(NL); j += kEnvThreads) s_lamf[j] = 0.f;
     if (!ok) s_bad[1] = 1;
     __syncthreads();
-    // G lanes per (r, eps) pair, as many as keep every thread busy, groups along r first (coalesced outputs,
-    // one atomic per warp and radius); each lane takes every G-th four lam values and keeps its smallest v', where it was, and its second smallest: with the second outside the
-    // window only that one value is formed in FP64, by all lanes at once.
-    const int pairs = rows * a.E, n4 = (NLs + 3) / 4;
-    int G = 1;
-    while (G < 32 && G < n4 && 2 * G * pairs <= kEnvThreads) G <<= 1;
-    const int per_pass = kEnvThreads / G, g = tid & (G - 1);
-    for (int p0 = 0; p0 < pairs; p0 += per_pass) {  // the same trips for every lane: the group's shuffles are warp-wide
-        const int p = p0 + tid / G;
-        const bool active = p < pairs;
-        const int e = active ? p / rows : 0, rl = active ? p % rows : 0;
-        const double* S = s_S + rl * lay.stride;
-        const double eps = s_eps[e];
-        const float4* lam4 = reinterpret_cast<const float4*>(s_lamf);
-        const float4* S4 = reinterpret_cast<const float4*>(s_Sf + rl * lay.stride_f);
-        bool fast = floats && s_bad[1] == 0;
-        const float ef = cut(eps, fast);
-        float m1 = INFINITY, m2 = INFINITY;
-        int j1 = 0;
-        for (int q = g; q < n4; q += G) {
-            const float4 l = lam4[q], s = S4[q];
-            const float v[4] = {fmaf(l.x, ef, s.x), fmaf(l.y, ef, s.y), fmaf(l.z, ef, s.z), fmaf(l.w, ef, s.w)};
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                m2 = fminf(m2, fmaxf(m1, v[i]));
-                if (v[i] < m1) j1 = 4 * q + i;
-                m1 = fminf(m1, v[i]);
-            }
-        }
-        for (int o = 1; o < G; o <<= 1) {
-            const float o1 = __shfl_xor_sync(0xffffffffu, m1, o), o2 = __shfl_xor_sync(0xffffffffu, m2, o);
-            const int oj = __shfl_xor_sync(0xffffffffu, j1, o);
-            m2 = fminf(fminf(m2, o2), fmaxf(m1, o1));
-            if (o1 < m1 || (o1 == m1 && oj < j1)) j1 = oj;
-            m1 = fminf(m1, o1);
-        }
-        fast = fast && m1 > kLamFloor;
-        const float thr = m1 * kLamWindow;
-        LamMin best;
-        if (fast && m2 > thr) {
-            best.v = __dadd_rn(__dmul_rn(s_lam[j1], eps), S[j1]);
-            best.j = j1;
-        }
-        const bool several = active && best.j == 0x7fffffff;
-        if (__any_sync(0xffffffffu, several)) {
-            LamMin r;
-            if (several)
-                for (int j = g; j < NLs; j += G)
-                    if (!fast || fmaf(s_lamf[j], ef, s_Sf[rl * lay.stride_f + j]) <= thr)
-                        r.take(s_lam[j], eps, S[j], j, fast, s_lam, S);
-            r.reduce(G);
-            if (several) best = r;
-        }
-        u64 key = ~0ull;
-        if (active && g == 0) key = write_pair<false>(a, best.v, best.j, m, k, e, r_cta0 + rl);
-        // the warp's minimum over each radius it holds, e0 (its first lane's) upwards
-        const int e0 = __shfl_sync(0xffffffffu, e, 0), e1 = __reduce_max_sync(0xffffffffu, e);
-        for (int ei = e0; ei <= e1; ei++) {
-            const u64 low = group_min(e == ei ? key : ~0ull, 32);
-            if (lane == 0 && low != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + ei) * a.K + k, low);
-        }
-    }
+    const LamRows rows_of = {s_S, s_lam, s_eps, s_Sf, s_lamf, lay.stride, lay.stride_f, rows, NLs, floats && s_bad[1] == 0};
+    lam_min_epilogue<false>(a, rows_of, r_cta0, m, k);
 }
 
 template <Prec P>
@@ -1147,52 +1201,98 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
     sh.LT = (NL + C::TL - 1) / C::TL;
     sh.RG = sh.LT >= kWarpsTarget ? 1 : kWarpsTarget / sh.LT;
     sh.threads = 32 * sh.LT * sh.RG;
-    sh.r_blocks = (R + sh.RG * C::TR - 1) / (sh.RG * C::TR);
+    sh.rows = sh.RG * C::TR;
+    sh.stages = C::STAGES;
+    sh.r_blocks = (R + sh.rows - 1) / sh.rows;
     sh.smem = smem_layout(sh.RG, C::TR, sh.LT * C::TL, E, C::CHUNK * C::BYTES, C::STAGES).total;
     return sh;
 }
 
-GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L) {
+// Rows per CTA and passes over the samples.  A pass is 256 cells (16 warps); more passes lay a CTA's rows
+// over more of them, so that fewer cells stand empty at the end, but leave fewer CTAs to fill the last wave.
+// The choice maximises cells filled x waves filled.  One pass of fewer warps instead of empty cells is worth
+// less than its cells: 13 warps per CTA held 75 % of the rate (5 classes x 1001 r x 200 lam x 3 regimes 2.27
+// ms in one pass, 1.90 in four; 2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
+template <bool PAIR>
+GridShape exact_shape(int variant, int32_t R, int32_t NL, int32_t E, int64_t classes, int sms) {
+    using X = ExactCfg<PAIR>;
+    constexpr int kCells = kExactWarps * kExactV;
+    GridShape best, sh;
+    sh.variant = variant;
+    sh.LT = sh.RG = 1;
+    double best_score = -1.0;
+    for (int passes = 1; passes <= kExactMaxPasses; passes++) {
+        const int rows = std::min(R, passes * kCells / NL);
+        if (rows < 1) continue;
+        const int tiles = (rows * NL + kExactV - 1) / kExactV;
+        sh.rows = rows;
+        sh.passes = (tiles + kExactWarps - 1) / kExactWarps;
+        const int warps = (tiles + sh.passes - 1) / sh.passes;
+        sh.threads = 32 * warps;
+        sh.r_blocks = (R + rows - 1) / rows;
+        // 96 KB of ring: three 32 KB chunks of pair sums (8192 samples; two of 32, 36 or 48 KB, four of 24
+        // and six of 16 measured 2 to 5 % slower) or two 48 KB chunks of (x', x') pairs; smaller chunks where
+        // the cells need the room
+        sh.stages = PAIR ? 3 : 2;
+        sh.chunk = X::kChunk;
+        do {
+            sh.smem = exact_smem(rows, NL, E, warps * sh.passes, sh.stages * sh.chunk * X::kBytes).total;
+        } while (sh.smem > kExactSmem && (sh.chunk -= 1024) > 0);
+        const double slots = 2.0 * sms, ctas = (double)classes * sh.r_blocks, waves = ctas / slots;
+        const double filled = (double)R * NL / ((double)sh.r_blocks * warps * sh.passes * kExactV);
+        const double rate = 0.55 + 0.45 * warps / kExactWarps;  // of full occupancy's
+        const double score = filled * (warps < kExactWarps ? rate : 1.0) * waves / std::ceil(waves);
+        if (score > best_score + 0.02) {
+            best_score = score;
+            best = sh;
+        }
+    }
+    return best;
+}
+
+GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, int64_t classes, int sms) {
     if (p == Prec::ENVELOPE) {
         GridShape sh;
         sh.variant = 4;
-        sh.LT = 1;
-        sh.RG = 1;
+        sh.LT = sh.RG = sh.stages = 1;
         sh.threads = kEnvThreads;
-        sh.r_blocks = (R + env_rows(NL) - 1) / env_rows(NL);
+        sh.rows = env_rows(NL);
+        sh.r_blocks = (R + sh.rows - 1) / sh.rows;
         sh.smem = env_smem(NL, E).total;
         return sh;
     }
     if (p == Prec::F64) return shape_for<CfgF64>(2, R, NL, E);
-    if (p == Prec::EXACT) {  // NL <= kExactLamBlock: larger grids launch in blocks
-        if (max_L > kPairMaxL) return NL <= kFewLam ? shape_for<CfgExactIntFewLam>(9, R, NL, E) : shape_for<CfgExactInt>(6, R, NL, E);
-        return NL <= kFewLam ? shape_for<CfgExactFewLam>(8, R, NL, E) : shape_for<CfgExact>(3, R, NL, E);
-    }
+    if (p == Prec::EXACT)
+        return max_L > kPairMaxL ? exact_shape<false>(6, R, NL, E, classes, sms) : exact_shape<true>(3, R, NL, E, classes, sms);
     if (NL <= kWarpsTarget * CfgF32::TL) return shape_for<CfgF32>(0, R, NL, E);
     return shape_for<CfgF32Wide>(1, R, NL, E);
 }
 
-// Raises the kernel's shared-memory limit to the largest layout its shapes can have: all of its warps,
-// 64 eps.
+namespace {
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// The largest layout the kernel's shapes can have: all of its warps, 64 eps.
 template <class C>
 cudaError_t prepare() {
     const int warps = C::MAXT / 32;
-    return cudaFuncSetAttribute(k_grid<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_layout(1, C::TR, warps * C::TL, 64, C::CHUNK * C::BYTES, C::STAGES).total + 256);
+    size_t most = 0;
+    for (int lt = 1; lt <= warps; lt++)
+        most = std::max(most, smem_layout(std::max(1, kWarpsTarget / lt), C::TR, lt * C::TL, 64, C::CHUNK * C::BYTES, C::STAGES).total);
+    return allow_smem((const void*)k_grid<C>, most);
 }
+
+}  // namespace
 
 cudaError_t grid_prepare(Prec p) {
     if (p == Prec::F64) return prepare<CfgF64>();
     if (p == Prec::EXACT) {
-        cudaError_t e = prepare<CfgExact>();
-        if (e == cudaSuccess) e = prepare<CfgExactInt>();
-        if (e == cudaSuccess) e = prepare<CfgExactFewLam>();
-        if (e == cudaSuccess) e = prepare<CfgExactIntFewLam>();
-        return e;
+        const cudaError_t e = allow_smem((const void*)k_exact<true>, kExactSmem);
+        return e == cudaSuccess ? allow_smem((const void*)k_exact<false>, kExactSmem) : e;
     }
-    if (p == Prec::ENVELOPE)
-        return cudaFuncSetAttribute(k_envelope, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)env_smem(256, 64).total);
+    if (p == Prec::ENVELOPE) return allow_smem((const void*)k_envelope, env_smem(256, 64).total);
     const cudaError_t e = prepare<CfgF32>();
     return e == cudaSuccess ? prepare<CfgF32Wide>() : e;
 }
@@ -1200,15 +1300,17 @@ cudaError_t grid_prepare(Prec p) {
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s) {
     a.LT = sh.LT;
     a.RG = sh.RG;
+    a.rows = sh.rows;
+    a.stages = sh.stages;
+    a.passes = sh.passes;
+    a.chunk = sh.chunk;
     a.r_blocks = sh.r_blocks;
     const int64_t nblocks = (int64_t)a.m_count * a.K * a.r_blocks;
     if (nblocks <= 0 || nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (p == Prec::ENVELOPE) k_envelope<<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (p == Prec::F64) k_grid<CfgF64><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT && sh.variant == 3) k_grid<CfgExact><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT && sh.variant == 8) k_grid<CfgExactFewLam><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT && sh.variant == 9) k_grid<CfgExactIntFewLam><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT) k_grid<CfgExactInt><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
+    else if (p == Prec::EXACT && sh.variant == 3) k_exact<true><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
+    else if (p == Prec::EXACT) k_exact<false><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (sh.variant == 0) k_grid<CfgF32><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else k_grid<CfgF32Wide><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     return cudaGetLastError();

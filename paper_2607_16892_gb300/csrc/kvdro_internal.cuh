@@ -91,8 +91,12 @@ struct GridArgs {
     const double* cp;           // [M]
     const double* cw;           // [M]
     int32_t K, R, NL, E, M;
-    int32_t LT;                 // lam tiles per CTA
-    int32_t RG;                 // r groups per CTA
+    int32_t LT;                 // lam tiles per CTA (FP32 and FP64 kernels)
+    int32_t RG;                 // r groups per CTA (FP32 and FP64 kernels)
+    int32_t rows;               // r values per CTA
+    int32_t stages;             // ring depth
+    int32_t passes;             // over the samples (exact kernel)
+    int32_t chunk;              // samples per staged chunk (exact kernel)
     int32_t r_blocks;           // CTAs per (m, k)
     int32_t m0, m_count;        // regime range covered by this launch
     int32_t f32_out;            // exact kernel: write S, cost and the argmin keys as FP32 (FP32 mode)
@@ -106,20 +110,7 @@ struct GridArgs {
     // the waits on it run out (-1 in production).
     long long wait_ns;
     int32_t test_skip_chunk;
-    // Lam blocks: a grid of more lam values than one launch takes runs as consecutive launches over
-    // blocks of it (ascending lam).  lam / NL are this block's values; lam0 is the index of its
-    // first value in the caller's grid of NL_out values.  With several blocks, part_val / part_idx
-    // ([m - m0][E][K][R]) carry each (r, eps) pair's minimum over the earlier blocks; the first
-    // block starts them, the last writes the outputs.  One block: part_val is null, lam0 = 0.
-    int32_t lam0, NL_out;
-    double* part_val;
-    int32_t* part_idx;
-    int32_t part_first, part_last;
 };
-
-// The largest lam grid one launch of the exact kernel takes (16 warps of 2 x 8 tiles); larger
-// grids run in blocks of it.
-constexpr int32_t kExactLamBlock = 128;
 
 struct FinalizeArgs {
     const unsigned long long* keys;
@@ -136,16 +127,21 @@ struct FinalizeArgs {
 };
 
 // grid.cu
-// Launch shape of the grid kernel for one (precision, grid) problem: which compiled variant,
-// lam tiles x r groups of warps per CTA, CTAs per (regime, class), dynamic shared memory.
+// Launch shape of the grid kernel for one (precision, grid) problem: which compiled variant, its
+// r values, warps and ring depth per CTA, CTAs per (regime, class), dynamic shared memory.
 struct GridShape {
     int variant;       // index of the compiled kernel instantiation
-    int LT, RG;        // lam tiles and r groups per CTA
-    int threads;       // 32 * LT * RG
+    int LT, RG;        // lam tiles and r groups per CTA (FP32 and FP64 kernels: LT * RG warps)
+    int rows, stages;  // r values per CTA, ring depth
+    int passes = 1;    // over the samples, and samples per staged chunk (exact kernel)
+    int chunk = 0;
+    int threads;
     int r_blocks;      // CTAs per (m, k)
     size_t smem;
 };
-GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L);  // max_L: largest support
+// max_L: largest support; classes: (regime, class) pairs that the request evaluates; sms: of the device
+GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, int64_t classes, int sms);
+cudaError_t sm_count(int* sms);  // of the current device (sort.cu)
 cudaError_t grid_prepare(Prec p);             // per-device attribute setup of every variant of p
 // Launches over regimes [a.m0, a.m0 + a.m_count); fills a.LT, a.RG, a.r_blocks from `sh`.
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s);

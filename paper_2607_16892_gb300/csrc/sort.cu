@@ -356,13 +356,18 @@ __global__ void k_gather_quantiles(const int32_t* sorted, const int64_t* offsets
 
 }  // namespace
 
+cudaError_t sm_count(int* sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
 // Histogram blocks of each class (written as a prefix over the classes): slices of at most
 // kHistSlice and at least kHistMinSlice samples, as many as fill whole waves of the device's
 // resident histogram blocks -- a last wave only a little filled would leave most SMs idle.
 cudaError_t hist_block_prefix(const int64_t* N, int32_t K, int32_t* prefix) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = sm_count(&sms);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_histogram, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kHistSmemBins * (int)sizeof(int32_t));

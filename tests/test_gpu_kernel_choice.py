@@ -115,3 +115,20 @@ def test_dual_on_each_side_of_the_smaller_cost(L, cp, cw):
     size = cw * L + cp * L + max(cp, cw) * L  # the lines that cross at a minimiser are no larger
     assert np.all(np.abs(cost - ref) <= 1e-12 * np.abs(ref) + 16 * np.finfo(float).eps * size)
     assert np.all((gamma >= 0) & (gamma <= max(cp, cw)))
+
+
+@pytest.mark.parametrize("nl", [9, 72, 100, 129, 200])
+def test_exact_passes_over_the_samples(nl, monkeypatch):
+    """CTAs whose rows take two to four passes (the chunk ring runs on across them, classes of one and of two
+    chunks), against the envelope's same integers; and a bounded wait that runs out inside such a CTA."""
+    rng = np.random.default_rng(nl)
+    w = make([rng.integers(0, 3001, 9001), rng.integers(0, 400, 333)], 3000, np.arange(0, 3001, 3), np.logspace(-3, 2, nl),
+             [0.0, 7.0, 90.0], [10.0, 4.0, 300.0], [1.0, 1.0, 1.0])
+    outputs = ("cost", "lam_idx", "r_idx", "min_cost", "fhat")
+    exact, env = run(w, kvdro.KVDRO_EXACT, outputs=outputs), run(w, kvdro.KVDRO_ENVELOPE, outputs=outputs)
+    for key, v in exact.items():
+        assert np.array_equal(v, env[key]), key
+    monkeypatch.setenv("KVDRO_TEST_SKIP_CHUNK", "1")
+    with pytest.raises(kvdro.KvdroError) as e:
+        run(w, kvdro.KVDRO_EXACT, outputs=outputs, host_outputs=True)
+    assert e.value.status == kvdro.KVDRO_ETIMEOUT
