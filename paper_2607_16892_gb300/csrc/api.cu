@@ -21,6 +21,7 @@ namespace kvdro {
 int64_t hist_slice_samples();
 int64_t expand_tile_positions();
 int64_t scan_tile_bins();
+bool scan_direct(int64_t scan_tiles);
 }  // namespace kvdro
 
 using kvdro::Prec;
@@ -65,7 +66,7 @@ struct kvdro_ctx {
     std::vector<int32_t> L, Lin, hist_blocks, exp_blocks;
     std::vector<double> inv_n;
 
-    Buf sorted, pairs, hist, csum, sumx, meta, errs, in_stage, grid_in, keys, cost64, out_stage, ranks, scan_tot,
+    Buf sorted, pairs, hist, cum, csum, sumx, meta, errs, in_stage, grid_in, keys, cost64, out_stage, ranks, scan_tot,
         tile_lo;
     void* pin = nullptr;  // pinned host staging
     size_t pin_bytes = 0;
@@ -79,6 +80,7 @@ struct kvdro_ctx {
     // device views into `meta`
     int64_t *d_off = nullptr, *d_pair_off = nullptr, *d_hist_off = nullptr, *d_N = nullptr;
     double* d_inv_n = nullptr;
+    int32_t* d_cum = nullptr;  // cumulative counts
     int32_t *d_L = nullptr, *d_Lin = nullptr, *d_hist_blocks = nullptr, *d_exp_blocks = nullptr;
 };
 
@@ -275,7 +277,7 @@ int kvdro_destroy(kvdro_ctx* ctx) {
     DeviceGuard g(ctx->device);
     if (ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
     cudaDeviceSynchronize();
-    for (Buf* b : {&ctx->sorted, &ctx->scan_tot, &ctx->pairs, &ctx->hist, &ctx->csum, &ctx->sumx, &ctx->meta, &ctx->errs, &ctx->in_stage,
+    for (Buf* b : {&ctx->sorted, &ctx->scan_tot, &ctx->pairs, &ctx->hist, &ctx->cum, &ctx->csum, &ctx->sumx, &ctx->meta, &ctx->errs, &ctx->in_stage,
                    &ctx->grid_in, &ctx->keys, &ctx->cost64, &ctx->out_stage, &ctx->ranks, &ctx->tile_lo})
         release(*b);
     if (ctx->pin) cudaFreeHost(ctx->pin);
@@ -358,6 +360,9 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     if ((rc = ensure(ctx, ctx->sumx, (size_t)K * 8))) return rc;
     if ((rc = ensure(ctx, ctx->errs, 2 * sizeof(int32_t)))) return rc;
     const int64_t scan_tiles = ((int64_t)max_L + 1 + kvdro::scan_tile_bins() - 1) / kvdro::scan_tile_bins();
+    const bool direct = kvdro::scan_direct(scan_tiles);
+    if (direct && (rc = ensure(ctx, ctx->cum, (size_t)ctx->hist_total * 4))) return rc;
+    ctx->d_cum = static_cast<int32_t*>(direct ? ctx->cum.p : ctx->hist.p);
     if ((rc = ensure(ctx, ctx->scan_tot, (size_t)K * scan_tiles * 16))) return rc;
     if ((rc = ensure(ctx, ctx->tile_lo, ((size_t)ctx->exp_blocks[K] + K) * 4))) return rc;
     const size_t meta_bytes = (size_t)(K + 1) * 8 * 3 + (size_t)K * 8 * 2 + (size_t)K * 4 * 2 + (size_t)(K + 1) * 4 * 2 + 64;
@@ -394,7 +399,6 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
         dlen = static_cast<const int32_t*>(ctx->in_stage.p);
     }
     KV_CUDA(cudaMemsetAsync(ctx->hist.p, 0, (size_t)ctx->hist_total * 4, s), "clearing histogram");
-    KV_CUDA(cudaMemsetAsync(ctx->sumx.p, 0, (size_t)K * 8, s), "clearing sums");
     KV_CUDA(cudaMemsetAsync(ctx->errs.p, 0, 2 * sizeof(int32_t), s), "clearing status");
 
     kvdro::SortArgs a;
@@ -406,6 +410,7 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     a.hist_blocks = ctx->d_hist_blocks;
     a.exp_blocks = ctx->d_exp_blocks;
     a.hist = static_cast<int32_t*>(ctx->hist.p);
+    a.cum = ctx->d_cum;
     a.csum = static_cast<int64_t*>(ctx->csum.p);
     a.sumx = static_cast<int64_t*>(ctx->sumx.p);
     a.sorted = static_cast<int32_t*>(ctx->sorted.p);
@@ -596,7 +601,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     a.sumx = static_cast<const int64_t*>(ctx->sumx.p);
     a.L = ctx->d_L;
     a.L_in = ctx->d_Lin;
-    a.cdf = static_cast<const int32_t*>(ctx->hist.p);
+    a.cdf = ctx->d_cum;
     a.csum = static_cast<const int64_t*>(ctx->csum.p);
     a.hist_off = ctx->d_hist_off;
     a.r = d_r;
@@ -663,7 +668,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     fa.r = d_r;
     fa.L_in = ctx->d_Lin;
     fa.N = ctx->d_N;
-    fa.cdf = static_cast<const int32_t*>(ctx->hist.p);
+    fa.cdf = ctx->d_cum;
     fa.hist_off = ctx->d_hist_off;
     fa.K = ctx->K;
     fa.R = R;
@@ -769,7 +774,7 @@ int kvdro_eval_dual(kvdro_ctx* ctx, int32_t R, const int32_t* r, int32_t E, cons
     KV_CUDA(cudaMemsetAsync(ctx->keys.p, 0xFF, (size_t)rows * 8, s), "clearing argmin keys");
 
     kvdro::DualArgs a;
-    a.cdf = static_cast<const int32_t*>(ctx->hist.p);
+    a.cdf = ctx->d_cum;
     a.csum = static_cast<const int64_t*>(ctx->csum.p);
     a.hist_off = ctx->d_hist_off;
     a.N = ctx->d_N;

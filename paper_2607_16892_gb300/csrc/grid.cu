@@ -1210,9 +1210,10 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
 
 // Rows per CTA and passes over the samples.  A pass is 256 cells (16 warps); more passes lay a CTA's rows
 // over more of them, so that fewer cells stand empty at the end, but leave fewer CTAs to fill the last wave.
-// The choice maximises cells filled x waves filled.  One pass of fewer warps instead of empty cells is worth
-// less than its cells: 13 warps per CTA held 75 % of the rate (5 classes x 1001 r x 200 lam x 3 regimes 2.27
-// ms in one pass, 1.90 in four; 2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
+// The choice maximises cells filled x waves filled.  A warp left out saves nothing while its scheduler still
+// holds as many as the others (13 to 16 warps take the same time), and fewer per scheduler run at a lower
+// rate: 5 classes x 1001 r x 200 lam x 3 regimes 2.27 ms in one pass of 13 warps, 1.90 in four passes of 16
+// (2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
 template <bool PAIR>
 GridShape exact_shape(int variant, int32_t R, int32_t NL, int32_t E, int64_t classes, int sms) {
     using X = ExactCfg<PAIR>;
@@ -1239,10 +1240,11 @@ GridShape exact_shape(int variant, int32_t R, int32_t NL, int32_t E, int64_t cla
             sh.smem = exact_smem(rows, NL, E, warps * sh.passes, sh.stages * sh.chunk * X::kBytes).total;
         } while (sh.smem > kExactSmem && (sh.chunk -= 1024) > 0);
         const double slots = 2.0 * sms, ctas = (double)classes * sh.r_blocks, waves = ctas / slots;
-        const double filled = (double)R * NL / ((double)sh.r_blocks * warps * sh.passes * kExactV);
-        const double rate = 0.55 + 0.45 * warps / kExactWarps;  // of full occupancy's
-        const double score = filled * (warps < kExactWarps ? rate : 1.0) * waves / std::ceil(waves);
-        if (score > best_score + 0.02) {
+        const int held = (warps + 3) / 4 * 4;  // warps that the fullest of the four schedulers accounts for
+        const double filled = (double)R * NL / ((double)sh.r_blocks * held * sh.passes * kExactV);
+        const double rate = 0.55 + 0.45 * held / kExactWarps;
+        const double score = filled * rate * waves / std::ceil(waves);
+        if (score > best_score + 0.01) {
             best_score = score;
             best = sh;
         }

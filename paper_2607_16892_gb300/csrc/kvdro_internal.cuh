@@ -28,9 +28,10 @@ struct SortArgs {
     const int64_t* pair_off;    // [K+1] start of class k's padded region, in samples
     const int32_t* hist_blocks; // [K+1] prefix of histogram blocks per class
     const int32_t* exp_blocks;  // [K+1] prefix of expand blocks per class
-    int32_t* hist;              // [hist_off[K]] counts, then cumulative counts (in place)
+    int32_t* hist;              // [hist_off[K]] counts, zero before the histogram
+    int32_t* cum;               // [hist_off[K]] cumulative counts; may be `hist` (must, past scan_direct's tiles)
     int64_t* csum;              // [hist_off[K]] cumulative sums sum_{x <= v} x, or nullptr to skip
-    int64_t* sumx;              // [K] sum of samples per class
+    int64_t* sumx;              // [K] sum of samples per class (written by the scan)
     int32_t* sorted;            // [offsets[K]]
     void* staged;               // pair_off[K] samples, 4 bytes each as pair sums or 8 as (x', x') pairs
     int32_t* err;               // [0] += out-of-range samples

@@ -240,7 +240,6 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     NA_CUDA(cudaMemcpyAsync(S + o_cp, c_p, (size_t)M * 8, cudaMemcpyHostToDevice, s));
     NA_CUDA(cudaMemcpyAsync(S + o_cw, c_w, (size_t)M * 8, cudaMemcpyHostToDevice, s));
     NA_CUDA(cudaMemsetAsync(S + o_err, 0, 2 * sizeof(int32_t), s));
-    NA_CUDA(cudaMemsetAsync(S + o_sumx, 0, (size_t)K * 8, s));
     NA_CUDA(cudaMemsetAsync(S + o_hist, 0, (size_t)hist_total * 4, s));
     NA_CUDA(cudaMemsetAsync(S + o_keys, 0xFF, (size_t)rows * 8, s));
     Meta mt;
@@ -268,7 +267,7 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     sa.pair_off = mt.pair_off;
     sa.hist_blocks = mt.hist_blocks;
     sa.exp_blocks = mt.exp_blocks;
-    sa.hist = reinterpret_cast<int32_t*>(S + o_hist);
+    sa.hist = sa.cum = reinterpret_cast<int32_t*>(S + o_hist);
     sa.csum = nullptr;  // cumulative sums are not needed here
     sa.sumx = reinterpret_cast<int64_t*>(S + o_sumx);
     sa.sorted = reinterpret_cast<int32_t*>(S + o_sorted);

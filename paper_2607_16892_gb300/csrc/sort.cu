@@ -17,16 +17,20 @@ namespace kvdro {
 namespace {
 
 constexpr int kHistThreads = 512;
-constexpr int64_t kHistSlice = 1 << 16;  // samples per histogram block
-constexpr int kHistSmemBins = 16384;     // bins [0, 16384) privatised in shared memory (64 KB)
-constexpr int kScanThreads = 1024;
-constexpr int64_t kScanTile = (int64_t)kScanThreads * 4;  // bins per scan block
-constexpr int kExpandThreads = 512;
-constexpr int kExpandPerThread = 8;
-constexpr int64_t kExpandTile = (int64_t)kExpandThreads * kExpandPerThread;
+constexpr int64_t kHistSlice = 65535;  // samples per histogram block: its counts fit 16 bits
+// Bins [0, 2 kHistWords) are privatised in shared memory (66 KB, three blocks per SM), bin v in the low and
+// v + kHistWords in the high half of word v: neighbouring values, the frequent ones, stay in words of their
+// own.  A class whose support they cover counts without the global path, whose mere presence in the loop
+// costs as much again: 32 M samples of support 32768 in 44 us (2.9 TB/s); 68 with the upper half counted in global memory.
+constexpr int kHistWords = 16448;
+constexpr int kScanThreads = 512;
+constexpr int kScanPer = 8;
+constexpr int64_t kScanTile = (int64_t)kScanThreads * kScanPer;  // bins per scan block
+constexpr int kExpandThreads = 256;
+constexpr int64_t kExpandTile = 4096;  // sorted positions per expansion block
 // Histogram slices get at least this many samples, so that counting outweighs clearing and
 // flushing the block's shared bins.
-constexpr int64_t kHistMinSlice = kHistSmemBins;
+constexpr int64_t kHistMinSlice = kHistWords;
 
 __device__ __forceinline__ int find_segment(const int32_t* prefix, int K, int b) {
     // largest k with prefix[k] <= b; prefix is strictly increasing, prefix[0] = 0
@@ -38,10 +42,47 @@ __device__ __forceinline__ int find_segment(const int32_t* prefix, int K, int b)
     return lo;
 }
 
+// Counts src[beg, end) into the block's bins; returns how many samples lie outside [0, L].  An unsigned
+// comparison is the whole range check (a negative x wraps above L).
+template <bool COVERED>
+__device__ __forceinline__ int count_slice(const int32_t* src, int64_t beg, int64_t end, uint32_t L, uint32_t* bins,
+                                           int32_t* gh) {
+    int bad = 0;
+    auto count = [&](int32_t x) {
+        const uint32_t u = (uint32_t)x;
+        const bool ok = u <= L;
+        bad += ok ? 0 : 1;
+        if (COVERED ? ok : ok && u < 2 * kHistWords) atomicAdd(bins + (u < kHistWords ? u : u - kHistWords), u < kHistWords ? 1u : 65536u);
+        if (!COVERED && ok && u >= 2 * kHistWords) atomicAdd(gh + u, 1);
+    };
+    // 16-byte loads of four samples over the slice's aligned middle (alignment is taken from the
+    // address: `lengths` is the caller's pointer): each thread loads its next two vectors before
+    // it counts the current two, so four loads are in flight while the atomics run; the unaligned
+    // head and the tail one sample at a time.
+    const int64_t mis = (int64_t)((reinterpret_cast<uintptr_t>(src + beg) >> 2) & 3);
+    const int64_t vbeg = min(end, beg + ((4 - mis) & 3));
+    const int nvec = (int)((end - vbeg) >> 2);
+    const int64_t vend = vbeg + 4 * (int64_t)nvec;
+    for (int64_t i = beg + threadIdx.x; i < vbeg; i += kHistThreads) count(__ldg(src + i));
+    const int4* v4 = reinterpret_cast<const int4*>(src + vbeg);
+    auto four = [&](const int4 v) { count(v.x), count(v.y), count(v.z), count(v.w); };
+    int q = threadIdx.x;
+    int4 u = q < nvec ? __ldg(v4 + q) : int4(), w = q + kHistThreads < nvec ? __ldg(v4 + q + kHistThreads) : int4();
+    for (; q + kHistThreads < nvec; q += 2 * kHistThreads) {
+        const int n = q + 2 * kHistThreads;
+        const int4 u2 = n < nvec ? __ldg(v4 + n) : int4(), w2 = n + kHistThreads < nvec ? __ldg(v4 + n + kHistThreads) : int4();
+        four(u);
+        four(w);
+        u = u2;
+        w = w2;
+    }
+    if (q < nvec) four(u);
+    for (int64_t i = vend + threadIdx.x; i < end; i += kHistThreads) count(__ldg(src + i));
+    return bad;
+}
+
 __global__ void __launch_bounds__(kHistThreads) k_histogram(SortArgs a) {
-    extern __shared__ int32_t sh_bins[];
-    __shared__ int32_t sh_bad[kHistThreads / 32];
-    __shared__ unsigned long long sh_sum[kHistThreads / 32];
+    extern __shared__ uint32_t sh_bins[];
     const int k = find_segment(a.hist_blocks, a.K, blockIdx.x);
     // the class's samples in equal slices, one per block (at most kHistSlice each)
     const int64_t nblk = a.hist_blocks[k + 1] - a.hist_blocks[k];
@@ -50,299 +91,250 @@ __global__ void __launch_bounds__(kHistThreads) k_histogram(SortArgs a) {
     const int64_t beg = a.offsets[k] + slice * slice_len;
     const int64_t end = min(a.offsets[k + 1], beg + slice_len);
     const int32_t Lk = a.L[k];
-    const int nb = min(Lk + 1, kHistSmemBins);
+    const int words = min(Lk + 1, kHistWords);
     int32_t* gh = a.hist + a.hist_off[k];
-    for (int v = threadIdx.x; v < nb; v += blockDim.x) sh_bins[v] = 0;
+    for (int v = threadIdx.x; v < words; v += kHistThreads) sh_bins[v] = 0;
     __syncthreads();
-    // Per sample: an unsigned comparison is the whole range check (a negative x wraps above L),
-    // and the two atomics are predicated, so a sample costs no branch.  A thread counts at most
-    // ceil(kHistSlice / kHistThreads) = 128 samples of at most 2^24, so its sum fits 32 bits.
-    int bad = 0;
-    uint32_t sum32 = 0;
-    auto count = [&](int32_t x) {
-        const bool ok = (uint32_t)x <= (uint32_t)Lk;
-        bad += ok ? 0 : 1;
-        sum32 += ok ? (uint32_t)x : 0u;
-        const bool in_smem = ok && x < nb, in_gmem = ok && x >= nb;
-        if (in_smem) atomicAdd(&sh_bins[x], 1);
-        if (in_gmem) atomicAdd(&gh[x], 1);
-    };
-    // 16-byte loads of four samples over the slice's aligned middle (alignment is taken from the
-    // address: `lengths` is the caller's pointer): each thread loads its next two vectors before
-    // it counts the current two, so four loads are in flight while the atomics run; the unaligned
-    // head and the tail one sample at a time.
-    const int32_t* src = a.lengths;
-    const int64_t mis = (int64_t)((reinterpret_cast<uintptr_t>(src + beg) >> 2) & 3);
-    const int64_t vbeg = min(end, beg + ((4 - mis) & 3));
-    const int64_t nvec = (end - vbeg) >> 2;
-    const int64_t vend = vbeg + 4 * nvec;
-    for (int64_t i = beg + threadIdx.x; i < vbeg; i += blockDim.x) count(__ldg(src + i));
-    const int4* v4 = reinterpret_cast<const int4*>(src + vbeg);
-    const int64_t bd = blockDim.x;
-    int64_t q = threadIdx.x;
-    int4 u = make_int4(0, 0, 0, 0), w = make_int4(0, 0, 0, 0);
-    bool hu = q < nvec, hw = q + bd < nvec;
-    if (hu) u = __ldg(v4 + q);
-    if (hw) w = __ldg(v4 + q + bd);
-    while (hu) {
-        const int64_t qn = q + 2 * bd;
-        const bool nu = qn < nvec, nw = qn + bd < nvec;
-        int4 u2 = make_int4(0, 0, 0, 0), w2 = make_int4(0, 0, 0, 0);
-        if (nu) u2 = __ldg(v4 + qn);
-        if (nw) w2 = __ldg(v4 + qn + bd);
-        count(u.x); count(u.y); count(u.z); count(u.w);
-        if (hw) {
-            count(w.x); count(w.y); count(w.z); count(w.w);
-        }
-        u = u2;
-        w = w2;
-        hu = nu;
-        hw = nw;
-        q = qn;
-    }
-    for (int64_t i = vend + threadIdx.x; i < end; i += blockDim.x) count(__ldg(src + i));
+    int bad = Lk < 2 * kHistWords ? count_slice<true>(a.lengths, beg, end, Lk, sh_bins, gh)
+                                  : count_slice<false>(a.lengths, beg, end, Lk, sh_bins, gh);
     __syncthreads();
-    for (int v = threadIdx.x; v < nb; v += blockDim.x) {
-        const int c = sh_bins[v];
-        if (c) atomicAdd(&gh[v], c);
+    for (int v = threadIdx.x; v < words; v += kHistThreads) {
+        const uint32_t c = sh_bins[v];
+        if (c & 0xffffu) atomicAdd(gh + v, (int32_t)(c & 0xffffu));
+        if (c >> 16) atomicAdd(gh + v + kHistWords, (int32_t)(c >> 16));
     }
-    unsigned long long sum = sum32;
-    for (int o = 16; o; o >>= 1) {
-        bad += __shfl_xor_sync(0xffffffffu, bad, o);
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    }
-    const int wid = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) { sh_bad[wid] = bad; sh_sum[wid] = sum; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tb = 0;
-        unsigned long long ts = 0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) { tb += sh_bad[i]; ts += sh_sum[i]; }
-        if (tb) atomicAdd(a.err, tb);
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.sumx + k), ts);
+    bad = __reduce_add_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0 && bad) atomicAdd(a.err, bad);
+}
+
+// The cumulative counts and sums of every class over tiles of kScanTile bins, one block per (tile, class)
+// so that every SM takes part: each tile's inclusive scan, offset by the class's earlier tiles, whose
+// totals (count, sum of v h[v]) come from a pass before it.  Where the cumulative counts have an array of
+// their own (up to 16 tiles a class) a block sums the earlier tiles' bins itself instead (they
+// lie in L2), which saves the pass: 32 classes x 32769 bins took
+// 6 + 15 us in two passes of 1024 threads with eleven barriers, 14 us now.
+struct CountSum {
+    int32_t c;
+    long long v;
+};
+__device__ __forceinline__ CountSum operator+(CountSum x, CountSum y) { return {x.c + y.c, x.v + y.v}; }
+
+__device__ __forceinline__ CountSum shfl_up(CountSum x, int o) {
+    return {__shfl_up_sync(0xffffffffu, x.c, o), __shfl_up_sync(0xffffffffu, x.v, o)};
+}
+__device__ __forceinline__ CountSum warp_sum(CountSum x) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        x = x + CountSum{__shfl_xor_sync(0xffffffffu, x.c, o), __shfl_xor_sync(0xffffffffu, x.v, o)};
+    return x;
+}
+
+// A lane's bins: kScanPer, 32 apart, from the warp's first (out of range: 0).
+__device__ __forceinline__ void load_bins(const int32_t* h, int64_t first, int64_t n, CountSum (&t)[kScanPer]) {
+#pragma unroll
+    for (int j = 0; j < kScanPer; j++) {
+        const int64_t i = first + 32 * j;
+        const int32_t x = i < n ? h[i] : 0;
+        t[j] = {x, i * x};
     }
 }
 
-// Block-wide inclusive scan of one value per thread; returns the thread's inclusive prefix and
-// leaves the block total in *total (all threads).
-template <typename T>
-__device__ __forceinline__ T block_inclusive_scan(T t, T* warp_tot, T* total) {
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    T incl = t;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const T y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (l >= o) incl += y;
-    }
-    if (l == 31) warp_tot[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-        T s = warp_tot[l];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const T y = __shfl_up_sync(0xffffffffu, s, o);
-            if (l >= o) s += y;
-        }
-        warp_tot[l] = s;
-    }
-    __syncthreads();
-    const T before = (w ? warp_tot[w - 1] : (T)0) + incl;
-    *total = warp_tot[kScanThreads / 32 - 1];
-    __syncthreads();
-    return before;
-}
-
-// Block-wide sum of one value per thread; every thread gets the total.
-template <typename T>
-__device__ __forceinline__ T block_sum(T t, T* warp_tot) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) warp_tot[w] = t;
-    __syncthreads();
-    T s = l < (int)(blockDim.x >> 5) ? warp_tot[l] : (T)0;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __syncthreads();  // warp_tot is reused by the caller
-    return s;
-}
-
-// The cumulative counts (and sums) of every class in two passes over tiles of kScanTile bins,
-// one block per (tile, class) so that every SM takes part: first each tile's count total (and
-// its sum of v h[v]), then each tile's inclusive scan, offset by the totals of the class's
-// earlier tiles.  The counts are scanned in place into C[v] = #{x <= v}; the sums go to
-// csum[v] = sum_{x <= v} x when it is requested.
 __global__ void __launch_bounds__(kScanThreads) k_scan_totals(SortArgs a) {
-    __shared__ long long warp_tot[kScanThreads / 32];
-    const int k = blockIdx.y;
+    __shared__ CountSum s_warp[kScanThreads / 32];
+    const int k = blockIdx.y, lane = threadIdx.x & 31;
     const int64_t n = (int64_t)a.L[k] + 1, b0 = (int64_t)blockIdx.x * kScanTile;
     if (b0 >= n) return;  // the class has fewer tiles
-    const int32_t* h = a.hist + a.hist_off[k];
-    long long c = 0, v = 0;
+    CountSum bins[kScanPer], t = {0, 0};
+    load_bins(a.hist + a.hist_off[k], b0 + (threadIdx.x >> 5) * (32 * kScanPer) + lane, n, bins);
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const int64_t i = b0 + (int64_t)threadIdx.x * 4 + j;
-        if (i < n) {
-            const long long hi = h[i];
-            c += hi;
-            v += i * hi;
+    for (int j = 0; j < kScanPer; j++) t = t + bins[j];
+    t = warp_sum(t);
+    if (lane == 0) s_warp[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const CountSum s = warp_sum(lane < kScanThreads / 32 ? s_warp[lane] : CountSum{0, 0});
+        if (lane == 0) {
+            const int64_t o = (int64_t)k * a.scan_tiles + blockIdx.x;
+            a.tile_tot[2 * o] = s.c;
+            a.tile_tot[2 * o + 1] = s.v;
         }
-    }
-    c = block_sum<long long>(c, warp_tot);
-    if (a.csum) v = block_sum<long long>(v, warp_tot);
-    if (threadIdx.x == 0) {
-        const int64_t o = (int64_t)k * a.scan_tiles + blockIdx.x;
-        a.tile_tot[2 * o] = c;
-        a.tile_tot[2 * o + 1] = v;
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(SortArgs a) {
-    __shared__ long long warp_tot[kScanThreads / 32];
-    __shared__ int32_t warp_tot32[kScanThreads / 32];
-    const int k = blockIdx.y;
+__global__ void __launch_bounds__(kScanThreads, 2) k_scan_apply(SortArgs a) {
+    __shared__ CountSum s_warp[kScanThreads / 32], s_carry[kScanThreads / 32];
+    const int k = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = (int64_t)a.L[k] + 1, b0 = (int64_t)blockIdx.x * kScanTile;
     if (b0 >= n) return;
-    int32_t* h = a.hist + a.hist_off[k];
-    // carry-in: the totals of this class's earlier tiles
-    long long cc = 0, cv = 0;
-    for (int u = threadIdx.x; u < (int)blockIdx.x; u += blockDim.x) {
-        const int64_t o = (int64_t)k * a.scan_tiles + u;
-        cc += a.tile_tot[2 * o];
-        cv += a.tile_tot[2 * o + 1];
-    }
-    cc = block_sum<long long>(cc, warp_tot);
-    if (a.csum) cv = block_sum<long long>(cv, warp_tot);
-    const int64_t i0 = b0 + (int64_t)threadIdx.x * 4;
-    int32_t cnt[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) cnt[j] = (i0 + j < n) ? h[i0 + j] : 0;
-    if (a.csum) {
-        long long* cs = reinterpret_cast<long long*>(a.csum + a.hist_off[k]);
-        long long w[4], t = 0;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            t += (long long)(i0 + j) * cnt[j];
-            w[j] = t;
+    const int32_t* h = a.hist + a.hist_off[k];
+    // the thread's share of the class's earlier tiles
+    CountSum carry = {0, 0};
+    if (a.cum != a.hist) {
+#pragma unroll 8
+        for (int i = threadIdx.x; i < (int)b0; i += kScanThreads) {
+            const int32_t x = h[i];
+            carry = carry + CountSum{x, (long long)i * x};
         }
-        long long total;
-        const long long incl = block_inclusive_scan<long long>(t, warp_tot, &total);
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-            if (i0 + j < n) cs[i0 + j] = cv + incl - t + w[j];
+    } else {
+        for (int u = threadIdx.x; u < (int)blockIdx.x; u += kScanThreads) {
+            const int64_t o = (int64_t)k * a.scan_tiles + u;
+            carry = carry + CountSum{(int32_t)a.tile_tot[2 * o], (long long)a.tile_tot[2 * o + 1]};
+        }
     }
-    int32_t w[4], t = 0;
+    // the warp's rows of 32 bins: a scan of each, offset by the rows before
+    const int64_t i0 = b0 + warp * (32 * kScanPer) + lane;
+    CountSum own[kScanPer], incl[kScanPer];
+    load_bins(h, i0, n, own);
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        t += cnt[j];
-        w[j] = t;
+    for (int j = 0; j < kScanPer; j++) incl[j] = own[j];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int j = 0; j < kScanPer; j++) {
+            const CountSum y = shfl_up(incl[j], o);
+            if (lane >= o) incl[j] = incl[j] + y;
+        }
+    CountSum row = {0, 0};
+#pragma unroll
+    for (int j = 0; j < kScanPer; j++) {
+        const CountSum total = {__shfl_sync(0xffffffffu, incl[j].c, 31), __shfl_sync(0xffffffffu, incl[j].v, 31)};
+        incl[j] = incl[j] + row;
+        row = row + total;
     }
-    int32_t total;
-    const int32_t incl = block_inclusive_scan<int32_t>(t, warp_tot32, &total);
+    carry = warp_sum(carry);
+    if (lane == 0) {
+        s_warp[warp] = row;
+        s_carry[warp] = carry;
+    }
+    __syncthreads();
+    CountSum before = {0, 0};  // the earlier tiles, and the tile's earlier warps
+    if (lane < kScanThreads / 32) {
+        before = s_carry[lane];
+        if (lane < warp) before = before + s_warp[lane];
+    }
+    before = warp_sum(before);
     // For the expansion: tile_lo[q] = the bin holding position q * kExpandTile for each tile q of
     // the class's sorted samples, and one more entry: the bin holding the last position, N - 1.
     // Every position lies in exactly one bin's run [C[v] - h[v], C[v]), so each entry is written once.
     const int64_t Nk = a.offsets[k + 1] - a.offsets[k];
     const int64_t tiles = (Nk + kExpandTile - 1) / kExpandTile;
     int32_t* tl = a.tile_lo + a.exp_blocks[k] + k;
+    long long* cs = a.csum ? reinterpret_cast<long long*>(a.csum + a.hist_off[k]) : nullptr;
+    int32_t* cum = a.cum + a.hist_off[k];
 #pragma unroll
-    for (int j = 0; j < 4; j++)
-        if (i0 + j < n) {
-            const int64_t hi = cc + incl - t + w[j], lo = hi - cnt[j];
-            h[i0 + j] = (int32_t)hi;
-            if (lo < hi) {
-                for (int64_t q = (lo + kExpandTile - 1) / kExpandTile; q * kExpandTile < hi && q < tiles; q++)
-                    tl[q] = (int32_t)(i0 + j);
-                if (lo <= Nk - 1 && Nk - 1 < hi) tl[tiles] = (int32_t)(i0 + j);
-            }
+    for (int j = 0; j < kScanPer; j++) {
+        const int64_t i = i0 + 32 * j;
+        if (i >= n) break;
+        const CountSum at = before + incl[j];
+        const int64_t hi = at.c, lo = hi - own[j].c;
+        cum[i] = (int32_t)hi;
+        if (cs) cs[i] = at.v;
+        if (i == n - 1) a.sumx[k] = at.v;
+        if (lo < hi) {
+            for (int64_t q = (lo + kExpandTile - 1) / kExpandTile; q * kExpandTile < hi && q < tiles; q++) tl[q] = (int32_t)i;
+            if (lo <= Nk - 1 && Nk - 1 < hi) tl[tiles] = (int32_t)i;
         }
+    }
 }
 
+// Smallest v in [lo, hi] with C[v] > p (C[hi] > p).
+__device__ __forceinline__ int32_t value_at(const int32_t* C, int32_t lo, int32_t hi, int32_t p) {
+    while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (__ldg(C + mid) > p) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
+// The sorted samples and their staged form, four consecutive positions per thread, 128 per warp and step.
+// A warp first searches the values at the ends of its steps, a lane each, among the bins of the tile's
+// position range (recorded by the scan).  Where they are the same -- runs of equal samples are long where
+// samples are many -- that is all; up to 31 bins apart each lane finds its first position among the run
+// ends that the lanes hold, and otherwise by a search of its own.  No shared memory, no
+// barrier, 16-byte stores: 32 M samples in 58 us (4.4 TB/s of stores); a running maximum over run
+// starts marked in shared memory took 86, a search per thread 75.
 __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
-    // One tile of kExpandTile output positions [p0, p0 + kExpandTile).  Its positions fall in the
-    // bins [tile_lo[q], tile_lo[q + 1]] (recorded by the scan).  The run of bin v starts at position
-    // C[v - 1]; marking each non-empty bin's run start inside the tile (and the first bin at the
-    // tile's first position) and taking the running maximum gives every position its value, since
-    // values ascend with position.  Stores are lane-contiguous (coalesced).
-    __shared__ int32_t sv[kExpandTile];
-    __shared__ int32_t s_wmax[kExpandThreads / 32];
+    constexpr int kWarps = kExpandThreads / 32, kSteps = (int)kExpandTile / 128 / kWarps;  // per warp
     const int k = find_segment(a.exp_blocks, a.K, blockIdx.x);
-    const int64_t q = blockIdx.x - a.exp_blocks[k];
-    const int64_t Nk = a.offsets[k + 1] - a.offsets[k];
-    const int64_t padk = a.pair_off[k + 1] - a.pair_off[k];
-    const int32_t* C = a.hist + a.hist_off[k];
-    const int32_t Lk = a.L[k];
-    const int64_t p0 = q * kExpandTile;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int64_t pend = min(Nk, p0 + kExpandTile);  // sample positions of this tile
-    if (a.inv_n && q == 0 && tid == 0) a.inv_n[k] = 1.0 / (double)Nk;
-    if (p0 < Nk) {  // block-uniform
-        const int32_t* tl = a.tile_lo + a.exp_blocks[k] + k;
-        const int32_t v_lo = tl[q], v_hi = tl[q + 1];
-        for (int i = tid; i < kExpandTile; i += kExpandThreads) sv[i] = i == 0 ? v_lo : -1;
-        __syncthreads();
-        // a non-empty bin after v_lo starts its run after p0 (C[v - 1] >= C[v_lo] > p0)
-        for (int64_t v = (int64_t)v_lo + 1 + tid; v <= v_hi; v += kExpandThreads) {
-            const int32_t start = __ldg(C + v - 1);
-            if (__ldg(C + v) > start && start < pend) sv[start - p0] = (int32_t)v;
+    const unsigned q = blockIdx.x - a.exp_blocks[k];
+    // positions fit 32 bits: a class has at most 2^31 - 1 samples, padded to a multiple of 128
+    const unsigned N = (unsigned)(a.offsets[k + 1] - a.offsets[k]), padk = (unsigned)(a.pair_off[k + 1] - a.pair_off[k]);
+    const int32_t* C = a.cum + a.hist_off[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (a.inv_n && q == 0 && threadIdx.x == 0) a.inv_n[k] = 1.0 / (double)N;
+    const unsigned p0 = q * (unsigned)kExpandTile;
+    const int32_t* tl = a.tile_lo + a.exp_blocks[k] + k;
+    // (samples out of range leave positions that no bin holds: entries not written by this load's scan)
+    auto bin = [&](unsigned i) { return p0 < N ? min(max(tl[i], 0), a.L[k]) : 0; };
+    const int32_t v_lo = bin(q), v_hi = bin(q + 1);
+    // lanes 2i, 2i + 1: the values at the start of the warp's step i and just past its end
+    int32_t ends = v_hi;
+    {
+        const unsigned p = p0 + 128 * (warp + kWarps * (lane >> 1) + (lane & 1));
+        if (lane < 2 * kSteps && p < N) ends = value_at(C, v_lo, v_hi, (int)p);
+    }
+    int32_t* sorted = a.sorted + a.offsets[k];
+    float* staged = static_cast<float*>(a.staged) + a.pair_off[k] * (a.pair_sums ? 1 : 2);
+    const bool aligned = (a.offsets[k] & 3) == 0;
+    const float off = stage_offset(a.L[k]);  // x + 2^23 is exact for L <= 2^22
+#pragma unroll 2
+    for (int i = 0; i < kSteps; i++) {
+        const unsigned first = p0 + 128 * (warp + kWarps * i), at = first + 4 * lane;
+        if (first >= padk) break;  // warp-uniform; padk is a multiple of 128
+        const int32_t vf = __shfl_sync(0xffffffffu, ends, 2 * i), vl = __shfl_sync(0xffffffffu, ends, 2 * i + 1);
+        if (vf == vl && first + 128 <= N && aligned && a.pair_sums) {  // one run
+            *reinterpret_cast<int4*>(sorted + at) = make_int4(vf, vf, vf, vf);
+            const float s = (float)(2 * vf);
+            *reinterpret_cast<float4*>(staged + at) = make_float4(s, s, 0.f, 0.f);
+            continue;
         }
-        __syncthreads();
-        // inclusive running maximum: kExpandPerThread consecutive entries per thread, then across
-        // the lanes of the warp and across the warps
-        int32_t m[kExpandPerThread], run = -1;
+        const int left = at < N ? (int)min(N - at, 4u) : 0;  // samples among the four
+        const int pos = (int)min(at, N - 1);
+        int32_t x[4] = {vf, vf, vf, vf};
+        if (vl - vf >= 32) {
+            x[0] = value_at(C, vf, vl, pos);
+            int32_t hi = __shfl_down_sync(0xffffffffu, x[0], 1);
+            if (lane == 31) hi = vl;
 #pragma unroll
-        for (int j = 0; j < kExpandPerThread; j++) {
-            run = max(run, sv[tid * kExpandPerThread + j]);
-            m[j] = run;
-        }
-        int32_t incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl = max(incl, y);
-        }
-        if (lane == 31) s_wmax[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            int32_t x = lane < kExpandThreads / 32 ? s_wmax[lane] : -1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x = max(x, y);
+            for (int j = 1; j < 4; j++) {
+                x[j] = x[j - 1];
+                if (j < left && x[j] < hi && __ldg(C + x[j]) <= pos + j) x[j] = value_at(C, x[j] + 1, hi, pos + j);
             }
-            if (lane < kExpandThreads / 32) s_wmax[lane] = x;
-        }
-        __syncthreads();
-        const int32_t lane_before = __shfl_up_sync(0xffffffffu, incl, 1);
-        const int32_t before = max(wid > 0 ? s_wmax[wid - 1] : -1, lane > 0 ? lane_before : -1);
+        } else if (vl != vf) {  // the ends of the runs of bins vf, vf + 1, ... a lane each, searched through shuffles
+            const int32_t end = vf + lane < vl ? __ldg(C + vf + lane) : 0x7fffffff;
+            int n = 0;
 #pragma unroll
-        for (int j = 0; j < kExpandPerThread; j++) sv[tid * kExpandPerThread + j] = max(before, m[j]);
-        __syncthreads();
-        int32_t* out = a.sorted + a.offsets[k];
-        for (int64_t i = tid; i < pend - p0; i += kExpandThreads) out[p0 + i] = sv[i];
-    }
-    const int64_t qend = min(padk, p0 + kExpandTile);  // padk and p0 are multiples of 128
-    if (a.pair_sums) {  // four positions per 16-byte store; 0 past the class's samples
-        float4* out = reinterpret_cast<float4*>(static_cast<float*>(a.staged) + a.pair_off[k]);
-        for (int64_t i = 4 * (int64_t)tid; p0 + i < qend; i += 4 * kExpandThreads) {
-            const int64_t pos = p0 + i;
-            int32_t x[4];
+            for (int s = 16; s; s >>= 1)
+                if (__shfl_sync(0xffffffffu, end, n + s - 1) <= pos) n += s;
+            const int32_t e0 = __shfl_sync(0xffffffffu, end, n), e1 = __shfl_sync(0xffffffffu, end, min(n + 1, 31));
+            x[0] = vf + n;
 #pragma unroll
-            for (int j = 0; j < 4; j++) x[j] = pos + j < Nk ? sv[i + j] : 0;
-            out[pos >> 2] = make_float4((float)(x[0] + x[1]), (float)(x[2] + x[3]), (float)abs(x[1] - x[0]),
-                                        (float)abs(x[3] - x[2]));
+            for (int j = 1; j < 4; j++) x[j] = x[0] + (pos + j >= e0);
+            if (pos + 3 >= e1 && n < 31)  // a run of fewer than four samples
+#pragma unroll
+                for (int j = 1; j < 4; j++) x[j] = j < left ? value_at(C, x[j - 1], vl, pos + j) : x[j];
         }
-        return;
-    }
-    // the tile's (x', x') pairs, two positions per 16-byte store; NaN past the class's samples
-    float2* pr = static_cast<float2*>(a.staged) + a.pair_off[k];
-    const float nan = __int_as_float(0x7fc00000);  // quiet NaN pad
-    const float off = stage_offset(Lk);              // x + 2^23 is exact for L <= 2^22
-    for (int64_t i = 2 * (int64_t)tid; p0 + i < qend; i += 2 * kExpandThreads) {
-        const int64_t pos = p0 + i;
-        const float f0 = pos < Nk ? (float)sv[i] + off : nan;
-        const float f1 = pos + 1 < Nk ? (float)sv[i + 1] + off : nan;
-        *reinterpret_cast<float4*>(pr + pos) = make_float4(f0, f0, f1, f1);  // qend is even
+        if (aligned && left == 4) {
+            *reinterpret_cast<int4*>(sorted + at) = make_int4(x[0], x[1], x[2], x[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (j < left) sorted[at + j] = x[j];
+        }
+        if (a.pair_sums) {  // 0 past the class's samples
+#pragma unroll
+            for (int j = 0; j < 4; j++) x[j] = j < left ? x[j] : 0;
+            *reinterpret_cast<float4*>(staged + at) =
+                make_float4((float)(x[0] + x[1]), (float)(x[2] + x[3]), (float)abs(x[1] - x[0]), (float)abs(x[3] - x[2]));
+        } else {  // (x', x') pairs; NaN past the class's samples
+            float f[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) f[j] = j < left ? (float)x[j] + off : __int_as_float(0x7fc00000);
+            float4* out = reinterpret_cast<float4*>(staged + 2 * (size_t)at);
+            out[0] = make_float4(f[0], f[0], f[1], f[1]);
+            out[1] = make_float4(f[2], f[2], f[3], f[3]);
+        }
     }
 }
 
@@ -370,10 +362,10 @@ cudaError_t hist_block_prefix(const int64_t* N, int32_t K, int32_t* prefix) {
     cudaError_t e = sm_count(&sms);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_histogram, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kHistSmemBins * (int)sizeof(int32_t));
+                                 kHistWords * (int)sizeof(int32_t));
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_histogram, kHistThreads,
-                                                          kHistSmemBins * sizeof(int32_t));
+                                                          kHistWords * sizeof(int32_t));
     if (e != cudaSuccess) return e;
     const int64_t slots = std::max<int64_t>(1, (int64_t)sms * per_sm);
     int64_t total = 0, base = 0;
@@ -394,22 +386,25 @@ cudaError_t hist_block_prefix(const int64_t* N, int32_t K, int32_t* prefix) {
 cudaError_t launch_histogram(const SortArgs& a, int32_t nblocks, cudaStream_t s) {
     // per-device attribute; cheap enough to set on every launch
     cudaError_t e = cudaFuncSetAttribute(k_histogram, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kHistSmemBins * (int)sizeof(int32_t));
+                                         kHistWords * (int)sizeof(int32_t));
     if (e != cudaSuccess) return e;
-    k_histogram<<<nblocks, kHistThreads, kHistSmemBins * sizeof(int32_t), s>>>(a);
+    k_histogram<<<nblocks, kHistThreads, kHistWords * sizeof(int32_t), s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const SortArgs& a, cudaStream_t s) {
     const dim3 grid((unsigned)a.scan_tiles, (unsigned)a.K);
-    k_scan_totals<<<grid, kScanThreads, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (a.cum == a.hist) {
+        k_scan_totals<<<grid, kScanThreads, 0, s>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     k_scan_apply<<<grid, kScanThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 int64_t scan_tile_bins() { return kScanTile; }
+bool scan_direct(int64_t scan_tiles) { return scan_tiles <= 16; }
 
 cudaError_t launch_expand(const SortArgs& a, int32_t nblocks, cudaStream_t s) {
     k_expand<<<nblocks, kExpandThreads, 0, s>>>(a);

@@ -132,3 +132,18 @@ def test_exact_passes_over_the_samples(nl, monkeypatch):
     with pytest.raises(kvdro.KvdroError) as e:
         run(w, kvdro.KVDRO_EXACT, outputs=outputs, host_outputs=True)
     assert e.value.status == kvdro.KVDRO_ETIMEOUT
+
+
+@pytest.mark.parametrize("L", [1, 31, 4095, 4096, 32766, 32895, 32896, 65534, 65535, 70000, 1 << 20])
+@pytest.mark.parametrize("n", [1, 3, 127, 129, 4096, 4099, 70001])
+def test_sort_supports_and_sizes(L, n):
+    """Supports on and around the histogram's shared bins (2 x 16448), the scan's tiles (4096) and the tiles up
+    to which it needs no pass of totals (16), class sizes around the expansion's steps and tiles, runs longer
+    and shorter than a lane's four positions, and a class whose offset is not a multiple of four."""
+    rng = np.random.default_rng(L + n)
+    x = [rng.integers(0, L + 1, n), np.minimum(rng.geometric(0.3, n + 1), L), np.full(n, L)]
+    w = make(x, L, [0, L], [1.0], [0.0], 1.0, 1.0)
+    got = run(w, kvdro.KVDRO_ENVELOPE, outputs=("sorted", "fhat", "S"))
+    assert np.array_equal(got["sorted"], np.concatenate([np.sort(v) for v in x]))
+    want = np.stack([[v.mean(), (L - v).mean()] for v in x])[None, :, :, None]  # at r = 0 and L, lam = 1 = c_p = c_w
+    np.testing.assert_allclose(got["S"], want, rtol=1e-12)
