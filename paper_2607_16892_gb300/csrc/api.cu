@@ -70,6 +70,7 @@ struct kvdro_ctx {
         tile_lo;
     void* pin = nullptr;  // pinned host staging
     size_t pin_bytes = 0;
+    void* land = nullptr;  // pinned: small results and the status words land here on their way to the caller
     cudaEvent_t pin_free = nullptr;  // completes when the last copy out of `pin` is done
     cudaEvent_t grid_t0 = nullptr, grid_t1 = nullptr;  // around the last grid-kernel launches
     // Copies of host outputs back to the caller, overlapped with later grid launches
@@ -180,6 +181,30 @@ int pinned(kvdro_ctx* ctx, size_t bytes, void** out) {
     return KVDRO_OK;
 }
 
+// Parameters of a call on their way to the device: written to `host`, then sent with the call's fills, in the
+// setup launch's arguments where they fit, else by a copy from pinned staging ahead of it.
+struct Params {
+    kvdro_ctx* ctx;
+    alignas(16) char small[16384];
+    char* host = small;
+    int rc = KVDRO_OK;
+    Params(kvdro_ctx* c, size_t bytes) : ctx(c) {
+        if (kvdro::setup_fits(bytes)) return;
+        void* p = nullptr;
+        rc = pinned(c, bytes, &p);
+        host = static_cast<char*>(p);
+    }
+    int send(void* dst, size_t bytes, const kvdro::Fill& f0, const kvdro::Fill& f1, cudaStream_t s) {
+        if (host != small) {
+            KV_CUDA(cudaMemcpyAsync(dst, host, bytes, cudaMemcpyHostToDevice, s), "uploading parameters");
+            KV_CUDA(cudaEventRecord(ctx->pin_free, s), "recording staging event");
+            if (f0.words + f1.words == 0) return KVDRO_OK;
+        }
+        KV_CUDA(kvdro::launch_setup(small, host == small ? bytes : 0, dst, f0, f1, s), "setup kernel");
+        return KVDRO_OK;
+    }
+};
+
 // Device-accessible (device or managed memory) versus host memory (pinned or pageable).
 bool is_device_ptr(const void* p) {
     cudaPointerAttributes at;
@@ -193,17 +218,46 @@ bool is_device_ptr(const void* p) {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Reads and clears the kernels' error word; KVDRO_ETIMEOUT if a bounded wait gave up.
-int check_kernel_errors(kvdro_ctx* ctx, cudaStream_t s) {
-    if (!ctx->errs.p) return KVDRO_OK;
-    int32_t h[2] = {0, 0};
-    KV_CUDA(cudaMemcpyAsync(h, ctx->errs.p, sizeof(h), cudaMemcpyDeviceToHost, s), "reading kernel status");
-    KV_CUDA(cudaStreamSynchronize(s), "reading kernel status");
+// Device results read back to the host: up to kLandBytes at a time in one copy, with the kernels' status words
+// behind them, and one wait.  (A copy into pageable memory for each output, a wait and another copy and wait
+// for the status took 30 us of a small call.)
+constexpr size_t kLandBytes = 64 << 10;
+
+int land(kvdro_ctx* ctx, const void* dev, size_t bytes, cudaStream_t s) {  // status words at ctx->land + kLandBytes
+    if (!ctx->land) {
+        ctx->allocs++;
+        if (ctx->fail_after > 0 && ctx->allocs == ctx->fail_after)
+            return fail(ctx, KVDRO_ENOMEM, "pinned allocation failed (injected by KVDRO_TEST_FAIL_ALLOC)");
+        const cudaError_t e = cudaHostAlloc(&ctx->land, kLandBytes + 16, cudaHostAllocDefault);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            ctx->land = nullptr;
+            return fail(ctx, KVDRO_ENOMEM, "cudaHostAlloc(%zu): %s", kLandBytes + 16, cudaGetErrorString(e));
+        }
+    }
+    if (bytes) KV_CUDA(cudaMemcpyAsync(ctx->land, dev, bytes, cudaMemcpyDeviceToHost, s), "copying results");
+    KV_CUDA(cudaMemcpyAsync(static_cast<char*>(ctx->land) + kLandBytes, ctx->errs.p, 8, cudaMemcpyDeviceToHost, s),
+            "reading kernel status");
+    KV_CUDA(cudaStreamSynchronize(s), "copying results");
+    return KVDRO_OK;
+}
+
+// The kernels' status words that the last land() brought, cleared on the device; KVDRO_ETIMEOUT if a bounded
+// wait gave up.
+int landed_status(kvdro_ctx* ctx, cudaStream_t s) {
+    int32_t h[2];
+    std::memcpy(h, static_cast<char*>(ctx->land) + kLandBytes, sizeof(h));
     if (h[1] & kvdro::kErrTimeout) {
         KV_CUDA(cudaMemsetAsync(static_cast<int32_t*>(ctx->errs.p) + 1, 0, sizeof(int32_t), s), "clearing status");
         return fail(ctx, KVDRO_ETIMEOUT, "a grid kernel gave up waiting for a staged sample chunk");
     }
     return KVDRO_OK;
+}
+
+int check_kernel_errors(kvdro_ctx* ctx, cudaStream_t s) {
+    if (!ctx->errs.p) return KVDRO_OK;
+    if (int rc = land(ctx, nullptr, 0, s)) return rc;
+    return landed_status(ctx, s);
 }
 
 // Every r must lie in [L_in, L_in + L_max] of every class (the reservation domain of Sec. 2.2),
@@ -281,6 +335,7 @@ int kvdro_destroy(kvdro_ctx* ctx) {
                    &ctx->grid_in, &ctx->keys, &ctx->cost64, &ctx->out_stage, &ctx->ranks, &ctx->tile_lo})
         release(*b);
     if (ctx->pin) cudaFreeHost(ctx->pin);
+    if (ctx->land) cudaFreeHost(ctx->land);
     if (ctx->pin_free) cudaEventDestroy(ctx->pin_free);
     if (ctx->grid_t0) cudaEventDestroy(ctx->grid_t0);
     if (ctx->grid_t1) cudaEventDestroy(ctx->grid_t1);
@@ -368,10 +423,10 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     const size_t meta_bytes = (size_t)(K + 1) * 8 * 3 + (size_t)K * 8 * 2 + (size_t)K * 4 * 2 + (size_t)(K + 1) * 4 * 2 + 64;
     if ((rc = ensure(ctx, ctx->meta, meta_bytes))) return rc;
 
-    // Metadata upload (one copy from pinned staging).
-    void* hp;
-    if ((rc = pinned(ctx, meta_bytes, &hp))) return rc;
-    char* h = static_cast<char*>(hp);
+    // Metadata, and what the sort starts from zero, in one launch.
+    Params pm(ctx, meta_bytes);
+    if (pm.rc) return pm.rc;
+    char* h = pm.host;
     char* d = static_cast<char*>(ctx->meta.p);
     size_t o = 0;
     auto put = [&](const void* src, size_t bytes, void** dview) {
@@ -388,8 +443,9 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     put(ctx->Lin.data(), K * 4, reinterpret_cast<void**>(&ctx->d_Lin));
     put(ctx->hist_blocks.data(), (K + 1) * 4, reinterpret_cast<void**>(&ctx->d_hist_blocks));
     put(ctx->exp_blocks.data(), (K + 1) * 4, reinterpret_cast<void**>(&ctx->d_exp_blocks));
-    KV_CUDA(cudaMemcpyAsync(ctx->meta.p, hp, o, cudaMemcpyHostToDevice, s), "uploading class metadata");
-    KV_CUDA(cudaEventRecord(ctx->pin_free, s), "recording staging event");
+    if ((rc = pm.send(ctx->meta.p, o, {static_cast<uint32_t*>(ctx->hist.p), ctx->hist_total, 0u},
+                      {static_cast<uint32_t*>(ctx->errs.p), 2, 0u}, s)))
+        return rc;
 
     const int32_t* dlen = lengths;
     if (!is_device_ptr(lengths)) {
@@ -398,8 +454,6 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
                 "uploading samples");
         dlen = static_cast<const int32_t*>(ctx->in_stage.p);
     }
-    KV_CUDA(cudaMemsetAsync(ctx->hist.p, 0, (size_t)ctx->hist_total * 4, s), "clearing histogram");
-    KV_CUDA(cudaMemsetAsync(ctx->errs.p, 0, 2 * sizeof(int32_t), s), "clearing status");
 
     kvdro::SortArgs a;
     a.lengths = dlen;
@@ -426,9 +480,9 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     KV_CUDA(kvdro::launch_scan(a, s), "scan kernel");
     KV_CUDA(kvdro::launch_expand(a, ctx->exp_blocks[K], s), "expand kernel");
 
+    if ((rc = land(ctx, nullptr, 0, s))) return rc;
     int32_t bad = 0;
-    KV_CUDA(cudaMemcpyAsync(&bad, ctx->errs.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "reading range check");
-    KV_CUDA(cudaStreamSynchronize(s), "loading samples");
+    std::memcpy(&bad, static_cast<char*>(ctx->land) + kLandBytes, sizeof(bad));
     if (bad != 0)
         return fail(ctx, KVDRO_EINVAL, "%d samples lie outside [0, L_max] of their class; no samples are loaded", bad);
     ctx->loaded = true;
@@ -451,10 +505,10 @@ int kvdro_quantiles(kvdro_ctx* ctx, int32_t F, const double* fractiles, int32_t*
     ctx->last_stream = s;
     const int64_t n = (int64_t)ctx->K * F;
     int rc;
-    if ((rc = ensure(ctx, ctx->ranks, (size_t)n * 4))) return rc;
-    void* hp;
-    if ((rc = pinned(ctx, (size_t)n * 4, &hp))) return rc;
-    int32_t* hr = static_cast<int32_t*>(hp);
+    if ((rc = ensure(ctx, ctx->ranks, align_up((size_t)n * 4, 8)))) return rc;  // written in words of 8 bytes
+    Params pm(ctx, (size_t)n * 4);
+    if (pm.rc) return pm.rc;
+    int32_t* hr = reinterpret_cast<int32_t*>(pm.host);
     for (int32_t k = 0; k < ctx->K; k++)
         for (int32_t f = 0; f < F; f++) {
             // lower empirical quantile: rank max(1, ceil(q N)) in FP64
@@ -464,8 +518,7 @@ int kvdro_quantiles(kvdro_ctx* ctx, int32_t F, const double* fractiles, int32_t*
             if (rk > ctx->N[k]) rk = ctx->N[k];
             hr[(int64_t)k * F + f] = (int32_t)rk;
         }
-    KV_CUDA(cudaMemcpyAsync(ctx->ranks.p, hp, (size_t)n * 4, cudaMemcpyHostToDevice, s), "uploading ranks");
-    KV_CUDA(cudaEventRecord(ctx->pin_free, s), "recording staging event");
+    if ((rc = pm.send(ctx->ranks.p, (size_t)n * 4, {}, {}, s))) return rc;
     const bool dev_out = is_device_ptr(out);
     int32_t* dout = out;
     if (!dev_out) {
@@ -475,7 +528,10 @@ int kvdro_quantiles(kvdro_ctx* ctx, int32_t F, const double* fractiles, int32_t*
     KV_CUDA(kvdro::launch_gather_quantiles(static_cast<const int32_t*>(ctx->sorted.p), ctx->d_off,
                                            static_cast<const int32_t*>(ctx->ranks.p), ctx->K, F, dout, s),
             "quantile kernel");
-    if (!dev_out) {
+    if (!dev_out && (size_t)n * 4 <= kLandBytes) {
+        if ((rc = land(ctx, dout, (size_t)n * 4, s))) return rc;
+        std::memcpy(out, ctx->land, (size_t)n * 4);
+    } else if (!dev_out) {
         KV_CUDA(cudaMemcpyAsync(out, dout, (size_t)n * 4, cudaMemcpyDeviceToHost, s), "copying quantiles");
         KV_CUDA(cudaStreamSynchronize(s), "copying quantiles");
     }
@@ -535,9 +591,9 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     const size_t gbytes = align_up((size_t)R * 4, 8) + 8 * ((size_t)NL + E + 2 * (size_t)M);
     int rc;
     if ((rc = ensure(ctx, ctx->grid_in, gbytes))) return rc;
-    void* hp;
-    if ((rc = pinned(ctx, gbytes, &hp))) return rc;
-    char* h = static_cast<char*>(hp);
+    Params pm(ctx, gbytes);
+    if (pm.rc) return pm.rc;
+    char* h = pm.host;
     char* d = static_cast<char*>(ctx->grid_in.p);
     size_t o = 0;
     auto put = [&](const void* src, size_t bytes) {
@@ -551,8 +607,6 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     const double* d_eps = static_cast<const double*>(put(eps, (size_t)E * 8));
     const double* d_cp = static_cast<const double*>(put(c_p, (size_t)M * 8));
     const double* d_cw = static_cast<const double*>(put(c_w, (size_t)M * 8));
-    KV_CUDA(cudaMemcpyAsync(ctx->grid_in.p, hp, o, cudaMemcpyHostToDevice, s), "uploading the grid");
-    KV_CUDA(cudaEventRecord(ctx->pin_free, s), "recording staging event");
 
     // Outputs: device pointers are written in place, host outputs go through device staging.
     const size_t es = P == Prec::F32 ? 4 : 8;
@@ -589,8 +643,10 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
         if ((rc = ensure(ctx, ctx->cost64, (size_t)cells_out * 8))) return rc;
         cost_dev = ctx->cost64.p;
     }
-    if ((rc = ensure(ctx, ctx->keys, (size_t)rows * 8))) return rc;
-    KV_CUDA(cudaMemsetAsync(ctx->keys.p, 0xFF, (size_t)rows * 8, s), "clearing argmin keys");
+    // argmin keys, then the finished CTAs of each (regime, class): all ones
+    const int64_t done_words = (int64_t)M * ctx->K;
+    if ((rc = ensure(ctx, ctx->keys, (size_t)rows * 8 + (size_t)done_words * 4))) return rc;
+    if ((rc = pm.send(ctx->grid_in.p, o, {static_cast<uint32_t*>(ctx->keys.p), 2 * rows + done_words, ~0u}, {}, s))) return rc;
 
     kvdro::GridArgs a;
     a.staged = ctx->pairs.p;
@@ -624,6 +680,23 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     // chunk.  It travels with this context's launches only.
     a.test_skip_chunk = ctx->skip_chunk;
     a.wait_ns = ctx->skip_chunk >= 0 ? kTestWaitNs : 0;
+    kvdro::FinalizeArgs& fa = a.fin;
+    fa.keys = static_cast<const unsigned long long*>(ctx->keys.p);
+    fa.cost = cost_dev;
+    fa.r = d_r;
+    fa.L_in = ctx->d_Lin;
+    fa.N = ctx->d_N;
+    fa.cdf = ctx->d_cum;
+    fa.hist_off = ctx->d_hist_off;
+    fa.K = ctx->K;
+    fa.R = R;
+    fa.E = E;
+    fa.M = M;
+    fa.r_idx = static_cast<int32_t*>(outs[3].dev);
+    fa.min_cost = outs[4].dev;
+    fa.fhat = static_cast<double*>(outs[5].dev);
+    // the last CTA of each (regime, class) finalises its rows
+    a.done = fa.r_idx || fa.min_cost || fa.fhat ? reinterpret_cast<uint32_t*>(a.keys + rows) : nullptr;
     int64_t m_step = std::max<int64_t>(1, 0x7fffffffLL / ((int64_t)ctx->K * shape.r_blocks));
     // Host outputs laid out regime-major (S, cost, lam index) go back in blocks of regimes on the
     // context's copy stream, each block as soon as its launches are done, so the copies overlap the
@@ -662,23 +735,14 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     KV_CUDA(cudaEventRecord(ctx->grid_t1, s), "recording grid end");
     ctx->grid_timed = true;
 
-    kvdro::FinalizeArgs fa;
-    fa.keys = static_cast<const unsigned long long*>(ctx->keys.p);
-    fa.cost = cost_dev;
-    fa.r = d_r;
-    fa.L_in = ctx->d_Lin;
-    fa.N = ctx->d_N;
-    fa.cdf = ctx->d_cum;
-    fa.hist_off = ctx->d_hist_off;
-    fa.K = ctx->K;
-    fa.R = R;
-    fa.E = E;
-    fa.M = M;
-    fa.r_idx = static_cast<int32_t*>(outs[3].dev);
-    fa.min_cost = outs[4].dev;
-    fa.fhat = static_cast<double*>(outs[5].dev);
-    if (fa.r_idx || fa.min_cost || fa.fhat) KV_CUDA(kvdro::launch_finalize(P, fa, s), "finalize kernel");
-
+    if (stage_bytes && !pipe && stage_bytes <= kLandBytes) {
+        if ((rc = land(ctx, ctx->out_stage.p, stage_bytes, s))) return rc;
+        for (const Out& x : outs)
+            if (x.user && x.host)
+                std::memcpy(x.user, static_cast<char*>(ctx->land) + (static_cast<char*>(x.dev) - static_cast<char*>(ctx->out_stage.p)),
+                            x.bytes);
+        return landed_status(ctx, s);
+    }
     if (stage_bytes) {
         if (pipe) {  // the regime blocks' copies, then the rest on the caller's stream
             KV_CUDA(cudaEventRecord(ctx->copy_done, ctx->copy_stream), "recording the copies");
@@ -720,9 +784,9 @@ int kvdro_eval_dual(kvdro_ctx* ctx, int32_t R, const int32_t* r, int32_t E, cons
     const size_t gbytes = align_up((size_t)R * 4, 8) + 8 * ((size_t)E + 2 * (size_t)M);
     int rc;
     if ((rc = ensure(ctx, ctx->grid_in, gbytes))) return rc;
-    void* hp;
-    if ((rc = pinned(ctx, gbytes, &hp))) return rc;
-    char* h = static_cast<char*>(hp);
+    Params pm(ctx, gbytes);
+    if (pm.rc) return pm.rc;
+    char* h = pm.host;
     char* d = static_cast<char*>(ctx->grid_in.p);
     size_t o = 0;
     auto put = [&](const void* src, size_t bytes) {
@@ -735,8 +799,6 @@ int kvdro_eval_dual(kvdro_ctx* ctx, int32_t R, const int32_t* r, int32_t E, cons
     const double* d_eps = static_cast<const double*>(put(eps, (size_t)E * 8));
     const double* d_cp = static_cast<const double*>(put(c_p, (size_t)M * 8));
     const double* d_cw = static_cast<const double*>(put(c_w, (size_t)M * 8));
-    KV_CUDA(cudaMemcpyAsync(ctx->grid_in.p, hp, o, cudaMemcpyHostToDevice, s), "uploading the grid");
-    KV_CUDA(cudaEventRecord(ctx->pin_free, s), "recording staging event");
 
     struct Out {
         void* user;
@@ -771,7 +833,7 @@ int kvdro_eval_dual(kvdro_ctx* ctx, int32_t R, const int32_t* r, int32_t E, cons
         cost_dev = ctx->cost64.p;
     }
     if ((rc = ensure(ctx, ctx->keys, (size_t)rows * 8))) return rc;
-    KV_CUDA(cudaMemsetAsync(ctx->keys.p, 0xFF, (size_t)rows * 8, s), "clearing argmin keys");
+    if ((rc = pm.send(ctx->grid_in.p, o, {static_cast<uint32_t*>(ctx->keys.p), 2 * rows, ~0u}, {}, s))) return rc;
 
     kvdro::DualArgs a;
     a.cdf = ctx->d_cum;

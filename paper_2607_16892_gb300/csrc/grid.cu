@@ -341,6 +341,44 @@ __device__ __forceinline__ u64 write_pair(const GridArgs& a, double best, int bj
     }
 }
 
+// Row i = (m, e, k) of the per-(regime, radius, class) outputs from its argmin key and, FP64, the cost there
+// (past L1: other CTAs wrote them).
+template <bool F32>
+__device__ __forceinline__ void finalize_row(const FinalizeArgs& a, int64_t i, int k) {
+    const u64 key = __ldcg(a.keys + i);
+    if (key == ~0ull) {  // no r evaluated (cannot happen for R >= 1); report an invalid index
+        if (a.r_idx) a.r_idx[i] = -1;
+        return;
+    }
+    const int ri = (int)(F32 ? (key & 0xffffffffull) : (key & 0xFFFFFull));
+    if (a.r_idx) a.r_idx[i] = ri;
+    if (a.min_cost) {
+        if constexpr (F32) static_cast<float*>(a.min_cost)[i] = __uint_as_float((uint32_t)(key >> 32));
+        else static_cast<double*>(a.min_cost)[i] = __ldcg(static_cast<const double*>(a.cost) + i * a.R + ri);
+    }
+    if (a.fhat) {
+        const int32_t v = a.r[ri] - a.L_in[k];
+        a.fhat[i] = (double)a.cdf[a.hist_off[k] + v] / (double)a.N[k];
+    }
+}
+
+// The last of the (regime, class)'s CTAs to get here finalises its rows: a launch of its own took 4 us of
+// the smallest grids' 34.  Every CTA's outputs and keys are ordered before its count (barrier, fence,
+// atomic), the last one's reads after.  Kept out of line: its registers are no concern of the sample loops.
+template <bool F32>
+__device__ __noinline__ void finish_rows(const GridArgs& a, int m, int k) {
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(a.done + (size_t)m * a.K + k, 1u) == (uint32_t)a.r_blocks - 2u;  // counts from all ones
+        __threadfence();
+    }
+    __syncthreads();
+    if (s_last)
+        for (int e = threadIdx.x; e < a.E; e += blockDim.x) finalize_row<F32>(a.fin, ((int64_t)m * a.E + e) * a.K + k, k);
+}
+
 // The CTA's rows of S in shared memory, as doubles and cut to floats (INFINITY past NL up to a multiple of
 // four), with the lam values likewise (0 past NL).
 struct LamRows {
@@ -418,6 +456,7 @@ __device__ __forceinline__ void lam_min_epilogue(const GridArgs& a, const LamRow
             if (lane == 0 && low != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + ei) * a.K + k, low);
         }
     }
+    if (a.done) finish_rows<F32OUT>(a, m, k);
 }
 
 // ---------------------------------------------------------------- the FP32- and FP64-arithmetic kernels
@@ -1168,28 +1207,10 @@ __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
     lam_min_epilogue<false>(a, rows_of, r_cta0, m, k);
 }
 
-template <Prec P>
+template <bool F32>
 __global__ void k_finalize(const FinalizeArgs a) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)a.M * a.E * a.K) return;
-    const int k = (int)(i % a.K);
-    const u64 key = a.keys[i];
-    if (key == ~0ull) {  // no r evaluated (cannot happen for R >= 1); report an invalid index
-        if (a.r_idx) a.r_idx[i] = -1;
-        return;
-    }
-    const int ri = (int)(P == Prec::F32 ? (key & 0xffffffffull) : (key & 0xFFFFFull));
-    if (a.r_idx) a.r_idx[i] = ri;
-    if (a.min_cost) {
-        if constexpr (P == Prec::F32)
-            static_cast<float*>(a.min_cost)[i] = __uint_as_float((uint32_t)(key >> 32));
-        else
-            static_cast<double*>(a.min_cost)[i] = static_cast<const double*>(a.cost)[i * a.R + ri];
-    }
-    if (a.fhat) {
-        const int32_t v = a.r[ri] - a.L_in[k];
-        a.fhat[i] = (double)a.cdf[a.hist_off[k] + v] / (double)a.N[k];
-    }
+    if (i < (int64_t)a.M * a.E * a.K) finalize_row<F32>(a, i, (int)(i % a.K));
 }
 
 }  // namespace
@@ -1322,8 +1343,8 @@ cudaError_t launch_finalize(Prec p, const FinalizeArgs& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.M * a.E * a.K;
     const int threads = 256;
     const unsigned blocks = (unsigned)((n + threads - 1) / threads);
-    if (p == Prec::F32) k_finalize<Prec::F32><<<blocks, threads, 0, s>>>(a);
-    else k_finalize<Prec::F64><<<blocks, threads, 0, s>>>(a);
+    if (p == Prec::F32) k_finalize<true><<<blocks, threads, 0, s>>>(a);
+    else k_finalize<false><<<blocks, threads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -74,6 +74,20 @@ constexpr float kStageOffset = 8388608.0f;  // 2^23
 constexpr int32_t kStageBits = 0x4B000000;  // bit pattern of 2^23
 __host__ __device__ inline float stage_offset(int32_t L) { return L <= kExactMaxL ? kStageOffset : 0.0f; }
 
+struct FinalizeArgs {
+    const unsigned long long* keys;  // [M][E][K] argmin keys
+    const void* cost;           // FP64: cost buffer to read min_cost from; FP32 unused
+    const int32_t* r;
+    const int32_t* L_in;
+    const int64_t* N;
+    const int32_t* cdf;
+    const int64_t* hist_off;
+    int32_t K, R, E, M;
+    int32_t* r_idx;             // [M][E][K]
+    void* min_cost;             // [M][E][K]
+    double* fhat;               // [M][E][K]
+};
+
 struct GridArgs {
     const void* staged;         // the padded samples
     const int64_t* pair_off;    // [K+1] in samples
@@ -111,20 +125,10 @@ struct GridArgs {
     // the waits on it run out (-1 in production).
     long long wait_ns;
     int32_t test_skip_chunk;
-};
-
-struct FinalizeArgs {
-    const unsigned long long* keys;
-    const void* cost;           // FP64: cost buffer to read min_cost from; FP32 unused
-    const int32_t* r;
-    const int32_t* L_in;
-    const int64_t* N;
-    const int32_t* cdf;
-    const int64_t* hist_off;
-    int32_t K, R, E, M;
-    int32_t* r_idx;             // [M][E][K]
-    void* min_cost;             // [M][E][K]
-    double* fhat;               // [M][E][K]
+    // With `done` ([M][K] words, all ones before the launch) the last CTA of each (regime, class) finalises
+    // its rows by `fin`; without, the caller launches the finalisation.
+    uint32_t* done;
+    FinalizeArgs fin;
 };
 
 // grid.cu
@@ -147,6 +151,16 @@ cudaError_t grid_prepare(Prec p);             // per-device attribute setup of e
 // Launches over regimes [a.m0, a.m0 + a.m_count); fills a.LT, a.RG, a.r_blocks from `sh`.
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s);
 cudaError_t launch_finalize(Prec p, const FinalizeArgs& a, cudaStream_t s);
+
+// setup.cu: one launch that writes `bytes` of host parameters to dst (setup_fits) and fills two arrays of
+// 32-bit words (16-byte aligned; 0 words to skip)
+struct Fill {
+    uint32_t* p;
+    int64_t words;
+    uint32_t value;
+};
+bool setup_fits(size_t bytes);
+cudaError_t launch_setup(const void* payload, size_t bytes, void* dst, const Fill& f0, const Fill& f1, cudaStream_t s);
 
 // dual.cu: exact minimisation over gamma >= 0 per (regime, radius, class, reservation)
 struct DualArgs {
