@@ -695,8 +695,12 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     fa.r_idx = static_cast<int32_t*>(outs[3].dev);
     fa.min_cost = outs[4].dev;
     fa.fhat = static_cast<double*>(outs[5].dev);
-    // the last CTA of each (regime, class) finalises its rows
-    a.done = fa.r_idx || fa.min_cost || fa.fhat ? reinterpret_cast<uint32_t*>(a.keys + rows) : nullptr;
+    // In small grids the last CTA of each (regime, class) finalises its rows: the launch saved is 4 us of the
+    // smallest call's 34; in large ones its barriers and counts cost more (131,072 CTAs of the envelope 3.73
+    // -> 3.88 ms), so they take the launch.
+    const bool finalize = fa.r_idx || fa.min_cost || fa.fhat;
+    const bool fused = (int64_t)M * ctx->K * shape.r_blocks <= 2048;
+    a.done = finalize && fused ? reinterpret_cast<uint32_t*>(a.keys + rows) : nullptr;
     int64_t m_step = std::max<int64_t>(1, 0x7fffffffLL / ((int64_t)ctx->K * shape.r_blocks));
     // Host outputs laid out regime-major (S, cost, lam index) go back in blocks of regimes on the
     // context's copy stream, each block as soon as its launches are done, so the copies overlap the
@@ -734,6 +738,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     }
     KV_CUDA(cudaEventRecord(ctx->grid_t1, s), "recording grid end");
     ctx->grid_timed = true;
+    if (finalize && !fused) KV_CUDA(kvdro::launch_finalize(P, fa, s), "finalize kernel");
 
     if (stage_bytes && !pipe && stage_bytes <= kLandBytes) {
         if ((rc = land(ctx, ctx->out_stage.p, stage_bytes, s))) return rc;

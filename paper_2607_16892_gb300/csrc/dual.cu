@@ -25,7 +25,7 @@
 namespace kvdro {
 namespace {
 
-constexpr int kDualThreads = 256;
+constexpr int kDualThreads = 128;
 
 // One (regime, class, reservation): the class's cumulative arrays and what the costs fix.
 struct Cell {
@@ -91,7 +91,7 @@ __device__ __forceinline__ double crossing(const Cell& c, int v, bool nu1, bool 
     return fma(fma(-d, q, num), r, q);
 }
 
-__global__ void __launch_bounds__(kDualThreads, 3) k_dual(const DualArgs a) {
+__global__ void __launch_bounds__(kDualThreads, 6) k_dual(const DualArgs a) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t total = (int64_t)a.M * a.E * a.K * a.R;
     const bool valid = i < total;

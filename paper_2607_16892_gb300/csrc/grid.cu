@@ -40,6 +40,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "kvdro_internal.cuh"
 
@@ -902,7 +903,10 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
             for (int j = 0; j < V; j++) acci[j] = __sad(bb, cci[j], __sad(ba, cci[j], acci[j]));
         }
     };
-    constexpr int kSeg = 8;  // loads per segment of a fixed trip count
+    // Loads per segment of a fixed trip count: long ones run 1.4 % faster (8 classes x 100,000 samples x 4096 r x
+    // 128 lam 16.15 -> 15.92 ms), short ones take the rest of a chunk, and all of it where long ones would
+    // fold much more often than the bound asks (the heavy tail's support of 131072: 39.5 ms against 44).
+    constexpr int kLongSeg = 32, kShortSeg = 8;
     int pending = 0;         // loads since the last fold
     auto room = [&](int loads) {  // fold first if the loads since the last fold would pass fe
         if (pending + loads > fe) {
@@ -910,6 +914,15 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
             pending = 0;
         }
         pending += loads;
+    };
+    auto segments = [&](const float4* q, int& t0, int t_end, auto seg) {
+        constexpr int kSeg = decltype(seg)::value;
+#pragma unroll 1
+        for (; t0 + kSeg <= t_end; t0 += kSeg) {
+            room(kSeg);
+#pragma unroll
+            for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
+        }
     };
     bool timeout = false;
     int at = 0, c = 0, s = 0;  // chunk over all passes, of the class, its stage
@@ -941,14 +954,8 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
             const int64_t left = a.N[k] - (int64_t)c * chunk;
             const int t_clean = PAIR ? nq : (left <= 0 ? 0 : (int)min((int64_t)nq, left / (32 * X::kPer)));
             int t0 = 0;
-            if (fe >= kSeg) {
-#pragma unroll 1
-                for (; t0 + kSeg <= t_clean; t0 += kSeg) {
-                    room(kSeg);
-#pragma unroll
-                    for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
-                }
-            }
+            if (fe >= 2 * kLongSeg) segments(q, t0, t_clean, std::integral_constant<int, kLongSeg>());
+            if (fe >= kShortSeg) segments(q, t0, t_clean, std::integral_constant<int, kShortSeg>());
 #pragma unroll 1
             for (; t0 < nq; t0++) {
                 room(1);
@@ -1048,17 +1055,25 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
 // lam alone is formed once per CTA, and the minimum over lam leaves about one value per
 // (r, eps) pair to FP64.
 //
-// A warp takes 2 passes of 32 / W rows, W lanes along lam each (W: NL rounded up to a power of two, at
-// most 32), so small lam grids fill the warp with rows.
+// A warp takes up to kEnvPasses passes of 32 / W rows, W lanes along lam each (W: NL rounded up to a power of
+// two, at most 32), so small lam grids fill the warp with rows.  More passes share the CTA's start and end
+// (128 regimes x 8 classes x 2048 r x 64 lam x 16 eps: 4 passes 3.33 ms, 3 3.58, 2 3.70); fewer where the
+// grid has too few rows to fill the SMs several times over, or rows so wide that two CTAs fill an SM's
+// shared memory (more than 64 lam).
 constexpr int kEnvThreads = 256;
-constexpr int kEnvPasses = 2;
+constexpr int kEnvPasses = 4;
 
 __host__ __device__ inline int env_width(int NL) {
     int w = 1;
     while (w < NL && w < 32) w <<= 1;
     return w;
 }
-__host__ __device__ inline int env_rows(int NL) { return kEnvPasses * kEnvThreads / env_width(NL); }
+inline int env_rows(int NL, int64_t R, int64_t classes, int sms) {
+    const int rows = kEnvThreads / env_width(NL);
+    int passes = NL <= 64 ? kEnvPasses : 2;
+    while (passes > 1 && classes * ((R + passes * rows - 1) / (passes * rows)) < 8 * (int64_t)sms) passes /= 2;
+    return passes * rows;
+}
 
 struct EnvRow {
     RowOffset off;
@@ -1070,9 +1085,9 @@ struct EnvSmem {
     size_t kap, eps, S, row, muf, kapf, lamf, Sf, total;
     int stride, stride_f;  // elements per row of S and Sf
 };
-__host__ __device__ inline EnvSmem env_smem(int NL, int E) {
+__host__ __device__ inline EnvSmem env_smem(int rows, int NL, int E) {
     EnvSmem s;
-    const int rows = env_rows(NL), n4 = four(NL);
+    const int n4 = four(NL);
     s.stride = NL | 1;  // odd: rows start in other banks
     s.stride_f = float_stride(NL);
     s.kap = 8 * (size_t)NL;
@@ -1091,7 +1106,7 @@ __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
     extern __shared__ __align__(16) unsigned char esm[];
     __shared__ int s_bad[2];  // some magnitude the floats do not hold: in the inputs, in S
     __shared__ int s_first_sat, s_unsorted;
-    const EnvSmem lay = env_smem(a.NL, a.E);
+    const EnvSmem lay = env_smem(a.rows, a.NL, a.E);
     double* s_lam = reinterpret_cast<double*>(esm);
     double* s_kap = reinterpret_cast<double*>(esm + lay.kap);
     double* s_eps = reinterpret_cast<double*>(esm + lay.eps);
@@ -1107,8 +1122,8 @@ __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
     b /= a.r_blocks;
     const int k = b % a.K;
     const int m = a.m0 + b / a.K;
-    const int NL = a.NL, W = env_width(NL), max_rows = env_rows(NL);
-    const int r_cta0 = rb * max_rows, rows = min(max_rows, a.R - r_cta0);
+    const int NL = a.NL, W = env_width(NL);
+    const int r_cta0 = rb * a.rows, rows = min(a.rows, a.R - r_cta0);
     const double cp = a.cp[m], cw = a.cw[m];
     const int L = a.L[k];
     const long long N = a.N[k], sumx = a.sumx[k];
@@ -1279,9 +1294,9 @@ GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, in
         sh.variant = 4;
         sh.LT = sh.RG = sh.stages = 1;
         sh.threads = kEnvThreads;
-        sh.rows = env_rows(NL);
+        sh.rows = env_rows(NL, R, classes, sms);
         sh.r_blocks = (R + sh.rows - 1) / sh.rows;
-        sh.smem = env_smem(NL, E).total;
+        sh.smem = env_smem(sh.rows, NL, E).total;
         return sh;
     }
     if (p == Prec::F64) return shape_for<CfgF64>(2, R, NL, E);
@@ -1315,7 +1330,11 @@ cudaError_t grid_prepare(Prec p) {
         const cudaError_t e = allow_smem((const void*)k_exact<true>, kExactSmem);
         return e == cudaSuccess ? allow_smem((const void*)k_exact<false>, kExactSmem) : e;
     }
-    if (p == Prec::ENVELOPE) return allow_smem((const void*)k_envelope, env_smem(256, 64).total);
+    if (p == Prec::ENVELOPE) {
+        size_t most = 0;
+        for (int nl = 1; nl <= 256; nl++) most = std::max(most, env_smem(env_rows(nl, 1 << 20, 1 << 20, 1), nl, 64).total);
+        return allow_smem((const void*)k_envelope, most);
+    }
     const cudaError_t e = prepare<CfgF32>();
     return e == cudaSuccess ? prepare<CfgF32Wide>() : e;
 }
