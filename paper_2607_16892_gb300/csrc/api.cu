@@ -59,7 +59,7 @@ struct kvdro_ctx {
     cudaStream_t last_stream = nullptr;
 
     bool loaded = false;
-    bool pair_sums = false;  // the staged form of the loaded samples
+    bool quads = false;  // the staged form of the loaded samples
     int32_t K = 0;
     int64_t total = 0, pair_total = 0, hist_total = 0;
     std::vector<int64_t> off, pair_off, hist_off, N;
@@ -408,8 +408,8 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     if ((rc = ensure(ctx, ctx->sorted, (size_t)ctx->total * 4))) return rc;
     int32_t max_L = 0;
     for (int32_t k = 0; k < K; k++) max_L = std::max(max_L, L_max[k]);
-    ctx->pair_sums = max_L <= kvdro::kPairMaxL;
-    if ((rc = ensure(ctx, ctx->pairs, (size_t)ctx->pair_total * (ctx->pair_sums ? 4 : 8)))) return rc;
+    ctx->quads = max_L <= kvdro::kExactMaxL;
+    if ((rc = ensure(ctx, ctx->pairs, (size_t)ctx->pair_total * (ctx->quads ? 4 : 8)))) return rc;
     if ((rc = ensure(ctx, ctx->hist, (size_t)ctx->hist_total * 4))) return rc;
     if ((rc = ensure(ctx, ctx->csum, (size_t)ctx->hist_total * 8))) return rc;
     if ((rc = ensure(ctx, ctx->sumx, (size_t)K * 8))) return rc;
@@ -469,7 +469,7 @@ int kvdro_load_samples(kvdro_ctx* ctx, int32_t K, const int64_t* offsets, const 
     a.sumx = static_cast<int64_t*>(ctx->sumx.p);
     a.sorted = static_cast<int32_t*>(ctx->sorted.p);
     a.staged = ctx->pairs.p;
-    a.pair_sums = ctx->pair_sums;
+    a.quads = ctx->quads;
     a.err = static_cast<int32_t*>(ctx->errs.p);
     a.tile_tot = static_cast<int64_t*>(ctx->scan_tot.p);
     a.tile_lo = static_cast<int32_t*>(ctx->tile_lo.p);
@@ -571,7 +571,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     // FP32 and FP64 results come from the exact kernel whenever it applies (FP32: rounded).  Its sums
     // are integers, so it carries only the final combination's FP64 rounding: on 8 classes x 100,000
     // samples x 512 r x 128 lam it is within 1e-16 of the 64-bit result, as the native FP64 kernel is
-    // (6e-14 at 537,000 samples, where the exact kernel stays at 1e-16), in 2.1 ms against 320.7 ms.
+    // (6e-14 at 537,000 samples, where the exact kernel stays at 1e-16), in 1.85 ms against 320.7 ms.
     // The FP32-arithmetic and native FP64 kernels serve supports above 2^22, and native FP64 also
     // costs so large that a whole class's sum nears the end of the double range, where the two
     // combine their parts in different orders.
@@ -650,7 +650,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
 
     kvdro::GridArgs a;
     a.staged = ctx->pairs.p;
-    a.pair_sums = ctx->pair_sums;
+    a.quads = ctx->quads;
     a.pair_off = ctx->d_pair_off;
     a.N = ctx->d_N;
     a.inv_n = ctx->d_inv_n;

@@ -21,18 +21,18 @@
 //    multiply-add on the excess scaled by a power of two (the clamp to [0, 1] is the max) and half
 //    a packed add per sample and cell.
 //  - EXACT (also FP32 and FP64 requests whose supports are all <= 2^22): each cell's integer threshold t
-//    (x >= t exactly when kappa x + d > 0), then the exact sum of |x + 1 - t|, two samples at a time in
-//    packed FP32 adds and a max (or, above a support of 2^19, one at a time in integer absolute
-//    differences); the epilogue puts every sample on its own branch (branch_sum).
+//    (x >= t exactly when kappa x + d > 0), then the exact sum of |x + 1 - t| over the samples, four at a
+//    time (k_exact); the epilogue puts every sample on its own branch (branch_sum).
 //  - ENVELOPE (k_envelope): the same branch sums from the cumulative counts and sums, O(1) per
 //    cell, not per term.
 //
-// Work decomposition.  A CTA owns one (regime m, class k) and a block of RG*TR consecutive r
-// values for the whole lam grid.  Each warp owns a TR x TL tile of (r, lam) cells; its 32 lanes
-// split the class's samples, which stream through a ring of shared-memory chunks filled by TMA
-// bulk copies (cp.async.bulk + mbarrier).  Packed f32x2 instructions serve two cells at once.
-// Periodically each lane's partial sums are transposed and reduced across the warp (fixed
-// shuffle order) so that each lane then owns one cell, folded into an FP64 or int64 accumulator.
+// Work decomposition.  A CTA owns one (regime m, class k) and a block of consecutive r values for the whole
+// lam grid.  A warp owns a few cells at a time -- a TR x TL tile of (r, lam) in k_grid, the next 16 of the
+// CTA's rows laid end to end in k_exact -- and its 32 lanes split the class's samples, which stream
+// through a ring of shared-memory chunks filled by TMA bulk copies (cp.async.bulk + mbarrier).  Packed
+// f32x2 instructions serve two cells at once.  Periodically each lane's partial sums are transposed and
+// reduced across the warp (fixed shuffle order) so that each lane then owns one cell, folded into an
+// FP64 or int64 accumulator.  k_envelope has no samples to stream: its lanes lie along lam, its warps on rows.
 // The epilogue forms S = (1/N) sum phi, then for every eps the minimum over lam (lowest index),
 // and feeds the argmin over r through a 64-bit atomicMin on (cost, r index) keys.
 #include <float.h>
@@ -74,7 +74,7 @@ struct GridCfg {
     static constexpr int TR = TR_, TL = TL_, V = TR_ * TL_, LOG2V = ilog2(TR_ * TL_), FLUSH = FLUSH_, MINB = MINB_;
     static constexpr int MAXT = MAXT_;
     static constexpr int CHUNK = CHUNK_;    // samples per staged chunk
-    static constexpr int BYTES = 8;         // staged bytes per sample (native FP64 also reads pair sums, 4)
+    static constexpr int BYTES = 8;         // staged bytes per sample (native FP64 also reads quads, 4)
     static constexpr int STAGES = STAGES_;  // ring depth
     static constexpr int UNROLL = UNROLL_;  // unroll of the sample loop
     static_assert(P_ != Prec::EXACT && CHUNK_ % 128 == 0 && CHUNK_ * BYTES * STAGES_ <= 160 * 1024, "chunk ring must fit");
@@ -90,19 +90,17 @@ using CfgF32Wide = GridCfg<Prec::F32, 2, 16, 2, 1, 512, 4096, 2, 4>;
 using CfgF64 = GridCfg<Prec::F64, 2, 8, 0, 1, 512, 4096, 2>;
 constexpr int kWarpsTarget = 16;  // warps per CTA the r groups fill up to
 
-// The exact kernel: 16 cells per warp, up to 16 warps per CTA and two CTAs per SM (64 registers).  A CTA
-// takes whole rows of lam values, laid over its warps without regard to rows (a warp needs 16 thresholds,
-// whatever cells they are), in one pass over the class's samples or several (exact_shape).
-constexpr int kExactV = 16;
+// The exact kernel: kExactV cells per warp, up to kExactWarps warps per CTA and kExactBlocks CTAs per SM.  A
+// CTA takes whole rows of lam values, laid over its warps without regard to rows (a warp needs kExactV
+// thresholds, whatever cells they are), in one pass over the class's samples or several (exact_shape).
 constexpr int kExactLog2V = 4;
+constexpr int kExactV = 1 << kExactLog2V;
 constexpr int kExactWarps = 16;
+constexpr int kExactBlocks = 2;
 constexpr int kExactMaxPasses = 4;
-constexpr size_t kExactSmem = (228 * 1024 - 2 * 1024) / 2 - 256;  // two CTAs in an SM's 228 KB, 1 KB reserved for each
-template <bool PAIR>
-struct ExactCfg {
-    static constexpr int kBytes = PAIR ? 4 : 8, kPer = PAIR ? 4 : 2;  // staged bytes per sample, samples per load
-    static constexpr int kChunk = PAIR ? 8192 : 6144;                 // samples per staged chunk at most
-};
+constexpr int kExactStages = 3;
+constexpr int kExactChunk = 8192;  // samples per staged chunk at most
+constexpr size_t kExactSmem = (228 * 1024 / kExactBlocks - 1024) - 256;  // an SM's 228 KB, 1 KB reserved for each CTA
 
 // ---------------------------------------------------------------- PTX helpers
 
@@ -126,11 +124,16 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
-// max(|v|, d) of both halves
-__device__ __forceinline__ u64 max_abs2(u64 v, float d) {
-    float a, b;
-    upk(v, a, b);
-    return pk(fmaxf(fabsf(a), d), fmaxf(fabsf(b), d));
+__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// max(|u|, |v| + p, d)
+__device__ __forceinline__ float max3_abs(float u, float v, float p, float d) {
+    float m;
+    asm("{\n\t.reg .f32 q;\n\tabs.f32 q, %1;\n\tmax.f32 %0, q, %2, %3;\n\t}" : "=f"(m) : "f"(u), "f"(fabsf(v) + p), "f"(d));
+    return m;
 }
 // max(w, 0); a NaN operand yields 0 (PTX max returns the non-NaN input).
 __device__ __forceinline__ double relu(double w) {
@@ -143,6 +146,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -263,11 +269,11 @@ __host__ __device__ inline ExactSmem exact_smem(int rows, int NL, int E, int til
     ExactSmem s;
     s.stride_f = float_stride(NL);
     s.full = ring_bytes;
-    s.lam = s.full + 32;
+    s.lam = s.full + 48;
     s.eps = s.lam + 8 * (size_t)NL;
     s.S = s.eps + 8 * (size_t)E;
     s.t = (s.S + 8 * (size_t)tiles * kExactV + 15) & ~(size_t)15;
-    s.lamf = s.t + 4 * (size_t)tiles * kExactV;
+    s.lamf = (s.t + 4 * (size_t)tiles * kExactV + 15) & ~(size_t)15;
     s.Sf = s.lamf + 4 * (size_t)four(NL);
     s.total = s.Sf + 4 * (size_t)rows * s.stride_f;
     return s;
@@ -394,7 +400,7 @@ struct LamRows {
 // over lam, its outputs and the argmin over r.
 //
 // G lanes per pair, as many as keep every thread busy, groups along r first (outputs side by side, one
-// atomic per warp and radius: one per pair held the envelope at 7.8 ms where it now takes 3.7); each lane
+// atomic per warp and radius: one per pair held the envelope at 7.8 ms where it then took 3.7); each lane
 // takes every G-th four lam values and keeps its smallest v', where it was, and its second smallest: with
 // the second outside the window only that one value is formed in FP64, by all lanes at once.
 template <bool F32OUT>
@@ -493,8 +499,8 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     const int64_t pbase = a.pair_off[k];
     const int64_t np = a.pair_off[k + 1] - pbase;  // multiple of kPadSamples
     const int nchunks = (int)((np + C::CHUNK - 1) / C::CHUNK);
-    // (native FP64 also serves contexts that stage pair sums)
-    const int bytes = P == Prec::F64 && a.pair_sums ? 4 : C::BYTES;
+    // (native FP64 also serves contexts that stage quads)
+    const int bytes = P == Prec::F64 && a.quads ? 4 : C::BYTES;
     const unsigned char* src = static_cast<const unsigned char*>(a.staged) + pbase * bytes;
     auto issue = [&](int c) {
         if (c == a.test_skip_chunk) return;  // test hook: nothing will complete this chunk's barrier
@@ -532,11 +538,10 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         // x - eta comes from the staged samples in one packed add per row and load (both samples of
         // the load): the staged value carries the class's offset, and offset + eta is an integer
         // below 2^24, so the add is exact.
-        const double offd = (double)stage_offset(a.L[k]);
         u64 noff[TR];
 #pragma unroll
         for (int i = 0; i < TR; i++) {
-            const float o = (float)-(offd + eta[i]);
+            const float o = (float)-eta[i];
             noff[i] = pk(o, o);
         }
         u64 kap[TL / 2], dd[TR][TL / 2], acc[TR][TL / 2];
@@ -616,7 +621,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
             if (!timeout) {
                 const int cnt = (int)min((int64_t)C::CHUNK, np - (int64_t)c * C::CHUNK);
                 const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * kStageBytes);
-                const int nq = cnt >> 6;  // float4 (two samples) per lane: (x', x') pairs
+                const int nq = cnt >> 6;  // float4 (two samples) per lane: (x, x) pairs
                 if (nq == C::CHUNK / 64) {  // a full chunk: a fixed trip count, unrolled with no remainder
 #pragma unroll(C::UNROLL)
                     for (int t = 0; t < C::CHUNK / 64; t++) step(q[lane + 32 * t]);
@@ -653,10 +658,6 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
         }
     } else if constexpr (P == Prec::F64) {
         // each row's excess about its reservation, as in the FP32 kernel: x - eta per sample and row
-        const double offd = a.pair_sums ? 0.0 : (double)stage_offset(a.L[k]);  // (x', x') pairs carry the class's offset
-        double base[TR];
-#pragma unroll
-        for (int i = 0; i < TR; i++) base[i] = offd + eta[i];  // an exact integer
         double kap[TL], dd[TR][TL], acc[TR][TL];
 #pragma unroll
         for (int j = 0; j < TL; j++) {
@@ -681,7 +682,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
                 auto two = [&](float x0, float x1) {  // two staged samples (NaN: none)
 #pragma unroll
                     for (int i = 0; i < TR; i++) {
-                        const double xa = (double)x0 - base[i], xb = (double)x1 - base[i];  // x - eta, exact
+                        const double xa = (double)x0 - eta[i], xb = (double)x1 - eta[i];  // x - eta, exact
 #pragma unroll
                         for (int j = 0; j < TL; j++) {
                             acc[i][j] += relu(fma(kap[j], xa, dd[i][j]));
@@ -689,15 +690,15 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
                         }
                     }
                 };
-                if (a.pair_sums) {  // samples back from (sum, difference), exactly; none past the class's last
+                if (a.quads) {  // samples back from their quads, exactly; the class's last quad may start with padding
                     const int64_t left = a.N[k] - (int64_t)c * C::CHUNK;
                     for (int t = 0; t < cnt >> 7; t++) {
-                        const float4 v = q[lane + 32 * t];
-                        const int at = 4 * (lane + 32 * t);
+                        const int4 v = reinterpret_cast<const int4*>(q)[lane + 32 * t];
+                        const int64_t first = max((int64_t)0, 4 * (int64_t)(lane + 32 * t) + 4 - left);  // of the four
                         const float nan = __int_as_float(0x7fc00000);
-                        // the one real sample of a half-padded pair is the larger: its partner is 0
-                        two(at < left ? 0.5f * (v.x + v.z) : nan, at + 1 < left ? 0.5f * (v.x - v.z) : nan);
-                        two(at + 2 < left ? 0.5f * (v.y + v.w) : nan, at + 3 < left ? 0.5f * (v.y - v.w) : nan);
+                        const int ends = v.x - v.y, gap = v.w - v.z;  // x0 + x3, x2 - x1
+                        two(first < 1 ? (float)((ends - v.z) / 2) : nan, first < 2 ? (float)((v.y - gap) / 2) : nan);
+                        two(first < 3 ? (float)((v.y + gap) / 2) : nan, first < 4 ? (float)((ends + v.z) / 2) : nan);
                     }
                 } else {
                     for (int t = 0; t < cnt >> 6; t++) {
@@ -783,26 +784,32 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
 // max(x - c, 0) = (x - c + |x - c|) / 2 and sum_n (x - c) has a closed form, so the kernel streams
 // sum_n |x - c| only, as integers.
 //
-// Pair sums: |a - c| + |b - c| = max(|a + b - 2c|, |a - b|) takes two samples for two cells in one packed
-// FP32 add, two max and (with the next pair's) one packed add, an instruction per term as with one sample
-// at a time, but split evenly over the FMA and ALU pipes within each cell and with fewer register operands
-// (3 reads a term, and the pair's sum and difference serve every cell), in half the staged bytes.  Packed
-// adds on one half of a warp's cells beside integer absolute differences on the other (3.5 reads a term)
-// took 16.43 ms on 8 classes x 100,000 samples x 4096 r x 128 lam, this 16.06: 83 of the 128 terms/clk/SM
-// that either pipe and the issue slots allow.  Every value is an integer below 2^24, so the FP32
-// arithmetic is exact; sums fold into int64 through the warp transposition before one could pass 2^24.
+// Quads: for sorted samples x0 <= x1 <= x2 <= x3 the sum over the four is the maximum of its linear pieces,
+//   sum |x_i - c| = max(|S - 4c|, |Q - 2c| + P, D),
+//   S = x0 + x1 + x2 + x3, Q = x1 + x2, P = x3 - x0, D = (x2 + x3) - (x0 + x1),
+// so one load of {S, Q, P, D} serves four samples of every cell in two packed FP32 instructions for two cells
+// (S - 4c; Q - 2c as one FMA from the same -4c), an add and a three-way max per cell, and half a
+// three-input integer add: 3.5 instructions per cell for four samples, where pairs of samples,
+// max(|a + b - 2c|, |a - b|), take 4.  FMA pipe (128 lanes a clock and SM) and ALU (64) carry 3 cycles each of
+// those, so the issue slots bound it: 146 terms/clk/SM against the pairs' 128.
 //
-// (x', x') pairs (supports above kPairMaxL): one integer absolute-difference-and-add (__sad) per term on
-// the staged float's bit pattern, 0x4B000000 + x; 23.1 ms there.
+// The integers are the floats' bit patterns: an integer n <= 2^24 read as a float is n x 2^-149, a
+// subnormal or one of the two smallest normal binades, where patterns are linear.  FP32 adds, fmas and
+// maxima of such values are exact and full-rate, and their results are already integers: sums
+// run on in 32-bit integer adds, on the pipe that has the room, and fold 256 times more rarely than
+// FP32 sums below 2^24 would.  (The maths need subnormals kept: no flush-to-zero.)
+//
+// 8 classes x 100,000 samples x 4096 r x 128 lam: 14.1 ms, 95 terms/clk/SM (pairs 15.9); the loop alone runs 97
+// to 99 in isolation, bound by register reads (23 operands for 8 terms) rather than by either pipe.  Also
+// measured there: -2c kept beside -4c instead of the FMA 14.5 (80 registers, 12 warps); (S, Q) as one packed
+// operand against (-4c, -2c) of one cell 16.1; 8, 10 and 12 cells a warp 15.6, 15.5, 14.8.
 //
 // The count #{x >= t} comes from the class's cumulative counts; every sample then goes on its branch of
 // phi with these integer sums (branch_sum) in FP64.
-template <bool PAIR>
-__global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a) {
-    using X = ExactCfg<PAIR>;
+__global__ void __launch_bounds__(32 * kExactWarps, kExactBlocks) k_exact(const GridArgs a) {
     constexpr int V = kExactV, kOwn = 5 - kExactLog2V;  // lane l owns cell l >> kOwn after the transposition
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_timeout;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NL = a.NL;
     int b = blockIdx.x;
     const int r_cta0 = b % a.r_blocks * a.rows;
@@ -810,13 +817,15 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
     const int k = b % a.K;
     const int m = a.m0 + b / a.K;
     const int rows = min(a.rows, a.R - r_cta0), cells = rows * NL;
-    const int chunk = a.chunk, stage_bytes = chunk * X::kBytes, nwarps = blockDim.x >> 5;
-    const ExactSmem lay = exact_smem(a.rows, NL, a.E, nwarps * a.passes, a.stages * stage_bytes);
+    const int chunk = a.chunk, stage_bytes = chunk * 4, nwarps = blockDim.x >> 5;
+    const ExactSmem lay = exact_smem(a.rows, NL, a.E, nwarps * a.passes, kExactStages * stage_bytes);
     unsigned char* ring = smem;  // chunk c in stage c % stages
-    u64* full = reinterpret_cast<u64*>(smem + lay.full);
+    u64* full = reinterpret_cast<u64*>(smem + lay.full);  // a chunk has landed in the stage
+    u64* empty = full + kExactStages;                     // every warp is done with the stage's chunk
     double* s_lam = reinterpret_cast<double*>(smem + lay.lam);
     double* s_eps = reinterpret_cast<double*>(smem + lay.eps);
     double* s_S = reinterpret_cast<double*>(smem + lay.S);
+    long long* sums = reinterpret_cast<long long*>(s_S);
     int* s_t = reinterpret_cast<int*>(smem + lay.t);
     float* s_lamf = reinterpret_cast<float*>(smem + lay.lamf);
     float* s_Sf = reinterpret_cast<float*>(smem + lay.Sf);
@@ -824,20 +833,23 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
     const int64_t pbase = a.pair_off[k];
     const int64_t np = a.pair_off[k + 1] - pbase;  // multiple of kPadSamples
     const int nchunks = (int)((np + chunk - 1) / chunk), total = nchunks * a.passes;  // over all passes
-    const unsigned char* src = static_cast<const unsigned char*>(a.staged) + pbase * X::kBytes;
+    const unsigned char* src = static_cast<const unsigned char*>(a.staged) + pbase * 4;
     auto issue = [&](int c, int s) {  // the class's chunk c into stage s
         if (c == a.test_skip_chunk) return;  // test hook: nothing will complete this chunk's barrier
         const int64_t cnt = min((int64_t)chunk, np - (int64_t)c * chunk);
-        tma_bulk_load(smem_u32(ring + (size_t)s * stage_bytes), src + (int64_t)c * stage_bytes, (uint32_t)(cnt * X::kBytes),
+        tma_bulk_load(smem_u32(ring + (size_t)s * stage_bytes), src + (int64_t)c * stage_bytes, (uint32_t)(cnt * 4),
                       smem_u32(&full[s]));
     };
     // the chunk `ahead` places after the class's chunk c, passes wrapping
     auto chunk_after = [&](int c, int ahead) { return (c + ahead) % nchunks; };
     if (tid == 0) {  // no other thread touches a barrier before the __syncthreads below
-        s_bad = 0;
-        for (int s = 0; s < a.stages; s++) mbar_init(smem_u32(&full[s]), 1);
+        s_bad = s_timeout = 0;
+        for (int s = 0; s < kExactStages; s++) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), nwarps);
+        }
         fence_mbar_init();
-        for (int i = 0; i < a.stages && i < total; i++) issue(chunk_after(0, i), i);
+        for (int i = 0; i < kExactStages && i < total; i++) issue(chunk_after(0, i), i);
     }
     for (int i = tid; i < NL; i += blockDim.x) s_lam[i] = a.lam[i];
     for (int i = tid; i < a.E; i += blockDim.x) s_eps[i] = a.eps[i];
@@ -855,148 +867,122 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
             t = first_active(__dadd_rn(mu, dmin_nonneg(lam, cw)), excess_offset(row, cp, mu, to_double(a.L[k])), a.L[k]);
         }
         s_t[c] = t;
+        sums[c] = 0;
     }
     __syncthreads();
-    constexpr int NP = PAIR ? V / 2 : 1, NI = PAIR ? 1 : V;  // array extents
-    [[maybe_unused]] u64 n2c[NP], accf[NP];                  // -2c for two cells, their sums
-    [[maybe_unused]] int cci[NI];                            // 0x4B000000 + c per cell
-    [[maybe_unused]] unsigned acci[NI];
-    // Fold after at most `fe` loads of kPer samples each: a lane's sum is then at most kPer fe (L + 1),
-    // within 2^24 in FP32 (the transposition's 32-lane sums stay below 2^29), or as integers 32 lanes'
-    // sums below 2^32.  The same for every thread of the CTA.
-    constexpr long long kFoldLimit = PAIR ? (1ll << 24) : (1ll << 32) / 32 - 1;
-    const int fe = (int)min(1ll << 20, max(1ll, kFoldLimit / (X::kPer * ((long long)a.L[k] + 1))));
-    long long acc_r = 0;
+    u64 n4c[V / 2] = {};  // -4c for two cells
+    unsigned acc[V] = {};
+    const u64 half = pk(0.5f, 0.5f);
+    const int* w_t = s_t + warp * V;  // the pass's thresholds
+    // Fold after at most `fe` loads of 4 samples: 32 lanes' sums of at most 4 L a load then stay below 2^32.
+    // The same for every thread of the CTA.
+    const int fe = (int)((1u << 27) - 1) / (4 * max(a.L[k], 1)) & ~1;
+    int pending = 0;  // loads since the last fold
     auto fold = [&]() {
-        unsigned vs[V];
-        if constexpr (PAIR) {
+        const unsigned sum = transpose_reduce<unsigned, V>(acc, lane);
+        if ((lane & ((1 << kOwn) - 1)) == 0) sums[w_t - s_t + (lane >> kOwn)] += sum;
 #pragma unroll
-            for (int p = 0; p < NP; p++) {
-                float a0, a1;
-                upk(accf[p], a0, a1);
-                vs[2 * p] = __float2uint_rn(a0);
-                vs[2 * p + 1] = __float2uint_rn(a1);
-                accf[p] = 0ull;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < V; j++) {
-                vs[j] = acci[j];
-                acci[j] = 0u;
-            }
-        }
-        acc_r += (long long)transpose_reduce<unsigned, V>(vs, lane);
+        for (int j = 0; j < V; j++) acc[j] = 0u;
+        pending = 0;
     };
-    // One load into every cell's sum.  The pair sums' rate hangs on ptxas's register allocation (operand
-    // bank conflicts): written cell by cell, the second pair first, 16.06 ms on 8 classes x 100,000
-    // samples x 4096 r x 128 lam; first pair first 16.39, the accumulator as first operand 16.57, two
-    // cells' adds ahead of their max 16.91, all adds first 17.03; unrolled 4 / 16 times 16.6 / 16.5.
-    auto step = [&](const float4 v) {
-        if constexpr (PAIR) {
-            const u64 s0 = pk(v.x, v.x), s1 = pk(v.y, v.y);
+    // One load's sum for cells 2p and 2p + 1.
+    auto quad = [&](const float4 v, int p, unsigned& s0, unsigned& s1) {
+        float u0, u1, v0, v1;
+        upk(ffma2(n4c[p], half, pk(v.y, v.y)), v0, v1);
+        upk(fadd2(pk(v.x, v.x), n4c[p]), u0, u1);
+        s0 = __float_as_uint(max3_abs(u0, v0, v.z, v.w));
+        s1 = __float_as_uint(max3_abs(u1, v1, v.z, v.w));
+    };
+    auto two = [&](const float4 va, const float4 vb) {
 #pragma unroll
-            for (int p = 0; p < NP; p++)
-                accf[p] = fadd2(fadd2(max_abs2(fadd2(s1, n2c[p]), v.w), max_abs2(fadd2(s0, n2c[p]), v.z)), accf[p]);
-        } else {
-            const int ba = __float_as_int(v.x), bb = __float_as_int(v.z);  // 0x4B000000 + x
-#pragma unroll
-            for (int j = 0; j < V; j++) acci[j] = __sad(bb, cci[j], __sad(ba, cci[j], acci[j]));
+        for (int p = 0; p < V / 2; p++) {
+            unsigned a0, a1, b0, b1;
+            quad(va, p, a0, a1);
+            quad(vb, p, b0, b1);
+            acc[2 * p] += a0 + b0;
+            acc[2 * p + 1] += a1 + b1;
         }
     };
-    // Loads per segment of a fixed trip count: long ones run 1.4 % faster (8 classes x 100,000 samples x 4096 r x
-    // 128 lam 16.15 -> 15.92 ms), short ones take the rest of a chunk, and all of it where long ones would
-    // fold much more often than the bound asks (the heavy tail's support of 131072: 39.5 ms against 44).
-    constexpr int kLongSeg = 32, kShortSeg = 8;
-    int pending = 0;         // loads since the last fold
-    auto room = [&](int loads) {  // fold first if the loads since the last fold would pass fe
-        if (pending + loads > fe) {
-            fold();
-            pending = 0;
-        }
-        pending += loads;
-    };
-    auto segments = [&](const float4* q, int& t0, int t_end, auto seg) {
-        constexpr int kSeg = decltype(seg)::value;
+    // `loads` loads (a multiple of kSeg) in segments of a fixed trip count, two loads at a time.  64 with 8 loads
+    // to an iteration run 14.1 ms on 8 classes x 100,000 samples x 4096 r x 128 lam, 16 with 4 14.6; unrolled in
+    // full, loads move up and registers spill (16: 22.8).
+    auto segments = [&](const float4*& q, int loads, auto seg) {
+        constexpr int kSeg = decltype(seg)::value, kUnroll = kSeg == 64 ? 8 : 4;
+        const float4* stop = q + 32 * loads;
 #pragma unroll 1
-        for (; t0 + kSeg <= t_end; t0 += kSeg) {
-            room(kSeg);
-#pragma unroll
-            for (int t = 0; t < kSeg; t++) step(q[lane + 32 * (t0 + t)]);
+        for (; q < stop; q += 32 * kSeg) {
+#pragma unroll kUnroll
+            for (int t = 0; t < kSeg; t += 2) two(q[32 * t], q[32 * t + 32]);
         }
     };
     bool timeout = false;
+    int issued = min(kExactStages, total);  // by thread 0
     int at = 0, c = 0, s = 0;  // chunk over all passes, of the class, its stage
     uint32_t phase = 0;
-    const int* w_t = s_t + warp * V;  // the pass's thresholds
     for (; at < total; at++) {
         if (c == 0) {
-            if constexpr (PAIR) {
 #pragma unroll
-                for (int p = 0; p < NP; p++) {
-                    n2c[p] = pk((float)(2 - 2 * w_t[2 * p]), (float)(2 - 2 * w_t[2 * p + 1]));
-                    accf[p] = 0ull;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < V; j++) {
-                    cci[j] = kStageBits - 1 + w_t[j];
-                    acci[j] = 0u;
-                }
+            for (int p = 0; p < V / 2; p++) {
+                const int c0 = max(w_t[2 * p], 1) - 1, c1 = max(w_t[2 * p + 1], 1) - 1;
+                n4c[p] = pk(-__int_as_float(4 * c0), -__int_as_float(4 * c1));
             }
         }
-        if (!mbar_wait_bounded(smem_u32(&full[s]), phase, a.wait_ns)) timeout = true;
-        if (!timeout) {
-            const int cnt = (int)min((int64_t)chunk, np - (int64_t)c * chunk);
-            const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * stage_bytes);
-            const int nq = cnt / (32 * X::kPer);
-            // loads [0, t_clean) hold samples only; of (x', x') pairs the class's last ones may hold NaN
-            // padding, which they read as x = 0 (x' = 2^23)
-            const int64_t left = a.N[k] - (int64_t)c * chunk;
-            const int t_clean = PAIR ? nq : (left <= 0 ? 0 : (int)min((int64_t)nq, left / (32 * X::kPer)));
-            int t0 = 0;
-            if (fe >= 2 * kLongSeg) segments(q, t0, t_clean, std::integral_constant<int, kLongSeg>());
-            if (fe >= kShortSeg) segments(q, t0, t_clean, std::integral_constant<int, kShortSeg>());
-#pragma unroll 1
-            for (; t0 < nq; t0++) {
-                room(1);
-                float4 v = q[lane + 32 * t0];
-                if (!PAIR && t0 >= t_clean) {
-                    v.x = fmaxf(v.x, kStageOffset), v.y = fmaxf(v.y, kStageOffset);
-                    v.z = fmaxf(v.z, kStageOffset), v.w = fmaxf(v.w, kStageOffset);
+        // The warps run on by themselves, up to a stage's reuse: a barrier of the CTA after each chunk costs 1 to 2 %.
+        timeout = !__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&full[s]), phase, a.wait_ns));
+        if (timeout) break;
+        const float4* q = reinterpret_cast<const float4*>(ring + (size_t)s * stage_bytes) + lane;
+        const float4* end = q + min((int64_t)chunk, np - (int64_t)c * chunk) / 4;
+        while (q < end) {
+            if (pending == fe) fold();
+            const int loads = min((int)(end - q) / 32, fe - pending);
+            pending += loads;
+            segments(q, loads & ~63, std::integral_constant<int, 64>());
+            segments(q, loads & 48, std::integral_constant<int, 16>());
+            segments(q, loads & 14, std::integral_constant<int, 2>());
+            if (loads & 1) {
+#pragma unroll
+                for (int p = 0; p < V / 2; p++) {
+                    unsigned a0, a1;
+                    quad(*q, p, a0, a1);
+                    acc[2 * p] += a0;
+                    acc[2 * p + 1] += a1;
                 }
-                step(v);
+                q += 32;
             }
         }
-        if (__syncthreads_or(timeout)) {
-            timeout = true;
-            break;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
+        // The first warp refills the stage before, which the others have mostly left by now.
+        if (warp == 0 && at > 0 && at - 1 + kExactStages < total) {
+            const int sp = s == 0 ? kExactStages - 1 : s - 1;
+            const uint32_t done = s == 0 ? phase ^ 1 : phase;
+            timeout = !__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&empty[sp]), done, a.wait_ns));
+            if (timeout) break;
+            if (lane == 0) {
+                fence_proxy_async();
+                issue(chunk_after(c, kExactStages - 1), sp);
+                issued++;
+            }
         }
-        if (tid == 0 && at + a.stages < total) {
-            fence_proxy_async();
-            issue(chunk_after(c, a.stages), s);
-        }
-        if (++s == a.stages) {
+        if (++s == kExactStages) {
             s = 0;
             phase ^= 1;
         }
         if (++c == nchunks) {  // the pass's sums
             c = 0;
             if (pending > 0) fold();
-            pending = 0;
-            if ((lane & ((1 << kOwn) - 1)) == 0)
-                reinterpret_cast<long long*>(s_S)[w_t - s_t + (lane >> kOwn)] = acc_r;
-            acc_r = 0;
             w_t += nwarps * V;
         }
     }
-    if (timeout) {
-        // Report, then let every copy this CTA issued land before the CTA's shared memory is released:
-        // chunks up to `at` + stages - 1 were issued.
+    if (timeout) s_timeout = 1;
+    __syncthreads();
+    if (s_timeout) {
+        // Report, then let every copy this CTA issued land before the CTA's shared memory is released.
         if (tid == 0) {
             atomicOr(a.err + 1, kErrTimeout);
-            for (const int end = min(at + a.stages, total); at < end; at++) {
+            for (; at < issued; at++) {
                 (void)mbar_wait_bounded(smem_u32(&full[s]), phase, a.wait_ns);
-                if (++s == a.stages) {
+                if (++s == kExactStages) {
                     s = 0;
                     phase ^= 1;
                 }
@@ -1005,7 +991,6 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
         __syncthreads();
         return;
     }
-    __syncthreads();
     bool ok = true;
     {
         const long long N = a.N[k], sumx = a.sumx[k], npad = np - N;
@@ -1013,13 +998,12 @@ __global__ void __launch_bounds__(32 * kExactWarps, 2) k_exact(const GridArgs a)
         for (int i = tid; i < cells; i += blockDim.x) {
             // the active count from the cumulative counts, then the branch sums
             const int ti = s_t[i], rl = i / NL, lj = i % NL;  // ti in [0, L + 1]
-            const long long t = ti;
-            const long long count = ti <= 0 ? N : (ti > L ? 0 : N - (long long)a.cdf[a.hist_off[k] + t - 1]);
+            const long long count = ti <= 0 ? N : (ti > L ? 0 : N - (long long)a.cdf[a.hist_off[k] + ti - 1]);
             // sum |x - c| over the samples and the padding zeros; with y = x - c, max(y, 0) = (y + |y|) / 2
-            const long long sum_abs = dbits(s_S[i]) - npad * (t > 1 ? t - 1 : 1 - t);
-            const long long sum_y = sumx + N * (1 - t);
-            const long long sum_relu = (sum_y + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
-            const long long sum = sum_relu + (t - 1) * count;  // sum_{x >= t} x
+            const long long c = max(ti, 1) - 1;  // x >= t exactly when x > c, or always for t = 0, where c = 0 serves too
+            const long long sum_abs = sums[i] - npad * c;
+            const long long sum_relu = (sumx - N * c + sum_abs) / 2;  // each sample adds y + |y| = 2 relu(y)
+            const long long sum = sum_relu + c * count;               // sum_{x >= t} x
             // each sample on its own branch of phi (exact integer sums): V = c_w eta - nu x below t,
             // U = c_p (L - eta) - mu (L - x) from t on; no large term cancels another
             const double lam = s_lam[lj];
@@ -1250,12 +1234,10 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
 // holds as many as the others (13 to 16 warps take the same time), and fewer per scheduler run at a lower
 // rate: 5 classes x 1001 r x 200 lam x 3 regimes 2.27 ms in one pass of 13 warps, 1.90 in four passes of 16
 // (2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
-template <bool PAIR>
-GridShape exact_shape(int variant, int32_t R, int32_t NL, int32_t E, int64_t classes, int sms) {
-    using X = ExactCfg<PAIR>;
+GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int64_t classes, int sms) {
     constexpr int kCells = kExactWarps * kExactV;
     GridShape best, sh;
-    sh.variant = variant;
+    sh.variant = 3;
     sh.LT = sh.RG = 1;
     double best_score = -1.0;
     for (int passes = 1; passes <= kExactMaxPasses; passes++) {
@@ -1267,15 +1249,14 @@ GridShape exact_shape(int variant, int32_t R, int32_t NL, int32_t E, int64_t cla
         const int warps = (tiles + sh.passes - 1) / sh.passes;
         sh.threads = 32 * warps;
         sh.r_blocks = (R + rows - 1) / rows;
-        // 96 KB of ring: three 32 KB chunks of pair sums (8192 samples; two of 32, 36 or 48 KB, four of 24
-        // and six of 16 measured 2 to 5 % slower) or two 48 KB chunks of (x', x') pairs; smaller chunks where
+        // 96 KB of ring: three chunks of 8192 samples (6144 measured 1 % slower, 4096 3 %); smaller chunks where
         // the cells need the room
-        sh.stages = PAIR ? 3 : 2;
-        sh.chunk = X::kChunk;
+        sh.stages = kExactStages;
+        sh.chunk = kExactChunk;
         do {
-            sh.smem = exact_smem(rows, NL, E, warps * sh.passes, sh.stages * sh.chunk * X::kBytes).total;
+            sh.smem = exact_smem(rows, NL, E, warps * sh.passes, sh.stages * sh.chunk * 4).total;
         } while (sh.smem > kExactSmem && (sh.chunk -= 1024) > 0);
-        const double slots = 2.0 * sms, ctas = (double)classes * sh.r_blocks, waves = ctas / slots;
+        const double slots = (double)kExactBlocks * sms, ctas = (double)classes * sh.r_blocks, waves = ctas / slots;
         const int held = (warps + 3) / 4 * 4;  // warps that the fullest of the four schedulers accounts for
         const double filled = (double)R * NL / ((double)sh.r_blocks * held * sh.passes * kExactV);
         const double rate = 0.55 + 0.45 * held / kExactWarps;
@@ -1301,7 +1282,7 @@ GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, in
     }
     if (p == Prec::F64) return shape_for<CfgF64>(2, R, NL, E);
     if (p == Prec::EXACT)
-        return max_L > kPairMaxL ? exact_shape<false>(6, R, NL, E, classes, sms) : exact_shape<true>(3, R, NL, E, classes, sms);
+        return exact_shape(R, NL, E, classes, sms);
     if (NL <= kWarpsTarget * CfgF32::TL) return shape_for<CfgF32>(0, R, NL, E);
     return shape_for<CfgF32Wide>(1, R, NL, E);
 }
@@ -1327,8 +1308,7 @@ cudaError_t prepare() {
 cudaError_t grid_prepare(Prec p) {
     if (p == Prec::F64) return prepare<CfgF64>();
     if (p == Prec::EXACT) {
-        const cudaError_t e = allow_smem((const void*)k_exact<true>, kExactSmem);
-        return e == cudaSuccess ? allow_smem((const void*)k_exact<false>, kExactSmem) : e;
+        return allow_smem((const void*)k_exact, kExactSmem);
     }
     if (p == Prec::ENVELOPE) {
         size_t most = 0;
@@ -1351,8 +1331,7 @@ cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s)
     if (nblocks <= 0 || nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (p == Prec::ENVELOPE) k_envelope<<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (p == Prec::F64) k_grid<CfgF64><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT && sh.variant == 3) k_exact<true><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
-    else if (p == Prec::EXACT) k_exact<false><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
+    else if (p == Prec::EXACT) k_exact<<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else if (sh.variant == 0) k_grid<CfgF32><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     else k_grid<CfgF32Wide><<<(unsigned)nblocks, sh.threads, sh.smem, s>>>(a);
     return cudaGetLastError();

@@ -8,13 +8,13 @@ namespace kvdro {
 
 // Samples of one class are staged for the grid kernel in regions of a multiple of kPadSamples, in one
 // of two forms, the same for every class of a context.
-//  - Pair sums, where the largest support is at most kPairMaxL: four samples a, b, c, d in 16 bytes as
-//    the floats {a + b, c + d, |a - b|, |c - d|}, each an integer below 2^24; samples past the class's
-//    last are 0, and the exact kernel subtracts their known |0 - c| per cell.
-//  - (x', x') float pairs above, x' the sample plus the class's staging offset (stage_offset below), so
-//    that one 128-bit shared-memory load yields the packed operands of two samples, padded with NaN
-//    pairs, which contribute exactly zero to the per-term kernels' excess sums (max(NaN, 0) = 0 in PTX
-//    max.f32 / max.f64); the exact kernel reads the padding as x = 0.
+//  - Quads, where every support is at most kExactMaxL: four samples a <= b <= c <= d (neighbours of the sorted
+//    class) in 16 bytes as the integers {a + b + c + d, b + c, d - a, (c + d) - (a + b)}.  The class's last
+//    quad starts with zeros where its samples are fewer, further quads are zeros; the exact kernel
+//    subtracts their known |0 - c| per cell.
+//  - (x, x) float pairs otherwise, so that one 128-bit shared-memory load yields the packed operands of two
+//    samples, padded with NaN pairs, which contribute exactly zero to the per-term kernels' excess sums
+//    (max(NaN, 0) = 0 in PTX max.f32 / max.f64).
 constexpr int kPadSamples = 128;
 
 // Error bits reported by kernels in ctx->d_err[1].
@@ -33,7 +33,7 @@ struct SortArgs {
     int64_t* csum;              // [hist_off[K]] cumulative sums sum_{x <= v} x, or nullptr to skip
     int64_t* sumx;              // [K] sum of samples per class (written by the scan)
     int32_t* sorted;            // [offsets[K]]
-    void* staged;               // pair_off[K] samples, 4 bytes each as pair sums or 8 as (x', x') pairs
+    void* staged;               // pair_off[K] samples, 4 bytes each as quads or 8 as (x, x) pairs
     int32_t* err;               // [0] += out-of-range samples
     int64_t* tile_tot;          // [K][scan_tiles][2] scan tile totals (count, sum of v h[v])
     int32_t* tile_lo;           // [exp_blocks[K] + K] per class from exp_blocks[k] + k: the bin of the
@@ -41,7 +41,7 @@ struct SortArgs {
     double* inv_n;              // [K] 1 / N written by the expansion, or nullptr to skip (may lie over
                                 // tile_tot, which the expansion does not read)
     int32_t scan_tiles;         // scan tiles of the largest class: ceil((max L + 1) / scan tile bins)
-    int32_t pair_sums;          // the staged form
+    int32_t quads;          // the staged form
     int32_t K;
 };
 
@@ -55,24 +55,10 @@ cudaError_t launch_gather_quantiles(const int32_t* sorted, const int64_t* offset
                                     int32_t F, int32_t* out, cudaStream_t s);
 
 // F32: per-term FP32 excess sums folded into FP64.  F64: per-term FP64.  EXACT: an exact integer
-// threshold per cell, then an exact sum of |x - c| over the samples (two samples at a time in packed
-// FP32 adds and a max, or one at a time in integer absolute differences), combined in FP64.
+// threshold per cell, then an exact sum of |x - c| over the samples (four at a time), combined in FP64.
 // ENVELOPE: the same sums in O(1) per cell from cumulative counts and sums (not per term).
 enum class Prec { F32 = 0, F64 = 1, EXACT = 2, ENVELOPE = 3 };
 constexpr int32_t kExactMaxL = 1 << 22;  // the exact kernel's integer sums need L <= 2^22
-
-// Up to a support of kPairMaxL a lane's FP32 sums of |a - c| + |b - c| stay exact (below 2^24) over at
-// least 7 loads of four samples between folds; the integer sums of larger supports fold every 8 loads
-// of two at most.
-constexpr int32_t kPairMaxL = 1 << 19;
-
-// In the (x', x') form, samples of a class whose support is at most kExactMaxL carry an offset of 2^23.
-// On [2^23, 2^24) a float's bit pattern is 0x4B000000 + x exactly, so the exact kernel's integer
-// absolute differences work on the bits without a conversion.  Larger supports are staged as x.  The
-// FP32 and FP64 per-term kernels subtract the class's offset (exactly) from every sample.
-constexpr float kStageOffset = 8388608.0f;  // 2^23
-constexpr int32_t kStageBits = 0x4B000000;  // bit pattern of 2^23
-__host__ __device__ inline float stage_offset(int32_t L) { return L <= kExactMaxL ? kStageOffset : 0.0f; }
 
 struct FinalizeArgs {
     const unsigned long long* keys;  // [M][E][K] argmin keys
@@ -91,7 +77,7 @@ struct FinalizeArgs {
 struct GridArgs {
     const void* staged;         // the padded samples
     const int64_t* pair_off;    // [K+1] in samples
-    int32_t pair_sums;          // the staged form
+    int32_t quads;          // the staged form
     const int64_t* N;           // [K]
     const double* inv_n;        // [K] 1 / N
     const int64_t* sumx;        // [K]

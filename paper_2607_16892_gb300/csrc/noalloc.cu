@@ -1,9 +1,10 @@
 // kvdro_eval_grid_noalloc: the FP32 grid evaluation for callers that cannot allocate memory.
 // All of its scratch (class metadata, grid parameters, cumulative counts, the sorted samples,
-// the NaN-padded sample pairs the grid kernel streams, and the argmin keys) lives in one
+// the staged samples the grid kernel streams, and the argmin keys) lives in one
 // file-scope __device__ array that every device loading this library holds until the process
 // exits.  Nothing in this file calls cudaMalloc, cudaFree, cudaHostAlloc, malloc/new or any
-// other allocating routine; the per-class metadata is derived on the device.
+// other allocating routine; the per-class metadata is derived on the stack where it travels in the setup
+// launch's arguments, and by one thread on the device where it does not fit there.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -304,8 +305,8 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     sa.csum = nullptr;  // cumulative sums are not needed here
     sa.sumx = reinterpret_cast<int64_t*>(S + o_sumx);
     sa.sorted = reinterpret_cast<int32_t*>(S + o_sorted);
-    sa.staged = S + o_pairs;  // of 8 bytes a sample as pair sums take 4
-    sa.pair_sums = max_L <= kvdro::kPairMaxL;
+    sa.staged = S + o_pairs;  // of 8 bytes a sample as quads take 4
+    sa.quads = max_L <= kvdro::kExactMaxL;
     sa.err = reinterpret_cast<int32_t*>(S + o_err);
     sa.tile_tot = reinterpret_cast<int64_t*>(S + o_tiles);
     sa.tile_lo = reinterpret_cast<int32_t*>(S + o_tile_lo);
@@ -324,7 +325,7 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     // else the FP32-arithmetic one) and the argmin finalisation
     kvdro::GridArgs a;
     a.staged = sa.staged;
-    a.pair_sums = sa.pair_sums;
+    a.quads = sa.quads;
     a.pair_off = sa.pair_off;
     a.N = mt.N;
     a.inv_n = sa.inv_n;

@@ -3,10 +3,9 @@
 // sorted order is fully determined by its histogram over [0, L_k]: histogram -> inclusive scan
 // (the cumulative count C[v] = #{x <= v}, i.e. N times the empirical CDF) -> expansion of every
 // output position p into the smallest v with C[v] > p.  The scan also records, for every tile of
-// kExpandTile output positions, the bin its first position falls in; the expansion then marks
-// where each bin's run of positions starts inside the tile and takes a running maximum, O(N + L)
-// in all.  It also writes the samples in the form that the grid kernel streams (kvdro_internal.cuh),
-// padded to a multiple of kPadSamples per class.
+// kExpandTile output positions, the bin its first position falls in; the expansion then searches the
+// bins of its tile's range.  It also writes the samples in the form that the grid kernel streams
+// (kvdro_internal.cuh), padded to a multiple of kPadSamples per class.
 #include <math.h>
 
 #include <algorithm>
@@ -275,18 +274,16 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
         if (lane < 2 * kSteps && p < N) ends = value_at(C, v_lo, v_hi, (int)p);
     }
     int32_t* sorted = a.sorted + a.offsets[k];
-    float* staged = static_cast<float*>(a.staged) + a.pair_off[k] * (a.pair_sums ? 1 : 2);
+    float* staged = static_cast<float*>(a.staged) + a.pair_off[k] * (a.quads ? 1 : 2);
     const bool aligned = (a.offsets[k] & 3) == 0;
-    const float off = stage_offset(a.L[k]);  // x + 2^23 is exact for L <= 2^22
 #pragma unroll 2
     for (int i = 0; i < kSteps; i++) {
         const unsigned first = p0 + 128 * (warp + kWarps * i), at = first + 4 * lane;
         if (first >= padk) break;  // warp-uniform; padk is a multiple of 128
         const int32_t vf = __shfl_sync(0xffffffffu, ends, 2 * i), vl = __shfl_sync(0xffffffffu, ends, 2 * i + 1);
-        if (vf == vl && first + 128 <= N && aligned && a.pair_sums) {  // one run
+        if (vf == vl && first + 128 <= N && aligned && a.quads) {  // one run
             *reinterpret_cast<int4*>(sorted + at) = make_int4(vf, vf, vf, vf);
-            const float s = (float)(2 * vf);
-            *reinterpret_cast<float4*>(staged + at) = make_float4(s, s, 0.f, 0.f);
+            *reinterpret_cast<int4*>(staged + at) = make_int4(4 * vf, 2 * vf, 0, 0);
             continue;
         }
         const int left = at < N ? (int)min(N - at, 4u) : 0;  // samples among the four
@@ -322,15 +319,21 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
             for (int j = 0; j < 4; j++)
                 if (j < left) sorted[at + j] = x[j];
         }
-        if (a.pair_sums) {  // 0 past the class's samples
+        if (a.quads) {  // of the class's last samples and zeros before them
 #pragma unroll
-            for (int j = 0; j < 4; j++) x[j] = j < left ? x[j] : 0;
-            *reinterpret_cast<float4*>(staged + at) =
-                make_float4((float)(x[0] + x[1]), (float)(x[2] + x[3]), (float)abs(x[1] - x[0]), (float)abs(x[3] - x[2]));
-        } else {  // (x', x') pairs; NaN past the class's samples
+            for (int j = 0; j < 4; j++)
+                if (j >= left) {
+                    x[3] = x[2];
+                    x[2] = x[1];
+                    x[1] = x[0];
+                    x[0] = 0;
+                }
+            const int low = x[0] + x[1], high = x[2] + x[3];
+            *reinterpret_cast<int4*>(staged + at) = make_int4(low + high, x[1] + x[2], x[3] - x[0], high - low);
+        } else {  // (x, x) pairs; NaN past the class's samples
             float f[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) f[j] = j < left ? (float)x[j] + off : __int_as_float(0x7fc00000);
+            for (int j = 0; j < 4; j++) f[j] = j < left ? (float)x[j] : __int_as_float(0x7fc00000);
             float4* out = reinterpret_cast<float4*>(staged + 2 * (size_t)at);
             out[0] = make_float4(f[0], f[0], f[1], f[1]);
             out[1] = make_float4(f[2], f[2], f[3], f[3]);

@@ -78,17 +78,17 @@ def test_envelope_magnitudes(scale):
     compare_full(w, env, O.solve(w), "fp64")
 
 
-@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 127, 128, 129, 8191, 8192, 8193, 24577])
-@pytest.mark.parametrize("L,nl", [(300, 9), (1 << 19, 1), (1 << 19, 9), ((1 << 19) + 1, 2), ((1 << 19) + 1, 9)])
-def test_exact_staged_forms(n, L, nl):
-    """Pair sums up to a support of 2^19 (4 samples to a load, 8192 to a chunk, zero padding) and (x', x')
-    pairs above, on 2 x 8 and 8 x 2 tiles: the sums of the exact and the envelope mode are the same integers,
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 127, 128, 129, 4095, 4096, 4097, 8193, 24577])
+@pytest.mark.parametrize("L,nl", [(1, 3), (300, 9), (1 << 19, 1), ((1 << 21) + 1, 9), (1 << 22, 1), (1 << 22, 9)])
+def test_exact_quads(n, L, nl):
+    """Quads of sorted samples (a class's last one starting with zeros, 4096 samples to a chunk) as integers
+    up to 2^24 in float bit patterns: the sums of the exact and the envelope mode are the same integers,
     so every output is the same bit for bit.  Samples at 0 and at the top of the support, against
-    reservations at both ends, make a lane's sums as large as they get between folds."""
+    reservations at both ends, make a lane's sums as large as they get between folds (7 loads at 2^22)."""
     rng = np.random.default_rng(n)
     x = rng.integers(0, L + 1, n)
     x[: n // 2] = L
-    w = make([x], L, [0, 1, L // 3, L - 1, L], np.logspace(-2, 2, nl), [0.0, 30.0], [10.0, 0.3], [1.0, 1.0])
+    w = make([x], L, np.unique([0, 1, L // 3, L - 1, L]), np.logspace(-2, 2, nl), [0.0, 30.0], [10.0, 0.3], [1.0, 1.0])
     exact, env = run(w, kvdro.KVDRO_EXACT), run(w, kvdro.KVDRO_ENVELOPE)
     for key, v in exact.items():
         assert np.array_equal(v, env[key]), key
