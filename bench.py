@@ -42,16 +42,14 @@ METRIC = "DRO cost terms/sec (class×r×λ×sample) on 1 GB300; % of FP32/HBM ro
 UNIT = "terms/s"
 DEFAULT_WORKLOAD = "regimes_k8_n2e5"
 SM_MAX_MHZ_RECIPE = 2070.0
-# Bound of the exact kernel's per-term work.  A term costs one instruction-lane on one of two
-# pipes: packed f32x2 adds on the FMA pipe (128 FP32 lanes/clk/SM, two lane-operations per term:
-# 64 terms/clk/SM) or an integer absolute-difference-and-add (sad) on the ALU pipe (64 lanes/clk/SM,
-# one per term: 64 terms/clk/SM).  The kernel splits every warp's cells between the two, so at
-# most 128 terms per clock per SM, which is also the issue limit (4 schedulers x 1 instruction per
-# clock x 32 lanes, one instruction per term and lane).  Measured on this GB300: packed f32x2 adds
-# alone 127.9 FP32 lane-ops/clk/SM, sad.s32 alone 63.4 terms/clk/SM.
-FMA_TERMS_PER_CLK_PER_SM = 128.0 / 2.0
-ALU_TERMS_PER_CLK_PER_SM = 64.0
-TERMS_PER_CLK_PER_SM = FMA_TERMS_PER_CLK_PER_SM + ALU_TERMS_PER_CLK_PER_SM
+# Bound of the exact kernel's per-term work.  Four samples of one cell take 3.5 instructions: half each of
+# a packed f32x2 add, a packed fma and a three-input integer add (shared by two cells or two loads), an FP32
+# add and a three-way max.  The packed ones and the add hold the FMA pipe (128 lanes/clk/SM) for 3
+# cycles of a scheduler, the max and the integer add the ALU pipe (64 lanes) for 3; the issue slots (4
+# schedulers, one instruction a clock) allow 128 x 4 / 3.5 terms per clock and SM.  Measured on this
+# GB300: packed f32x2 adds 127.9 FP32 lane-ops/clk/SM, max, three-way max and integer add 59 lanes each.
+INST_PER_TERM_FLOOR = 3.5 / 4.0
+TERMS_PER_CLK_PER_SM = 128.0 / INST_PER_TERM_FLOOR
 # The per-term bound of the three-candidate supremum as written: two FMAs, two maxima and one add
 # per term, 5 FP32 lane-operations on 128 FP32 lanes per clock per SM.
 PAPER_FORM_LANE_OPS_PER_TERM = 5.0
@@ -60,10 +58,13 @@ PAPER_FORM_LANE_OPS_PER_TERM = 5.0
 FP32_PHI_TERMS_PER_CLK_PER_SM = 128.0 / 2.0
 # What the exact kernel evaluates per term: once a cell's exact integer threshold t is known
 # (x >= t exactly when the excess kappa x + d is positive), the excess sum is
-# kappa sum_{x >= t} x + d #{x >= t}, and the kernel streams sum_n |x_n - (t - 1)| to get it.
+# kappa sum_{x >= t} x + d #{x >= t}, and the kernel streams sum_n |x_n - (t - 1)| to get it, four
+# sorted samples x0 <= x1 <= x2 <= x3 at a time as the maximum of their five lines:
+# max(|S - 4c|, |Q - 2c| + P, D) with S their sum, Q = x1 + x2, P = x3 - x0, D = x2 + x3 - x0 - x1.
 # That sum also has an O(1) closed form from the cumulative counts and sums the same context holds
 # (the envelope mode returns the same S that way).
-PER_TERM_OP = "|x - c| summed exactly per (cell, sample), c = t - 1 the cell's integer threshold; not the 3-candidate phi"
+PER_TERM_OP = ("|x - c| summed exactly over every (cell, sample), four samples at a time, c = t - 1 the cell's "
+               "integer threshold; not the 3-candidate phi")
 GRID_SOURCE = os.path.join(ROOT, "paper_2607_16892_gb300", "csrc", "grid.cu")
 PROFILE = os.path.join(ROOT, "profiles", "k_grid_exact_regimes_k8_n2e5.md")
 LAUNCHES_PER_STEP = 7  # histogram, scan totals, scan, expand, quantile gather, grid, argmin finalise
@@ -212,7 +213,7 @@ def secondary_figures(kv, w, ctx, stream, sms, reps=2):
                                             f"{SM_MAX_MHZ_RECIPE:.0f} MHz"},
             "envelope": {"what": "O(1) per cell from cumulative counts and sums; not per term",
                          "cells": M * K * R * NL, "kernel_ms": env_ms, "cells_per_s": M * K * R * NL / (env_ms / 1e3)},
-            "exact_dual": {"what": "min over gamma >= 0 by bisection, O(1) per probe; not per term",
+            "exact_dual": {"what": "min over gamma >= 0 by a search over integer thresholds, O(1) per probe; not per term",
                            "cells": M * E * K * R, "kernel_ms": dual_ms, "cells_per_s": M * E * K * R / (dual_ms / 1e3)}}
 
 
@@ -436,10 +437,10 @@ def run_ours(args):
     peak_paper = sms * 128.0 / PAPER_FORM_LANE_OPS_PER_TERM * SM_MAX_MHZ_RECIPE * 1e6
     traffic, inst_per_term = profile_figures()
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": UNIT, "frac": achieved / peak,
-                "traffic": traffic, "kernel": "k_grid<EXACT> (FP32 outputs)",
+                "traffic": traffic, "kernel": "k_exact (FP32 outputs)",
                 "kernel_ms_mean": kernel_ms, "per_term_op": PER_TERM_OP,
-                "peak_basis": f"{sms} SMs x ({FMA_TERMS_PER_CLK_PER_SM:.0f} terms/clk/SM on packed "
-                              f"FP32 adds + {ALU_TERMS_PER_CLK_PER_SM:.0f} on integer sad) x {SM_MAX_MHZ_RECIPE:.0f} MHz",
+                "peak_basis": f"{sms} SMs x {TERMS_PER_CLK_PER_SM:.1f} terms/clk/SM (issue: 3.5 instructions per four "
+                              f"samples and cell) x {SM_MAX_MHZ_RECIPE:.0f} MHz",
                 "frac_survey_basis": achieved / peak_paper,
                 "survey_basis": f"{sms} SMs x 128 FP32 lanes / {PAPER_FORM_LANE_OPS_PER_TERM:.0f} lane-ops per term of "
                                 f"the 3-candidate phi (2 FMA, 2 max, 1 add) x {SM_MAX_MHZ_RECIPE:.0f} MHz = "

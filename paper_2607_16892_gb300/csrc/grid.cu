@@ -132,7 +132,7 @@ __device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
 // max(|u|, |v| + p, d)
 __device__ __forceinline__ float max3_abs(float u, float v, float p, float d) {
     float m;
-    asm("{\n\t.reg .f32 q;\n\tabs.f32 q, %1;\n\tmax.f32 %0, q, %2, %3;\n\t}" : "=f"(m) : "f"(u), "f"(fabsf(v) + p), "f"(d));
+    asm("{\n\t.reg .f32 q;\n\tabs.f32 q, %1;\n\tmax.f32 %0, %3, q, %2;\n\t}" : "=f"(m) : "f"(u), "f"(fabsf(v) + p), "f"(d));
     return m;
 }
 // max(w, 0); a NaN operand yields 0 (PTX max returns the non-NaN input).
@@ -799,9 +799,11 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
 // run on in 32-bit integer adds, on the pipe that has the room, and fold 256 times more rarely than
 // FP32 sums below 2^24 would.  (The maths need subnormals kept: no flush-to-zero.)
 //
-// 8 classes x 100,000 samples x 4096 r x 128 lam: 14.1 ms, 95 terms/clk/SM (pairs 15.9); the loop alone runs 97
-// to 99 in isolation, bound by register reads (23 operands for 8 terms) rather than by either pipe.  Also
-// measured there: -2c kept beside -4c instead of the FMA 14.5 (80 registers, 12 warps); (S, Q) as one packed
+// 8 classes x 100,000 samples x 4096 r x 128 lam: 13.64 ms, 98 terms/clk/SM (pairs 15.92); the loop alone runs at
+// 97 to 99 in isolation, bound by register reads (23 operands for 8 terms) and their banks rather than by
+// either pipe, so the order of operands counts: 13.65 to 14.05 over the six orders of the maximum's, 13.64
+// with the second load's cells ahead of the first's.  Also measured, with the maximum's operands as written
+// above (14.1 so): -2c kept beside -4c instead of the FMA 14.5 (80 registers, 12 warps); (S, Q) as one packed
 // operand against (-4c, -2c) of one cell 16.1; 8, 10 and 12 cells a warp 15.6, 15.5, 14.8.
 //
 // The count #{x >= t} comes from the class's cumulative counts; every sample then goes on its branch of
@@ -897,15 +899,15 @@ __global__ void __launch_bounds__(32 * kExactWarps, kExactBlocks) k_exact(const 
 #pragma unroll
         for (int p = 0; p < V / 2; p++) {
             unsigned a0, a1, b0, b1;
-            quad(va, p, a0, a1);
             quad(vb, p, b0, b1);
+            quad(va, p, a0, a1);
             acc[2 * p] += a0 + b0;
             acc[2 * p + 1] += a1 + b1;
         }
     };
     // `loads` loads (a multiple of kSeg) in segments of a fixed trip count, two loads at a time.  64 with 8 loads
-    // to an iteration run 14.1 ms on 8 classes x 100,000 samples x 4096 r x 128 lam, 16 with 4 14.6; unrolled in
-    // full, loads move up and registers spill (16: 22.8).
+    // to an iteration run 13.65 ms on 8 classes x 100,000 samples x 4096 r x 128 lam, 4 or 16 14.1; segments of 16 with
+    // 8 spill registers (15.1).
     auto segments = [&](const float4*& q, int loads, auto seg) {
         constexpr int kSeg = decltype(seg)::value, kUnroll = kSeg == 64 ? 8 : 4;
         const float4* stop = q + 32 * loads;
