@@ -571,7 +571,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     // FP32 and FP64 results come from the exact kernel whenever it applies (FP32: rounded).  Its sums
     // are integers, so it carries only the final combination's FP64 rounding: on 8 classes x 100,000
     // samples x 512 r x 128 lam it is within 1e-16 of the 64-bit result, as the native FP64 kernel is
-    // (6e-14 at 537,000 samples, where the exact kernel stays at 1e-16), in 1.85 ms against 320.7 ms.
+    // (6e-14 at 537,000 samples, where the exact kernel stays at 1e-16), in 1.8 ms against 320.7 ms.
     // The FP32-arithmetic and native FP64 kernels serve supports above 2^22, and native FP64 also
     // costs so large that a whole class's sum nears the end of the double range, where the two
     // combine their parts in different orders.

@@ -134,14 +134,16 @@ def test_exact_passes_over_the_samples(nl, monkeypatch):
     assert e.value.status == kvdro.KVDRO_ETIMEOUT
 
 
-@pytest.mark.parametrize("L", [1, 31, 4095, 4096, 32766, 32895, 32896, 65534, 65535, 70000, 1 << 20])
+@pytest.mark.parametrize("L", [1, 31, 511, 513, 4095, 4096, 32766, 32895, 32896, 40961, 65534, 65535, 70000, 1 << 20])
 @pytest.mark.parametrize("n", [1, 3, 127, 129, 4096, 4099, 70001])
 def test_sort_supports_and_sizes(L, n):
     """Supports on and around the histogram's shared bins (2 x 16448), the scan's tiles (4096) and the tiles up
     to which it needs no pass of totals (16), class sizes around the expansion's steps and tiles, runs longer
-    and shorter than a lane's four positions, and a class whose offset is not a multiple of four."""
+    and shorter than a lane's four positions, a class whose offset is not a multiple of four, and one long run
+    among single samples (tiles laid out in shared memory: 512 to 40960 bins)."""
     rng = np.random.default_rng(L + n)
-    x = [rng.integers(0, L + 1, n), np.minimum(rng.geometric(0.3, n + 1), L), np.full(n, L)]
+    x = [rng.integers(0, L + 1, n), np.minimum(rng.geometric(0.3, n + 1), L), np.full(n, L),
+         np.concatenate([np.full(n, L // 3), rng.integers(0, L + 1, n // 2 + 1)])]
     w = make(x, L, [0, L], [1.0], [0.0], 1.0, 1.0)
     got = run(w, kvdro.KVDRO_ENVELOPE, outputs=("sorted", "fhat", "S"))
     assert np.array_equal(got["sorted"], np.concatenate([np.sort(v) for v in x]))
