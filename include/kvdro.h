@@ -62,10 +62,9 @@ typedef enum {
                             L_max * N passes 1e300) they are the KVDRO_EXACT results, whose sums
                             carry no rounding; otherwise per-term arithmetic and sums in FP64 */
     KVDRO_EXACT = 2,     /* per term, exact integer arithmetic on exact integer thresholds
-                            (|x + 1 - t| summed exactly, half of the cells in packed FP32 adds,
-                            half in integer absolute differences); exact integer counts and
-                            sums combined once per cell in FP64, so results carry FP64 rounding
-                            only.  Needs every L_max <= 2^22. */
+                            (|x + 1 - t| summed exactly, four samples at a time); exact integer
+                            counts and sums combined once per cell in FP64, so results carry
+                            FP64 rounding only.  Needs every L_max <= 2^22. */
     KVDRO_ENVELOPE = 3   /* not per term: each cell's sample sum from the sorted samples'
                             cumulative counts and sums at its exact threshold, O(1) per cell,
                             FP64 outputs with FP64 rounding only */
@@ -113,11 +112,7 @@ int kvdro_quantiles(kvdro_ctx* ctx, int32_t F, const double* fractiles, int32_t*
  * KVDRO_FP32 and double for the other modes.
  *   R, r       host int32[R], 1 <= R <= 2^20; every r must satisfy L_in_k <= r <= L_in_k + L_k for
  *              every class (the reservation domain of Sec. 2.2).
- *   NL, lam    host double[NL], finite, >= 0; 1 <= NL <= 256 (128 for KVDRO_FP64).  The exact
- *              kernel (KVDRO_EXACT, and FP32 and FP64 as above) takes 128 lam values
- *              per launch; a larger grid runs as consecutive launches over blocks of 128 with the
- *              running minimum in context scratch (12 bytes per (regime, eps, class, r), at most
- *              256 MB at a time).
+ *   NL, lam    host double[NL], finite, >= 0; 1 <= NL <= 256 (128 for KVDRO_FP64).
  *   E, eps     host double[E], finite, >= 0; 1 <= E <= 64.
  *   M, c_p,c_w host double[M] each, finite, >= 0; 1 <= M <= 65536.
  * Outputs (each may be NULL to skip it; host or device).  With M > 1, host S, cost and lam_idx
@@ -141,10 +136,10 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
  * radius, class and reservation, min over gamma >= 0 of gamma*eps + S(eta, gamma) (App. A,
  * eq. app_kantorovich; the value of the epigraph LP of eq. app_lp, which equals the worst case
  * over the Wasserstein ball by the strong duality of App. A Step 2).  The objective is convex
- * and piecewise linear in gamma with its minimiser in [0, max(c_p, c_w)]; the library bisects on
- * its right derivative over the ordered bit patterns of the nonnegative doubles (at most 63
- * steps, down to two adjacent doubles at any scale) with every evaluation O(1) from the sorted
- * samples' cumulative counts and sums, so results carry FP64 rounding only.  The result is
+ * and piecewise linear in gamma with its minimiser in [0, max(c_p, c_w)]; the library
+ * searches on the sign of its right derivative, over the integer thresholds between which it is
+ * constant and then over the ordered bit patterns of the nonnegative doubles (down to two adjacent
+ * doubles at any scale), with every evaluation O(1) from the sorted samples' cumulative counts and sums, so results carry FP64 rounding only.  The result is
  * never below the empirical cost (1/N) sum_n Q(eta, x_n), computed exactly from integer sums:
  * that bound holds at every gamma (App. A) and is the value itself at eps = 0.
  * Arguments as kvdro_eval_grid; outputs (each may be NULL; host or device):
@@ -186,8 +181,9 @@ int kvdro_last_grid_ms(kvdro_ctx* ctx, float* ms);
  * Calls share the array: it keeps the last call's contents (the call clears what must start at
  * zero), and calls whose GPU work overlaps in time race on it -- serialise them, e.g. on one
  * stream.  A problem whose scratch would exceed the array (about 12 bytes per sample plus
- * 4 bytes per support point and 8 bytes per (regime, radius, class) row, and with more than 128
- * lam values 12 bytes per (regime, radius, class, r) cell) is rejected with KVDRO_EINVAL and a
+ * 4 bytes per support point and 8 bytes per (regime, radius, class) row; with more than 128 lam
+ * values and every L_max <= 2^22 the limit also counts 12 bytes per (regime, radius, class, r) cell,
+ * which the call does not use) is rejected with KVDRO_EINVAL and a
  * message.
  *
  * Arguments are those of kvdro_load_samples and kvdro_eval_grid with precision KVDRO_FP32,
