@@ -29,7 +29,7 @@ constexpr int kExpandThreads = 256;
 constexpr int64_t kExpandTile = 4096;  // sorted positions per expansion block
 // Tiles whose positions lie among at least kSparseBins bins lay their runs out in shared memory instead of
 // searching: 1.6 M samples of support 32768 in 24 us instead of 36 (search; 35 with a limit of 16384 bins), 3,000
-// of support 8192 in 10 instead of 18, 32 M in 51 instead of 57.  From 256, 512 or 1024 bins on the same within
+// of support 8192 in 10 instead of 18, 32 M in 52 instead of 57.  From 256, 512 or 1024 bins on the same within
 // 2 us.  Past kSparseMost the bins' loads outweigh the search (16 M of support 131072: 73 against 63).
 constexpr int kSparseBins = 512;
 constexpr int kSparseMost = 40960;
@@ -259,7 +259,7 @@ __device__ __forceinline__ int32_t value_at(const int32_t* C, int32_t lo, int32_
 // position range (recorded by the scan).  Where they are the same -- runs of equal samples are long where
 // samples are many -- that is all; up to 31 bins apart each lane finds its first position among the run
 // ends that the lanes hold, and otherwise by a search of its own: no shared memory, no
-// barrier.  16-byte stores: 32 M samples in 51 us (5.0 TB/s of stores); a running maximum over run
+// barrier.  16-byte stores: 32 M samples in 52 us (4.9 TB/s of stores); a running maximum over run
 // starts marked in shared memory took 86, a search per thread 75.
 __global__ void __launch_bounds__(kExpandThreads) k_expand(SortArgs a) {
     constexpr int kWarps = kExpandThreads / 32, kSteps = (int)kExpandTile / 128 / kWarps;  // per warp
