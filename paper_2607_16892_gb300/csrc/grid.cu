@@ -286,8 +286,9 @@ __host__ __device__ inline ExactSmem exact_smem(int rows, int NL, int E, int til
 // within [v (1 - 2.6 x 2^-23), v (1 + 2^-23)], so a lam attaining the minimum has v' at most
 // (1 + 2^-20) times the smallest v', and only those values -- one as a rule -- are formed in FP64, in
 // ascending order, except one whose lam and S are both no smaller than the best's, which cannot be
-// below it.  Where the floats do not hold (a negative S, magnitudes above 2^100, a minimum below
-// 2^-80 that the cut of smaller parts to zero could matter to) every value is formed.
+// below it.  Where the floats do not hold every value is formed: a negative S, magnitudes above 2^100, a
+// nonzero lam or eps below 2^-100 (the other factor may be so large that their product decides), or
+// a minimum below 2^-80, which an S cut to zero, below 2^-100, could matter to.
 constexpr float kLamWindow = 1.f + 0x1p-19f;
 constexpr float kLamFloor = 0x1p-80f;
 
@@ -298,6 +299,13 @@ __device__ __forceinline__ float cut(double v, bool& ok) {
     const unsigned e = (unsigned)((unsigned long long)b >> 52);  // sign and exponent
     ok = ok && e <= 1023u + 100u;
     return e >= 1023u - 100u ? narrow(b) : 0.f;
+}
+// The same for a factor, lam or eps: `ok` is also cleared for a nonzero value below 2^-100.
+__device__ __forceinline__ float cut_factor(double v, bool& ok) {
+    const long long b = dbits(v);
+    if ((b << 1) == 0) return 0.f;
+    ok = ok && b > 0 && narrowable(b);
+    return narrow(b);
 }
 
 struct LamMin {
@@ -393,7 +401,7 @@ struct LamRows {
     const float *Sf, *lamf;
     int stride, stride_f;
     int rows, NL;
-    bool floats;  // every lam and S is >= 0 and small enough for its float
+    bool floats;  // every lam and S is >= 0 and its float holds
 };
 
 // The end of every grid kernel, by all threads of the CTA (whole warps): for each (r, eps) pair the minimum
@@ -418,7 +426,7 @@ __device__ __forceinline__ void lam_min_epilogue(const GridArgs& a, const LamRow
         const float* Sf = x.Sf + rl * x.stride_f;
         const double eps = x.eps[e];
         bool fast = x.floats;
-        const float ef = cut(eps, fast);
+        const float ef = cut_factor(eps, fast);
         float m1 = INFINITY, m2 = INFINITY;
         int j1 = 0;
         for (int q = g; q < n4; q += G) {
@@ -771,7 +779,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     // the floats past the last lam value; `ok` over the CTA
     for (int i = tid; i < a.RG * TR * 4; i += blockDim.x)
         if (a.NL + (i & 3) < four(a.NL)) s_Sf[(i >> 2) * lay.stride_f + a.NL + (i & 3)] = INFINITY;
-    for (int j = tid; j < four(a.NL); j += blockDim.x) s_lamf[j] = j < a.NL ? cut(s_lam[j], ok) : 0.f;
+    for (int j = tid; j < four(a.NL); j += blockDim.x) s_lamf[j] = j < a.NL ? cut_factor(s_lam[j], ok) : 0.f;
     const bool floats = __syncthreads_and(ok);
     const LamRows rows = {s_S, s_lam, s_eps, s_Sf, s_lamf, NLpad, lay.stride_f, min(a.RG * TR, a.R - r_cta0), a.NL, floats};
     lam_min_epilogue<P == Prec::F32>(a, rows, r_cta0, m, k);
@@ -1022,7 +1030,7 @@ __global__ void __launch_bounds__(32 * kExactWarps, kExactBlocks) k_exact(const 
         }
         for (int i = tid; i < rows * 4; i += blockDim.x)
             if (NL + (i & 3) < four(NL)) s_Sf[(i >> 2) * lay.stride_f + NL + (i & 3)] = INFINITY;
-        for (int j = tid; j < four(NL); j += blockDim.x) s_lamf[j] = j < NL ? cut(s_lam[j], ok) : 0.f;
+        for (int j = tid; j < four(NL); j += blockDim.x) s_lamf[j] = j < NL ? cut_factor(s_lam[j], ok) : 0.f;
     }
     if (!ok) s_bad = 1;
     __syncthreads();
@@ -1140,7 +1148,7 @@ __global__ void __launch_bounds__(kEnvThreads) k_envelope(const GridArgs a) {
         s_kap[i] = kap;
         if (dbits(l) >= dbits(cp) && dbits(l) >= dbits(cw)) atomicMin(&s_first_sat, i);
         if (i > 0 && !(dbits(a.lam[i - 1]) <= dbits(l))) s_unsorted = 1;
-        s_lamf[i] = cut(l, ok);
+        s_lamf[i] = cut_factor(l, ok);
         s_muf[i] = cut(mu, ok);
         s_kapf[i] = cut(kap, ok);
     }

@@ -149,3 +149,28 @@ def test_sort_supports_and_sizes(L, n):
     assert np.array_equal(got["sorted"], np.concatenate([np.sort(v) for v in x]))
     want = np.stack([[v.mean(), (L - v).mean()] for v in x])[None, :, :, None]  # at r = 0 and L, lam = 1 = c_p = c_w
     np.testing.assert_allclose(got["S"], want, rtol=1e-12)
+
+
+MODES = {"fp32": kvdro.KVDRO_FP32, "fp64": kvdro.KVDRO_FP64, "exact": kvdro.KVDRO_EXACT, "envelope": kvdro.KVDRO_ENVELOPE}
+
+
+def _tiny_factor_cases(L):
+    """One factor of lam * eps below 2^-100, the other so large that the product decides the minimum."""
+    rng = np.random.default_rng(8)
+    at = np.full(40, 100)
+    return [make([at], L, [L // 3, 2 * L // 3], [0.0, 7e-31], [1e3, 1e6], 1e-26, 1e-26),
+            make([at], L, [L // 3, 2 * L // 3], [1e-32, 7e-31, 7.8e-31, 7.9e-31], [0.0, 1e2, 1e3, 1e6], [1e-26, 2e-26], [1e-26, 1e-26]),
+            make([rng.integers(0, L + 1, 300)], L, [L // 2], [9.9995, 1e30], [7e-31], 10.0, 1.0),
+            make([rng.integers(0, L + 1, 300)], L, [L // 4, L // 2], np.concatenate([np.linspace(9.99, 10.0, 30), [1e27, 1e30]]),
+                 [0.0, 1e-300, 7e-31, 7.9e-31], 10.0, 1.0)]
+
+
+@pytest.mark.parametrize("mode,L", [("fp32", 900), ("fp64", 900), ("exact", 900), ("envelope", 900),
+                                    ("fp32", (1 << 22) + 3), ("fp64", (1 << 22) + 3), ("noalloc", 900)])
+def test_products_of_a_tiny_and_a_large_factor(mode, L):
+    """A lam or a radius that a float look at the minimum takes for zero still counts through its product
+    with the other, in every kernel: exact, FP32 and FP64 arithmetic, envelope, and the allocation-free call."""
+    from tests.test_zz_no_alloc import _noalloc
+    for w in _tiny_factor_cases(L):
+        got = _noalloc(w) if mode == "noalloc" else run(w, MODES[mode])
+        compare_full(w, got, O.solve(w), "fp32" if mode in ("fp32", "noalloc") else "fp64")
