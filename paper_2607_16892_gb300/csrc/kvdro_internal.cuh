@@ -201,11 +201,12 @@ __device__ __forceinline__ float narrow(long long b) {
     return __uint_as_float((unsigned)((b & 0x7fffffffffffffffll) >> 29) - (896u << 23));
 }
 
-// Order key of a double: equal for equal values (-0 is taken as +0) and ordered as the values are
-// for every non-NaN double.
+// Order key of a double: equal for equal values (-0 is taken as +0), ordered as the values are, and above them
+// all for a NaN (a sum past the double range, whose own sign bit is set), which is no minimum.
 __device__ __forceinline__ long long order_key(double v) {
     long long b = __double_as_longlong(v);
     if (b == (long long)0x8000000000000000ull) b = 0;
+    if (((unsigned long long)b << 1) > 0xffe0000000000000ull) return 0x7fffffffffffffffll;
     return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 

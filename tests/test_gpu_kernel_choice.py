@@ -174,3 +174,30 @@ def test_products_of_a_tiny_and_a_large_factor(mode, L):
     for w in _tiny_factor_cases(L):
         got = _noalloc(w) if mode == "noalloc" else run(w, MODES[mode])
         compare_full(w, got, O.solve(w), "fp32" if mode in ("fp32", "noalloc") else "fp64")
+
+
+@pytest.mark.parametrize("mode", ["fp32", "fp64", "exact", "envelope"])
+def test_sums_past_the_double_range_leave_the_finite_ones(mode):
+    """c_p so large that the class sums of small multipliers pass the double range: their S is infinite or not
+    a number, and the minimum over lam is taken over the others, here from lam = c_p on, where 15 of the 500
+    samples lie 1 to 5 above r."""
+    x = np.concatenate([np.full(485, 10), np.repeat(np.arange(891, 896), 3)])
+    w = make([x], 900, [890], [0.0, 1e290, 1e305, 2e305], [0.0], 1e305, 0.0)
+    got = run(w, MODES[mode], outputs=("cost", "lam_idx", "r_idx", "min_cost"))
+    assert got["lam_idx"].tolist() == [[[[2]]]] and got["r_idx"].tolist() == [[[0]]]
+    if mode != "fp32":  # beyond FP32
+        np.testing.assert_allclose([got["cost"].item(), got["min_cost"].item()], 1e305 / 500 * 45, rtol=1e-12)
+
+
+def test_dual_values_past_the_double_range_are_not_the_empirical_cost():
+    """The same samples at a radius that puts the minimiser at gamma = 0, where g = 1e306 and its class sum is past
+    the double range: the result is no number, or the value, but not the empirical cost of 9e303 below it."""
+    x = np.concatenate([np.full(485, 10), np.repeat(np.arange(891, 896), 3)])
+    ctx = kvdro.kvdro_create(0)
+    try:
+        kvdro.kvdro_load_samples(ctx, 1, np.array([0, 500]), torch.from_numpy(x.astype(np.int32)).cuda(), [900])
+        cost = np.empty((1, 1, 1, 1))
+        kvdro.kvdro_eval_dual(ctx, 1, [890], 1, [1e6], 1, [1e305], [0.0], cost=cost)
+    finally:
+        kvdro.kvdro_destroy(ctx)
+    assert np.isnan(cost.item()) or abs(cost.item() - 1e306) <= 1e-12 * 1e306
