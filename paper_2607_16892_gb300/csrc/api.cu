@@ -552,11 +552,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
                  : precision == KVDRO_EXACT ? Prec::EXACT : Prec::ENVELOPE;
     const int32_t maxNL = P == Prec::F64 ? kMaxNLf64 : kMaxNLf32;
     bool exact_ok = true;  // every class's support fits the exact kernel's integer sums
-    int32_t max_L = 0;
-    for (int32_t k = 0; k < ctx->K; k++) {
-        exact_ok = exact_ok && ctx->L[k] <= kvdro::kExactMaxL;
-        max_L = std::max(max_L, ctx->L[k]);
-    }
+    for (int32_t k = 0; k < ctx->K; k++) exact_ok = exact_ok && ctx->L[k] <= kvdro::kExactMaxL;
     if (P == Prec::EXACT && !exact_ok)
         return fail(ctx, KVDRO_EINVAL, "KVDRO_EXACT needs L_max <= 2^22 for every class");
     if (R < 1 || R > kMaxR) return fail(ctx, KVDRO_EINVAL, "R = %d outside [1, 2^20]", R);
@@ -585,7 +581,7 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     if (!g.ok) return fail(ctx, KVDRO_ECUDA, "cannot select device %d", ctx->device);
     ctx->last_stream = s;
 
-    const kvdro::GridShape shape = kvdro::grid_shape(KP, R, NL, E, max_L, (int64_t)M * ctx->K, ctx->sms);
+    const kvdro::GridShape shape = kvdro::grid_shape(KP, R, NL, E, ctx->K, M, ctx->sms);
 
     // Grid parameters in one upload.
     const size_t gbytes = align_up((size_t)R * 4, 8) + 8 * ((size_t)NL + E + 2 * (size_t)M);

@@ -1244,7 +1244,7 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
 // holds as many as the others (13 to 16 warps take the same time), and fewer per scheduler run at a lower
 // rate: 5 classes x 1001 r x 200 lam x 3 regimes 2.27 ms in one pass of 13 warps, 1.90 in four passes of 16
 // (2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
-GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int64_t classes, int sms) {
+GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int32_t K, int64_t classes, int sms) {
     constexpr int kCells = kExactWarps * kExactV;
     GridShape best, sh;
     sh.variant = 3;
@@ -1259,6 +1259,7 @@ GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int64_t classes, int sms
         const int warps = (tiles + sh.passes - 1) / sh.passes;
         sh.threads = 32 * warps;
         sh.r_blocks = (R + rows - 1) / rows;
+        if ((int64_t)K * sh.r_blocks > 0x7fffffffLL) continue;  // a launch holds one regime's CTAs (four passes always do)
         // 96 KB of ring: three chunks of 8192 samples (6144 measured 1 % slower, 4096 3 %); smaller chunks where
         // the cells need the room
         sh.stages = kExactStages;
@@ -1279,7 +1280,8 @@ GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int64_t classes, int sms
     return best;
 }
 
-GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, int64_t classes, int sms) {
+GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t K, int32_t M, int sms) {
+    const int64_t classes = (int64_t)M * K;
     if (p == Prec::ENVELOPE) {
         GridShape sh;
         sh.variant = 4;
@@ -1291,8 +1293,7 @@ GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, in
         return sh;
     }
     if (p == Prec::F64) return shape_for<CfgF64>(2, R, NL, E);
-    if (p == Prec::EXACT)
-        return exact_shape(R, NL, E, classes, sms);
+    if (p == Prec::EXACT) return exact_shape(R, NL, E, K, classes, sms);
     if (NL <= kWarpsTarget * CfgF32::TL) return shape_for<CfgF32>(0, R, NL, E);
     return shape_for<CfgF32Wide>(1, R, NL, E);
 }

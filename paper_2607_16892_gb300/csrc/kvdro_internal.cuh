@@ -130,8 +130,8 @@ struct GridShape {
     int r_blocks;      // CTAs per (m, k)
     size_t smem;
 };
-// max_L: largest support; classes: (regime, class) pairs that the request evaluates; sms: of the device
-GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t max_L, int64_t classes, int sms);
+// K, M: classes and regimes that the request evaluates; sms: of the device
+GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t K, int32_t M, int sms);
 cudaError_t sm_count(int* sms);  // of the current device (sort.cu)
 cudaError_t grid_prepare(Prec p);             // per-device attribute setup of every variant of p
 // Launches over regimes [a.m0, a.m0 + a.m_count); fills a.LT, a.RG, a.r_blocks from `sh`.

@@ -190,11 +190,7 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     const size_t o_pairs = take((size_t)pair_total * 8);
     const size_t o_keys = take((size_t)rows * 8);
     bool exact_ok = true;
-    int32_t max_L = 0;
-    for (int32_t k = 0; k < K; k++) {
-        exact_ok = exact_ok && L_max[k] <= kvdro::kExactMaxL;
-        max_L = L_max[k] > max_L ? L_max[k] : max_L;
-    }
+    for (int32_t k = 0; k < K; k++) exact_ok = exact_ok && L_max[k] <= kvdro::kExactMaxL;
     // The documented limit counts 12 bytes per (regime, radius, class, r) cell above 128 lam values.
     const size_t counted_cells = exact_ok && NL > 128 ? (size_t)rows * R : 0;
     (void)take(counted_cells * 8), (void)take(counted_cells * 4);
@@ -221,7 +217,7 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
         return report(err, err_len, KVDRO_ECUDA, "reading the device's SM count failed");
     }
     const kvdro::Prec kp = exact_ok ? kvdro::Prec::EXACT : kvdro::Prec::F32;
-    const kvdro::GridShape shape = kvdro::grid_shape(kp, R, NL, E, max_L, (int64_t)M * K, sms);
+    const kvdro::GridShape shape = kvdro::grid_shape(kp, R, NL, E, K, M, sms);
     const int64_t per_m = (int64_t)K * shape.r_blocks;
     const int64_t m_step = per_m > 0x7fffffffLL ? 1 : 0x7fffffffLL / per_m;
     char* S = static_cast<char*>(base);
@@ -306,7 +302,7 @@ extern "C" int kvdro_eval_grid_noalloc(int32_t K, const int64_t* offsets, const 
     sa.sumx = reinterpret_cast<int64_t*>(S + o_sumx);
     sa.sorted = reinterpret_cast<int32_t*>(S + o_sorted);
     sa.staged = S + o_pairs;  // of 8 bytes a sample as quads take 4
-    sa.quads = max_L <= kvdro::kExactMaxL;
+    sa.quads = exact_ok;
     sa.err = reinterpret_cast<int32_t*>(S + o_err);
     sa.tile_tot = reinterpret_cast<int64_t*>(S + o_tiles);
     sa.tile_lo = reinterpret_cast<int32_t*>(S + o_tile_lo);
