@@ -379,7 +379,8 @@ __device__ __forceinline__ void finalize_row(const FinalizeArgs& a, int64_t i, i
 
 // The last of the (regime, class)'s CTAs to get here finalises its rows: a launch of its own took 4 us of
 // the smallest grids' 34.  Every CTA's outputs and keys are ordered before its count (barrier, fence,
-// atomic), the last one's reads after.  Kept out of line: its registers are no concern of the sample loops.
+// atomic), the last one's reads after.  A CTA that gave up a wait counts too, so rows are finalised whatever came of
+// them.  Kept out of line: its registers are no concern of the sample loops.
 template <bool F32>
 __device__ __noinline__ void finish_rows(const GridArgs& a, int m, int k) {
     __shared__ int s_last;
@@ -746,6 +747,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
                 (void)mbar_wait_bounded(smem_u32(&full[c % C::STAGES]), (uint32_t)((c / C::STAGES) & 1), a.wait_ns);
         }
         __syncthreads();
+        if (a.done) finish_rows<P == Prec::F32>(a, m, k);
         return;
     }
 
@@ -999,6 +1001,8 @@ __global__ void __launch_bounds__(32 * kExactWarps, kExactBlocks) k_exact(const 
             }
         }
         __syncthreads();
+        if (a.done && a.f32_out) finish_rows<true>(a, m, k);
+        else if (a.done) finish_rows<false>(a, m, k);
         return;
     }
     bool ok = true;

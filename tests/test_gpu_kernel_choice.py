@@ -201,3 +201,29 @@ def test_dual_values_past_the_double_range_are_not_the_empirical_cost():
     finally:
         kvdro.kvdro_destroy(ctx)
     assert np.isnan(cost.item()) or abs(cost.item() - 1e306) <= 1e-12 * 1e306
+
+
+@pytest.mark.parametrize("mode,L", [("fp32", 1000), ("exact", 1000), ("fp32", (1 << 22) + 1), ("fp64", (1 << 22) + 1)])
+def test_rows_after_a_wait_that_runs_out(mode, L, monkeypatch):
+    """With the first chunk's copy left out every CTA of the exact kernel, and above 2^22 of the FP32- and
+    FP64-arithmetic kernels, gives up: no r was evaluated, and r_idx says so (-1) whether the rows are
+    finalised by the last CTA or by a launch.  With the second, the classes of one chunk have their results."""
+    rng = np.random.default_rng(3)
+    w = make([rng.integers(0, 900, 20000), rng.integers(0, 900, 77)], L, [10, 200, 600], [0.5, 5.0], [0.0, 10.0], 10.0, 1.0)
+    ref = O.solve(w)
+    for skip in (0, 1):
+        monkeypatch.setenv("KVDRO_TEST_SKIP_CHUNK", str(skip))
+        ctx = kvdro.kvdro_create(0)
+        monkeypatch.delenv("KVDRO_TEST_SKIP_CHUNK")
+        try:
+            kvdro.kvdro_load_samples(ctx, w.K, w.offsets, torch.from_numpy(w.samples).cuda(), w.L, w.L_in)
+            r_idx = torch.full((1, 2, 2), 7, dtype=torch.int32, device="cuda")
+            kvdro.kvdro_eval_grid(ctx, MODES[mode], 3, w.r, 2, w.lam, 2, w.eps, 1, w.cp, w.cw, r_idx=r_idx)
+            with pytest.raises(kvdro.KvdroError) as e:
+                kvdro.kvdro_sync(ctx)
+            assert e.value.status == kvdro.KVDRO_ETIMEOUT
+        finally:
+            kvdro.kvdro_destroy(ctx)
+        got = r_idx.cpu().numpy()[0]
+        assert np.all(got[:, 0] == -1)
+        assert np.array_equal(got[:, 1], ref["r_idx"][0, :, 1] if skip else [-1, -1])
