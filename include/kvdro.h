@@ -177,7 +177,8 @@ int kvdro_last_grid_ms(kvdro_ctx* ctx, float* ms);
  * Instead of a context, it works in one static device array of KVDRO_NOALLOC_SCRATCH_BYTES
  * bytes, defined in the library; every GPU that loads the library holds that array until the
  * process exits.  The first call on a device (with that device current) resolves the array's
- * device address and sets a kernel attribute; make that first call before any stream capture.
+ * device address, sets kernel attributes and loads every kernel that a call can choose; make that
+ * first call while device memory is free for the kernels' code and before any stream capture.
  * Calls share the array: it keeps the last call's contents (the call clears what must start at
  * zero), and calls whose GPU work overlaps in time race on it -- serialise them, e.g. on one
  * stream.  A problem whose scratch would exceed the array (about 12 bytes per sample plus

@@ -1330,8 +1330,10 @@ cudaError_t grid_prepare(Prec p) {
         for (int nl = 1; nl <= 256; nl++) most = std::max(most, env_smem(env_rows(nl, 1 << 20, 1 << 20, 1), nl, 64).total);
         return allow_smem((const void*)k_envelope, most);
     }
-    const cudaError_t e = prepare<CfgF32>();
-    return e == cudaSuccess ? prepare<CfgF32Wide>() : e;
+    cudaFuncAttributes at;
+    cudaError_t e = prepare<CfgF32>();
+    if (e == cudaSuccess) e = prepare<CfgF32Wide>();
+    return e == cudaSuccess ? cudaFuncGetAttributes(&at, (const void*)k_finalize<true>) : e;
 }
 
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s) {

@@ -133,7 +133,7 @@ struct GridShape {
 // K, M: classes and regimes that the request evaluates; sms: of the device
 GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t K, int32_t M, int sms);
 cudaError_t sm_count(int* sms);  // of the current device (sort.cu)
-cudaError_t grid_prepare(Prec p);             // per-device attribute setup of every variant of p
+cudaError_t grid_prepare(Prec p);  // per-device attributes of every variant of p, and F32's finalisation loaded
 // Launches over regimes [a.m0, a.m0 + a.m_count); fills a.LT, a.RG, a.r_blocks from `sh`.
 cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s);
 cudaError_t launch_finalize(Prec p, const FinalizeArgs& a, cudaStream_t s);
@@ -146,6 +146,7 @@ struct Fill {
     uint32_t value;
 };
 bool setup_fits(size_t bytes);
+cudaError_t setup_prepare();  // loads every variant on the current device
 cudaError_t launch_setup(const void* payload, size_t bytes, void* dst, const Fill& f0, const Fill& f1, cudaStream_t s);
 
 // dual.cu: exact minimisation over gamma >= 0 per (regime, radius, class, reservation)

@@ -78,8 +78,9 @@ int report(char* err, int32_t err_len, int code, const char* msg) {
     return code;
 }
 
-// Once per device, with that device current: resolve the scratch's device address and raise the
-// grid kernel's dynamic shared-memory limit.
+// Once per device, with that device current: resolve the scratch's device address, raise the grid kernels'
+// dynamic shared-memory limit, and load what a first call may not launch -- the parameters' size chooses
+// among the setup launches -- since CUDA otherwise loads a kernel, into device memory, when it first runs.
 int setup_device(int dev, void** out, char* err, int32_t err_len) {
     if (dev < 0 || dev >= kMaxDevices) return report(err, err_len, KVDRO_EINVAL, "device ordinal out of range");
     std::lock_guard<std::mutex> lock(g_setup_mu);
@@ -90,9 +91,11 @@ int setup_device(int dev, void** out, char* err, int32_t err_len) {
             cudaGetLastError();
             return report(err, err_len, KVDRO_ECUDA, "cudaGetSymbolAddress of the static scratch failed");
         }
-        if (kvdro::grid_prepare(kvdro::Prec::F32) != cudaSuccess || kvdro::grid_prepare(kvdro::Prec::EXACT) != cudaSuccess) {
+        cudaFuncAttributes at;
+        if (kvdro::grid_prepare(kvdro::Prec::F32) != cudaSuccess || kvdro::grid_prepare(kvdro::Prec::EXACT) != cudaSuccess ||
+            kvdro::setup_prepare() != cudaSuccess || cudaFuncGetAttributes(&at, (const void*)k_noalloc_meta) != cudaSuccess) {
             cudaGetLastError();
-            return report(err, err_len, KVDRO_ECUDA, "setting the grid kernel's shared-memory limit failed");
+            return report(err, err_len, KVDRO_ECUDA, "preparing the kernels failed");
         }
         g_scratch_addr[dev] = p;
     }

@@ -3,6 +3,7 @@
 // launch of their own and a switch between the copy and the compute engines (about 4 us a call together),
 // and the staging buffer has to be waited for before the next call may fill it.
 #include <cstring>
+#include <initializer_list>
 
 #include "kvdro_internal.cuh"
 
@@ -38,6 +39,13 @@ cudaError_t launch(const void* payload, size_t bytes, void* dst, const Fill& f0,
 }
 
 }  // namespace
+
+cudaError_t setup_prepare() {
+    cudaFuncAttributes at;
+    for (const void* kernel : {(const void*)k_setup<2048>, (const void*)k_setup<4032>, (const void*)k_setup<16384>})
+        if (const cudaError_t e = cudaFuncGetAttributes(&at, kernel)) return e;
+    return cudaSuccess;
+}
 
 bool setup_fits(size_t bytes) { return bytes <= 16384; }
 

@@ -10,6 +10,9 @@ one above).  This file is collected last so that a stop-at-first-failure run has
 every other test.
 """
 
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -130,3 +133,62 @@ def test_noalloc_reports_a_wait_that_runs_out(monkeypatch):
     assert e.value.status == kvdro.KVDRO_ETIMEOUT and "gave up waiting" in str(e.value)
     monkeypatch.delenv("KVDRO_TEST_SKIP_CHUNK")
     compare_full(w, _noalloc(w), O.solve(w), "fp32")
+
+
+# The library's sources as one module, whose functions and their state the driver lists without loading them.
+LOADED = r"""
+#include "setup.cu"
+#include "sort.cu"
+#include "grid.cu"
+#include "noalloc.cu"
+#include <cuda.h>
+#include <vector>
+__global__ void anchor() {}
+int main() {
+    const int64_t off[2] = {0, 100};
+    const int32_t L = 50, r = 3;
+    const double one = 1.0;
+    int32_t* x;
+    float* cost;
+    cudaMalloc(&x, 400);
+    cudaMemset(x, 0, 400);
+    cudaMalloc(&cost, 4);
+    char err[200];
+    if (kvdro_eval_grid_noalloc(1, off, x, &L, nullptr, 1, &r, 1, &one, 1, &one, 1, &one, &one, cost, nullptr, nullptr, nullptr,
+                                nullptr, nullptr, err, 200)) {
+        printf("%s\n", err);
+        return 1;
+    }
+    cudaFunction_t f;
+    CUmodule m;
+    unsigned n = 0;
+    if (cudaGetFuncBySymbol(&f, (const void*)anchor) || cuFuncGetModule(&m, (CUfunction)f) || cuModuleGetFunctionCount(&n, m)) return 2;
+    std::vector<CUfunction> all(n);
+    if (cuModuleEnumerateFunctions(all.data(), n, m)) return 3;
+    for (CUfunction g : all) {
+        const char* name;
+        CUfunctionLoadingState s;
+        if (cuFuncGetName(&name, g) || cuFuncIsLoaded(&s, g)) return 4;
+        printf("%d %s\n", (int)s, name);
+    }
+    return 0;
+}
+"""
+
+
+def test_the_first_call_loads_every_kernel_that_a_later_one_may_choose(tmp_path):
+    """CUDA loads a kernel's code, into device memory, when it is first used: after one small call without row
+    outputs none is left that a call with more parameters, more lam values, a larger support or row
+    outputs runs."""
+    from paper_2607_16892_gb300 import build as kbuild
+    src, exe = tmp_path / "loaded.cu", str(tmp_path / "loaded")
+    src.write_text(LOADED)
+    subprocess.run([kbuild.nvcc(), *kbuild.ARCH, "-std=c++17", "-I", os.path.join(kbuild.ROOT, "include"), "-I", kbuild.CSRC,
+                    str(src), "-o", exe, "-lcuda"], check=True, capture_output=True, timeout=300)
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=120, env={**os.environ, "CUDA_MODULE_LOADING": "LAZY"})
+    assert out.returncode == 0, (out.returncode, out.stdout, out.stderr)
+    state = {name: int(s) for s, name in (line.split() for line in out.stdout.splitlines())}
+    for part, count in (("k_setup", 3), ("k_noalloc_meta", 1), ("k_histogram", 1), ("k_scan_totals", 1), ("k_scan_apply", 1),
+                        ("k_expand", 1), ("k_exact", 1), ("k_finalizeILb1E", 1), ("k_gridINS0_7GridCfgILNS_4PrecE0E", 2)):
+        mine = {n: s for n, s in state.items() if part in n}
+        assert len(mine) == count and all(s == 1 for s in mine.values()), (part, mine)
