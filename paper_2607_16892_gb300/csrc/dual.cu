@@ -93,7 +93,7 @@ __device__ __forceinline__ double crossing(const Cell& c, int v, bool nu1, bool 
 }
 
 __global__ void __launch_bounds__(kDualThreads, 6) k_dual(const DualArgs a) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t total = (int64_t)a.M * a.E * a.K * a.R;
     const bool valid = i < total;
     int64_t t = valid ? i : total - 1;
@@ -227,11 +227,16 @@ __global__ void __launch_bounds__(kDualThreads, 6) k_dual(const DualArgs a) {
 
 }  // namespace
 
+// Rows of 2^31 - 1 blocks; lanes of the last one past the cells repeat the last cell.
+dim3 dual_grid(int64_t cells) {
+    const int64_t blocks = (cells + kDualThreads - 1) / kDualThreads, x = blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL;
+    return dim3((unsigned)x, (unsigned)((blocks + x - 1) / x));
+}
+
 cudaError_t launch_dual(const DualArgs& a, cudaStream_t s) {
     const int64_t total = (int64_t)a.M * a.E * a.K * a.R;
-    const int64_t blocks = (total + kDualThreads - 1) / kDualThreads;
-    if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    k_dual<<<(unsigned)blocks, kDualThreads, 0, s>>>(a);
+    if (total <= 0) return cudaErrorInvalidConfiguration;
+    k_dual<<<dual_grid(total), kDualThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -168,8 +168,8 @@ struct DualArgs {
     double* gamma;              // optional [M][E][K][R]
     unsigned long long* keys;   // [M][E][K], initialised to all ones
 };
+dim3 dual_grid(int64_t cells);
 cudaError_t launch_dual(const DualArgs& a, cudaStream_t s);
-
 
 #ifdef __CUDACC__
 // Every FP64-pipe instruction -- add, multiply, FMA, compare, minimum and each conversion from or to

@@ -40,3 +40,26 @@ def test_the_largest_grid_of_one_regime_fits_a_launch(tmp_path):
     fills its warps best, take more rows where 4096 classes x 2^20 reservations need it."""
     out = run_program(tmp_path, PROGRAM)
     assert out.returncode == 0, out.stdout
+
+
+DUAL = r"""
+#include <cstdio>
+#include "kvdro_internal.cuh"
+int main() {
+    const long long most = 0x7fffffffLL * 256;  // cells that the entry point takes
+    for (long long cells : {1LL, 127LL, 128LL, 129LL, most / 2 - 127, most / 2, most / 2 + 1, most - 128, most}) {
+        const dim3 g = kvdro::dual_grid(cells);
+        if (g.x > 0x7fffffffu || g.y > 65535 || g.z != 1 || (long long)g.x * g.y * 128 < cells) {
+            std::printf("%lld cells: %u x %u blocks\n", cells, g.x, g.y);
+            return 1;
+        }
+    }
+    return 0;
+}
+"""
+
+
+def test_the_dual_launch_covers_every_cell_that_the_entry_point_takes(tmp_path):
+    """Up to 2^31 - 1 times 256 cells, in blocks of 128."""
+    out = run_program(tmp_path, DUAL)
+    assert out.returncode == 0, out.stdout
