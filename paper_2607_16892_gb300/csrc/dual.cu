@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kDualThreads, 6) k_dual(const DualArgs a) {
                         else if (p != up) out = false;
                         if (out) {
                             x = up ? hb - step : lb + step;
-                            step = min(step << 3, 1ll << 60);
+                            step = min(step, 1ll << 57) << 3;  // at most 2^60
                             out = x > lb && x < hb;
                         }
                         if (!out) x = lb + (hb - lb) / 2;
