@@ -4,7 +4,8 @@ The envelope evaluator of the oracle (the same finite sum regrouped by affine pi
 exact cumulative counts, pinned in test_oracle_pins.py) gives every cell of the full grids;
 the direct per-term evaluator checks randomly drawn cells of the same runs.  The regime
 sweep (all 1024 regimes) runs exactly as bench.py times it (FP32, the same outputs); the
-8-class workload runs in FP32, exact and native FP64 over its full grid.
+8-class workload runs in FP32, exact and FP64 over its full grid, all by the exact kernel, and at every 16th
+r by native FP64.
 """
 
 import os
@@ -105,12 +106,25 @@ def test_heavy_tail_k16_n1e6_exact_full_grid():
 
 
 def test_lognormal_k8_n1e5_fp64_full_grid():
-    """FP64 requests on every cell of the 8-class grid (4096 r x 128 lam)."""
+    """FP64 requests on every cell of the 8-class grid (4096 r x 128 lam), which the exact kernel serves."""
     w = lognormal_workload_k8_n1e5()
     gpu = run(w, kvdro.KVDRO_FP64)
     rep = compare_full(w, gpu, oracle_from_S(w, O.envelope_grid(w)), "fp64")
     rep["direct"] = direct_cells(w, gpu["S"], 4096, RTOL["fp64"], 2)
     rep["direct_at_r_star"] = chosen_r_cells(w, gpu["S"], gpu["r_idx"], RTOL["fp64"], 12)
+    print(rep)
+
+
+def test_lognormal_k8_n1e5_native_fp64():
+    """Native FP64 arithmetic per term, which serves supports above 2^22: the 8 classes x 100,000 samples with
+    the support declared 2^22 + 1, every 16th r, every lam."""
+    w = lognormal_workload_k8_n1e5()
+    w.L = np.full(w.K, (1 << 22) + 1, np.int32)
+    w.r = w.r[::16].copy()
+    gpu = run(w, kvdro.KVDRO_FP64)
+    rep = compare_full(w, gpu, oracle_from_S(w, O.envelope_grid(w)), "fp64")
+    rep["direct"] = direct_cells(w, gpu["S"], 4096, RTOL["fp64"], 4)
+    rep["direct_at_r_star"] = chosen_r_cells(w, gpu["S"], gpu["r_idx"], RTOL["fp64"], 14)
     print(rep)
 
 

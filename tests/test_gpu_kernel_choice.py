@@ -78,13 +78,13 @@ def test_envelope_magnitudes(scale):
     compare_full(w, env, O.solve(w), "fp64")
 
 
-@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 127, 128, 129, 4095, 4096, 4097, 8193, 24577])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 127, 128, 129, 4095, 4096, 4097, 8191, 8192, 8193, 24577])
 @pytest.mark.parametrize("L,nl", [(1, 3), (300, 9), (1 << 19, 1), ((1 << 21) + 1, 9), (1 << 22, 1), (1 << 22, 9)])
 def test_exact_quads(n, L, nl):
-    """Quads of sorted samples (a class's last one starting with zeros, 4096 samples to a chunk) as integers
+    """Quads of sorted samples (a class's last one starting with zeros, 8192 samples to a chunk) as integers
     up to 2^24 in float bit patterns: the sums of the exact and the envelope mode are the same integers,
     so every output is the same bit for bit.  Samples at 0 and at the top of the support, against
-    reservations at both ends, make a lane's sums as large as they get between folds (7 loads at 2^22)."""
+    reservations at both ends, make a lane's sums as large as they get between folds (6 loads at 2^22)."""
     rng = np.random.default_rng(n)
     x = rng.integers(0, L + 1, n)
     x[: n // 2] = L
@@ -227,3 +227,13 @@ def test_rows_after_a_wait_that_runs_out(mode, L, monkeypatch):
         got = r_idx.cpu().numpy()[0]
         assert np.all(got[:, 0] == -1)
         assert np.array_equal(got[:, 1], ref["r_idx"][0, :, 1] if skip else [-1, -1])
+
+
+@pytest.mark.parametrize("sizes", [(4095, 4097), (8193,), (8191, 12289), (3, 3 * 4096 + 4093, 5 * 4096 + 2)])
+def test_native_fp64_on_quads_over_several_chunks(sizes):
+    """Costs past the exact kernel's bound run native FP64 on staged quads: samples taken back from them in
+    every chunk of a ring of two, class sizes on either side of a chunk and of a quad."""
+    rng = np.random.default_rng(sum(sizes))
+    w = make([rng.integers(0, 901, n) for n in sizes], 900, [0, 5, 450, 899, 900], 1e296 * np.logspace(-3, 1, 21), [0.0, 3.0, 50.0],
+             [1e296, 1e295], [3e295, 1e296])
+    compare_full(w, run(w, kvdro.KVDRO_FP64), O.solve(w), "fp64")

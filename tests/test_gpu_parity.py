@@ -116,8 +116,8 @@ def test_host_buffers_match_device_buffers(prec):
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "exact", "envelope"])
 def test_host_outputs_copied_in_regime_blocks_match_device_outputs(prec):
     """With many regimes, host outputs come back in blocks of regimes on the context's copy
-    stream while later blocks evaluate: 37 regimes make blocks of 3 with a ragged last one, and
-    150 lam values (100 in FP64) make the exact kernel run two lam blocks per regime block."""
+    stream while later blocks evaluate: 37 regimes make blocks of 3 with a ragged last one; 150 lam
+    values (100 in FP64), so that the exact kernel's warps hold cells of several rows."""
     w = random_case(23, K=2, N=(2500, 90), L=(900, 900), R=13, n_lam=100 if prec == "fp64" else 150, n_eps=3, M=37,
                     lam_range=(1e-3, 50.0), eps_max=200.0)
     mode = kvdro.KVDRO_ENVELOPE if prec == "envelope" else P[prec]
@@ -235,9 +235,10 @@ def test_a_wait_that_runs_out_reports_etimeout_and_the_device_stays_usable(monke
     """Failure detection without a fault: a test hook leaves one chunk's copy unissued, so nothing
     completes that barrier; every CTA's bounded wait (about 1 ms under the hook) gives up, the CTA
     drains the copies it did issue and sets the error bit, and the call reports KVDRO_ETIMEOUT.
-    Afterwards the same CUDA context evaluates correctly."""
+    Afterwards the same CUDA context evaluates correctly.  Both precisions run the exact kernel here; the
+    waits of the FP32- and FP64-arithmetic kernels are in test_rows_after_a_wait_that_runs_out."""
     rng = np.random.default_rng(3)
-    w = make([rng.integers(0, 900, 20000)], 1000, [10, 200, 600], [0.5, 5.0], [0.0, 10.0], 10.0, 1.0)  # 4 staged chunks in the exact kernel, 5 in the FP64 one
+    w = make([rng.integers(0, 900, 20000)], 1000, [10, 200, 600], [0.5, 5.0], [0.0, 10.0], 10.0, 1.0)  # 3 staged chunks
     monkeypatch.setenv("KVDRO_TEST_SKIP_CHUNK", "2")
     ctx = kvdro.kvdro_create(0)
     monkeypatch.delenv("KVDRO_TEST_SKIP_CHUNK")
@@ -297,8 +298,8 @@ def test_the_wait_hook_of_one_context_leaves_another_on_the_same_device_unaffect
 
 @pytest.mark.parametrize("prec", ["exact", "fp32"])
 def test_lam_blocks_keep_the_lowest_index_on_ties_across_a_block_boundary(prec):
-    """More than 128 lam values run as consecutive launches over blocks of 128.  Here the second
-    block repeats the first block's last value (lam = 3) 128 times.  Equal lam values give
+    """256 lam values, one row to a pass of the exact kernel: the second half repeats the first half's
+    last value (lam = 3) 128 times, in warps and lanes of their own.  Equal lam values give
     bit-identical objectives, so a minimum reached at lam = 3 must report index 127 (at eps = 0
     with c_p = 10 most cells reach it: S does not increase in lam) and no index above 127 may
     appear; the rest matches the oracle."""
@@ -316,9 +317,9 @@ def test_lam_blocks_keep_the_lowest_index_on_ties_across_a_block_boundary(prec):
 @pytest.mark.parametrize("prec", ["exact", "fp32"])
 @pytest.mark.parametrize("nl,L", [(1, 3000), (2, 3000), (129, 3000), (130, 3000), (1, (1 << 20) + 5), (129, (1 << 20) + 5)])
 def test_one_or_two_lam_values_and_blocks_ending_in_them(prec, nl, L):
-    """A grid of one or two lam values -- or a block of 128 followed by one or two -- takes the
-    8 r x 2 lam tiles (all-integer); a ragged r count (not a multiple of the CTA's 128 rows) and a
-    support above 2^19 included."""
+    """A grid of one or two lam values puts 128 or 256 rows in a pass of the exact kernel, one of 129 or 130
+    a single row or, over several passes, a few; a ragged r count (no multiple of the CTA's rows) and
+    a support above 2^20 included."""
     rng = np.random.default_rng(nl + L % 97)
     w = make([np.concatenate([[0, L], rng.integers(0, L + 1, 4100)]), rng.integers(0, L + 1, 333)], L,
              np.unique(np.linspace(0, L, 203).round()).astype(np.int32), np.logspace(-3, 2, nl),
@@ -366,7 +367,7 @@ def test_multipliers_costs_and_radii_far_above_fp32_range(prec):
 def test_fp32_results_are_the_exact_results_rounded(nl):
     """With every support at most 2^22 an FP32 request runs the exact kernel and rounds its
     results: S, cost and the minimum cost are the FP64 exact-mode values cast to FP32, bit for bit
-    (lam counts on both sides of the 128 / 256 tile variants)."""
+    (lam counts that fill the exact kernel's warps and that do not)."""
     w = random_case(21, K=3, N=(3000, 517, 40), L=(4000, 4000, 4000), R=29, n_lam=nl, n_eps=3, M=2,
                     lam_range=(1e-3, 300.0), eps_max=500.0)
     f32, ex = run(w, P["fp32"]), run(w, P["exact"])
@@ -377,8 +378,8 @@ def test_fp32_results_are_the_exact_results_rounded(nl):
 
 @pytest.mark.parametrize("prec", ["exact", "fp32"])
 def test_exact_kernel_at_its_largest_support(prec):
-    """L = 2^22, the largest support the exact kernel takes: its FP32 sums fold after every
-    load; samples at 0 and at L, cells with every sample active (lam = 0) and none active."""
+    """L = 2^22, the largest support the exact kernel takes: its integer sums fold after six
+    loads; samples at 0 and at L, cells with every sample active (lam = 0) and none active."""
     L = 1 << 22
     rng = np.random.default_rng(12)
     w = make([np.concatenate([[0, 0, L, L], rng.integers(0, L + 1, 2500)]), rng.integers(L - 3000, L + 1, 700)], L,
@@ -389,9 +390,8 @@ def test_exact_kernel_at_its_largest_support(prec):
 
 @pytest.mark.parametrize("L,nl", [(1 << 19, 40), ((1 << 19) + 1, 40), ((1 << 20) + 3, 200)])
 def test_exact_variants_either_side_of_the_integer_split(L, nl):
-    """Supports up to 2^19 run half of every row's columns on packed FP32 adds; above, every
-    column on integer absolute differences (narrow tiles, and wide ones for 200 lam values).
-    Both forms are exact."""
+    """Supports on either side of 2^19 and above 2^20, with lam counts that fill the exact kernel's warps and
+    that do not: exact integer sums in float bit patterns at every support up to 2^22."""
     rng = np.random.default_rng(41)
     w = make([np.concatenate([[0, L], rng.integers(0, L + 1, 3000)]), rng.integers(L - 9000, L + 1, 500)], L,
              [0, 1, L // 3, L - 1, L], np.logspace(-3, 2, nl), [0.0, 700.0], [10.0, 0.5], [1.0, 3.0])
@@ -400,7 +400,7 @@ def test_exact_variants_either_side_of_the_integer_split(L, nl):
 
 
 def test_integer_variant_with_input_lengths_and_ragged_classes():
-    """The all-integer variant (support above 2^19) with per-class input lengths, a class of 1 and
+    """The exact kernel at a support above 2^20 with per-class input lengths, a class of 1 and
     one of 67 samples (padding in its only load), and a support point at each end."""
     L = (1 << 20) + 17
     rng = np.random.default_rng(43)
@@ -412,8 +412,8 @@ def test_integer_variant_with_input_lengths_and_ragged_classes():
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_staging_offsets_differ_by_class(prec):
-    """A class staged as x + 2^23 (support at most 2^22) beside one staged as x (support above
-    2^22) in one request: the FP32-arithmetic and FP64 kernels remove each class's own offset."""
+    """A class with a support of at most 2^22 beside one above it in one request: both are staged as (x, x)
+    pairs, and the FP32-arithmetic and FP64 kernels serve them."""
     L_small, L_big = 3000, (1 << 22) + 100
     rng = np.random.default_rng(31)
     w = make([np.concatenate([[0, L_small], rng.integers(0, L_small + 1, 2000)]),
@@ -551,15 +551,15 @@ def test_random_large_shapes_every_mode(seed):
         compare_full(w, run(w, P[mode]), ora, "fp32" if mode == "fp32" else "fp64")
 
 
-@pytest.mark.parametrize("L", [65534, 32767, 16382, 131070])
+@pytest.mark.parametrize("L", [65534, 32767, 16382, 131070, (1 << 18) - 1, (1 << 21) - 1, (1 << 22) - 1])
 def test_exact_sums_stay_exact_at_the_fold_bound(L):
-    """The exact kernel folds its packed FP32 sums after fe loads, fe the largest power of two with
-    2 fe (L + 1) <= 2^24; each L here sits just below such a bound, so a lane's sums reach nearly
-    2^24 by the fold.  Samples crowd the top of the support and the reservations its bottom (every
-    |x - c| near L, odd and even), and the classes end in a large ragged chunk after one, two or
-    three full ones, so the loads since the last fold do not restart at a chunk boundary.  One load
-    past the bound rounds the sums: the exact mode must still meet the envelope mode (same integer
-    sums, O(1) per cell) to 1e-12 and the oracle to 1e-9."""
+    """The exact kernel folds its 32-bit integer sums after fe loads of four samples a lane, fe the largest even
+    number with 32 lanes x 4 fe L < 2^32.  A power of two just above L brings the two sides together: at
+    2^18 - 1, 2^21 - 1 and 2^22 - 1 (fe = 128, 16, 8) the classes here hold several folds, and two more loads
+    before one would wrap; the smaller supports fold at the end of the class alone.  Samples crowd the top of
+    the support and the reservations its bottom (every |x - c| near L, odd and even), and the classes end in
+    ragged chunks, so the loads since the last fold do not restart at a chunk boundary.  The exact mode must
+    meet the envelope mode (same integer sums, O(1) per cell) to 1e-12 and the oracle to 1e-9."""
     rng = np.random.default_rng(L)
     sizes = (12144, 3 * 6144 + 6100, 2 * 6144 + 6100, 4 * 4096 + 4000)
     cls = [L - rng.integers(0, 1 + L // 64, n) for n in sizes]
@@ -574,13 +574,14 @@ def test_exact_sums_stay_exact_at_the_fold_bound(L):
 
 @pytest.mark.parametrize("L", [900, 1 << 20, (1 << 22) + 3])
 def test_class_sizes_at_chunk_and_padding_boundaries(L):
-    """Classes whose sizes sit on and around the staged chunk sizes (6144 samples in the exact
-    kernels, 4096 in the FP32 and FP64 ones) and the 128-sample padding unit, one sample each side:
-    the fast full-chunk path, the ragged last chunk and the padded tail all meet the oracle.  The
-    supports select the mixed exact kernel (900), the all-integer one (2^20) and, above 2^22, the
-    FP32-arithmetic kernel for FP32 requests."""
+    """Classes whose sizes sit on and around the staged chunk sizes (8192 samples in the exact
+    kernel, 4096 in the FP32- and FP64-arithmetic ones), rings of two and three of them, and the 128-sample
+    padding unit, one sample each side: full chunks, the ragged last chunk and the padded tail
+    all meet the oracle.  The supports select the exact kernel (900 and 2^20) and, above 2^22, the
+    FP32- and FP64-arithmetic ones."""
     rng = np.random.default_rng(L)
-    sizes = (1, 127, 128, 129, 4095, 4096, 4097, 6143, 6144, 6145, 12288, 12289)
+    sizes = (1, 127, 128, 129, 4095, 4096, 4097, 6143, 6144, 6145, 8191, 8192, 8193, 12288, 12289, 16383, 16384, 16385, 24575,
+             24576, 24577)
     cls = [np.minimum(L, rng.integers(0, min(L, 5000) + 1, n)) for n in sizes]
     w = make(cls, L, np.unique(np.linspace(0, L, 11).astype(np.int64)), [0.02, 0.5, 1.0, 4.0, 30.0], [0.0, 7.0, 90.0],
              [6.0, 1.0], [1.0, 3.0], name=f"sizes{L}")

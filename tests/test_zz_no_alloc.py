@@ -4,9 +4,8 @@ The no-allocation entry point serves callers that cannot allocate device memory 
 need a reservation answer (for example a serving engine whose free memory all belongs to its
 KV-cache pool).  It must give the same results as the context-based entry point, also when
 the previous call left other data in its shared static scratch, and the oracle's results
-within the FP32 tolerance, for every kernel it can choose (the exact kernel with packed and
-integer columns up to a support of 2^19, the all-integer one up to 2^22, the FP32-arithmetic
-one above).  This file is collected last so that a stop-at-first-failure run has already run
+within the FP32 tolerance, for every kernel it can choose (the exact kernel up to a support of 2^22, the
+FP32-arithmetic one above).  This file is collected last so that a stop-at-first-failure run has already run
 every other test.
 """
 
@@ -112,8 +111,7 @@ def test_noalloc_matches_the_oracle():
 
 @pytest.mark.parametrize("L,K", [((1 << 20) + 3, 2), ((1 << 22) + 4096, 1)])
 def test_noalloc_large_supports_match_the_oracle(L, K):
-    """A support in (2^19, 2^22] takes the all-integer exact kernel; one above 2^22 the
-    FP32-arithmetic kernel.  Both through the static scratch, against the oracle."""
+    """A support up to 2^22 takes the exact kernel; one above 2^22 the FP32-arithmetic kernel.  Both through the static scratch, against the oracle."""
     w = _classes_on(L, K, 44 + K)
     compare_full(w, _noalloc(w), O.solve(w), "fp32")
 
@@ -123,7 +121,7 @@ def test_noalloc_reports_a_wait_that_runs_out(monkeypatch):
     never issued; the call returns KVDRO_ETIMEOUT (its outputs are incomplete) instead of
     KVDRO_OK, and the next call without the hook is correct."""
     rng = np.random.default_rng(5)
-    cls = rng.integers(0, 900, 20000).astype(np.int32)  # four staged chunks
+    cls = rng.integers(0, 900, 20000).astype(np.int32)  # three staged chunks
     w = Workload(name="wait", samples=cls, offsets=np.array([0, cls.size], np.int64), L=np.array([1000], np.int32),
                  L_in=np.zeros(1, np.int32), r=np.array([10, 200, 600], np.int32), lam=np.array([0.5, 5.0]),
                  eps=np.array([0.0, 10.0]), cp=np.array([10.0]), cw=np.array([1.0]), fractiles=np.array([0.5]))
