@@ -51,7 +51,8 @@ typedef enum {
     KVDRO_ENOMEM = -2,   /* a device or pinned-host allocation failed */
     KVDRO_ECUDA = -3,    /* a CUDA call failed (message in kvdro_last_error) */
     KVDRO_ESTATE = -4,   /* call out of order, e.g. eval before samples are loaded */
-    KVDRO_ETIMEOUT = -5  /* a kernel gave up a bounded wait and reported it */
+    KVDRO_ETIMEOUT = -5  /* a kernel gave up a bounded wait and reported it; the outputs are then
+                            incomplete (r_idx is -1 where no r was evaluated) */
 } kvdro_status;
 
 typedef enum {
@@ -159,8 +160,8 @@ int kvdro_sorted_samples(const kvdro_ctx* ctx, int32_t* out, void* stream);
 /*
  * Device time, in milliseconds, of the grid-kernel launches of the last kvdro_eval_grid() or
  * kvdro_eval_dual() call on this context, measured with CUDA events recorded on that call's
- * stream immediately before and after them (the argmin finalisation and the output copies are
- * outside).  Blocks until the second event has completed.  KVDRO_ESTATE if nothing has been
+ * stream immediately before and after them (the output copies are outside, and so is the argmin
+ * finalisation, but for small grids, whose last CTAs do it).  Blocks until the second event has completed.  KVDRO_ESTATE if nothing has been
  * evaluated yet.
  */
 int kvdro_last_grid_ms(kvdro_ctx* ctx, float* ms);

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kDualThreads, 6) k_dual(const DualArgs a) {
     const unsigned long long key = ((unsigned long long)(above ? gb : 0ll) & ~0xFFFFFull) | (unsigned long long)ri;
     // one atomic per warp where its lanes hold one row of r values (a lane past the end repeats the last cell)
     if (__all_sync(0xffffffffu, row == __shfl_sync(0xffffffffu, row, 0))) {
-        const unsigned long long low = group_min(key, 32);
+        const unsigned long long low = warp_min(key);
         if ((threadIdx.x & 31) == 0) atomicMin(a.keys + row, low);
     } else {
         atomicMin(a.keys + row, key);

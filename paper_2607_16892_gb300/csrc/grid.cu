@@ -468,7 +468,7 @@ __device__ __forceinline__ void lam_min_epilogue(const GridArgs& a, const LamRow
         // the warp's minimum over each radius it holds, e0 (its first lane's) upwards
         const int e0 = __shfl_sync(0xffffffffu, e, 0), e1 = __reduce_max_sync(0xffffffffu, e);
         for (int ei = e0; ei <= e1; ei++) {
-            const u64 low = group_min(e == ei ? key : ~0ull, 32);
+            const u64 low = warp_min(e == ei ? key : ~0ull);
             if (lane == 0 && low != ~0ull) atomicMin(a.keys + ((size_t)m * a.E + ei) * a.K + k, low);
         }
     }
@@ -545,8 +545,7 @@ __global__ void __launch_bounds__(C::MAXT, C::MINB) k_grid(const GridArgs a) {
     if constexpr (P == Prec::F32) {
         // Each row's excess is taken about its reservation: kappa (x - eta) + W(eta) (excess_at_eta).
         // x - eta comes from the staged samples in one packed add per row and load (both samples of
-        // the load): the staged value carries the class's offset, and offset + eta is an integer
-        // below 2^24, so the add is exact.
+        // the load); both are integers up to 2^24, so the add is exact.
         u64 noff[TR];
 #pragma unroll
         for (int i = 0; i < TR; i++) {
@@ -1056,8 +1055,9 @@ __global__ void __launch_bounds__(32 * kExactWarps, kExactBlocks) k_exact(const 
 // A warp takes up to kEnvPasses passes of 32 / W rows, W lanes along lam each (W: NL rounded up to a power of
 // two, at most 32), so small lam grids fill the warp with rows.  More passes share the CTA's start and end
 // (128 regimes x 8 classes x 2048 r x 64 lam x 16 eps: 4 passes 3.33 ms, 3 3.58, 2 3.70); fewer where the
-// grid has too few rows to fill the SMs several times over, or rows so wide that two CTAs fill an SM's
-// shared memory (more than 64 lam).
+// grid leaves an SM fewer than eight CTAs, or rows so wide that two CTAs fill an SM's shared memory (more
+// than 64 lam).  With 1, 4, 8, 16 and 64 CTAs in eight's place: 8 classes x 2048 r x 64 lam x 16 eps x 2 regimes 90.1, 90.0,
+// 89.4, 96.6 and 96.7 us, 4 regimes 141.9, 141.9, 142.0, 145.0 and 168.2; one regime x 8 eps 57.0, 56.7, 59.6, 59.5 and 59.4.
 constexpr int kEnvThreads = 256;
 constexpr int kEnvPasses = 4;
 
@@ -1077,7 +1077,7 @@ struct EnvRow {
     RowOffset off;
     double pv, ev, pu, eu;  // c_w eta N and c_p (L - eta) N: rounded product and its error
     float cp_le, cw_eta;
-    int eta, pad;
+    int eta;
 };
 struct EnvSmem {
     size_t kap, eps, S, row, muf, kapf, lamf, Sf, total;
@@ -1236,7 +1236,6 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
     sh.RG = sh.LT >= kWarpsTarget ? 1 : kWarpsTarget / sh.LT;
     sh.threads = 32 * sh.LT * sh.RG;
     sh.rows = sh.RG * C::TR;
-    sh.stages = C::STAGES;
     sh.r_blocks = (R + sh.rows - 1) / sh.rows;
     sh.smem = smem_layout(sh.RG, C::TR, sh.LT * C::TL, E, C::CHUNK * C::BYTES, C::STAGES).total;
     return sh;
@@ -1247,7 +1246,11 @@ GridShape shape_for(int variant, int32_t R, int32_t NL, int32_t E) {
 // The choice maximises cells filled x waves filled.  A warp left out saves nothing while its scheduler still
 // holds as many as the others (13 to 16 warps take the same time), and fewer per scheduler run at a lower
 // rate: 5 classes x 1001 r x 200 lam x 3 regimes 2.27 ms in one pass of 13 warps, 1.90 in four passes of 16
-// (2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).
+// (2.09 in 2 r x 8 lam tiles with a second launch past 128 lam).  At 5 classes x 40,000 samples x 1001 r x 3 regimes and
+// 13 lam counts from 1 to 250 the choice takes at most 3 % longer than the best of the four (33 lam: 769 us in one
+// pass, 748 in two; 129: 2791 in three, 3145 in one).  In grids under two waves it can miss: one regime x 200 r, one
+// pass against the choice, 129 lam 252 and 313 us, 150 lam 268 and 337 (366 in blocks of 128 lam, the form before);
+// 72 lam 128 in two passes and 165.
 GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int32_t K, int64_t classes, int sms) {
     constexpr int kCells = kExactWarps * kExactV;
     GridShape best, sh;
@@ -1266,10 +1269,9 @@ GridShape exact_shape(int32_t R, int32_t NL, int32_t E, int32_t K, int64_t class
         if ((int64_t)K * sh.r_blocks > 0x7fffffffLL) continue;  // a launch holds one regime's CTAs (four passes always do)
         // 96 KB of ring: three chunks of 8192 samples (6144 measured 1 % slower, 4096 3 %); smaller chunks where
         // the cells need the room
-        sh.stages = kExactStages;
         sh.chunk = kExactChunk;
         do {
-            sh.smem = exact_smem(rows, NL, E, warps * sh.passes, sh.stages * sh.chunk * 4).total;
+            sh.smem = exact_smem(rows, NL, E, warps * sh.passes, kExactStages * sh.chunk * 4).total;
         } while (sh.smem > kExactSmem && (sh.chunk -= 1024) > 0);
         const double slots = (double)kExactBlocks * sms, ctas = (double)classes * sh.r_blocks, waves = ctas / slots;
         const int held = (warps + 3) / 4 * 4;  // warps that the fullest of the four schedulers accounts for
@@ -1289,7 +1291,7 @@ GridShape grid_shape(Prec p, int32_t R, int32_t NL, int32_t E, int32_t K, int32_
     if (p == Prec::ENVELOPE) {
         GridShape sh;
         sh.variant = 4;
-        sh.LT = sh.RG = sh.stages = 1;
+        sh.LT = sh.RG = 1;
         sh.threads = kEnvThreads;
         sh.rows = env_rows(NL, R, classes, sms);
         sh.r_blocks = (R + sh.rows - 1) / sh.rows;
@@ -1340,7 +1342,6 @@ cudaError_t launch_grid(Prec p, const GridShape& sh, GridArgs a, cudaStream_t s)
     a.LT = sh.LT;
     a.RG = sh.RG;
     a.rows = sh.rows;
-    a.stages = sh.stages;
     a.passes = sh.passes;
     a.chunk = sh.chunk;
     a.r_blocks = sh.r_blocks;

@@ -95,7 +95,6 @@ struct GridArgs {
     int32_t LT;                 // lam tiles per CTA (FP32 and FP64 kernels)
     int32_t RG;                 // r groups per CTA (FP32 and FP64 kernels)
     int32_t rows;               // r values per CTA
-    int32_t stages;             // ring depth
     int32_t passes;             // over the samples (exact kernel)
     int32_t chunk;              // samples per staged chunk (exact kernel)
     int32_t r_blocks;           // CTAs per (m, k)
@@ -119,11 +118,11 @@ struct GridArgs {
 
 // grid.cu
 // Launch shape of the grid kernel for one (precision, grid) problem: which compiled variant, its
-// r values, warps and ring depth per CTA, CTAs per (regime, class), dynamic shared memory.
+// r values and warps per CTA, CTAs per (regime, class), dynamic shared memory.
 struct GridShape {
     int variant;       // index of the compiled kernel instantiation
     int LT, RG;        // lam tiles and r groups per CTA (FP32 and FP64 kernels: LT * RG warps)
-    int rows, stages;  // r values per CTA, ring depth
+    int rows;          // r values per CTA
     int passes = 1;    // over the samples, and samples per staged chunk (exact kernel)
     int chunk = 0;
     int threads;
@@ -211,9 +210,9 @@ __device__ __forceinline__ long long order_key(double v) {
     return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-// The smaller key over groups of G lanes (a power of two), in every lane.
-__device__ __forceinline__ unsigned long long group_min(unsigned long long key, int G) {
-    for (int o = 1; o < G; o <<= 1) {
+// The smallest key of the warp, in every lane.
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long key) {
+    for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
         key = other < key ? other : key;
     }
