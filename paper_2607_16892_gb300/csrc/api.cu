@@ -691,13 +691,11 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     fa.r_idx = static_cast<int32_t*>(outs[3].dev);
     fa.min_cost = outs[4].dev;
     fa.fhat = static_cast<double*>(outs[5].dev);
-    // In grids whose CTAs are all resident, two per SM, the last CTA of each (regime, class) finalises its rows: a
-    // launch saved.  In larger ones the barriers and counts of every CTA cost more than the launch.  4 classes
-    // x 1000 samples x 64 lam x 8 eps, last CTA against launch: exact kernel 64 CTAs 22.7 and 25.2 us, 256 27.1 and
-    // 27.6, 512 39.6 and 38.9, 1024 61.6 and 56.7, 2048 100.5 and 95.6; envelope 64 25.4 and 26.2, 256 39.2 and
-    // 39.1, 512 59.4 and 55.9.
+    // In small grids the last CTA of each (regime, class) finalises its rows: the launch saved is 4 us of the
+    // smallest call's 34; in large ones its barriers and counts cost more (131,072 CTAs of the envelope 3.73
+    // -> 3.88 ms), so they take the launch.
     const bool finalize = fa.r_idx || fa.min_cost || fa.fhat;
-    const bool fused = (int64_t)M * ctx->K * shape.r_blocks <= 2 * (int64_t)ctx->sms;
+    const bool fused = (int64_t)M * ctx->K * shape.r_blocks <= 2048;
     a.done = finalize && fused ? reinterpret_cast<uint32_t*>(a.keys + rows) : nullptr;
     int64_t m_step = std::max<int64_t>(1, 0x7fffffffLL / ((int64_t)ctx->K * shape.r_blocks));
     // Host outputs laid out regime-major (S, cost, lam index) go back in blocks of regimes on the
