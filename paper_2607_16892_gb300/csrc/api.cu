@@ -691,9 +691,13 @@ int kvdro_eval_grid(kvdro_ctx* ctx, int precision, int32_t R, const int32_t* r, 
     fa.r_idx = static_cast<int32_t*>(outs[3].dev);
     fa.min_cost = outs[4].dev;
     fa.fhat = static_cast<double*>(outs[5].dev);
-    // In small grids the last CTA of each (regime, class) finalises its rows: the launch saved is 4 us of the
-    // smallest call's 34; in large ones its barriers and counts cost more (131,072 CTAs of the envelope 3.73
-    // -> 3.88 ms), so they take the launch.
+    // In grids of up to 2048 CTAs the last CTA of each (regime, class) finalises its rows: a launch saved, 1 to 2 us
+    // while every CTA is resident.  Past that its barriers and count add 2 us to every wave, which CTAs of many
+    // samples hide and short ones do not.  4 classes x 2 regimes, last CTA against launch: exact kernel, 300
+    // samples 256 CTAs 24.6 and 25.6 us, 304 35.2 and 35.6, 400 32.8 and 31.9, 800 45.5 and 43.4, 1600 75.6 and 68.6; 20,000
+    // samples 256 75.9 and 76.3, 800 185.1 and 185.6, 1600 324.0 and 323.6; two classes x 101,336, 492 CTAs 283.9 and
+    // 285.1.  Envelope, four CTAs per SM, 304 23.0 and 24.0, 600 27.9 and 28.9, 800 37.0 and 36.6, 1600 49.9 and 47.5;
+    // 131,072 3.88 and 3.73 ms.
     const bool finalize = fa.r_idx || fa.min_cost || fa.fhat;
     const bool fused = (int64_t)M * ctx->K * shape.r_blocks <= 2048;
     a.done = finalize && fused ? reinterpret_cast<uint32_t*>(a.keys + rows) : nullptr;

@@ -237,3 +237,16 @@ def test_native_fp64_on_quads_over_several_chunks(sizes):
     w = make([rng.integers(0, 901, n) for n in sizes], 900, [0, 5, 450, 899, 900], 1e296 * np.logspace(-3, 1, 21), [0.0, 3.0, 50.0],
              [1e296, 1e295], [3e295, 1e296])
     compare_full(w, run(w, kvdro.KVDRO_FP64), O.solve(w), "fp64")
+
+
+@pytest.mark.parametrize("blocks", [255, 256, 257, 514])
+def test_rows_finalised_by_the_last_cta_and_by_a_launch(blocks):
+    """4 classes x 2 regimes x `blocks` CTAs of the exact kernel, up to 2048 of them finalised by the last CTA of
+    each (regime, class), above by a launch, against the envelope, half as many CTAs."""
+    rng = np.random.default_rng(blocks)
+    w = make([rng.integers(0, 3001, n) for n in (300, 77, 4, 1)], 3000, np.arange(4 * blocks), np.logspace(-3, 2, 64),
+             [0.0, 7.0, 90.0], [10.0, 4.0], [1.0, 1.0])
+    outputs = ("cost", "lam_idx", "r_idx", "min_cost", "fhat")
+    exact, env = run(w, kvdro.KVDRO_EXACT, outputs=outputs), run(w, kvdro.KVDRO_ENVELOPE, outputs=outputs)
+    for key, v in exact.items():
+        assert np.array_equal(v, env[key]), key
